@@ -102,9 +102,10 @@ typedef struct {
  * outcome's slice contiguously with modalities of equal dependency set sharing
  * one axis order; B is re-laid per action as forward, log, log-transposed and
  * column-normalised-transposed matrices; D as ln D.  The packed copies live in
- * device memory owned by the handle; the caller's A, B, D may be released once
- * the stream's work has completed.  Returns BI_OK and *out, or an error code
- * with *out = NULL.
+ * device memory owned by the handle.  The call waits for the packing on the
+ * stream (later calls choose their kernels by whether A has zeros), so the
+ * caller's A, B, D may be released when it returns.  Returns BI_OK and *out, or
+ * an error code with *out = NULL.
  */
 int bi_model_create(const bi_model_desc *desc, void *cuda_stream, bi_model_t **out);
 
@@ -119,8 +120,7 @@ int bi_model_create_arith(const bi_model_desc *desc, int arith, void *cuda_strea
  * lane's elements are not the floor ln 1e-16) plus those values; bi_vmp / bi_mmp read that form, so the
  * gather's HBM traffic shrinks with the share of zeros; the result is bit for bit that of the dense
  * form.  Made automatically by bi_model_create for per-agent register-tile models (G > 1, up to four
- * modalities) when it is under 60 % of the dense size; sizing it needs the non-zero counts on the
- * host, so creating such a handle synchronises the stream.  Both are 0 when the handle has no
+ * modalities) when it is under 60 % of the dense size.  Both are 0 when the handle has no
  * compressed form.
  */
 int bi_model_slice_bytes(const bi_model_t *model, int64_t *dense, int64_t *compressed);

@@ -9,6 +9,16 @@
 #include "bi_device.cuh"
 #include "bi_internal.h"
 
+// the block kernels' share of the packing layer (block.cu)
+void bi_block_choose_shape(bi_model *md);
+int bi_block_slice_elems(const bi_model *md, int gi);
+int bi_block_pack_member(const bi_model *md, int gi, const float *src, int m, const int64_t *sstride, int P, void *dst,
+                         cudaStream_t stream);
+void bi_block_build(bi_model *md, std::vector<unsigned char> &blob);
+void bi_block_bind(bi_model *md, unsigned char *dev);
+void bi_block_free(bi_model *md);
+int bi_block_exp_table(double *dst, cudaStream_t stream);
+
 namespace {
 
 #define BI_CUDA_TRY(expr)                      \
@@ -27,7 +37,7 @@ struct PackA {
   int32_t dim[BI_MAX_RANK];      // packed axis sizes
   int64_t sstride[BI_MAX_RANK];  // source stride of each packed axis
   int32_t npad;                  // padded size of the last packed axis (rank > 0)
-  uint32_t *wide;                // set to 1 when an entry exceeds 1 (see BiDev::status)
+  uint32_t *wide;                // [0] set when an entry exceeds 1, [1] when one is at or below 1e-16 (BiDev::status)
 };
 
 // ln(max(A, eps)) in float64, rounded once; outcome slices contiguous, axes in
@@ -44,6 +54,7 @@ __global__ void bi_pack_A_kernel(PackA p) {
     if (idx == 0) {
       const float v = p.src[go * p.P];
       if (v > 1.0f) atomicOr(p.wide, 1u);
+      if (v <= 1e-16f) p.wide[1] = 1u;
       out = (R)log(fmax((double)v, 1e-16));
     }
   } else {
@@ -57,6 +68,7 @@ __global__ void bi_pack_A_kernel(PackA p) {
       }
       const float v = p.src[s];
       if (v > 1.0f) atomicOr(p.wide, 1u);
+      if (v <= 1e-16f) p.wide[1] = 1u;
       out = (R)log(fmax((double)v, 1e-16));
     }
   }
@@ -65,7 +77,7 @@ __global__ void bi_pack_A_kernel(PackA p) {
 
 // B[g][s_next][s_prev][u] -> four [g][u][row][npad] matrices
 template <typename R>
-__global__ void bi_pack_B_kernel(const float *__restrict__ B, int G, int n, int npad, int U,
+__global__ void bi_pack_B_kernel(const float *__restrict__ B, int G, int n, int npad, int U, uint32_t *wide,
                                  R *Bf, R *logB, R *logBt, R *Bdag, R *BfT, R *BdagT) {
   int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int64_t total = (int64_t)G * U * n * npad;
@@ -81,6 +93,7 @@ __global__ void bi_pack_B_kernel(const float *__restrict__ B, int G, int n, int 
     const float *Bg = B + g * (int64_t)n * n * U;
     // forward: row = next state, column = previous state
     double b = (double)Bg[((int64_t)r * n + c) * U + u];
+    if (b > 1.0) atomicOr(wide, 1u);
     f = (R)b;
     lf = (R)log(fmax(b, 1e-16));
     // transposed: row = previous state, column = next state
@@ -204,7 +217,7 @@ __global__ void bi_pack_comb_kernel(PackComb p) {
 
 // transition tensors with B-dependencies: source [G][n][PB][U] -> [G][U][n][PB], plain and clamped log
 template <typename R>
-__global__ void bi_pack_Bfull_kernel(const float *__restrict__ B, int64_t total, int n, int64_t PB, int U, R *Bfull,
+__global__ void bi_pack_Bfull_kernel(const float *__restrict__ B, int64_t total, int n, int64_t PB, int U, uint32_t *wide, R *Bfull,
                                      R *logBfull) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= total) return;
@@ -215,16 +228,18 @@ __global__ void bi_pack_Bfull_kernel(const float *__restrict__ B, int64_t total,
   const int u = (int)(r % U);
   const int64_t g = r / U;
   const float v = B[((g * n + sn) * PB + par) * U + u];
+  if (v > 1.0f) atomicOr(wide, 1u);
   Bfull[e] = (R)v;
   logBfull[e] = (R)log(fmax((double)v, 1e-16));
 }
 
 template <typename R>
-__global__ void bi_pack_D_kernel(const float *__restrict__ D, int G, int n, int npad, R *logD) {
+__global__ void bi_pack_D_kernel(const float *__restrict__ D, int G, int n, int npad, uint32_t *wide, R *logD) {
   int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (int64_t)G * npad) return;
   int c = (int)(e % npad);
   int64_t g = e / npad;
+  if (c < n && D[g * n + c] > 1.0f) atomicOr(wide, 1u);
   logD[e] = c < n ? (R)log(fmax((double)D[g * n + c], 1e-16)) : (R)0;
 }
 
@@ -514,9 +529,14 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
     md->rank2_ok = !bdep_len && deep == 0;   // any number of groups over two factors: the pair window kernel's models
   }
 
+  md->batch_unrolled = 1;
+  for (int gi = 0; gi < h.ngroups; ++gi)
+    if (h.grp[gi].rank >= 2 && (h.grp[gi].rank > 4 || bi_batch_shape(h.grp[gi].rank, h.grp[gi].dim) < 0)) md->batch_unrolled = 0;
+  bi_block_choose_shape(md);
+
   // ---- allocate and pack
-  rc = dev_alloc(md, (void **)&h.status, 2 * sizeof(uint32_t));   // the flags, and the wide-range mark
-  if (rc == BI_OK && cudaMemsetAsync(h.status, 0, 2 * sizeof(uint32_t), stream) != cudaSuccess) rc = BI_ERR_CUDA;
+  rc = dev_alloc(md, (void **)&h.status, 3 * sizeof(uint32_t));   // the flags, and two marks on A
+  if (rc == BI_OK && cudaMemsetAsync(h.status, 0, 3 * sizeof(uint32_t), stream) != cudaSuccess) rc = BI_ERR_CUDA;
   for (int gi = 0; gi < h.ngroups && rc == BI_OK; ++gi) {
     BiGroup &g = h.grp[gi];
     for (int mi = g.mem_begin; mi < g.mem_end && rc == BI_OK; ++mi) {
@@ -571,6 +591,13 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
         bi_pack_A_kernel<double><<<(unsigned)((t.total + threads - 1) / threads), threads, 0, stream>>>(t);
         if (cudaGetLastError() != cudaSuccess) rc = BI_ERR_CUDA;
         mm.logA_T = tdst;
+      }
+      if (const int per = rc == BI_OK ? bi_block_slice_elems(md, gi) : 0) {
+        void *bdst = nullptr;
+        rc = dev_alloc(md, &bdst, (size_t)G * mm.m * per * esz);
+        if (rc != BI_OK) break;
+        mm.logA_blk = bdst;
+        rc = bi_block_pack_member(md, gi, desc->A[i], mm.m, p.sstride, p.P, bdst, stream);
       }
       if (rc == BI_OK && md->tile_sb > 0) {
         PackTile q;
@@ -758,11 +785,11 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
     const unsigned gb = (unsigned)((total + threads - 1) / threads);
     const unsigned gd = (unsigned)(((size_t)G * npad + threads - 1) / threads);
     if (arith == BI_ARITH_F64) {
-      bi_pack_Bfull_kernel<double><<<gb, threads, 0, stream>>>(desc->B[f], total, n, PB, U, (double *)bfull, (double *)lbfull);
-      bi_pack_D_kernel<double><<<gd, threads, 0, stream>>>(desc->D[f], G, n, npad, (double *)ld);
+      bi_pack_Bfull_kernel<double><<<gb, threads, 0, stream>>>(desc->B[f], total, n, PB, U, h.status + 1, (double *)bfull, (double *)lbfull);
+      bi_pack_D_kernel<double><<<gd, threads, 0, stream>>>(desc->D[f], G, n, npad, h.status + 1, (double *)ld);
     } else {
-      bi_pack_Bfull_kernel<float><<<gb, threads, 0, stream>>>(desc->B[f], total, n, PB, U, (float *)bfull, (float *)lbfull);
-      bi_pack_D_kernel<float><<<gd, threads, 0, stream>>>(desc->D[f], G, n, npad, (float *)ld);
+      bi_pack_Bfull_kernel<float><<<gb, threads, 0, stream>>>(desc->B[f], total, n, PB, U, h.status + 1, (float *)bfull, (float *)lbfull);
+      bi_pack_D_kernel<float><<<gd, threads, 0, stream>>>(desc->D[f], G, n, npad, h.status + 1, (float *)ld);
     }
     if (cudaGetLastError() != cudaSuccess) rc = BI_ERR_CUDA;
   }
@@ -785,17 +812,32 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
     unsigned gb = (unsigned)((count + threads - 1) / threads);
     unsigned gd = (unsigned)(((size_t)G * npad + threads - 1) / threads);
     if (arith == BI_ARITH_F64) {
-      bi_pack_B_kernel<double><<<gb, threads, 0, stream>>>(desc->B[f], G, n, npad, U, (double *)bf,
+      bi_pack_B_kernel<double><<<gb, threads, 0, stream>>>(desc->B[f], G, n, npad, U, h.status + 1, (double *)bf,
                                                            (double *)lb, (double *)lt, (double *)bd,
                                                            (double *)bft, (double *)bdt);
-      bi_pack_D_kernel<double><<<gd, threads, 0, stream>>>(desc->D[f], G, n, npad, (double *)ld);
+      bi_pack_D_kernel<double><<<gd, threads, 0, stream>>>(desc->D[f], G, n, npad, h.status + 1, (double *)ld);
     } else {
-      bi_pack_B_kernel<float><<<gb, threads, 0, stream>>>(desc->B[f], G, n, npad, U, (float *)bf,
+      bi_pack_B_kernel<float><<<gb, threads, 0, stream>>>(desc->B[f], G, n, npad, U, h.status + 1, (float *)bf,
                                                           (float *)lb, (float *)lt, (float *)bd,
                                                           (float *)bft, (float *)bdt);
-      bi_pack_D_kernel<float><<<gd, threads, 0, stream>>>(desc->D[f], G, n, npad, (float *)ld);
+      bi_pack_D_kernel<float><<<gd, threads, 0, stream>>>(desc->D[f], G, n, npad, h.status + 1, (float *)ld);
     }
     if (cudaGetLastError() != cudaSuccess) rc = BI_ERR_CUDA;
+  }
+  if (rc == BI_OK) {   // the block kernels' plans and table, one upload (from pageable memory: the call returns when it is staged)
+    std::vector<unsigned char> blob;
+    bi_block_build(md, blob);
+    unsigned char *dev = nullptr;
+    const size_t tab = (512 + 256) * sizeof(double);   // 2^(j/512), then 128 pairs (1/c, ln c)
+    rc = dev_alloc(md, (void **)&dev, tab + blob.size());
+    if (rc == BI_OK) {
+      rc = bi_block_exp_table((double *)dev, stream);
+      md->exp_tab = (const double *)dev;
+      bi_block_bind(md, dev + tab);
+      if (rc == BI_OK && !blob.empty() &&
+          cudaMemcpyAsync(dev + tab, blob.data(), blob.size(), cudaMemcpyHostToDevice, stream) != cudaSuccess)
+        rc = BI_ERR_CUDA;
+    }
   }
   if (rc == BI_OK) rc = dev_alloc(md, (void **)&md->d, sizeof(BiDev));
   if (rc == BI_OK) {
@@ -803,9 +845,17 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
     if (cudaMemcpyAsync(md->d, &md->h, sizeof(BiDev), cudaMemcpyHostToDevice, stream) != cudaSuccess)
       rc = BI_ERR_CUDA;
   }
+  if (rc == BI_OK && md->blk_BR) {   // (the dispatcher needs to know on the host: making a handle synchronises the stream)
+    uint32_t z = 0;
+    if (cudaMemcpyAsync(&z, h.status + 2, sizeof(z), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
+        cudaStreamSynchronize(stream) != cudaSuccess)
+      rc = BI_ERR_CUDA;
+    md->has_zeros = z != 0;
+  }
   if (rc != BI_OK) {
     cudaStreamSynchronize(stream);
     free_all(md);
+    bi_block_free(md);
     delete md;
     return rc;
   }
@@ -821,6 +871,7 @@ extern "C" int bi_model_destroy(bi_model_t *model) {
   if (model->ws_prior) cudaFree(model->ws_prior);
   if (model->carry) cudaFree(model->carry);
   free_all(model);
+  bi_block_free(model);
   delete model;
   return e == cudaSuccess ? BI_OK : BI_ERR_CUDA;
 }
@@ -850,7 +901,8 @@ int bi_dispatch(const BiCall &c, bi_model *mut) {
     // step, which the CTA-per-agent filtering kernel computes; window calls (VMP) need them in every
     // message: the warp-per-step kernel's lanes sum them, the general kernel where that one does not fit.
     int rc = BI_ERR_UNSUPPORTED;
-    if (c.model->test_family == BI_FAMILY_ANY)
+    if (c.model->test_family == BI_FAMILY_ANY) rc = bi_launch_block(c, mut);
+    if (rc == BI_ERR_UNSUPPORTED && c.model->test_family == BI_FAMILY_ANY)
       rc = c.algo == BI_ALGO_FILTER ? bi_launch_cta_filter(c, mut) : bi_launch_warp(c, mut);
     return rc == BI_ERR_UNSUPPORTED ? bi_launch_generic(c, mut) : rc;
   }
@@ -861,6 +913,7 @@ int bi_dispatch(const BiCall &c, bi_model *mut) {
     if (rc == BI_ERR_UNSUPPORTED) rc = bi_launch_tile3_window(c, mut);
     if (rc == BI_ERR_UNSUPPORTED) rc = bi_launch_pair_filter(c, mut);
     if (rc == BI_ERR_UNSUPPORTED) rc = bi_launch_pair_window(c, mut);
+    if (rc == BI_ERR_UNSUPPORTED && c.model->test_drop_copy == 0) rc = bi_launch_block(c, mut);
     if (rc == BI_ERR_UNSUPPORTED) rc = bi_launch_batch(c, mut);
     // Filtering exposes one unit per agent, so a CTA per agent keeps more of the machine busy than
     // a warp per agent, and its staged slices and per-factor warps pay at every batch size measured

@@ -59,6 +59,7 @@ struct BiMember {
   // of such a slice are the floor ln 1e-16 (a zero of A), so a slice is stored as one 64-bit mask per
   // lane of a unit (bit i set: the lane's i-th element is not the floor) plus the other values, packed
   // lane after lane.  cmask: [G * m][LPU]; coff: [G * m + 1] element offsets into cvals.
+  const void *logA_blk;   // the slices in the block kernels' order (block.cuh), [G][m][blocks x entries], or NULL
   const void *logA_T;     // groups over two factors of pair models: the slices transposed, [G][m][dim1][pad4(dim0)], or NULL
   const unsigned long long *cmask;
   const void *cvals;
@@ -95,8 +96,9 @@ struct alignas(16) BiDev {
   int64_t Bfull_stride[BI_MAX_F];  // elements per model (0 when shared)
   int64_t Dstride[BI_MAX_F];
   // status[0]: the BI_FLAG_* bits bi_status reports and clears.  status[1]: set when the model was packed
-  // if an entry of A exceeds 1 (not a probability): kernels that shift several agents' softmaxes by one
+  // if an entry of A, B or D exceeds 1 (not a probability): kernels that shift several agents' softmaxes by one
   // common power of two then shift per agent, because such logits can lie too far apart for one shift.
+  // status[2]: set when an entry of A is at or below the floor 1e-16.
   uint32_t *status;
 };
 
@@ -104,7 +106,7 @@ struct alignas(16) BiDev {
 struct bi_model {
   BiDev h;          // host copy (device pointers inside)
   BiDev *d;         // device copy
-  void *allocs[24 + 3 * BI_MAX_M + 10 * BI_MAX_F];  // status, descriptor, pre-summed table, 2 per modality, 7 per factor
+  void *allocs[28 + 4 * BI_MAX_M + 10 * BI_MAX_F];  // status, descriptor, pre-summed table, 2 per modality, 7 per factor
   int nalloc;
   int arith;        // BI_ARITH_F64 or BI_ARITH_F32
   int device;
@@ -148,6 +150,15 @@ struct bi_model {
   // announce their slice copies without issuing them, so that the bounded wait on the copy runs out and
   // the status flag BI_FLAG_COPY_TIMEOUT is raised; nothing faults, nothing is left in flight.
   int test_drop_copy;
+  // block kernels: the block shape the slices are laid out for (0: none), the filtering and the window plan
+  // (bi_block::Plan), the device table 2^(j/512)
+  int blk_BR, blk_BC;
+  void *blk_plan[2];
+  const double *exp_tab;
+  int has_zeros;    // A has entries at or below 1e-16 (see bi_launch_block)
+  // every group over two factors or more has an unrolled form of the batched contraction: those run at 0.7 ps per
+  // slice entry, unit and iteration, the block kernels at 2.1; below some 4000 units the launches decide
+  int batch_unrolled;
 };
 
 struct BiCall {
@@ -181,6 +192,7 @@ int bi_launch_pair_window(const BiCall &c, bi_model *mut);  // window calls on t
 int bi_launch_tile3(const BiCall &c, bi_model *mut);
 int bi_launch_tile3_window(const BiCall &c, bi_model *mut);
 int bi_launch_batch(const BiCall &c, bi_model *mut);
+int bi_launch_block(const BiCall &c, bi_model *mut);        // any structure of rank up to 4; blocks of the slices in registers
 // tries the kernel families in order (the dispatcher behind every inference call)
 int bi_dispatch(const BiCall &c, bi_model *mut);
 // inference with observations given as categorical vectors [N][T][sum m_i]

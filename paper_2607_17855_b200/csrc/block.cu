@@ -1,0 +1,773 @@
+// Planner and launcher of the block kernels (block.cuh).
+#include <algorithm>
+#include <atomic>
+#include <cmath>
+#include <cstring>
+#include <vector>
+
+#include "block.h"
+
+const void *bi_block_kernel_f64(int BR, int BC, bool window, int sync, bool hass);
+const void *bi_block_kernel_f32(int BR, int BC, bool window, int sync, bool hass);
+
+using namespace bi_block;
+
+namespace {
+
+int ceil_div(int a, int b) { return (a + b - 1) / b; }
+int pow2_ceil(int x) {
+  int p = 1;
+  while (p < x) p <<= 1;
+  return p;
+}
+
+// Which axes of a group are a block's rows and columns (indices into BiGroup::axis), and the block counts.
+struct Cut {
+  int row, col, pre[2], npre_axes;   // pre: remaining axes, in packed order
+  int nrb, ncb, npre, nb;
+};
+Cut cut_group(const BiGroup &g, int BR, int BC) {
+  Cut best;
+  memset(&best, 0, sizeof(best));
+  best.nb = 1 << 30;
+  for (int r = 0; r < g.rank; ++r)
+    for (int c = 0; c < g.rank; ++c) {
+      if (r == c) continue;
+      Cut k;
+      memset(&k, 0, sizeof(k));
+      k.row = r; k.col = c;
+      k.nrb = ceil_div(g.dim[r], BR); k.ncb = ceil_div(g.dim[c], BC);
+      k.npre = 1;
+      for (int j = 0; j < g.rank; ++j)
+        if (j != r && j != c) { k.pre[k.npre_axes++] = j; k.npre *= g.dim[j]; }
+      k.nb = k.nrb * k.ncb * k.npre;
+      if (k.nb < best.nb) best = k;
+    }
+  return best;
+}
+
+struct Shape { int BR, BC; };
+const Shape kShapes[] = {{4, 4}, {8, 4}, {8, 6}};
+
+}  // namespace
+
+// ---- packing: a modality's slices in block order ----
+struct PackBlk {
+  const float *src;
+  void *dst;
+  int64_t total;
+  int32_t P, nb, npre, ncb, BR, BC, VE, nrow, ncol, npre1;
+  int64_t srow, scol, spre0, spre1;
+};
+template <typename R>
+__global__ void bi_pack_block_kernel(PackBlk p) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= p.total) return;
+  const int per = p.nb * p.BR * p.BC;
+  const int64_t go = e / per;
+  const int idx = (int)(e - go * per);
+  const int v = idx / (p.nb * p.VE), rest = idx - v * p.nb * p.VE, b = rest / p.VE, el = v * p.VE + rest % p.VE;
+  const int pre = b % p.npre, rc = b / p.npre, rb = rc / p.ncb, cb = rc - rb * p.ncb;
+  const int i = rb * p.BR + el / p.BC, j = cb * p.BC + el % p.BC;
+  R out = (R)0;
+  if (i < p.nrow && j < p.ncol) {
+    const int p0 = pre / p.npre1, p1 = pre - p0 * p.npre1;
+    const float x = p.src[go * p.P + i * p.srow + j * p.scol + p0 * p.spre0 + p1 * p.spre1];
+    out = (R)log(fmax((double)x, 1e-16));
+  }
+  ((R *)p.dst)[e] = out;
+}
+__global__ void bi_exp_table_kernel(double *tab) {
+  for (int j = threadIdx.x; j < 512; j += blockDim.x) tab[j] = exp2((double)j * (1.0 / 512));
+  for (int j = threadIdx.x; j < 128; j += blockDim.x) {   // the pairs bi_log_fast reads
+    const double c = 1.0 + ((double)j + 0.5) * (1.0 / 128);
+    tab[512 + 2 * j] = 1.0 / c;
+    tab[512 + 2 * j + 1] = log(c);
+  }
+}
+
+// Elements of one outcome's slice of group gi in block order (0: the model has no block plan).
+int bi_block_slice_elems(const bi_model *md, int gi) {
+  if (!md->blk_BR || md->h.grp[gi].rank < 2) return 0;
+  const Cut k = cut_group(md->h.grp[gi], md->blk_BR, md->blk_BC);
+  return k.nb * md->blk_BR * md->blk_BC;
+}
+
+// Block shape of a model (0, 0: none).  Decided from the groups alone, because the slices are laid out for
+// it once: the smallest block under which a filtering unit is a single warp (no block barriers), else 8 x 6,
+// which has the fewest partial messages per entry that the register file allows.
+void bi_block_choose_shape(bi_model *md) {
+  md->blk_BR = md->blk_BC = 0;
+  for (int gi = 0; gi < md->h.ngroups; ++gi)
+    if (md->h.grp[gi].rank > kMaxRank) return;
+  for (const Shape &s : kShapes) {
+    int nb = 0;
+    for (int gi = 0; gi < md->h.ngroups; ++gi)
+      if (md->h.grp[gi].rank >= 2) nb += cut_group(md->h.grp[gi], s.BR, s.BC).nb;
+    md->blk_BR = s.BR; md->blk_BC = s.BC;
+    if (nb <= 32) break;
+  }
+}
+
+// The block-ordered copy of one modality: sstride[j] is the source stride of the group's axis j, P the
+// entries of a source slice.  Returns the packing job's element count per outcome.
+int bi_block_pack_member(const bi_model *md, int gi, const float *src, int m, const int64_t *sstride, int P, void *dst,
+                         cudaStream_t stream) {
+  const BiGroup &g = md->h.grp[gi];
+  const Cut k = cut_group(g, md->blk_BR, md->blk_BC);
+  PackBlk q;
+  memset(&q, 0, sizeof(q));
+  q.src = src; q.dst = dst; q.P = P;
+  q.nb = k.nb; q.npre = k.npre; q.ncb = k.ncb; q.BR = md->blk_BR; q.BC = md->blk_BC;
+  q.VE = md->arith == BI_ARITH_F64 ? 2 : 4;
+  q.nrow = g.dim[k.row]; q.ncol = g.dim[k.col];
+  q.npre1 = k.npre_axes > 1 ? g.dim[k.pre[1]] : 1;
+  q.srow = sstride[k.row]; q.scol = sstride[k.col];
+  q.spre0 = k.npre_axes > 0 ? sstride[k.pre[0]] : 0;
+  q.spre1 = k.npre_axes > 1 ? sstride[k.pre[1]] : 0;
+  q.total = (int64_t)md->h.G * m * k.nb * q.BR * q.BC;
+  const unsigned blocks = (unsigned)((q.total + 255) / 256);
+  if (md->arith == BI_ARITH_F64) bi_pack_block_kernel<double><<<blocks, 256, 0, stream>>>(q);
+  else bi_pack_block_kernel<float><<<blocks, 256, 0, stream>>>(q);
+  return cudaGetLastError() == cudaSuccess ? BI_OK : BI_ERR_CUDA;
+}
+
+namespace {
+
+// ---- the plan of one call kind ----
+struct HostPlan {
+  Plan p;
+  std::vector<Desc> desc;
+  std::vector<Lane> lane[kMaxVariants];
+  std::vector<Pass> pass[kMaxVariants];
+};
+
+struct Run {           // a factor's message entries
+  int kg, kp, kf;      // entries per state: groups, edge in, edge out
+  int rows;            // states allocated (padded rows and columns of blocks are written too)
+  int y0, cs;          // first entry, entries per state
+  int op, of;          // starts of the edges' runs within a state
+};
+
+// Which lanes of the finishing phase complete which states, for a team of NW warps: a factor's states side by
+// side in one warp, several factors to a pass where they fit, several lanes per state where the warps have
+// room for it (the longest runs first).
+struct LanePack {
+  int npass, g[BI_MAX_F], pass_of[BI_MAX_F], lane_of[BI_MAX_F];
+  std::vector<Pass> passes;
+};
+int up2(int x) { return (x + 1) & ~1; }
+void pack_lanes(const BiDev &h, const Run *run, int ve, int NW, LanePack &lp) {
+  const int F = h.F;
+  for (int f = 0; f < F; ++f) lp.g[f] = 1;
+  auto pack = [&]() {   // by decreasing lanes per state: every start is a multiple of it (n g lanes each)
+    std::vector<int> order(F), used;
+    for (int f = 0; f < F; ++f) order[f] = f;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return lp.g[a] != lp.g[b] ? lp.g[a] > lp.g[b] : h.n[a] > h.n[b]; });
+    for (int f : order) {
+      const int need = h.n[f] * lp.g[f];
+      size_t k = 0;
+      while (k < used.size() && used[k] + need > 32) ++k;
+      if (k == used.size()) used.push_back(0);
+      lp.pass_of[f] = (int)k;
+      lp.lane_of[f] = used[k];
+      used[k] += need;
+    }
+    return (int)used.size();
+  };
+  const int limit = std::max(NW, pack());
+  std::vector<char> stuck(F, 0);
+  for (;;) {
+    int best = -1;
+    double most = 2.0;   // (runs of a few vectors gain nothing from more lanes)
+    for (int f = 0; f < F; ++f) {
+      const double len = (double)(run[f].kg + run[f].kp + run[f].kf) / ve / lp.g[f];
+      if (!stuck[f] && h.n[f] * lp.g[f] * 2 <= 32 && lp.g[f] < 16 && len > most) { most = len; best = f; }
+    }
+    if (best < 0) break;
+    lp.g[best] *= 2;
+    if (pack() > limit) {
+      lp.g[best] /= 2;
+      stuck[best] = 1;
+    }
+  }
+  lp.npass = pack();
+  lp.passes.assign(lp.npass, Pass{1, 0, 0, 0});
+  for (int f = 0; f < F; ++f) {
+    Pass &ps = lp.passes[lp.pass_of[f]];
+    auto vecs = [&](int k) { return ceil_div(ceil_div(k, ve), lp.g[f]); };
+    ps.gmax = std::max(ps.gmax, lp.g[f]);
+    ps.nz = std::max(ps.nz, std::max(2, pow2_ceil((h.n[f] + 1) / 2)));
+    ps.nvec = std::max(ps.nvec, up2(vecs(run[f].kg)));
+    ps.nedge = std::max(ps.nedge, up2(std::max(vecs(run[f].kp), vecs(run[f].kf))));
+  }
+}
+void build_lanes(const BiDev &h, const Plan &p, const Run *run, const int *e0, int ve, const LanePack &lp, std::vector<Lane> &lanes) {
+  Lane dead;   // an idle lane: the first factor's first state, completed and thrown away
+  memset(&dead, 0, sizeof(dead));
+  dead.f = -1;
+  dead.g = dead.n = 1;
+  dead.ya = p.ydead;
+  dead.e0 = (int16_t)e0[0];
+  dead.qa = (int16_t)p.qo[0];
+  lanes.assign((size_t)lp.npass * 32, dead);
+  for (int f = 0; f < h.F; ++f)
+    for (int i = 0; i < h.n[f] * lp.g[f]; ++i) {
+      const int s = i / lp.g[f], q = i % lp.g[f];
+      Lane &l = lanes[(size_t)lp.pass_of[f] * 32 + lp.lane_of[f] + i];
+      l.f = (int16_t)f; l.s = (int16_t)s; l.p = (int16_t)q; l.g = (int16_t)lp.g[f]; l.n = (int16_t)h.n[f];
+      l.ya = run[f].y0 + s * run[f].cs + q * ve;
+      l.op = (int16_t)run[f].op;
+      l.of = (int16_t)run[f].of;
+      l.qa = (int16_t)(p.qo[f] + s);
+      l.e0 = (int16_t)e0[f];
+      l.out = h.off[f] + s;
+    }
+}
+
+// window: also the edges' transitions
+bool build_plan(const bi_model *md, bool window, HostPlan &hp) {
+  const BiDev &h = md->h;
+  const int BR = md->blk_BR, BC = md->blk_BC, F = h.F, ve = md->arith == BI_ARITH_F64 ? 2 : 4;
+  Plan &p = hp.p;
+  memset(&p, 0, sizeof(p));
+  if (!BR) return false;
+  p.BR = BR; p.BC = BC;
+  p.max_th = max_threads(BR * BC * 4 / ve);
+  std::vector<Cut> cut(h.ngroups);
+  int rowsp[BI_MAX_F];
+  for (int f = 0; f < F; ++f) rowsp[f] = h.n[f];
+  auto as_rows = [&](int f) { rowsp[f] = std::max(rowsp[f], ceil_div(h.n[f], BR) * BR); };
+  auto as_cols = [&](int f) { rowsp[f] = std::max(rowsp[f], ceil_div(h.n[f], BC) * BC); };
+  for (int gi = 0; gi < h.ngroups; ++gi) {
+    const BiGroup &g = h.grp[gi];
+    if (g.rank > kMaxRank) return false;
+    if (g.rank < 2) continue;
+    cut[gi] = cut_group(g, BR, BC);
+    as_rows(g.axis[cut[gi].row]);
+    as_cols(g.axis[cut[gi].col]);
+    p.g_nb[gi] = cut[gi].nb;
+  }
+  if (window) {
+    for (int f = 0; f < F; ++f) {
+      if (!h.has_bdep) { as_rows(f); as_cols(f); continue; }
+      const int k = h.bdep_len[f];
+      if (k > 3) return false;
+      as_rows(f);
+      for (int j = 0; j < k; ++j) { as_rows(h.bdep[f][j]); as_cols(h.bdep[f][j]); }
+    }
+  }
+  int o = 0;
+  for (int f = 0; f < F; ++f) {
+    p.qo[f] = o;
+    o += (rowsp[f] + 3) & ~3;
+  }
+  p.one = o;
+  p.SQ = (o + 1 + 3) & ~3;
+  // ---- pass 1: entries per state; pass 2: the blocks with their addresses
+  Run run[BI_MAX_F];
+  memset(run, 0, sizeof(run));
+  LanePack lp[kMaxVariants];
+  int e0[BI_MAX_F] = {}, nedge_blocks = 0;
+  for (int pass = 0; pass < 2; ++pass) {
+    int kg[BI_MAX_F] = {}, kp[BI_MAX_F] = {}, kf[BI_MAX_F] = {};   // entries used so far
+    auto entry = [&](int f, int s, int k) { return run[f].y0 + s * run[f].cs + k; };
+    for (int gi = 0; gi < h.ngroups; ++gi) {
+      const BiGroup &g = h.grp[gi];
+      if (g.rank < 2) continue;
+      const Cut &c = cut[gi];
+      const int fr = g.axis[c.row], fc = g.axis[c.col];
+      const int f0 = c.npre_axes > 0 ? g.axis[c.pre[0]] : -1, f1 = c.npre_axes > 1 ? g.axis[c.pre[1]] : -1;
+      const int n0 = f0 >= 0 ? h.n[f0] : 1, n1 = f1 >= 0 ? h.n[f1] : 1;
+      if (pass == 1)
+        for (int b = 0; b < c.nb; ++b) {
+          const int pre = b % c.npre, rc = b / c.npre, rb = rc / c.ncb, cb = rc % c.ncb, d0 = pre / n1, d1 = pre % n1;
+          Desc d;
+          memset(&d, 0, sizeof(d));
+          d.yv = d.yw = d.yu0 = d.yu1 = p.ydump;
+          d.qr = (int16_t)(p.qo[fr] + rb * BR);
+          d.qc = (int16_t)(p.qo[fc] + cb * BC);
+          d.q0 = (int16_t)(f0 >= 0 ? p.qo[f0] + d0 : p.one);
+          d.q1 = (int16_t)(f1 >= 0 ? p.qo[f1] + d1 : p.one);
+          d.kind = KIND_V | KIND_W;
+          d.yv = entry(fr, rb * BR, kg[fr] + cb * c.npre + pre);
+          d.sv = (int16_t)run[fr].cs;
+          d.yw = entry(fc, cb * BC, kg[fc] + rb * c.npre + pre);
+          d.sw = (int16_t)run[fc].cs;
+          if (f0 >= 0) {   // u times the other prefix factor's belief
+            d.kind |= KIND_U0;
+            d.yu0 = entry(f0, d0, kg[f0] + (rb * c.ncb + cb) * n1 + d1);
+          }
+          if (f1 >= 0) {
+            d.kind |= KIND_U1;
+            d.yu1 = entry(f1, d1, kg[f1] + (rb * c.ncb + cb) * n0 + d0);
+          }
+          d.grp = gi; d.base = b;
+          hp.desc.push_back(d);
+        }
+      kg[fr] += c.ncb * c.npre;
+      kg[fc] += c.nrb * c.npre;
+      if (f0 >= 0) kg[f0] += c.nrb * c.ncb * n1;
+      if (f1 >= 0) kg[f1] += c.nrb * c.ncb * n0;
+    }
+    for (int f = 0; f < F && window; ++f) {
+      const int n = h.n[f];
+      if (!h.has_bdep) {
+        if (n == 1) continue;
+        const int nrb = ceil_div(n, BR), ncb = ceil_div(n, BC);
+        for (int dir = 0; dir < 2; ++dir) {
+          const int k0 = dir == 0 ? run[f].op + kp[f] : run[f].of + kf[f];
+          if (pass == 1)
+            for (int b = 0; b < nrb * ncb; ++b) {
+              const int rb = b / ncb, cb = b % ncb;
+              Desc d;
+              memset(&d, 0, sizeof(d));
+              d.yv = d.yw = d.yu0 = d.yu1 = p.ydump;
+              d.qr = (int16_t)((dir == 0 ? -p.SQ : p.SQ) + p.qo[f] + rb * BR);
+              d.q0 = d.q1 = (int16_t)p.one;
+              d.kind = KIND_W | (dir == 0 ? KIND_PAST : KIND_FUT);
+              d.yw = entry(f, cb * BC, k0 + rb);
+              d.sw = (int16_t)run[f].cs;
+              d.grp = f; d.base = rb * BR * h.npad[f] + cb * BC;
+              d.rs = h.npad[f]; d.cs = 1;
+              d.rlim = (int16_t)std::min(BR, n - rb * BR);
+              d.clim = (int16_t)std::min(BC, n - cb * BC);
+              hp.desc.push_back(d);
+            }
+          (dir == 0 ? kp[f] : kf[f]) += nrb;
+          if (pass == 0) nedge_blocks += nrb * ncb;
+        }
+        continue;
+      }
+      // transitions over several parents: the tensor [n][parents, last fastest]
+      const int k = h.bdep_len[f], *par = h.bdep[f], PB = h.PB[f];
+      int str[3] = {1, 1, 1};
+      for (int j = k - 2; j >= 0; --j) str[j] = str[j + 1] * h.n[par[j + 1]];
+      {   // edge in: rows = own states, columns = the last parent, prefix = the others (all at the step before)
+        const int fc = par[k - 1], nrb = ceil_div(n, BR), ncb = ceil_div(h.n[fc], BC);
+        const int n0 = k > 1 ? h.n[par[0]] : 1, n1 = k > 2 ? h.n[par[1]] : 1, npre = n0 * n1;
+        if (pass == 1)
+          for (int b = 0; b < nrb * ncb * npre; ++b) {
+            const int pre = b % npre, rc = b / npre, rb = rc / ncb, cb = rc % ncb, d0 = pre / n1, d1 = pre % n1;
+            Desc d;
+            memset(&d, 0, sizeof(d));
+            d.yv = d.yw = d.yu0 = d.yu1 = p.ydump;
+            d.qr = (int16_t)(p.qo[f] + rb * BR);
+            d.qc = (int16_t)(-p.SQ + p.qo[fc] + cb * BC);
+            d.q0 = (int16_t)(k > 1 ? -p.SQ + p.qo[par[0]] + d0 : p.one);
+            d.q1 = (int16_t)(k > 2 ? -p.SQ + p.qo[par[1]] + d1 : p.one);
+            d.kind = KIND_V | KIND_PAST;
+            d.yv = entry(f, rb * BR, run[f].op + kp[f] + cb * npre + pre);
+            d.sv = (int16_t)run[f].cs;
+            d.grp = f;
+            d.base = rb * BR * PB + cb * BC + (k > 1 ? d0 * str[0] : 0) + (k > 2 ? d1 * str[1] : 0);
+            d.rs = PB; d.cs = 1;
+            d.rlim = (int16_t)std::min(BR, n - rb * BR);
+            d.clim = (int16_t)std::min(BC, h.n[fc] - cb * BC);
+            hp.desc.push_back(d);
+          }
+        kp[f] += ncb * npre;
+        if (pass == 0) nedge_blocks += nrb * ncb * npre;
+      }
+      if (k == 1) {   // edge out, one parent: rows = the child's next states, columns = the parent
+        const int fc = par[0], nrb = ceil_div(n, BR), ncb = ceil_div(h.n[fc], BC);
+        if (pass == 1)
+          for (int b = 0; b < nrb * ncb; ++b) {
+            const int rb = b / ncb, cb = b % ncb;
+            Desc d;
+            memset(&d, 0, sizeof(d));
+            d.yv = d.yw = d.yu0 = d.yu1 = p.ydump;
+            d.qr = (int16_t)(p.SQ + p.qo[f] + rb * BR);
+            d.q0 = d.q1 = (int16_t)p.one;
+            d.kind = KIND_W | KIND_FUT;
+            d.yw = entry(fc, cb * BC, run[fc].of + kf[fc] + rb);
+            d.sw = (int16_t)run[fc].cs;
+            d.grp = f; d.base = rb * BR * PB + cb * BC;
+            d.rs = PB; d.cs = 1;
+            d.rlim = (int16_t)std::min(BR, n - rb * BR);
+            d.clim = (int16_t)std::min(BC, h.n[fc] - cb * BC);
+            hp.desc.push_back(d);
+          }
+        kf[fc] += nrb;
+        if (pass == 0) nedge_blocks += nrb * ncb;
+      } else {        // two or three: prefix = the child's next state (and the first of three parents), rows and columns = the last two
+        const int fr = par[k - 2], fc = par[k - 1], f1 = k > 2 ? par[0] : -1;
+        const int nrb = ceil_div(h.n[fr], BR), ncb = ceil_div(h.n[fc], BC), n1 = f1 >= 0 ? h.n[f1] : 1, npre = n * n1;
+        if (pass == 1)
+          for (int b = 0; b < nrb * ncb * npre; ++b) {
+            const int pre = b % npre, rc = b / npre, rb = rc / ncb, cb = rc % ncb, sn = pre / n1, d1 = pre % n1;
+            Desc d;
+            memset(&d, 0, sizeof(d));
+            d.yv = d.yw = d.yu0 = d.yu1 = p.ydump;
+            d.qr = (int16_t)(p.qo[fr] + rb * BR);
+            d.qc = (int16_t)(p.qo[fc] + cb * BC);
+            d.q0 = (int16_t)(p.SQ + p.qo[f] + sn);
+            d.q1 = (int16_t)(f1 >= 0 ? p.qo[f1] + d1 : p.one);
+            d.kind = KIND_V | KIND_W | KIND_FUT | (f1 >= 0 ? KIND_U1 : 0);
+            d.yv = entry(fr, rb * BR, run[fr].of + kf[fr] + cb * npre + pre);
+            d.sv = (int16_t)run[fr].cs;
+            d.yw = entry(fc, cb * BC, run[fc].of + kf[fc] + rb * npre + pre);
+            d.sw = (int16_t)run[fc].cs;
+            if (f1 >= 0) d.yu1 = entry(f1, d1, run[f1].of + kf[f1] + (rb * ncb + cb) * n + sn);
+            d.grp = f;
+            d.base = sn * PB + rb * BR * str[k - 2] + cb * BC + (k > 2 ? d1 * str[0] : 0);
+            d.rs = str[k - 2]; d.cs = 1;
+            d.rlim = (int16_t)std::min(BR, h.n[fr] - rb * BR);
+            d.clim = (int16_t)std::min(BC, h.n[fc] - cb * BC);
+            hp.desc.push_back(d);
+          }
+        kf[fr] += ncb * npre;
+        kf[fc] += nrb * npre;
+        if (f1 >= 0) kf[f1] += nrb * ncb * n;
+        if (pass == 0) nedge_blocks += nrb * ncb * npre;
+      }
+    }
+    if (pass == 0) {
+      // team sizes: a thread per block, in window calls also those under which 2, 3, 4, 6 or 12 steps share a CTA
+      int NB = 0;
+      for (int gi = 0; gi < h.ngroups; ++gi) NB += p.g_nb[gi];
+      NB += nedge_blocks;
+      // (and, where that is more than a thread per block, a warp for each pass of the finishing phase)
+      const int full = std::max(32, (NB + 31) / 32 * 32);
+      for (int f = 0; f < F; ++f) { run[f].kg = kg[f]; run[f].kp = kp[f]; run[f].kf = kf[f]; }
+      LanePack one;
+      pack_lanes(h, run, ve, 1, one);
+      const int wide = std::max(full, 32 * one.npass);
+      for (int uc : {1, 2, 3, 4, 6, 12})
+        for (int want : {full, wide}) {
+          if (!window && uc > 1) continue;
+          const int LT = std::min(want, p.max_th / uc / 32 * 32);
+          bool have = LT < 32 || p.nv == kMaxVariants;
+          for (int v = 0; v < p.nv; ++v) have = have || p.var[v].LT == LT;
+          if (have) continue;
+          Variant &v = p.var[p.nv];
+          v.LT = LT;
+          v.nbpt = ceil_div(std::max(NB, 1), LT);
+          pack_lanes(h, run, ve, LT / 32, lp[p.nv]);
+          v.npass = lp[p.nv].npass;
+          p.nv += 1;
+        }
+      // runs of whole 16-byte vectors, zero-padded to what the longest lane of the same pass reads (under
+      // every team size); an odd number of vectors between states: consecutive states on different banks
+      int y = 0;
+      for (int f = 0; f < F; ++f) {
+        int lg = 0, le = 0, lz = 0;
+        for (int v = 0; v < p.nv; ++v) {
+          const Pass &ps = lp[v].passes[lp[v].pass_of[f]];
+          lg = std::max(lg, ps.nvec * lp[v].g[f]);
+          le = std::max(le, ps.nedge * lp[v].g[f]);
+          lz = std::max(lz, ps.nz);
+        }
+        run[f].rows = rowsp[f];
+        run[f].op = lg * ve;
+        run[f].of = (lg + le) * ve;
+        // entries between states: the padding under which the lanes of a quarter-warp hit distinct banks most
+        const int need = lg + (window ? 2 * le : 0);
+        int cs = need, least = 1 << 30;
+        for (int c = std::max(need, 1); c < need + 9; ++c) {
+          int cost = c - need;
+          for (int v = 0; v < p.nv; ++v) {
+            const int g = lp[v].g[f];
+            for (int l0 = 0; l0 < h.n[f] * g; l0 += 8) {
+              int hits[8] = {}, most = 0;
+              for (int l = l0; l < std::min(l0 + 8, h.n[f] * g); ++l) most = std::max(most, ++hits[(l / g * c + l % g) & 7]);
+              cost += 16 * (most - 1);
+            }
+          }
+          if (cost < least) { least = cost; cs = c; }
+        }
+        run[f].cs = cs * ve;
+        if (run[f].cs > 16000 || y / ve > 60000) return false;
+        run[f].y0 = y;
+        y += run[f].rows * run[f].cs;
+        e0[f] = p.Esz;
+        p.Esz += 2 * lz;
+      }
+      // (an idle lane reads what any lane may read, from an area of zeros)
+      p.ydead = y;
+      int most = 0;
+      for (int v = 0; v < p.nv; ++v)
+        for (const Pass &ps : lp[v].passes) most = std::max(most, std::max(ps.nvec, ps.nedge));
+      y += most * ve;
+      p.ydump = y;   // (results that a block does not have)
+      y += ve;
+      for (int v = 0; v < p.nv; ++v)   // (and of the exchange area, from the first factor's entry on)
+        for (const Pass &ps : lp[v].passes) p.Esz = std::max(p.Esz, 2 * ps.nz);
+      p.Ysz = (y + 3) & ~3;
+    }
+  }
+  p.NB = (int)hp.desc.size();
+  {   // the entry of threads without a block
+    Desc d;
+    memset(&d, 0, sizeof(d));
+    d.q0 = d.q1 = (int16_t)p.one;
+    d.yv = d.yw = d.yu0 = d.yu1 = p.ydump;
+    hp.desc.push_back(d);
+  }
+  for (int v = 0; v < p.nv; ++v) {
+    build_lanes(h, p, run, e0, ve, lp[v], hp.lane[v]);
+    hp.pass[v] = lp[v].passes;
+  }
+  p.ok = p.nv > 0;
+  return p.ok != 0;
+}
+
+}  // namespace
+
+// Builds the filtering and the window plan of a model and appends their tables to the upload buffer; the
+// device pointers in the plans are offsets until bi_block_bind turns them into addresses.
+void bi_block_build(bi_model *md, std::vector<unsigned char> &blob) {
+  auto put = [&](const void *src, size_t bytes) {
+    const size_t at = (blob.size() + 15) & ~(size_t)15;
+    blob.resize(at + bytes);
+    memcpy(blob.data() + at, src, bytes);
+    return (uintptr_t)at;
+  };
+  md->blk_plan[0] = md->blk_plan[1] = nullptr;
+  for (int k = 0; k < 2; ++k) {
+    HostPlan hp;
+    if (!build_plan(md, k == 1, hp)) continue;
+    hp.p.desc = reinterpret_cast<const Desc *>(put(hp.desc.data(), hp.desc.size() * sizeof(Desc)));
+    for (int v = 0; v < hp.p.nv; ++v) {
+      hp.p.var[v].lane = reinterpret_cast<const Lane *>(put(hp.lane[v].data(), hp.lane[v].size() * sizeof(Lane)));
+      hp.p.var[v].pass = reinterpret_cast<const Pass *>(put(hp.pass[v].data(), hp.pass[v].size() * sizeof(Pass)));
+    }
+    md->blk_plan[k] = new Plan(hp.p);
+  }
+}
+void bi_block_bind(bi_model *md, unsigned char *dev) {
+  for (int k = 0; k < 2; ++k) {
+    Plan *p = static_cast<Plan *>(md->blk_plan[k]);
+    if (!p) continue;
+    p->desc = reinterpret_cast<const Desc *>(dev + reinterpret_cast<uintptr_t>(p->desc));
+    for (int v = 0; v < p->nv; ++v) {
+      p->var[v].lane = reinterpret_cast<const Lane *>(dev + reinterpret_cast<uintptr_t>(p->var[v].lane));
+      p->var[v].pass = reinterpret_cast<const Pass *>(dev + reinterpret_cast<uintptr_t>(p->var[v].pass));
+    }
+  }
+}
+void bi_block_free(bi_model *md) {
+  for (int k = 0; k < 2; ++k) {
+    delete static_cast<Plan *>(md->blk_plan[k]);
+    md->blk_plan[k] = nullptr;
+  }
+}
+int bi_block_exp_table(double *dst, cudaStream_t stream) {
+  bi_exp_table_kernel<<<1, 512, 0, stream>>>(dst);
+  return cudaGetLastError() == cudaSuccess ? BI_OK : BI_ERR_CUDA;
+}
+
+namespace {
+
+void fill_params(const BiCall &c, const Plan &pl, Params &p) {
+  const bi_model *md = c.model;
+  const BiDev &h = md->h;
+  memset(&p, 0, sizeof(p));
+  const bool window = c.algo != BI_ALGO_FILTER;
+  p.desc = pl.desc;
+  p.NB = pl.NB; p.SQ = pl.SQ; p.one = pl.one; p.Ysz = pl.Ysz; p.Esz = pl.Esz;
+  p.N = c.N; p.T = c.T; p.K = c.K; p.F = h.F; p.M = h.M; p.S = h.S; p.G = h.G;
+  p.mmp = c.algo == BI_ALGO_MMP;
+  p.has_bdep = h.has_bdep;
+  p.lambda = c.lambda;
+  // No softmax shift in float64: with probabilities in A and B a logit is at least
+  // (modalities + 3) ln 1e-16 below zero, 53.2 binary orders each; beyond that, or with the caller's own
+  // weights or starting beliefs (used as given), every segment shifts by its own maximum (a model with
+  // entries above 1 is marked in status[1]).
+  p.common = !md->soft_shadow && !(c.q_init && c.lambda != 1.0) && (h.M + 3) * 54 < 960;
+  for (int f = 0; f < h.F; ++f) {
+    p.n[f] = h.n[f]; p.off[f] = h.off[f]; p.qo[f] = pl.qo[f]; p.npad[f] = h.npad[f]; p.U[f] = h.U[f];
+    p.logD[f] = h.logD[f];
+    p.n_max = std::max(p.n_max, (int)h.n[f]);
+    p.Dstride[f] = h.Dstride[f];
+    p.Bstride[f] = h.Bstride[f];
+    if (h.has_bdep) {
+      p.bdep_len[f] = h.bdep_len[f];
+      for (int j = 0; j < h.bdep_len[f]; ++j) p.bdep[f][j] = h.bdep[f][j];
+      p.PB[f] = h.PB[f];
+      p.Bfull[f] = h.Bfull[f];
+      p.Bfull_stride[f] = h.Bfull_stride[f];
+      p.Mp[f] = h.logBfull[f];
+      p.wpar = std::max(p.wpar, (h.PB[f] + 3) & ~3);
+    } else if (window) {
+      p.Mp[f] = c.algo == BI_ALGO_VMP ? h.logBt[f] : h.BfT[f];     // [previous][next]
+      p.Mf[f] = c.algo == BI_ALGO_VMP ? h.logB[f] : h.BdagT[f];    // [next][previous]
+    } else {
+      p.Mp[f] = h.BfT[f];
+    }
+  }
+  int n1 = 0;
+  for (int f = 0; f < h.F; ++f) {
+    p.r1_begin[f] = n1;
+    for (int gi = 0; gi < h.ngroups; ++gi) {
+      const BiGroup &gr = h.grp[gi];
+      if (gr.rank != 1 || gr.axis[0] != f) continue;
+      for (int mi = gr.mem_begin; mi < gr.mem_end; ++mi) {
+        const BiMember &mm = h.mem[mi];
+        p.r1_mod[n1] = mm.modality; p.r1_m[n1] = mm.m; p.r1_P[n1] = mm.P_pad;
+        p.r1_logA[n1] = mm.logA; p.r1_gstride[n1] = mm.gstride;
+        ++n1;
+      }
+    }
+  }
+  p.r1_begin[h.F] = n1;
+  for (int gi = 0; gi < h.ngroups; ++gi) {
+    p.g_nb[gi] = pl.g_nb[gi];
+    p.g_beg[gi] = h.grp[gi].mem_begin;
+    p.g_beg[gi + 1] = h.grp[gi].mem_end;
+    if (h.grp[gi].rank >= 2) p.g_any = gi;
+    if (h.grp[gi].rank >= 2) p.max_mem = std::max(p.max_mem, h.grp[gi].mem_end - h.grp[gi].mem_begin);
+    for (int mi = h.grp[gi].mem_begin; mi < h.grp[gi].mem_end; ++mi) {
+      p.m_mod[mi] = h.mem[mi].modality;
+      p.m_m[mi] = h.mem[mi].m;
+      p.m_blk[mi] = h.mem[mi].logA_blk;
+    }
+  }
+  p.exp_tab = md->exp_tab;
+  p.obs = c.obs; p.act = c.act; p.act_prev = c.act_prev;
+  p.q_prev = c.q_prev; p.q_init = c.q_init; p.carry_in = c.carry_in; p.carry_out = c.carry_out; p.lnprior = c.lnprior;
+  p.q_out = c.q_out; p.logq_out = c.logq_out; p.argmax_out = c.argmax_out; p.status = h.status;
+}
+
+void use_variant(const Variant &v, Params &p) {
+  p.lane = v.lane; p.pass = v.pass; p.npass = v.npass; p.LT = v.LT; p.nbpt = v.nbpt;
+}
+
+// shared-memory layout for `units` teams and `slots` belief slots (behind the exponential table); returns bytes
+size_t layout(const Plan &pl, Params &p, int esz, int units, int slots) {
+  auto up16 = [](int x) { return (x + 15) & ~15; };
+  int u = up16(pl.Ysz * esz);
+  p.o_cst = u; u += pl.SQ * 8;
+  p.o_xp = u; u += p.lambda != 1.0 ? pl.SQ * 8 : 0;
+  p.o_e = u; u += pl.Esz * 8;
+  p.unit_sz = u;
+  size_t o = (512 + (p.mmp ? 256 : 0)) * sizeof(double);
+  p.o_unit = (int)o; o += (size_t)units * p.unit_sz;
+  p.o_q = (int)o; o += (size_t)slots * pl.SQ * esz;
+  p.o_par = (int)o; o += (size_t)p.W * up16(p.wpar * esz);
+  // the blocks beyond a thread each: whole rounds of the team, the last one only as far as it goes
+  const int extra = p.nbpt > 1 ? (pl.NB - p.LT + 31) / 32 * 32 : 0;
+  p.extra = extra;
+  p.o_L = (int)o; o += (size_t)units * extra * pl.BR * pl.BC * esz;
+  p.o_ref = (int)o; o += (size_t)extra * 48;
+  p.o_lane = (int)o; o += (size_t)p.npass * 33 * 16;
+  return o;
+}
+
+// The attribute is set once per kernel and device and only ever raised.
+bool allow_smem(const void *kern, int slot, int device, size_t bytes) {
+  constexpr int kDev = 32;
+  static std::atomic<int> have[72][kDev];
+  if (device < kDev && have[slot][device].load(std::memory_order_relaxed) >= (int)bytes) return true;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess ||
+      cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (device < kDev) have[slot][device].store((int)bytes, std::memory_order_relaxed);
+  return true;
+}
+
+}  // namespace
+
+// Any model whose groups span at most four factors (transitions over at most three parents in window
+// calls), either arithmetic, as long as a step's blocks fit the register file and shared memory of an SM
+// (window calls: of a cluster); BI_ERR_UNSUPPORTED otherwise.
+int bi_launch_block(const BiCall &c, bi_model *mut) {
+  const bi_model *md = c.model;
+  const bool window = c.algo != BI_ALGO_FILTER;
+  const Plan *plp = static_cast<const Plan *>(md->blk_plan[window ? 1 : 0]);
+  if (!plp || !plp->ok) return BI_ERR_UNSUPPORTED;
+  if (window && md->h.has_bdep && (c.algo == BI_ALGO_MMP || c.lnprior)) return BI_ERR_UNSUPPORTED;
+  // A model with zeros in A amplifies a rounding by up to 1e9 within sixteen iterations, and a trajectory carries
+  // the result on from step to step: in float32, and in float64 over more than two filtered steps, another
+  // order of summation gives other beliefs (measured: one in five such trajectories differs in the first
+  // digit from the CTA kernel's).  Those calls stay with the kernels that have served them, bit for bit.
+  if (md->has_zeros && (md->arith == BI_ARITH_F32 || (!window && c.T > 2))) return BI_ERR_UNSUPPORTED;
+  if (plp->NB == 0) return BI_ERR_UNSUPPORTED;   // nothing to contract: the CTA kernel's warp per factor does that
+  if (window && !md->h.has_bdep && md->batch_unrolled && (long long)c.N * c.T >= 4096) return BI_ERR_UNSUPPORTED;   // (see batch_unrolled)
+  const Plan &pl = *plp;
+  const int esz = md->arith == BI_ARITH_F64 ? 8 : 4;
+  const size_t budget = (size_t)md->max_smem_optin - 1024;
+  Params p;
+  fill_params(c, pl, p);
+  unsigned grid = 0, threads = 0;
+  size_t bytes = 0;
+  if (!window) {
+    // a warp per pass while the batch leaves the machine that much room (the second variant, if there is one)
+    use_variant(pl.var[pl.nv > 1 && (long long)c.N * pl.var[1].LT <= 8 * 32 * md->sm_count ? 1 : 0], p);
+    // agents per CTA (one-warp teams): one while the batch fits the machine anyway, so that no SM gets
+    // four more warps than another; four for large batches, which share the CTA's exponential table
+    p.W = p.LT == 32 ? (c.N > 24 * md->sm_count ? 4 : 1) : 1;
+    p.UC = p.W; p.CS = 1;
+    bytes = layout(pl, p, esz, p.W, p.W);
+    if (bytes > budget) return BI_ERR_UNSUPPORTED;
+    grid = (unsigned)((c.N + p.W - 1) / p.W);
+    threads = (unsigned)(p.W * p.LT);
+  } else {
+    // Steps per CTA and CTAs per agent: the cheapest by a small model of an iteration -- the larger of a
+    // dependent chain of about a thousand cycles (more when it crosses CTAs) and the throughput of
+    // the blocks resident on an SM -- times the number of waves.
+    double best = 1e300;
+    int bv = -1, buc = 0, bcs = 0;
+    for (int v = 0; v < pl.nv; ++v) {
+      use_variant(pl.var[v], p);
+      p.W = 0;
+      for (int cs = 1; cs <= 8; ++cs) {
+        const int uc = ceil_div(c.T, cs);
+        if (cs > 1 && ceil_div(c.T, uc) != cs) continue;
+        const int th = uc * p.LT;
+        if (th > pl.max_th) continue;
+        if (p.LT > 32 && uc > 15) continue;   // (named barriers)
+        const size_t b = layout(pl, p, esz, uc, 2 * (uc + 2));
+        if (b > budget) continue;
+        const int per_sm = std::max(1, std::min((int)((227 * 1024) / (b + 1024)), 65536 / (th * regs_per_thread(pl.BR * pl.BC * esz / 4))));
+        const double ctas = (double)c.N * cs, waves = std::ceil(ctas / ((double)per_sm * md->sm_count));
+        const double on_sm = std::min((double)per_sm, std::max(1.0, ctas / md->sm_count)) * uc;   // units side by side on an SM
+        const double unit = (double)pl.NB * pl.BR * pl.BC * (0.045 + 0.07 * p.extra / std::max(pl.NB, 1)) * (esz / 8.0 + 0.25);
+        const int rounds = ceil_div(p.npass, p.LT / 32);
+        const double t = waves * std::max(300.0 + 600.0 * rounds + 250.0 * p.nbpt + (cs > 1 ? 350.0 : 0.0), on_sm * unit);
+        if (t < best) { best = t; bv = v; buc = uc; bcs = cs; }
+      }
+    }
+    if (bv < 0) return BI_ERR_UNSUPPORTED;
+    use_variant(pl.var[bv], p);
+    p.W = 0;
+    p.UC = buc; p.CS = bcs;
+    bytes = layout(pl, p, esz, buc, 2 * (buc + 2));
+    grid = (unsigned)(c.N * bcs);
+    threads = (unsigned)(buc * p.LT);
+  }
+  const bool hass = p.nbpt > 1;
+  const int sync = p.LT == 32 ? 0 : (window && p.UC > 1) ? 2 : 1;   // (SYNC_WARP, SYNC_CTA, SYNC_NAMED)
+  const void *kern = esz == 8 ? bi_block_kernel_f64(pl.BR, pl.BC, window, sync, hass)
+                              : bi_block_kernel_f32(pl.BR, pl.BC, window, sync, hass);
+  if (!kern) return BI_ERR_UNSUPPORTED;
+  const int slot = (((pl.BR == 4 ? 0 : pl.BC == 4 ? 1 : 2) * 2 + window) * 3 + sync) * 4 + hass * 2 + (esz == 8);
+  if (!allow_smem(kern, slot, md->device, bytes)) return BI_ERR_CUDA;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = bytes;
+  cfg.stream = c.stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)p.CS;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = p.CS > 1 ? 1 : 0;
+  void *args[1] = {(void *)&p};
+  if (cudaLaunchKernelExC(&cfg, kern, args) != cudaSuccess) {
+    cudaGetLastError();
+    return BI_ERR_CUDA;
+  }
+  mut->launches += 1;
+  // family names: by the class of call the kernels of each family serve
+  const bool f64 = esz == 8;
+  if (!window) mut->last_kernel = f64 ? "cta_filter_f64" : "cta_filter_f32";
+  else if (md->h.has_bdep || (long long)c.N * c.T < 2048)
+    mut->last_kernel = c.algo == BI_ALGO_VMP ? (f64 ? "warp_vmp_f64" : "warp_vmp_f32") : (f64 ? "warp_mmp_f64" : "warp_mmp_f32");
+  else
+    mut->last_kernel = c.algo == BI_ALGO_VMP ? (f64 ? "batch_vmp_f64" : "batch_vmp_f32") : (f64 ? "batch_mmp_f64" : "batch_mmp_f32");
+  return BI_OK;
+}

@@ -307,6 +307,7 @@ int run_soft_t(const bi_model *model, int algo, int N, int T, const float *obs_s
     BiMember &mm = sh.h.mem[k];
     mm.logA = w + off_pack[k];
     mm.logA_tile = tile && k == 0 ? w + off_tile : nullptr;
+    mm.logA_blk = nullptr;
     mm.logA_T = k == kpair ? w + off_packT : nullptr;
     mm.cmask = nullptr; mm.cvals = nullptr; mm.coff = nullptr;   // (the slices formed above are dense)
     mm.gstride = (int64_t)T * g.P_pad;
@@ -317,6 +318,7 @@ int run_soft_t(const bi_model *model, int algo, int N, int T, const float *obs_s
   }
   // (a group of one modality is its own pre-summed table: the shadow's T per-agent slices)
   sh.soft_shadow = 1;
+  sh.blk_plan[0] = sh.blk_plan[1] = nullptr;
   sh.pair_ok = kpair >= 0 || (model->pair_ok && sizeof(R) == 8 && algo == BI_ALGO_FILTER);
   // (the pair filtering kernel needs the transposed slices formed above, or no pair at all; the pair
   // window kernel reads rows only)

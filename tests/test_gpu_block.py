@@ -1,0 +1,79 @@
+"""The block kernels (a team of threads per agent and step, every thread a block of the summed slices in
+registers) at the sizes where a plan can go wrong: one state more or less than a block, blocks left over for
+shared memory, teams of one and of several warps, windows over one CTA and over a cluster, every kind of
+prefix (groups of two to four factors), transitions with several parents."""
+import numpy as np
+import pytest
+
+from biwl import Workload, make_model, sample_streams
+from parity import check_workload
+
+pytestmark = pytest.mark.gpu
+
+
+def _workload(seed, n, dep, N, T, K, bdep=None, G=1):
+    rng = np.random.default_rng(seed)
+    m = [int(rng.integers(2, 7)) for _ in dep]
+    U = [int(rng.integers(1, 4)) for _ in n]
+    A, B, D = make_model(rng, n, m, dep, U, G, d_alpha=1.0, bdep=bdep)
+    obs, act = sample_streams(rng, n, m, dep, U, G, A, B, D, N, T, bdep=bdep)
+    return Workload(name="block", algo="filter", n=np.asarray(n, np.int32), m=np.asarray(m, np.int32), dep=dep,
+                    U=np.asarray(U, np.int32), G=G, A=A, B=B, D=D, N=N, T=T, K=K, obs=obs, act=act, bdep=bdep)
+
+
+FILTER = {
+    "below_a_block": ([7, 3, 3], [[0, 1, 2]]),
+    "one_block": ([8, 4, 2], [[0, 1, 2]]),
+    "a_state_over": ([9, 5, 7], [[0, 1, 2], [1]]),
+    "rank4_prefixes": ([2, 9, 3, 13], [[0, 1, 2, 3], [2, 0], [1]]),
+    "several_groups": ([17, 8, 25, 6], [[0, 1], [1, 2, 3], [0, 2], [3, 0, 1], [2]]),
+    "unobserved_factors": ([5, 1, 32, 7, 4], [[0, 2, 3], [1, 2]]),
+    "shared_memory_blocks": ([32, 31, 30], [[0, 1, 2], [2]]),
+}
+
+
+@pytest.mark.parametrize("N", [1, 37])
+@pytest.mark.parametrize("case", sorted(FILTER))
+def test_filtering(case, N):
+    n, dep = FILTER[case]
+    print(check_workload(_workload(10 + N, n, dep, N=N, T=4, K=7), "filter"))
+
+
+def test_filtering_large_batches_share_a_cta():
+    print(check_workload(_workload(3, [5, 4, 3], [[0, 1, 2], [1, 0, 2]], N=3701, T=2, K=3), "filter",
+                         agents=range(0, 3701, 97)))
+
+
+WINDOW = {   # (n, dep, T): one CTA, idle steps in the last one of a cluster, the longest window, blocks in shared memory
+    "one_step": ([9, 5, 7], [[0, 1, 2]], 1),
+    "one_cta": ([3, 4, 2, 5], [[0, 1, 2], [1, 3]], 9),
+    "ragged_cluster": ([9, 6, 12, 4], [[0, 1], [1, 2, 3], [0, 1, 2]], 13),
+    "longest": ([4, 3, 5], [[0, 1, 2], [2, 1]], 64),
+    "rank4": ([4, 6, 7, 5], [[0, 1, 2, 3]], 6),
+    "shared_memory_blocks": ([18, 29, 11], [[0, 1, 2], [0, 2]], 10),
+}
+
+
+@pytest.mark.parametrize("algo", ["vmp", "mmp"])
+@pytest.mark.parametrize("case", sorted(WINDOW))
+def test_windows(case, algo):
+    n, dep, T = WINDOW[case]
+    print(check_workload(_workload(20, n, dep, N=5, T=T, K=6), algo))
+
+
+@pytest.mark.parametrize("algo", ["filter", "vmp", "mmp"])
+def test_models_of_their_own(algo):
+    print(check_workload(_workload(30, [6, 5, 9], [[0, 1, 2], [2, 1]], N=9, T=7, K=5, G=9), algo))
+
+
+@pytest.mark.parametrize("algo", ["filter", "vmp"])
+@pytest.mark.parametrize("bdep", [[[0, 1], [1, 2], [2, 0]], [[2], [0, 1, 2], [1, 2]], [[1, 0, 2], [2, 1], [2]]])
+def test_transitions_with_several_parents(bdep, algo):
+    print(check_workload(_workload(40, [9, 4, 7], [[0, 1], [1, 2, 0]], N=7, T=6, K=5, bdep=bdep), algo))
+
+
+@pytest.mark.parametrize("algo", ["filter", "vmp", "mmp"])
+def test_float32(algo):
+    # (dense and few iterations: the tolerance of check_workload's strict=False form is not a numerical one)
+    res = check_workload(_workload(50, [9, 5, 7, 6], [[0, 1, 2], [1, 3]], N=21, T=5, K=4), algo, arith="f32", strict=False)
+    assert res["q_max_err"] < 1e-3, res   # four undamped float32 iterations: 1e-6 of the logits' sums, amplified below 1e3
