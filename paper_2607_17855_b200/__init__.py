@@ -15,6 +15,7 @@ from typing import List, Optional, Sequence
 from .build import LIB, build  # noqa: F401
 
 _lib = None
+_fns = {}   # the inference calls by name, filled when the library is loaded
 
 BI_OK = 0
 ERRORS = {0: "BI_OK", -1: "BI_ERR_INVALID_ARG", -2: "BI_ERR_SHAPE", -3: "BI_ERR_UNSUPPORTED",
@@ -102,6 +103,9 @@ def lib():
         L.bi_filter_static.argtypes = [ctypes.POINTER(_Desc), ctypes.c_int32, ctypes.c_int32, ctypes.c_void_p,
                                        ctypes.c_void_p, ctypes.c_int32, ctypes.c_void_p, ctypes.c_void_p,
                                        ctypes.c_void_p, ctypes.c_void_p]
+        for name in ("bi_filter", "bi_filter_from", "bi_filter_continue", "bi_vmp", "bi_mmp", "bi_vmp_warm", "bi_mmp_warm",
+                     "bi_vmp_from", "bi_mmp_from", "bi_filter_soft", "bi_vmp_soft", "bi_mmp_soft"):
+            _fns[name] = getattr(L, name)
         _lib = L
     return _lib
 
@@ -111,10 +115,29 @@ def _i32(vals):
     return arr
 
 
+_raw_stream = None
+
+
 def _stream_ptr(stream=None):
-    import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    """Address of the given stream, or of the current device's current one.  (A call on a single small agent
+    takes the GPU a few microseconds, so the way there is kept short: no stream object is made.)"""
+    global _raw_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None:
+        import torch
+        torch.cuda.current_stream()   # (initialises CUDA)
+        get, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        _raw_stream = (lambda: get(device())) if get and device else (lambda: torch.cuda.current_stream().cuda_stream)
+    return _raw_stream()
+
+
+def _ptr(t):
+    return t.data_ptr() if t is not None else None
+
+
+def _act_ptr(act):
+    return act.data_ptr() if act is not None and act.numel() > 0 else None
 
 
 class Model:
@@ -178,18 +201,16 @@ class Model:
             pass
 
     # ---- inference -----------------------------------------------------------
-    def _run(self, name, obs, act, iters, q_out, logq_out, argmax_out, stream):
+    def _out(self, obs, q_out):
+        if q_out is not None:
+            return q_out
         import torch
-        N, T = int(obs.shape[0]), int(obs.shape[1])
-        if q_out is None:
-            q_out = torch.empty((N, T, self.S), dtype=torch.float32, device=obs.device)
-        fn = getattr(lib(), name)
-        rc = fn(self._h, N, T, ctypes.c_void_p(obs.data_ptr()),
-                ctypes.c_void_p(act.data_ptr() if act is not None and act.numel() > 0 else None),
-                int(iters), ctypes.c_void_p(q_out.data_ptr()),
-                ctypes.c_void_p(logq_out.data_ptr() if logq_out is not None else None),
-                ctypes.c_void_p(argmax_out.data_ptr() if argmax_out is not None else None),
-                _stream_ptr(stream))
+        return torch.empty((obs.shape[0], obs.shape[1], self.S), dtype=torch.float32, device=obs.device)
+
+    def _run(self, name, obs, act, iters, q_out, logq_out, argmax_out, stream):
+        q_out = self._out(obs, q_out)
+        rc = _fns[name](self._h, obs.shape[0], obs.shape[1], obs.data_ptr(), _act_ptr(act), int(iters), q_out.data_ptr(),
+                        _ptr(logq_out), _ptr(argmax_out), _stream_ptr(stream))
         if rc != BI_OK:
             raise BiError(rc, name)
         return q_out
@@ -202,17 +223,10 @@ class Model:
                        stream=None):
         """Filtering continued from ``q_prev`` float32 ``[N,S]`` (the belief of the step before
         this window) and ``act_prev`` int32 ``[N,F]`` (the action taken there)."""
-        import torch
-        N, T = int(obs.shape[0]), int(obs.shape[1])
-        if q_out is None:
-            q_out = torch.empty((N, T, self.S), dtype=torch.float32, device=obs.device)
-        rc = lib().bi_filter_from(self._h, N, T, ctypes.c_void_p(obs.data_ptr()),
-                                  ctypes.c_void_p(act.data_ptr() if act is not None and act.numel() > 0 else None),
-                                  ctypes.c_void_p(q_prev.data_ptr()), ctypes.c_void_p(act_prev.data_ptr()),
-                                  int(iters), ctypes.c_void_p(q_out.data_ptr()),
-                                  ctypes.c_void_p(logq_out.data_ptr() if logq_out is not None else None),
-                                  ctypes.c_void_p(argmax_out.data_ptr() if argmax_out is not None else None),
-                                  _stream_ptr(stream))
+        q_out = self._out(obs, q_out)
+        rc = _fns["bi_filter_from"](self._h, obs.shape[0], obs.shape[1], obs.data_ptr(), _act_ptr(act), q_prev.data_ptr(),
+                                    act_prev.data_ptr(), int(iters), q_out.data_ptr(), _ptr(logq_out), _ptr(argmax_out),
+                                    _stream_ptr(stream))
         if rc != BI_OK:
             raise BiError(rc, "bi_filter_from")
         return q_out
@@ -222,17 +236,10 @@ class Model:
         """Filtering continued from the belief this handle kept from its previous filtering call
         (full precision: consecutive blocks equal the single call bit for bit); ``act_prev`` int32
         ``[N,F]`` is the action taken at that call's last step."""
-        import torch
-        N, T = int(obs.shape[0]), int(obs.shape[1])
-        if q_out is None:
-            q_out = torch.empty((N, T, self.S), dtype=torch.float32, device=obs.device)
-        rc = lib().bi_filter_continue(self._h, N, T, ctypes.c_void_p(obs.data_ptr()),
-                                      ctypes.c_void_p(act.data_ptr() if act is not None and act.numel() > 0 else None),
-                                      ctypes.c_void_p(act_prev.data_ptr()), int(iters),
-                                      ctypes.c_void_p(q_out.data_ptr()),
-                                      ctypes.c_void_p(logq_out.data_ptr() if logq_out is not None else None),
-                                      ctypes.c_void_p(argmax_out.data_ptr() if argmax_out is not None else None),
-                                      _stream_ptr(stream))
+        q_out = self._out(obs, q_out)
+        rc = _fns["bi_filter_continue"](self._h, obs.shape[0], obs.shape[1], obs.data_ptr(), _act_ptr(act),
+                                        act_prev.data_ptr(), int(iters), q_out.data_ptr(), _ptr(logq_out),
+                                        _ptr(argmax_out), _stream_ptr(stream))
         if rc != BI_OK:
             raise BiError(rc, "bi_filter_continue")
         return q_out
@@ -246,16 +253,9 @@ class Model:
         return self._run("bi_mmp", obs, act, iters, q_out, logq_out, argmax_out, stream)
 
     def _run_warm(self, name, obs, act, q_init, iters, q_out, logq_out, argmax_out, stream):
-        import torch
-        N, T = int(obs.shape[0]), int(obs.shape[1])
-        if q_out is None:
-            q_out = torch.empty((N, T, self.S), dtype=torch.float32, device=obs.device)
-        rc = getattr(lib(), name)(self._h, N, T, ctypes.c_void_p(obs.data_ptr()),
-                                  ctypes.c_void_p(act.data_ptr() if act is not None and act.numel() > 0 else None),
-                                  ctypes.c_void_p(q_init.data_ptr()), int(iters), ctypes.c_void_p(q_out.data_ptr()),
-                                  ctypes.c_void_p(logq_out.data_ptr() if logq_out is not None else None),
-                                  ctypes.c_void_p(argmax_out.data_ptr() if argmax_out is not None else None),
-                                  _stream_ptr(stream))
+        q_out = self._out(obs, q_out)
+        rc = _fns[name](self._h, obs.shape[0], obs.shape[1], obs.data_ptr(), _act_ptr(act), q_init.data_ptr(), int(iters),
+                        q_out.data_ptr(), _ptr(logq_out), _ptr(argmax_out), _stream_ptr(stream))
         if rc != BI_OK:
             raise BiError(rc, name)
         return q_out
@@ -274,19 +274,11 @@ class Model:
         ``q_prev`` float32 ``[N,S]`` and ``act_prev`` int32 ``[N,F]``."""
         if algo == "filter":
             return self.bi_filter_from(obs, act, q_prev, act_prev, iters, q_out, logq_out, argmax_out, stream)
-        import torch
-        N, T = int(obs.shape[0]), int(obs.shape[1])
-        if q_out is None:
-            q_out = torch.empty((N, T, self.S), dtype=torch.float32, device=obs.device)
+        q_out = self._out(obs, q_out)
         name = "bi_vmp_from" if algo == "vmp" else "bi_mmp_from"
-        rc = getattr(lib(), name)(self._h, N, T, ctypes.c_void_p(obs.data_ptr()),
-                                  ctypes.c_void_p(act.data_ptr() if act is not None and act.numel() > 0 else None),
-                                  ctypes.c_void_p(q_prev.data_ptr()), ctypes.c_void_p(act_prev.data_ptr()),
-                                  ctypes.c_void_p(q_init.data_ptr() if q_init is not None else None), int(iters),
-                                  ctypes.c_void_p(q_out.data_ptr()),
-                                  ctypes.c_void_p(logq_out.data_ptr() if logq_out is not None else None),
-                                  ctypes.c_void_p(argmax_out.data_ptr() if argmax_out is not None else None),
-                                  _stream_ptr(stream))
+        rc = _fns[name](self._h, obs.shape[0], obs.shape[1], obs.data_ptr(), _act_ptr(act), q_prev.data_ptr(),
+                        act_prev.data_ptr(), _ptr(q_init), int(iters), q_out.data_ptr(), _ptr(logq_out),
+                        _ptr(argmax_out), _stream_ptr(stream))
         if rc != BI_OK:
             raise BiError(rc, name)
         return q_out
