@@ -366,7 +366,8 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
   if (const char *e = getenv("BI_TEST_DROP_COPY")) md->test_drop_copy = atoi(e) > 0 ? atoi(e) : 0;   // testing aids,
   if (const char *e = getenv("BI_TEST_FAMILY")) {                                                  // read here only
     md->test_family = !strcmp(e, "warp") ? BI_FAMILY_WARP : !strcmp(e, "generic") ? BI_FAMILY_GENERIC
-                      : !strcmp(e, "cta") ? BI_FAMILY_CTA : !strcmp(e, "batch") ? BI_FAMILY_BATCH : BI_FAMILY_ANY;
+                      : !strcmp(e, "cta") ? BI_FAMILY_CTA : !strcmp(e, "batch") ? BI_FAMILY_BATCH
+                      : !strcmp(e, "block") ? BI_FAMILY_BLOCK : BI_FAMILY_ANY;
   }
   md->last_kernel = "";
   md->arith = arith;
@@ -923,6 +924,7 @@ int bi_dispatch(const BiCall &c, bi_model *mut) {
     // shared memory.
     if (rc == BI_ERR_UNSUPPORTED && c.algo == BI_ALGO_FILTER) rc = bi_launch_cta_filter(c, mut);
   }
+  if (only == BI_FAMILY_BLOCK) rc = bi_launch_block(c, mut);
   if (only == BI_FAMILY_CTA && c.algo == BI_ALGO_FILTER) rc = bi_launch_cta_filter(c, mut);
   if (only == BI_FAMILY_BATCH) {   // the batched window kernels and what follows them
     rc = bi_launch_batch(c, mut);

@@ -115,7 +115,7 @@ __device__ __forceinline__ void bi_exp_tab_init(float *, int) {}
 //   Permission to use, copy, modify, and distribute this software is freely granted,
 //   provided that this notice is preserved.
 // ---- table-driven exp and log in float64, for kernels whose pace is set by FP64 instructions ----
-// Tables in shared memory, filled by the block (bi_fast_tabs_init, then a block-wide barrier).
+// Tables in shared memory, copied by the block (bi_fast_tabs_init, then a block-wide barrier).
 //   exp: x = k ln2/512 + r with k = round(x 512/ln 2), |r| <= ln2/1024; exp(x) = 2^(k >> 9) *
 //        2^((k & 511)/512) * (1 + r + r^2/2 + r^3/6): 7 operations, within 1e-14 relative.  k ln2/512 is
 //        exact inside the fused multiply-add, so one constant serves the reduction (error |x| 1.1e-16).
@@ -124,14 +124,25 @@ __device__ __forceinline__ void bi_exp_tab_init(float *, int) {}
 //        9 operations (25 for the table-free form below), absolute error below 1e-15 for the
 //        probabilities and normalisers it is used on (|k| <= 54).
 constexpr int BI_EXP_TAB = 512, BI_EXP_BITS = 9, BI_LOG_TAB = 128;
-__device__ __forceinline__ void bi_fast_tabs_init(double *exp_tab, double2 *log_tab, int tid, int nthreads) {
-  for (int j = tid; j < BI_EXP_TAB; j += nthreads) exp_tab[j] = exp2((double)j * (1.0 / BI_EXP_TAB));
+// (Both are computed once, when the handle is made -- bi_fast_tabs_compute -- and copied by every block: computing
+// them in each block took a microsecond of the single-agent calls and of every block of the window kernels.)
+__device__ __forceinline__ void bi_exp_tab_copy(double *exp_tab, const double *__restrict__ src, int tid, int nthreads) {
+  for (int j = tid; j < BI_EXP_TAB / 2; j += nthreads)
+    reinterpret_cast<double2 *>(exp_tab)[j] = __ldg(reinterpret_cast<const double2 *>(src) + j);
+}
+__device__ __forceinline__ void bi_fast_tabs_init(double *exp_tab, double2 *log_tab, const double *__restrict__ src, int tid, int nthreads) {
+  bi_exp_tab_copy(exp_tab, src, tid, nthreads);
+  for (int j = tid; j < BI_LOG_TAB; j += nthreads) log_tab[j] = __ldg(reinterpret_cast<const double2 *>(src + BI_EXP_TAB) + j);
+}
+__device__ __forceinline__ void bi_fast_tabs_init(float *, float2 *, const double *, int, int) {}
+__device__ __forceinline__ void bi_fast_tabs_compute(double *dst, int tid, int nthreads) {
+  for (int j = tid; j < BI_EXP_TAB; j += nthreads) dst[j] = exp2((double)j * (1.0 / BI_EXP_TAB));
   for (int j = tid; j < BI_LOG_TAB; j += nthreads) {
     const double c = 1.0 + ((double)j + 0.5) * (1.0 / BI_LOG_TAB);
-    log_tab[j] = make_double2(1.0 / c, log(c));
+    dst[BI_EXP_TAB + 2 * j] = 1.0 / c;
+    dst[BI_EXP_TAB + 2 * j + 1] = log(c);
   }
 }
-__device__ __forceinline__ void bi_fast_tabs_init(float *, float2 *, int, int) {}
 // exact zero below -700 (the true value is below 1e-304)
 __device__ __forceinline__ double bi_exp_fast(double x, const double *__restrict__ tab) {
   const double KL = 738.6598609351493, LK = 0.0013538030870311431, MAGIC = 6755399441055744.0;

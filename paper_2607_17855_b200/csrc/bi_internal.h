@@ -10,7 +10,7 @@
 #define BI_MAX_GROUPS BI_MAX_M
 
 enum { BI_ALGO_FILTER = 0, BI_ALGO_VMP = 1, BI_ALGO_MMP = 2 };
-enum { BI_FAMILY_ANY = 0, BI_FAMILY_WARP = 1, BI_FAMILY_GENERIC = 2, BI_FAMILY_CTA = 3, BI_FAMILY_BATCH = 4 };
+enum { BI_FAMILY_ANY = 0, BI_FAMILY_WARP = 1, BI_FAMILY_GENERIC = 2, BI_FAMILY_CTA = 3, BI_FAMILY_BATCH = 4, BI_FAMILY_BLOCK = 5 };
 
 static __host__ __device__ inline int bi_pad4(int x) { return (x + 3) & ~3; }
 // Row stride in shared memory for rows of npad elements (npad a multiple of 4, elements of esize
@@ -142,8 +142,8 @@ struct bi_model {
   void *carry;      // last belief of the latest filtering call, [carry_N][S] in the arithmetic type, or NULL
   size_t carry_bytes;
   int carry_N;      // agents of that call (0: none yet)
-  // Testing aid, read from the environment once, when the handle is made (BI_TEST_FAMILY = "batch", "cta", "warp"
-  // or "generic"): calls skip the kernel families ahead of the named one, so that the general kernels can
+  // Testing aid, read from the environment once, when the handle is made (BI_TEST_FAMILY = "block", "batch", "cta",
+  // "warp" or "generic"): calls skip the kernel families ahead of the named one, so that the general kernels can
   // be checked on inputs small enough for the oracle.  0 = normal dispatch.
   int test_family;
   // Testing aid (BI_TEST_DROP_COPY = n, read when the handle is made): the next n batched window calls

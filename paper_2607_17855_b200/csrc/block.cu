@@ -5,6 +5,7 @@
 #include <cstring>
 #include <vector>
 
+#include "bi_device.cuh"
 #include "block.h"
 
 const void *bi_block_kernel_f64(int BR, int BC, bool window, int sync, bool hass);
@@ -77,14 +78,7 @@ __global__ void bi_pack_block_kernel(PackBlk p) {
   }
   ((R *)p.dst)[e] = out;
 }
-__global__ void bi_exp_table_kernel(double *tab) {
-  for (int j = threadIdx.x; j < 512; j += blockDim.x) tab[j] = exp2((double)j * (1.0 / 512));
-  for (int j = threadIdx.x; j < 128; j += blockDim.x) {   // the pairs bi_log_fast reads
-    const double c = 1.0 + ((double)j + 0.5) * (1.0 / 128);
-    tab[512 + 2 * j] = 1.0 / c;
-    tab[512 + 2 * j + 1] = log(c);
-  }
-}
+__global__ void bi_exp_table_kernel(double *tab) { bi_fast_tabs_compute(tab, threadIdx.x, blockDim.x); }
 
 // Elements of one outcome's slice of group gi in block order (0: the model has no block plan).
 int bi_block_slice_elems(const bi_model *md, int gi) {
@@ -435,7 +429,7 @@ bool build_plan(const bi_model *md, bool window, HostPlan &hp) {
       const int wide = std::max(full, 32 * one.npass);
       for (int uc : {1, 2, 3, 4, 6, 12})
         for (int want : {full, wide}) {
-          if (!window && uc > 1) continue;
+          if (!window && uc > 4) continue;   // (filtering: teams of which up to four share an SM)
           const int LT = std::min(want, p.max_th / uc / 32 * 32);
           bool have = LT < 32 || p.nv == kMaxVariants;
           for (int v = 0; v < p.nv; ++v) have = have || p.var[v].LT == LT;
@@ -694,8 +688,25 @@ int bi_launch_block(const BiCall &c, bi_model *mut) {
   unsigned grid = 0, threads = 0;
   size_t bytes = 0;
   if (!window) {
-    // a warp per pass while the batch leaves the machine that much room (the second variant, if there is one)
-    use_variant(pl.var[pl.nv > 1 && (long long)c.N * pl.var[1].LT <= 8 * 32 * md->sm_count ? 1 : 0], p);
+    // Team size: cycles of an iteration (a phase for each round of blocks and of passes), plus what the teams
+    // beside it on the SM add, times the waves of teams.  (Five coupled factors, 204 blocks, 256 agents: teams
+    // of 224 threads in two waves 486 us, of 192 and 128 side by side 436 and 420 us, of 96 526 us.)
+    double best = 1e300;
+    int v0 = 0;
+    for (int v = 0; v < pl.nv; ++v) {
+      use_variant(pl.var[v], p);
+      p.W = 1;
+      const size_t b = layout(pl, p, esz, 1, 1);
+      if (b > budget) continue;
+      const int per_sm = std::max(1, std::min((int)((227 * 1024) / (b + 1024)), 65536 / (p.LT * regs_per_thread(pl.BR * pl.BC * esz / 4))));
+      const int waves = ceil_div(c.N, per_sm * md->sm_count), on_sm = std::min(per_sm, ceil_div(c.N, md->sm_count));
+      const double alone = 900.0 + 900.0 * ceil_div(p.npass, p.LT / 32) + 600.0 * p.nbpt;
+      const double beside = pl.NB / 32.0 * pl.BR * pl.BC * 2.6 + 120.0 * p.npass;
+      const double t = waves * (alone + (on_sm - 1) * beside);
+      if (t < best) { best = t; v0 = v; }
+    }
+    if (best >= 1e300) return BI_ERR_UNSUPPORTED;
+    use_variant(pl.var[v0], p);
     // agents per CTA (one-warp teams): one while the batch fits the machine anyway, so that no SM gets
     // four more warps than another; four for large batches, which share the CTA's exponential table
     p.W = p.LT == 32 ? (c.N > 24 * md->sm_count ? 4 : 1) : 1;
@@ -726,7 +737,7 @@ int bi_launch_block(const BiCall &c, bi_model *mut) {
         const double on_sm = std::min((double)per_sm, std::max(1.0, ctas / md->sm_count)) * uc;   // units side by side on an SM
         const double unit = (double)pl.NB * pl.BR * pl.BC * (0.045 + 0.07 * p.extra / std::max(pl.NB, 1)) * (esz / 8.0 + 0.25);
         const int rounds = ceil_div(p.npass, p.LT / 32);
-        const double t = waves * std::max(300.0 + 600.0 * rounds + 250.0 * p.nbpt + (cs > 1 ? 350.0 : 0.0), on_sm * unit);
+        const double t = waves * std::max(300.0 + 600.0 * rounds + 450.0 * p.nbpt + (cs > 1 ? 350.0 : 0.0), on_sm * unit);
         if (t < best) { best = t; bv = v; buc = uc; bcs = cs; }
       }
     }

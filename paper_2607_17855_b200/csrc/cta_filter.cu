@@ -257,7 +257,7 @@ bi_cta_filter_kernel(const BiDev *__restrict__ mdp, int T, const int32_t *__rest
                      const int32_t *__restrict__ act, const float *q_prev,
                      const int32_t *__restrict__ act_prev, const void *carry_in, void *carry_out, double lambda,
                      int K, float *q_out, float *__restrict__ logq_out, int32_t *__restrict__ argmax_out,
-                     const CtaGeom sm) {
+                     const double *__restrict__ exp_src, const CtaGeom sm) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   R *smem = reinterpret_cast<R *>(smem_raw);
   {  // the model's description, read from shared memory from here on
@@ -317,7 +317,7 @@ bi_cta_filter_kernel(const BiDev *__restrict__ mdp, int T, const int32_t *__rest
   const double *exp_tab = nullptr;
   if constexpr (sizeof(R) == 8) {
     double *tab = reinterpret_cast<double *>(smem + sm.exptab);
-    for (int j = tid; j < tile3_f64::EXP_TAB; j += NT) tab[j] = exp2((double)j * (1.0 / tile3_f64::EXP_TAB));
+    bi_exp_tab_copy(tab, exp_src, tid, NT);
     exp_tab = tab;
   }
   __syncthreads();
@@ -704,7 +704,7 @@ int launch_cta_filter_t(const BiCall &c, bi_model *mut) {
       cudaSuccess)
     return BI_ERR_CUDA;
   kern<<<c.N, NT, sm.total_bytes, c.stream>>>(md->d, c.T, c.obs, c.act, c.q_prev, c.act_prev, c.carry_in, c.carry_out, c.lambda, c.K, c.q_out,
-                                               c.logq_out, c.argmax_out, sm);
+                                               c.logq_out, c.argmax_out, md->exp_tab, sm);
   if (cudaGetLastError() != cudaSuccess) return BI_ERR_CUDA;
   mut->launches += 1;
   mut->last_kernel = sizeof(R) == 8 ? "cta_filter_f64" : "cta_filter_f32";

@@ -52,6 +52,7 @@ struct PairParams {
   float *q_out, *logq_out;
   int32_t *argmax_out;
   uint32_t *status;
+  const double *exp_tab;   // the handle's tables (bi_fast_tabs_compute)
 };
 
 template <int LPU>
@@ -93,7 +94,7 @@ __global__ void __launch_bounds__(WARPS * 32) bi_pair_filter_kernel(const PairPa
   __shared__ __align__(16) R exp_tab[EXP_TAB];
   __shared__ __align__(16) R sm_q[WARPS * UPW][QS];
   __shared__ __align__(16) R sm_e[WARPS * UPW][2 * LPU];   // e_a, e_b of the pair
-  for (int j = threadIdx.x; j < EXP_TAB; j += blockDim.x) exp_tab[j] = exp2((double)j * (1.0 / EXP_TAB));
+  bi_exp_tab_copy(exp_tab, p.exp_tab, threadIdx.x, blockDim.x);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int unit = lane / LPU, u = lane % LPU;
   int agent = (blockIdx.x * WARPS + warp) * UPW + unit;
@@ -350,7 +351,7 @@ int bi_launch_pair_filter(const BiCall &c, bi_model *mut) {
   }
   p.obs = c.obs; p.act = c.act; p.act_prev = c.act_prev; p.q_prev = c.q_prev;
   p.carry_in = (const R *)c.carry_in; p.carry_out = (R *)c.carry_out;
-  p.q_out = c.q_out; p.logq_out = c.logq_out; p.argmax_out = c.argmax_out; p.status = h.status;
+  p.q_out = c.q_out; p.logq_out = c.logq_out; p.argmax_out = c.argmax_out; p.status = h.status; p.exp_tab = md->exp_tab;
   int rc;
   if (nmax <= 4) rc = launch<4>(p, c.stream);
   else if (nmax <= 8) rc = launch<8>(p, c.stream);

@@ -57,6 +57,7 @@ struct PairWinParams {
   float *q_out, *logq_out;
   int32_t *argmax_out;
   uint32_t *status;
+  const double *exp_tab;   // the handle's tables (bi_fast_tabs_compute)
   int32_t units;   // step slots per CTA (whole warps)
   // staged slices of the two-factor groups: `nar` rows of `ls` entries each (the groups' largest first
   // axis; their largest padded second axis plus one: an odd stride, so rows and columns are both read
@@ -124,7 +125,7 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 320 ? 2 : 1) bi_pair_window_kern
   R *Ls = xpv + (DAMPED ? p.units * slot_sz : 0);               // [units][ng][LPU][LS] the pair groups' summed slices, row-major
   const R lam = p.lambda, oml = 1.0 - lam;
   int32_t *aoff = reinterpret_cast<int32_t *>(Ls + (((size_t)p.units * p.ng * NAR * LS + 1) & ~(size_t)1));   // [units][F][2] matrix offsets of the two edges
-  for (int j = threadIdx.x; j < EXP_TAB; j += blockDim.x) exp_tab[j] = exp2((double)j * (1.0 / EXP_TAB));
+  bi_exp_tab_copy(exp_tab, p.exp_tab, threadIdx.x, blockDim.x);
 
   const int agent = blockIdx.x, g = p.G == 1 ? 0 : agent;
   const int tl = threadIdx.x / LPU, s = threadIdx.x % LPU;
@@ -369,7 +370,7 @@ int bi_launch_pair_window(const BiCall &c, bi_model *mut) {
     p.ls = std::max(p.ls, p.npb[gj] + 1);
   }
   p.obs = c.obs; p.act = c.act; p.q_init = c.q_init; p.lnprior = (const R *)c.lnprior;
-  p.q_out = c.q_out; p.logq_out = c.logq_out; p.argmax_out = c.argmax_out; p.status = h.status;
+  p.q_out = c.q_out; p.logq_out = c.logq_out; p.argmax_out = c.argmax_out; p.status = h.status; p.exp_tab = md->exp_tab;
   int rc;
   if (nmax <= 4) rc = launch<4>(p, md, c.stream);
   else if (nmax <= 8) rc = launch<8>(p, md, c.stream);

@@ -38,6 +38,7 @@ struct Tile3Params {
   float *q_out, *logq_out;
   int32_t *argmax_out;
   uint32_t *status;
+  const double *exp_tab;     // the handle's tables (bi_fast_tabs_compute)
   double lambda;             // damping step (1 = plain update)
   int32_t unit_shift;        // softmax shifts per agent even where a warp-wide one would do (see BiDev::status)
 };
@@ -96,5 +97,5 @@ static inline void bi_tile3_fill_params(const BiCall &c, Tile3Params &p) {
   p.N = c.N; p.T = c.T; p.K = c.K; p.M = h.M; p.S = h.S; p.G = h.G;
   p.obs = c.obs; p.act = c.act; p.q_out = c.q_out; p.logq_out = c.logq_out;
   p.q_prev = c.q_prev; p.act_prev = c.act_prev; p.carry_in = c.carry_in; p.carry_out = c.carry_out; p.q_init = c.q_init; p.lnprior = c.lnprior; p.lambda = c.lambda; p.F = c.model->h.F;
-  p.argmax_out = c.argmax_out; p.status = h.status;
+  p.argmax_out = c.argmax_out; p.status = h.status; p.exp_tab = md->exp_tab;
 }

@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(32) bi_tile3_filter_f64_kernel(const Tile3Para
   __shared__ __align__(16) R sm_tp[UPW][LPU * G::TPR + 2];
   __shared__ __align__(16) R sm_se[UPW][G::SE];
   const int lane = threadIdx.x;
-  for (int j = lane; j < EXP_TAB; j += 32) exp_tab[j] = exp2((double)j * (1.0 / EXP_TAB));
+  bi_exp_tab_copy(exp_tab, p.exp_tab, lane, 32);
   // One warp-wide reduction finds the softmax shift of all the warp's agents at once, unless the model's
   // logits can lie too far apart for a common shift (many modalities, entries of A above 1, observation
   // vectors with the caller's weights): then every agent takes its own.

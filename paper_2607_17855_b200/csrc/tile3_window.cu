@@ -88,7 +88,7 @@ bi_tile3_window_kernel(const Tile3Params p, const WindowGeom geo) {
   using R2 = typename std::conditional<sizeof(R) == 8, double2, float2>::type;
   __shared__ __align__(16) R exp_tab[sizeof(R) == 8 ? BI_EXP_TAB : 2];
   __shared__ __align__(16) R2 log_tab[sizeof(R) == 8 ? BI_LOG_TAB : 1];
-  bi_fast_tabs_init(exp_tab, log_tab, (int)threadIdx.x, (int)blockDim.x);
+  bi_fast_tabs_init(exp_tab, log_tab, p.exp_tab, (int)threadIdx.x, (int)blockDim.x);
   int rank = 0;
   if (CLUSTER) rank = (int)cg::this_cluster().block_rank();
   const int agent = blockIdx.x / geo.CS;
