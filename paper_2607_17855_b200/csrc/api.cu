@@ -11,7 +11,6 @@
 
 // the block kernels' share of the packing layer (block.cu)
 void bi_block_choose_shape(bi_model *md);
-int bi_block_slice_elems(const bi_model *md, int gi);
 int bi_block_pack_member(const bi_model *md, int gi, const float *src, int m, const int64_t *sstride, int P, void *dst,
                          cudaStream_t stream);
 void bi_block_build(bi_model *md, std::vector<unsigned char> &blob);

@@ -664,6 +664,15 @@ bool allow_smem(const void *kern, int slot, int device, size_t bytes) {
 
 }  // namespace
 
+// A model with zeros in A amplifies a rounding by up to 1e9 within sixteen iterations, and a trajectory carries
+// the result on from step to step: in float32, and in float64 over more than two filtered steps, another
+// order of summation gives other beliefs (measured: one in five such trajectories differs in the first
+// digit from the CTA kernel's).  Those calls stay with the kernels that have served them, bit for bit.
+bool bi_block_serves(const bi_model *md, int algo, int T) {
+  const bool window = algo != BI_ALGO_FILTER;
+  return md->blk_plan[window ? 1 : 0] && !(md->has_zeros && (md->arith == BI_ARITH_F32 || (!window && T > 2)));
+}
+
 // Any model whose groups span at most four factors (transitions over at most three parents in window
 // calls), either arithmetic, as long as a step's blocks fit the register file and shared memory of an SM
 // (window calls: of a cluster); BI_ERR_UNSUPPORTED otherwise.
@@ -673,11 +682,7 @@ int bi_launch_block(const BiCall &c, bi_model *mut) {
   const Plan *plp = static_cast<const Plan *>(md->blk_plan[window ? 1 : 0]);
   if (!plp || !plp->ok) return BI_ERR_UNSUPPORTED;
   if (window && md->h.has_bdep && (c.algo == BI_ALGO_MMP || c.lnprior)) return BI_ERR_UNSUPPORTED;
-  // A model with zeros in A amplifies a rounding by up to 1e9 within sixteen iterations, and a trajectory carries
-  // the result on from step to step: in float32, and in float64 over more than two filtered steps, another
-  // order of summation gives other beliefs (measured: one in five such trajectories differs in the first
-  // digit from the CTA kernel's).  Those calls stay with the kernels that have served them, bit for bit.
-  if (md->has_zeros && (md->arith == BI_ARITH_F32 || (!window && c.T > 2))) return BI_ERR_UNSUPPORTED;
+  if (!bi_block_serves(md, c.algo, c.T)) return BI_ERR_UNSUPPORTED;
   if (plp->NB == 0) return BI_ERR_UNSUPPORTED;   // nothing to contract: the CTA kernel's warp per factor does that
   if (window && !md->h.has_bdep && md->batch_unrolled && (long long)c.N * c.T >= 4096) return BI_ERR_UNSUPPORTED;   // (see batch_unrolled)
   const Plan &pl = *plp;

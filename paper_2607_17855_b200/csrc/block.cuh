@@ -341,8 +341,8 @@ __device__ __forceinline__ void finish(const Params &p, const LaneRef &l, int cs
     __syncwarp();
     const int n = __ldg(&cold->n);
     double m = -CUDART_INF;
-#pragma unroll 8
-    for (int r = 0; r < 32; ++r) m = bi_max(m, at<double>(l.ez + 8 * min(r, n - 1)));
+#pragma unroll 4
+    for (int r = 0; r < 2 * ps.w; ++r) m = bi_max(m, at<double>(l.ez + 8 * min(r, n - 1)));
     __syncwarp();
     xs -= m;
   }
@@ -531,16 +531,21 @@ bi_block_filter_kernel(const __grid_constant__ Params p) {
         const int ur = t == 0 ? __ldg(p.act_prev + (size_t)a * p.F + f) : __ldg(p.act + ((size_t)a * (p.T - 1) + (t - 1)) * p.F + f);
         const int u = clamp_flag(ur, p.U[f], p.status, BI_FLAG_ACT_RANGE);
         const R *Xu = (const R *)p.Bfull[f] + (size_t)g * p.Bfull_stride[f] + (size_t)u * n * PB;
-        for (int s = warp; s < n; s += NW) {
+        // eight lanes per next state, four states to a warp (with one warp per state a lone warp spends its time in
+        // reductions)
+        for (int s0 = 4 * warp; s0 < n; s0 += 4 * NW) {
+          const int s = min(s0 + (lane >> 3), n - 1), e8 = lane & 7;
           const R *row = Xu + (size_t)s * PB;
           R acc = (R)0;
 #pragma unroll 4
-          for (int e0 = 0; e0 < PB; e0 += 32) {
-            const int e = min(e0 + lane, PB - 1);
-            acc = fma(__ldg(row + e), e0 + lane < PB ? at<R>(par + e * E) : (R)0, acc);
+          for (int e0 = 0; e0 < PB; e0 += 8) {
+            const int e = min(e0 + e8, PB - 1);
+            acc = fma(__ldg(row + e), e0 + e8 < PB ? at<R>(par + e * E) : (R)0, acc);
           }
-          acc = warp_sum(acc);
-          if (lane == 0) at<double>(cst + (p.qo[f] + s) * 8) = (double)bi_log(bi_max(acc, (R)BI_EPS));
+          acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+          acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+          acc += __shfl_xor_sync(0xffffffffu, acc, 4);
+          if (e8 == 0) at<double>(cst + (p.qo[f] + s) * 8) = (double)bi_log(bi_max(acc, (R)BI_EPS));
         }
         team_sync<SYNC>(LT, team);
       }

@@ -229,6 +229,16 @@ int run_soft_t(const bi_model *model, int algo, int N, int T, const float *obs_s
     off_packT = need;
     need += up256(NT * PT * sizeof(R));
   }
+  // A call that the block kernels serve: their groups' slices are formed in block order instead (a rank-1
+  // group's stay packed; the packed ones of the others follow only if those kernels decline the call).
+  const bool block = !tile && bi_block_serves(model, algo, T) &&
+                     (sizeof(R) == 4 || !(algo == BI_ALGO_FILTER ? model->pair_ok : model->rank2_ok));
+  size_t off_blk[BI_MAX_GROUPS] = {};
+  for (int k = 0; k < h.ngroups && block; ++k)
+    if (h.grp[k].rank >= 2) {
+      off_blk[k] = need;
+      need += up256(NT * bi_block_slice_elems(model, k) * sizeof(R));
+    }
   const size_t off_obs = need;
   need += up256(NT * h.ngroups * sizeof(int32_t));
   const size_t off_desc = need;
@@ -257,19 +267,20 @@ int run_soft_t(const bi_model *model, int algo, int N, int T, const float *obs_s
       return BI_ERR_CUDA;
   int launches = 0;
   // layout 0: every group's packed slices; 1: the lane-interleaved slices of a tile model; 2: the
-  // pair's slices with the axes exchanged
-  auto form = [&](int layout) {
-    for (int k = layout == 2 ? kpair : 0; k < (layout == 1 ? 1 : layout == 2 ? kpair + 1 : h.ngroups); ++k) {
+  // pair's slices with the axes exchanged; 3: block order, packed for groups over one factor
+  auto form = [&](int what) {
+    for (int k = what == 2 ? kpair : 0; k < (what == 1 ? 1 : what == 2 ? kpair + 1 : h.ngroups); ++k) {
       const BiGroup &g = h.grp[k];
+      const int layout = what == 3 && g.rank < 2 ? 0 : what;
       SoftJob J;
       memset(&J, 0, sizeof(J));
       J.nmem = g.mem_end - g.mem_begin;
-      J.P = layout == 1 ? model->tile_P : layout == 2 ? (int)PT : g.P_pad;
+      J.P = layout == 1 ? model->tile_P : layout == 2 ? (int)PT : layout == 3 ? bi_block_slice_elems(model, k) : g.P_pad;
       J.T = T; J.Mtot = Mtot; J.soft = obs_soft;
-      J.dst = w + (layout == 1 ? off_tile : layout == 2 ? off_packT : off_pack[k]);
+      J.dst = w + (layout == 1 ? off_tile : layout == 2 ? off_packT : layout == 3 ? off_blk[k] : off_pack[k]);
       for (int i = 0; i < J.nmem; ++i) {
         const BiMember &mm = h.mem[g.mem_begin + i];
-        J.mem[i].src = layout == 1 ? mm.logA_tile : layout == 2 ? mm.logA_T : mm.logA;
+        J.mem[i].src = layout == 1 ? mm.logA_tile : layout == 2 ? mm.logA_T : layout == 3 ? mm.logA_blk : mm.logA;
         J.mem[i].gstride = h.G == 1 ? 0 : (int64_t)mm.m * J.P;
         J.mem[i].m = mm.m;
         J.mem[i].moff = moff[mm.modality];
@@ -288,7 +299,7 @@ int run_soft_t(const bi_model *model, int algo, int N, int T, const float *obs_s
       ++launches;
     }
   };
-  form(tile ? 1 : 0);
+  form(tile ? 1 : block ? 3 : 0);
   if (kpair >= 0) form(2);
   int32_t *obs_idx = reinterpret_cast<int32_t *>(w + off_obs);
   bi_soft_step_index_kernel<<<256, 256, 0, stream>>>(obs_idx, N, T, h.ngroups);
@@ -307,7 +318,7 @@ int run_soft_t(const bi_model *model, int algo, int N, int T, const float *obs_s
     BiMember &mm = sh.h.mem[k];
     mm.logA = w + off_pack[k];
     mm.logA_tile = tile && k == 0 ? w + off_tile : nullptr;
-    mm.logA_blk = nullptr;
+    mm.logA_blk = block && g.rank >= 2 ? w + off_blk[k] : nullptr;
     mm.logA_T = k == kpair ? w + off_packT : nullptr;
     mm.cmask = nullptr; mm.cvals = nullptr; mm.coff = nullptr;   // (the slices formed above are dense)
     mm.gstride = (int64_t)T * g.P_pad;
@@ -318,7 +329,7 @@ int run_soft_t(const bi_model *model, int algo, int N, int T, const float *obs_s
   }
   // (a group of one modality is its own pre-summed table: the shadow's T per-agent slices)
   sh.soft_shadow = 1;
-  sh.blk_plan[0] = sh.blk_plan[1] = nullptr;
+  if (!block) sh.blk_plan[0] = sh.blk_plan[1] = nullptr;
   sh.pair_ok = kpair >= 0 || (model->pair_ok && sizeof(R) == 8 && algo == BI_ALGO_FILTER);
   // (the pair filtering kernel needs the transposed slices formed above, or no pair at all; the pair
   // window kernel reads rows only)
@@ -347,7 +358,16 @@ int run_soft_t(const bi_model *model, int algo, int N, int T, const float *obs_s
       if (rc == BI_ERR_UNSUPPORTED) rc = bi_launch_generic(c, &sh);
     }
   } else {
-    rc = bi_dispatch(c, &sh);
+    rc = BI_ERR_UNSUPPORTED;
+    if (block && model->test_family == BI_FAMILY_ANY) rc = bi_launch_block(c, &sh);
+    if (rc == BI_ERR_UNSUPPORTED) {
+      if (block) {
+        form(0);
+        if (cudaGetLastError() != cudaSuccess) return BI_ERR_CUDA;
+        sh.blk_plan[0] = sh.blk_plan[1] = nullptr;
+      }
+      rc = bi_dispatch(c, &sh);
+    }
   }
   mut->ws = sh.ws;
   mut->ws_bytes = sh.ws_bytes;
