@@ -232,6 +232,16 @@ __global__ void bi_pack_Bfull_kernel(const float *__restrict__ B, int64_t total,
   logBfull[e] = (R)log(fmax((double)v, 1e-16));
 }
 
+// the logarithms with the last parent's axis padded to npad (zeros): rows of the batched contraction
+template <typename R>
+__global__ void bi_pack_Bedge_kernel(const R *__restrict__ logBfull, int64_t rows, int nlast, int npad, R *out) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= rows * npad) return;
+  const int64_t r = e / npad;
+  const int c = (int)(e - r * npad);
+  out[e] = c < nlast ? logBfull[r * nlast + c] : (R)0;
+}
+
 template <typename R>
 __global__ void bi_pack_D_kernel(const float *__restrict__ D, int G, int n, int npad, uint32_t *wide, R *logD) {
   int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -791,6 +801,16 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
       bi_pack_Bfull_kernel<float><<<gb, threads, 0, stream>>>(desc->B[f], total, n, PB, U, h.status + 1, (float *)bfull, (float *)lbfull);
       bi_pack_D_kernel<float><<<gd, threads, 0, stream>>>(desc->D[f], G, n, npad, h.status + 1, (float *)ld);
     }
+    if (G == 1) {
+      const int nlast = h.n[h.bdep[f][bdep_len[f] - 1]], np = bi_pad4(nlast);
+      const int64_t rows = total / nlast;
+      void *be;
+      if ((rc = dev_alloc(md, &be, (size_t)rows * np * esz)) != BI_OK) break;
+      h.logBedge[f] = be;
+      const unsigned ge = (unsigned)((rows * np + threads - 1) / threads);
+      if (arith == BI_ARITH_F64) bi_pack_Bedge_kernel<double><<<ge, threads, 0, stream>>>((const double *)lbfull, rows, nlast, np, (double *)be);
+      else bi_pack_Bedge_kernel<float><<<ge, threads, 0, stream>>>((const float *)lbfull, rows, nlast, np, (float *)be);
+    }
     if (cudaGetLastError() != cudaSuccess) rc = BI_ERR_CUDA;
   }
   for (int f = 0; f < F && rc == BI_OK && !bdep_len; ++f) {
@@ -902,6 +922,8 @@ int bi_dispatch(const BiCall &c, bi_model *mut) {
     // message: the warp-per-step kernel's lanes sum them, the general kernel where that one does not fit.
     int rc = BI_ERR_UNSUPPORTED;
     if (c.model->test_family == BI_FAMILY_ANY) rc = bi_launch_block(c, mut);
+    if ((c.model->test_family == BI_FAMILY_ANY && rc == BI_ERR_UNSUPPORTED) || c.model->test_family == BI_FAMILY_BATCH)
+      rc = bi_launch_batch(c, mut);
     if (rc == BI_ERR_UNSUPPORTED && c.model->test_family == BI_FAMILY_ANY)
       rc = c.algo == BI_ALGO_FILTER ? bi_launch_cta_filter(c, mut) : bi_launch_warp(c, mut);
     return rc == BI_ERR_UNSUPPORTED ? bi_launch_generic(c, mut) : rc;

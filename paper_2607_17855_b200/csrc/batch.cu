@@ -19,6 +19,7 @@
 // (its accumulators in registers, those of the outer axes in per-thread columns
 // of shared memory, the outer loops an odometer shared by the whole CTA).
 #include <algorithm>
+#include <climits>
 #include <cstring>
 
 #include <type_traits>
@@ -57,11 +58,17 @@ struct BatchMember {
   int64_t gstride;         // elements per agent's model (per-agent models), 0 when shared
   int32_t task0;           // first task slot of this member
   int32_t split;           // unrolled forms: threads per unit (1, 2 or 4), each taking a range of the first axis
+  // Where the messages of each axis go, relative to the unit's row of this member's plane.  (A transition
+  // tensor of a model with several parents per transition is a member too: its first axis is the child's state at
+  // the next step -- the next unit's beliefs, and messages to the next unit's row of a plane of their own.)
+  int32_t edge;            // 0, or 1 + the factor whose transition this is: its "outcome" is the action
+  int64_t oout[BI_MAX_RANK];
 };
 
 struct BatchParams {
-  BatchMember mem[BI_MAX_M];
+  BatchMember mem[BI_MAX_M + BI_MAX_F];
   int32_t nmem;            // members of rank >= 2
+  int32_t task_base;       // first task of this launch
   int32_t NU, Sp, ntask, tu;   // tu: units per contraction CTA
   int32_t sc_off;          // unrolled forms: element offset of the split tasks' scratch columns behind the slice
   int32_t lbuf, so_max;    // any-shape form: elements of the slice staging buffer; most outer states of a member
@@ -71,7 +78,8 @@ struct BatchParams {
   void *qbuf;              // [2][NU][Sp] beliefs
   uint32_t *status;        // the handle's status word
   const int32_t *obs;      // [NU][M] (per-agent models: every unit reads its own slice)
-  int32_t M, T;
+  const int32_t *act;      // [N][T-1][F] (transition members)
+  int32_t M, T, F;
   int32_t drop_copy;       // testing aid: the contraction announces its slice copy and does not issue it
 };
 
@@ -233,9 +241,17 @@ bi_batch_bucket_kernel(BatchParams P, const int32_t *__restrict__ obs, int M, ui
   int32_t *count = sh, *cursor = sh + m;
   for (int i = threadIdx.x; i < m; i += blockDim.x) count[i] = 0;
   __syncthreads();
+  // the outcome that buckets a unit: the observed one, or for a transition the action taken at the unit's step
+  // (a window's last step has none)
+  auto outcome = [&](int u) {
+    if (!mm.edge) return obs[(size_t)u * M + mm.modality];
+    const int a = u / P.T, t = u - a * P.T;
+    return t + 1 < P.T ? max(P.act[((size_t)a * (P.T - 1) + t) * P.F + mm.edge - 1], -1) : INT_MIN;
+  };
   for (int u = threadIdx.x; u < NU; u += blockDim.x) {
-    const int o = clamp_flag(obs[(size_t)u * M + mm.modality], m, status, BI_FLAG_OBS_RANGE);
-    atomicAdd(&count[o], 1);
+    const int v = outcome(u);
+    if (mm.edge && v == INT_MIN) continue;
+    atomicAdd(&count[clamp_flag(v, m, status, mm.edge ? BI_FLAG_ACT_RANGE : BI_FLAG_OBS_RANGE)], 1);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -252,7 +268,8 @@ bi_batch_bucket_kernel(BatchParams P, const int32_t *__restrict__ obs, int M, ui
   __syncthreads();
   int32_t *pm = perm + (size_t)blockIdx.x * NU;
   for (int u = threadIdx.x; u < NU; u += blockDim.x) {
-    int o = obs[(size_t)u * M + mm.modality];
+    int o = outcome(u);
+    if (mm.edge && o == INT_MIN) continue;
     o = o < 0 ? 0 : (o >= m ? m - 1 : o);
     pm[atomicAdd(&cursor[o], 1)] = u;
   }
@@ -279,9 +296,10 @@ bi_batch_contract_kernel(BatchParams P, int cur, int first) {
     bi_grid_launch_dependents();
   }
   int mi = 0;
-  while (mi + 1 < P.nmem && (int)blockIdx.x >= P.mem[mi + 1].task0) ++mi;
+  const int slot = (int)blockIdx.x + P.task_base;
+  while (mi + 1 < P.nmem && slot >= P.mem[mi + 1].task0) ++mi;
   const BatchMember &mm = P.mem[mi];
-  const int4 tk = P.task[blockIdx.x];
+  const int4 tk = P.task[slot];
   if (tk.z == 0) {   // an unused task slot (an exiting CTA counts as having released its dependents)
     return;
   }
@@ -477,7 +495,7 @@ __device__ __forceinline__ void contract_rt(const BatchMember &mm, const R *__re
     for (int k = 1; k < rs; ++k) sum += col[k * tu];
     int j = 0;
     while (j + 1 < K1 && st >= mm.ooff[j + 1]) ++j;
-    ((R *)P.ellp)[((size_t)mi * P.NU + unit_s[uu]) * P.Sp + mm.offp[j] + (st - mm.ooff[j])] = sum;
+    ((R *)P.ellp)[(int64_t)((size_t)mi * P.NU + unit_s[uu]) * P.Sp + mm.oout[j] + (st - mm.ooff[j])] = sum;
   }
   __syncthreads();
 #pragma unroll
@@ -489,7 +507,7 @@ __device__ __forceinline__ void contract_rt(const BatchMember &mm, const R *__re
     const R *col = as + (size_t)st * nt + uu;
     R sum = col[0];
     for (int k = 1; k < rs; ++k) sum += col[k * tu];
-    ((R *)P.ellp)[((size_t)mi * P.NU + unit_s[uu]) * P.Sp + mm.offp[K1] + st] = sum;
+    ((R *)P.ellp)[(int64_t)((size_t)mi * P.NU + unit_s[uu]) * P.Sp + mm.oout[K1] + st] = sum;
   }
 }
 
@@ -509,9 +527,10 @@ bi_batch_contract_rt_kernel(BatchParams P, int cur, int first) {
   R *as = qs + (size_t)P.so_max * P.tu;                     // [so_max][threads] message accumulators, per thread
   int *unit_s = reinterpret_cast<int *>(as + (size_t)P.so_max * blockDim.x);
   int mi = 0;
-  while (mi + 1 < P.nmem && (int)blockIdx.x >= P.mem[mi + 1].task0) ++mi;
+  const int slot = (int)blockIdx.x + P.task_base;
+  while (mi + 1 < P.nmem && slot >= P.mem[mi + 1].task0) ++mi;
   const BatchMember &mm = P.mem[mi];
-  const int4 tk = P.task[blockIdx.x];
+  const int4 tk = P.task[slot];
   if (tk.z == 0) return;
   const R *slice = (const R *)mm.logA + (size_t)tk.x * mm.P_pad;
   switch (mm.ncp) {
@@ -540,6 +559,8 @@ struct UpdateArgs {
   const float *q_init;        // warm start (for the first damped step's ln q), or NULL
   uint32_t fmask[BI_MAX_F];   // members (rank >= 2) whose group contains factor f
   uint32_t r1mask[BI_MAX_F];  // descriptor members (modalities) that depend on factor f alone
+  int32_t child_plane;        // transition members: the plane of the messages to the children (-1: none of that kind)
+  uint32_t pmask[BI_MAX_F];   // ... and the members with factor f among the parents
 };
 
 // Both transition messages' dot products at once: dp = sum_r Mp[r][s] qp[r] and df = sum_r Mf[r][s] qf[r],
@@ -650,6 +671,11 @@ bi_batch_update_kernel(const BiDev *__restrict__ mdp, BatchParams P, UpdateArgs 
       const R *ep = (const R *)P.ellp + (size_t)unit * Sp + p;   // member j's entry: NU * Sp elements further per j
       const size_t mstride = (size_t)NU * Sp;
       for (uint32_t mk = I.fmask; mk; mk &= mk - 1) x += ep[(__ffs(mk) - 1) * mstride];
+      if (A.child_plane >= 0) {   // transitions with several parents: their messages were contracted with the slices
+        if (t > 0) x += ep[A.child_plane * mstride];
+        if (t + 1 < T)
+          for (uint32_t mk = A.pmask[f]; mk; mk &= mk - 1) x += ep[(__ffs(mk) - 1) * mstride];
+      }
       for (uint32_t mk = I.r1mask; mk; mk &= mk - 1) {   // single-factor modalities: the slice is the message
         const BiMember &mm = md.mem[__ffs(mk) - 1];
         const int o = clamp_flag(ob[mm.modality], mm.m, md.status, BI_FLAG_OBS_RANGE);
@@ -671,6 +697,8 @@ bi_batch_update_kernel(const BiDev *__restrict__ mdp, BatchParams P, UpdateArgs 
     R x = -bi_inf<R>();
     if (s < n) {
       x = base[op + s];
+    }
+    if (s < n && A.child_plane < 0) {
       // both edges are evaluated (a window's end reads zeros and discards the result)
       const int up = t > 0 ? clamp_flag(acp[f], I.U, md.status, BI_FLAG_ACT_RANGE) : 0;
       const int uf = t + 1 < T ? clamp_flag(acp[F + f], I.U, md.status, BI_FLAG_ACT_RANGE) : 0;
@@ -760,6 +788,7 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
   // members of rank >= 2, largest slices first (their tasks are the longest)
   int order[BI_MAX_M], cnt = 0;
   const bool per_unit = h.G != 1;   // per-agent models: every unit contracts its own slice
+  A.child_plane = -1;
   bool any_shape = per_unit;        // (also set when some group has no unrolled form)
   for (int gi = 0; gi < h.ngroups; ++gi) {
     const BiGroup &g = h.grp[gi];
@@ -778,12 +807,14 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
     while (!(order[j] >= h.grp[gi].mem_begin && order[j] < h.grp[gi].mem_end)) ++gi;
     const BiGroup &g = h.grp[gi];
     BatchMember &bm = P.mem[j];
+    bm.edge = 0;
     bm.logA = mm.logA; bm.m = mm.m; bm.P_pad = mm.P_pad; bm.modality = mm.modality;
     bm.gstride = mm.gstride;
     bm.shape = shape_of(g); bm.rank = g.rank;
     int so = 0, rows = 1;
     for (int k = 0; k < g.rank; ++k) {
       bm.offp[k] = h.offp[g.axis[k]];
+      bm.oout[k] = h.offp[g.axis[k]];
       bm.dim[k] = g.dim[k];
       bm.ooff[k] = so;
       if (k + 1 < g.rank) { so += g.dim[k]; rows *= g.dim[k]; }
@@ -798,11 +829,47 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
     max_slice = std::max(max_slice, (size_t)mm.P_pad * sizeof(R));
     max_m = std::max(max_m, mm.m);
   }
+  // transitions with several parents: members behind the slices, always on the any-shape form
+  const int nslice = cnt;
+  const size_t max_slice_u = max_slice;
+  if (h.has_bdep) A.child_plane = cnt + h.F;   // (also for windows of one step, which have no transitions at all)
+  if (h.has_bdep && c.T > 1) {
+    for (int f = 0; f < h.F; ++f, ++cnt) {
+      BatchMember &bm = P.mem[cnt];
+      const int k = h.bdep_len[f], r = k + 1;
+      if (r > BI_MAX_RANK || per_unit) return BI_ERR_UNSUPPORTED;
+      bm.edge = 1 + f;
+      bm.logA = h.logBedge[f]; bm.m = h.U[f];
+      bm.modality = 0; bm.gstride = 0;
+      bm.shape = -1; bm.rank = r; bm.split = 1;
+      // first axis: the child's next state (one unit on), then the parents in list order, the last one padded
+      int so = 0, rows = 1;
+      for (int j = 0; j < r; ++j) {
+        const int fa = j == 0 ? f : h.bdep[f][j - 1];
+        bm.dim[j] = h.n[fa];
+        bm.offp[j] = h.offp[fa] + (j == 0 ? h.Sp : 0);
+        bm.oout[j] = h.offp[fa];
+        if (j == 0) bm.oout[j] += ((int64_t)(A.child_plane - cnt) * NU + 1) * h.Sp;
+        else A.pmask[fa] |= 1u << cnt;
+        bm.ooff[j] = so;
+        if (j + 1 < r) { so += bm.dim[j]; rows *= bm.dim[j]; }
+      }
+      bm.ncp = bi_pad4(bm.dim[r - 1]);
+      bm.rows = rows;
+      bm.P_pad = rows * bm.ncp;
+      so_max = std::max(so_max, so);
+      ncp_max = std::max(ncp_max, (int)bm.ncp);
+      max_slice = std::max(max_slice, (size_t)bm.P_pad * sizeof(R));
+      max_m = std::max(max_m, (int)bm.m);
+    }
+  }
+  const bool edges = cnt > nslice;
+  const bool use_rt = any_shape || edges;   // (the unrolled form for the slices, if they have it, beside the any-shape one)
   if (max_m > 4096) return BI_ERR_UNSUPPORTED;
   // shared memory and shape of a contraction CTA
   size_t csmem = max_slice;
   int rs = 1;
-  if (any_shape) {
+  if (use_rt) {
     // row splits: enough warps for about two per scheduler when the batch is small
     if (tu == 32) rs = NU <= 32 * 4 * md->sm_count ? 8 : 4;
     else if (tu == 64) rs = 2;
@@ -833,8 +900,9 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
   // get one more of its warps than the rest do not set the time.  (Measured on a rank-4 group of 4800
   // entries, 20 480 units: 1.32 ms per call unsplit, 1.23 ms in halves, 1.27 ms in quarters; lanes of one
   // warp sharing a unit, which turns the slice rows' broadcast loads into four different rows, 2.3 ms.)
+  size_t usmem = max_slice_u;   // the unrolled form's
   if (!any_shape)
-    for (int j = 0; j < cnt; ++j) {
+    for (int j = 0; j < nslice; ++j) {
       BatchMember &bm = P.mem[j];
       const long long fm = 2LL * bm.P_pad;
       int sp = fm >= 4000 ? 2 : 1;
@@ -845,23 +913,24 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
       if (sp > 1) {
         int ns = 0;
         for (int k = 1; k < bm.rank; ++k) ns += bm.dim[k];
-        P.sc_off = (int)((max_slice / sizeof(R) + 1) & ~(size_t)1);
-        csmem = std::max(csmem, ((size_t)P.sc_off + (size_t)ns * tu) * sizeof(R));
+        P.sc_off = (int)((max_slice_u / sizeof(R) + 1) & ~(size_t)1);
+        usmem = std::max(usmem, ((size_t)P.sc_off + (size_t)ns * tu) * sizeof(R));
       }
     }
-  if (csmem > (size_t)md->max_smem_optin - 1024) return BI_ERR_UNSUPPORTED;
+  if (std::max(use_rt ? csmem : 0, any_shape ? 0 : usmem) > (size_t)md->max_smem_optin - 1024) return BI_ERR_UNSUPPORTED;
   int ntask = 0;
   for (int j = 0; j < cnt; ++j) {
     P.mem[j].task0 = ntask;
     const int tum = tu / P.mem[j].split;
     ntask += (NU + tum - 1) / tum + P.mem[j].m;
   }
+  const int ntask_slices = edges ? P.mem[nslice].task0 : ntask;
   P.nmem = cnt; P.NU = NU; P.Sp = h.Sp; P.ntask = ntask;
 
   // ---- workspace (stream-ordered; kept in the handle and grown on demand)
   const size_t b_perm = up256((size_t)cnt * NU * sizeof(int32_t));
   const size_t b_task = up256((size_t)ntask * sizeof(int4));
-  const size_t b_ellp = up256((size_t)cnt * NU * h.Sp * sizeof(R));
+  const size_t b_ellp = up256((size_t)(cnt + (edges ? 1 : 0)) * NU * h.Sp * sizeof(R));
   const size_t b_q = up256(2 * (size_t)NU * h.Sp * sizeof(R));
   const size_t b_x = c.lambda != 1.0 ? up256((size_t)NU * h.Sp * sizeof(R)) : 0;
   const size_t need = b_perm + b_task + b_ellp + b_q + b_x;
@@ -890,7 +959,7 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
     P.drop_copy = 1;
     mut->test_drop_copy -= 1;
   }
-  P.obs = c.obs; P.M = h.M; P.T = c.T;
+  P.obs = c.obs; P.M = h.M; P.T = c.T; P.F = h.F; P.act = c.act;
   A.obs = c.obs; A.act = c.act; A.q_out = c.q_out; A.logq_out = c.logq_out; A.argmax_out = c.argmax_out;
   A.T = c.T;
   A.lnprior = c.lnprior;
@@ -903,12 +972,13 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
     bi_batch_identity_tasks_kernel<<<dim3(64, cnt), 256, 0, c.stream>>>(P, perm, task);
   else if (cnt > 0)
     bi_batch_bucket_kernel<<<cnt, 1024, 2 * max_m * sizeof(int32_t), c.stream>>>(P, c.obs, h.M, h.status, perm, task);
-  void (*contract)(BatchParams, int, int) =
-      per_unit    ? (ncp_max <= 16 ? bi_batch_contract_rt_kernel<R, true, 16> : bi_batch_contract_rt_kernel<R, true, 32>)
-      : any_shape ? (ncp_max <= 16 ? bi_batch_contract_rt_kernel<R, false, 16> : bi_batch_contract_rt_kernel<R, false, 32>)
-                  : bi_batch_contract_kernel<R>;
-  if (cudaFuncSetAttribute((const void *)contract, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem) !=
-      cudaSuccess)
+  typedef void (*ContractKernel)(BatchParams, int, int);
+  const ContractKernel rt = per_unit ? (ncp_max <= 16 ? bi_batch_contract_rt_kernel<R, true, 16> : bi_batch_contract_rt_kernel<R, true, 32>)
+                                     : (ncp_max <= 16 ? bi_batch_contract_rt_kernel<R, false, 16> : bi_batch_contract_rt_kernel<R, false, 32>);
+  const ContractKernel unrolled = bi_batch_contract_kernel<R>;
+  if (use_rt && cudaFuncSetAttribute((const void *)rt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem) != cudaSuccess)
+    return BI_ERR_CUDA;
+  if (!any_shape && cudaFuncSetAttribute((const void *)unrolled, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)usmem) != cudaSuccess)
     return BI_ERR_CUDA;
   for (int gi = 0; gi < h.ngroups; ++gi) {
     const BiGroup &g = h.grp[gi];
@@ -948,11 +1018,21 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
     cfg.stream = c.stream;
     cfg.attrs = pdl;
     cfg.numAttrs = 1;
-    if (cnt > 0) {
-      cfg.gridDim = dim3((unsigned)ntask);
+    // the slices on their unrolled form where they all have one, everything else on the any-shape form
+    const int n_unrolled = any_shape ? 0 : ntask_slices;
+    if (n_unrolled > 0) {
+      cfg.gridDim = dim3((unsigned)n_unrolled);
+      cfg.blockDim = dim3((unsigned)tu);
+      cfg.dynamicSmemBytes = usmem;
+      P.task_base = 0;
+      if (cudaLaunchKernelEx(&cfg, unrolled, P, cur, (int)(k == 0)) != cudaSuccess) return BI_ERR_CUDA;
+    }
+    if (ntask > n_unrolled) {
+      cfg.gridDim = dim3((unsigned)(ntask - n_unrolled));
       cfg.blockDim = dim3((unsigned)(tu * rs));
       cfg.dynamicSmemBytes = csmem;
-      if (cudaLaunchKernelEx(&cfg, contract, P, cur, (int)(k == 0)) != cudaSuccess) return BI_ERR_CUDA;
+      P.task_base = n_unrolled;
+      if (cudaLaunchKernelEx(&cfg, rt, P, cur, (int)(k == 0)) != cudaSuccess) return BI_ERR_CUDA;
     }
     cfg.gridDim = dim3((unsigned)(fw ? NU : (NU + upb - 1) / upb));
     cfg.blockDim = dim3((unsigned)(fw ? 32 * h.F : 128));
@@ -961,7 +1041,7 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
       return BI_ERR_CUDA;
   }
   if (cudaGetLastError() != cudaSuccess) return BI_ERR_CUDA;
-  mut->launches += cnt > 0 ? 2 + 2 * c.K : 1 + c.K;
+  mut->launches += 1 + (cnt > 0) + c.K * (1 + (!any_shape && nslice > 0) + (any_shape ? cnt > 0 : edges));
   const bool f64 = sizeof(R) == 8;
   mut->last_kernel = c.algo == BI_ALGO_VMP ? (f64 ? "batch_vmp_f64" : "batch_vmp_f32")
                                            : (f64 ? "batch_mmp_f64" : "batch_mmp_f32");
@@ -984,6 +1064,8 @@ int bi_batch_shape(int rank, const int *dim) {
 int bi_launch_batch(const BiCall &c, bi_model *mut) {
   const bi_model *md = c.model;
   if (c.algo == BI_ALGO_FILTER) return BI_ERR_UNSUPPORTED;
+  if (md->h.has_bdep && (c.algo != BI_ALGO_VMP || md->h.G != 1 || !md->h.logBedge[0] || (md->arith == BI_ARITH_F32 && md->has_zeros)))
+    return BI_ERR_UNSUPPORTED;   // (with zeros in A the order of float32 sums is kept, see bi_block_serves)
   if (md->h.G != 1) {
     // per-agent models: the slices are re-read every iteration, which pays only while they stay in L2
     // (measured on config 3's model with per-step slices: faster than the warp-per-step kernels at

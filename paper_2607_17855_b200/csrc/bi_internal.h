@@ -94,6 +94,7 @@ struct alignas(16) BiDev {
   const void *Bfull[BI_MAX_F];     // B[s_next, parents, u]
   const void *logBfull[BI_MAX_F];  // ln max(., 1e-16) of the same
   int64_t Bfull_stride[BI_MAX_F];  // elements per model (0 when shared)
+  const void *logBedge[BI_MAX_F];  // shared models: logBfull with the last parent padded to a multiple of 4, [U][n][..][pad4], or NULL
   int64_t Dstride[BI_MAX_F];
   // status[0]: the BI_FLAG_* bits bi_status reports and clears.  status[1]: set when the model was packed
   // if an entry of A, B or D exceeds 1 (not a probability): kernels that shift several agents' softmaxes by one
@@ -106,7 +107,7 @@ struct alignas(16) BiDev {
 struct bi_model {
   BiDev h;          // host copy (device pointers inside)
   BiDev *d;         // device copy
-  void *allocs[28 + 4 * BI_MAX_M + 10 * BI_MAX_F];  // status, descriptor, pre-summed table, 2 per modality, 7 per factor
+  void *allocs[28 + 4 * BI_MAX_M + 11 * BI_MAX_F];  // status, descriptor, pre-summed table, 2 per modality, 7 per factor
   int nalloc;
   int arith;        // BI_ARITH_F64 or BI_ARITH_F32
   int device;

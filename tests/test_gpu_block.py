@@ -72,6 +72,20 @@ def test_transitions_with_several_parents(bdep, algo):
     print(check_workload(_workload(40, [9, 4, 7], [[0, 1], [1, 2, 0]], N=7, T=6, K=5, bdep=bdep), algo))
 
 
+@pytest.mark.parametrize("n, dep, bdep, T", [
+    ([9, 4, 7], [[0, 1], [1, 2, 0]], [[0, 1], [2], [2, 0, 1]], 7),           # any-shape slices, one to three parents
+    ([10, 10, 8, 6], [[0, 1], [0, 2, 3]], [[0, 1], [1, 2], [2, 3], [3, 0]], 8),   # unrolled slices beside the transitions
+    ([3, 2, 4, 2, 3], [[0], [3]], [[1, 0, 2, 3], [1], [4, 2], [3], [0]], 1),      # no slice to contract, one step
+    ([3, 2, 4, 2, 3], [[0], [3]], [[1, 0, 2, 3], [1], [4, 2], [3], [0]], 9),      # four parents, a pure copy of another factor
+])
+def test_batched_transitions_with_several_parents(n, dep, bdep, T):
+    from test_gpu_parity import family_forced
+    N = 2100 if T == 1 else 2100 // T + 60
+    with family_forced("batch"):
+        res = check_workload(_workload(60 + T, n, dep, N=N, T=T, K=5, bdep=bdep), "vmp", agents=range(0, N, 23))
+    assert res["kernel"] == "batch_vmp_f64", res
+
+
 @pytest.mark.parametrize("algo", ["filter", "vmp", "mmp"])
 def test_float32(algo):
     # (dense and few iterations: the tolerance of check_workload's strict=False form is not a numerical one)
