@@ -745,6 +745,222 @@ bi_batch_update_kernel(const BiDev *__restrict__ mdp, BatchParams P, UpdateArgs 
   }
 }
 
+// The same for batches that fill the machine with one thread per (unit, factor), on shared models.  A CTA takes 32
+// consecutive units, a warp per factor and a lane per unit.  The units' rows (messages summed over the members,
+// the neighbours' beliefs) are one contiguous run of memory: they come through shared memory with coalesced
+// loads, the new beliefs leave the same way.  A lane keeps its unit's states of the factor in registers, so sums and
+// softmax need no shuffles; the factors' transition matrices, every action's, sit in shared memory (a pad of
+// 16 bytes between actions puts the rows that a warp's units read for different actions on different banks, so
+// a 16-byte load serves 32 units with two entries each).  The lane-group form above issues a 16-lane dot product
+// per unit and state and waits for it: 20 480 units of 34 states took 38 us.
+// NP: states in registers (the model's largest factor, padded).
+struct UnitUpdate {   // shared-memory layout, elements
+  int32_t mat[BI_MAX_F], xs, qs, stride;   // matrices of each factor; the units' logits; beliefs of units -1 .. 32; row stride
+};
+template <typename R>
+__device__ __forceinline__ void vec_add(R *x, const R *p) {
+  if constexpr (sizeof(R) == 8) {
+    const double2 v = *reinterpret_cast<const double2 *>(p);
+    x[0] += v.x; x[1] += v.y;
+  } else {
+    const float4 v = *reinterpret_cast<const float4 *>(p);
+    x[0] += v.x; x[1] += v.y; x[2] += v.z; x[3] += v.w;
+  }
+}
+template <typename R, int ALGO, int NP, bool FINAL, bool DAMPED>
+__global__ void __launch_bounds__(32 * BI_MAX_F)
+bi_batch_update_unit_kernel(const BiDev *__restrict__ mdp, BatchParams P, UpdateArgs A, UnitUpdate L) {
+  extern __shared__ __align__(16) unsigned char upd_smem[];
+  __shared__ unsigned char pfac[BI_MAX_F * 32];   // factor of each padded state position
+  R *sm = reinterpret_cast<R *>(upd_smem);
+  const BiDev &md = *mdp;
+  constexpr int VE = 16 / (int)sizeof(R);
+  const int F = md.F, Sp = md.Sp, S = md.S, M = md.M, T = A.T, NU = P.NU;
+  const int f = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int n = md.n[f], np = md.npad[f], op = md.offp[f], off = md.off[f], U = md.U[f];
+  const int msz = np * np, mst = msz + VE;   // (rows padded like columns; the padding rows are zero)
+  R *M0 = sm + L.mat[f], *M1 = M0 + (size_t)U * mst;
+  if (A.child_plane < 0) {
+    const R *s0 = (const R *)(ALGO == BI_ALGO_VMP ? md.logBt[f] : md.BfT[f]);   // [previous][next]
+    const R *s1 = (const R *)(ALGO == BI_ALGO_VMP ? md.logB[f] : md.BdagT[f]);   // [next][previous]
+    for (int u = 0; u < U; ++u)
+      for (int e = lane; e < msz; e += 32) {
+        const bool in = e < n * np;
+        M0[u * mst + e] = in ? __ldg(s0 + (size_t)u * n * np + e) : (R)0;
+        M1[u * mst + e] = in ? __ldg(s1 + (size_t)u * n * np + e) : (R)0;
+      }
+  }
+  for (int p = lane; p < np; p += 32) pfac[op + p] = (unsigned char)f;
+  __syncthreads();
+  bi_grid_wait();   // the contraction's messages (and, for the beliefs, everything before it)
+  bi_grid_launch_dependents();
+  // ---- rows in: summed messages, and the beliefs of the units from one before to one after
+  const int u0 = blockIdx.x * 32, nu = min(32, NU - u0), hv = Sp / VE;
+  const size_t mstride = (size_t)NU * Sp;
+  for (int i = threadIdx.x; i < nu * hv; i += blockDim.x) {
+    const int ul = i / hv, p = (i - ul * hv) * VE, fp = pfac[p];
+    const R *ep = (const R *)P.ellp + (size_t)u0 * Sp + (size_t)i * VE;   // member j's entry: NU * Sp elements further per j
+    R x[VE];
+#pragma unroll
+    for (int e = 0; e < VE; ++e) x[e] = (R)0;
+    uint32_t mk = A.fmask[fp];
+    if (A.child_plane >= 0) {   // transitions with several parents: their messages were contracted with the slices
+      const int t = (u0 + ul) % T;
+      if (t > 0) vec_add(x, ep + A.child_plane * mstride);
+      if (t + 1 < T) mk |= A.pmask[fp];
+    }
+    for (; mk; mk &= mk - 1) vec_add(x, ep + (__ffs(mk) - 1) * mstride);
+#pragma unroll
+    for (int e = 0; e < VE; ++e) sm[L.xs + ul * L.stride + p + e] = x[e];
+  }
+  if (A.child_plane < 0) {
+    const R *qc = (const R *)P.qbuf + (size_t)A.cur * NU * Sp;
+    for (int i = threadIdx.x; i < (nu + 2) * hv; i += blockDim.x) {
+      const int ul = i / hv, p = (i - ul * hv) * VE, u = u0 + ul - 1;
+      R x[VE];
+#pragma unroll
+      for (int e = 0; e < VE; ++e) x[e] = (R)0;
+      if (u >= 0 && u < NU) vec_add(x, qc + (size_t)u * Sp + p);
+#pragma unroll
+      for (int e = 0; e < VE; ++e) sm[L.qs + ul * L.stride + p + e] = x[e];
+    }
+  }
+  __syncthreads();
+  // ---- one unit and factor per lane
+  const bool live = lane < nu;
+  const int ul = live ? lane : 0, unit = u0 + ul;
+  const int a = unit / T, t = unit - a * T;
+  const bool has_prev = t > 0, has_next = t + 1 < T;
+  R *xrow = sm + L.xs + ul * L.stride + op;
+  R x[NP];
+#pragma unroll
+  for (int s = 0; s < NP; ++s) x[s] = (R)0;
+  auto add_row = [&](const R *row) {
+#pragma unroll
+    for (int s = 0; s < NP; s += VE)
+      if (s < np) vec_add(x + s, row + s);
+  };
+  add_row(xrow);
+  for (uint32_t mk = A.r1mask[f]; mk; mk &= mk - 1) {
+    const BiMember &mm = md.mem[__ffs(mk) - 1];
+    const int o = clamp_flag(A.obs[(size_t)unit * M + mm.modality], mm.m, md.status, BI_FLAG_OBS_RANGE);
+    add_row((const R *)mm.logA + (size_t)o * mm.P_pad);
+  }
+  if (!has_prev) {
+    if (A.lnprior) {
+#pragma unroll
+      for (int s = 0; s < NP; ++s)
+        if (s < n) x[s] += ((const R *)A.lnprior)[(size_t)a * S + off + s];
+    } else {
+      add_row((const R *)md.logD[f]);
+    }
+  }
+  // both transition messages: acc[s] += sum_r M[r][s] q[r] (a window's ends add nothing)
+  if (A.child_plane < 0) {
+    const int32_t *acp = A.act + ((ptrdiff_t)a * (T - 1) + (t - 1)) * F + f;
+    auto edge = [&](bool real, const R *Mx, const int32_t *ac, const R *q, R (&acc)[NP]) {
+      const int u = real ? clamp_flag(*ac, U, md.status, BI_FLAG_ACT_RANGE) : 0;
+      const R *row = Mx + u * mst;
+#pragma unroll 2
+      for (int r = 0; r < np; r += VE, row += VE * np) {
+        R w[VE];
+        lds_vec(q + r, w);
+#pragma unroll
+        for (int k = 0; k < VE; ++k) {
+          const R wk = real ? w[k] : (R)0;
+#pragma unroll
+          for (int s = 0; s < NP; s += VE) {
+            if (s < np) {
+              R m[VE];
+              lds_vec(row + k * np + s, m);
+#pragma unroll
+              for (int e = 0; e < VE; ++e) acc[s + e] = fma(m[e], wk, acc[s + e]);
+            }
+          }
+        }
+      }
+    };
+    const R *q0 = sm + L.qs + ul * L.stride + op, *q1 = q0 + 2 * L.stride;
+    if (ALGO == BI_ALGO_VMP) {
+      edge(has_prev, M0, acp, q0, x);
+      edge(has_next, M1, acp + F, q1, x);
+    } else {
+#pragma unroll 1
+      for (int d = 0; d < 2; ++d) {
+        const bool real = d == 0 ? has_prev : has_next;
+        R m[NP];
+#pragma unroll
+        for (int s = 0; s < NP; ++s) m[s] = (R)0;
+        edge(real, d == 0 ? M0 : M1, d == 0 ? acp : acp + F, d == 0 ? q0 : q1, m);
+#pragma unroll
+        for (int s = 0; s < NP; ++s)
+          if (s < n) x[s] += real ? (R)0.5 * bi_log_inline(bi_max(m[s], (R)BI_EPS)) : (R)0;
+      }
+    }
+  }
+  if (DAMPED) {   // as in the lane-group form
+    R *xp = (R *)A.xprev + (size_t)unit * Sp + op;
+#pragma unroll
+    for (int s = 0; s < NP; ++s) {
+      if (s < n && live) {
+        R prev = (R)0;
+        if (!A.first) prev = xp[s];
+        else if (A.q_init) prev = bi_log(bi_max((R)A.q_init[(size_t)unit * S + off + s], (R)BI_EPS));
+        x[s] = fma((R)A.lambda, x[s], ((R)1 - (R)A.lambda) * prev);
+        xp[s] = x[s];
+      }
+    }
+  }
+  R mx;
+  if (FINAL) {
+    mx = x[0];
+#pragma unroll
+    for (int s = 1; s < NP; ++s)
+      if (s < n) mx = bi_max(mx, x[s]);
+  } else {   // (any shift near the maximum keeps the exponentials in range)
+    float m = (float)x[0];
+#pragma unroll
+    for (int s = 1; s < NP; ++s)
+      if (s < n) m = fmaxf(m, (float)x[s]);
+    mx = (R)m;
+  }
+  R e[NP], z0 = (R)0, z1 = (R)0;
+#pragma unroll
+  for (int s = 0; s < NP; ++s) {
+    e[s] = s < n ? bi_exp_inline(x[s] - mx) : (R)0;
+    if (s & 1) z1 += e[s];
+    else z0 += e[s];
+  }
+  const R z = z0 + z1, rz = bi_rcp(z);
+#pragma unroll
+  for (int s = 0; s < NP; ++s)
+    if (s < np && live) xrow[s] = e[s] * rz;   // (the lane's own entries: nobody else reads them before the barrier)
+  if (FINAL && live) {
+    const R lz = A.logq_out ? bi_log(z) : (R)0;
+    int am = 0;
+    bool found = false;
+#pragma unroll
+    for (int s = 0; s < NP; ++s) {
+      if (s < n) {
+        A.q_out[(size_t)unit * S + off + s] = (float)(e[s] * rz);
+        if (A.logq_out) A.logq_out[(size_t)unit * S + off + s] = (float)(x[s] - mx - lz);
+        if (!found && x[s] == mx) { am = s; found = true; }
+      }
+    }
+    if (A.argmax_out) A.argmax_out[(size_t)unit * F + f] = am;
+  }
+  if (!FINAL) {   // rows out
+    __syncthreads();
+    R *qn = (R *)P.qbuf + ((size_t)(A.cur ^ 1) * NU + u0) * Sp;
+    for (int i = threadIdx.x; i < nu * hv; i += blockDim.x) {
+      const int ul2 = i / hv, p = (i - ul2 * hv) * VE;
+      const R *src = sm + L.xs + ul2 * L.stride + p;
+      if constexpr (sizeof(R) == 8) *reinterpret_cast<double2 *>(qn + (size_t)i * VE) = *reinterpret_cast<const double2 *>(src);
+      else *reinterpret_cast<float4 *>(qn + (size_t)i * VE) = *reinterpret_cast<const float4 *>(src);
+    }
+  }
+}
+
 template <typename R>
 __global__ void bi_batch_init_kernel(const BiDev *__restrict__ mdp, R *q, int NU, const float *__restrict__ q_init) {
   const BiDev &md = *mdp;
@@ -1005,6 +1221,43 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
 #undef BI_UPD
   };
   const UpdateKernel update_mid = pick(false), update_last = pick(true);
+  // a lane per unit and a warp per factor: shared models of up to 16 states per factor whose matrices fit beside
+  // the units' rows twice per SM, from about two CTAs per SM on (below that the form above has more warps)
+  typedef void (*UnitKernel)(const BiDev *, BatchParams, UpdateArgs, UnitUpdate);
+  UnitKernel unit_mid = nullptr, unit_last = nullptr;
+  UnitUpdate UL;
+  memset(&UL, 0, sizeof(UL));
+  size_t unit_smem = 0;
+  if (h.G == 1 && nmax <= 16 && NU >= 64 * md->sm_count) {
+    constexpr int VE = 16 / (int)sizeof(R);
+    size_t o = 0;
+    for (int f = 0; f < h.F; ++f) {
+      UL.mat[f] = (int)o;
+      if (!h.has_bdep) o += 2 * (size_t)h.U[f] * ((size_t)h.npad[f] * h.npad[f] + VE);
+      if (o > 100 * 1024) break;
+    }
+    UL.stride = ((h.Sp / VE) | 1) * VE;   // an odd number of 16-byte units: the lanes' rows on different banks
+    UL.xs = (int)o; o += 32 * (size_t)UL.stride;
+    UL.qs = (int)o; o += h.has_bdep ? 0 : 34 * (size_t)UL.stride;
+    unit_smem = o * sizeof(R);
+    if (unit_smem <= 100 * 1024) {
+      auto pick_unit = [&](bool fin) -> UnitKernel {
+#define BI_UPT(AL, NPV) \
+    (fin ? (damped ? (UnitKernel)bi_batch_update_unit_kernel<R, AL, NPV, true, true>   \
+                   : (UnitKernel)bi_batch_update_unit_kernel<R, AL, NPV, true, false>) \
+         : (damped ? (UnitKernel)bi_batch_update_unit_kernel<R, AL, NPV, false, true>  \
+                   : (UnitKernel)bi_batch_update_unit_kernel<R, AL, NPV, false, false>))
+        if (c.algo == BI_ALGO_VMP) return nmax <= 8 ? BI_UPT(BI_ALGO_VMP, 8) : nmax <= 12 ? BI_UPT(BI_ALGO_VMP, 12) : BI_UPT(BI_ALGO_VMP, 16);
+        return nmax <= 8 ? BI_UPT(BI_ALGO_MMP, 8) : nmax <= 12 ? BI_UPT(BI_ALGO_MMP, 12) : BI_UPT(BI_ALGO_MMP, 16);
+#undef BI_UPT
+      };
+      unit_mid = pick_unit(false);
+      unit_last = pick_unit(true);
+      for (UnitKernel k : {unit_mid, unit_last})
+        if (cudaFuncSetAttribute((const void *)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)unit_smem) != cudaSuccess)
+          return BI_ERR_CUDA;
+    }
+  }
   // every launch of the loop may be scheduled while its predecessor drains (see bi_grid_wait)
   cudaLaunchAttribute pdl[1];
   pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1033,6 +1286,13 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
       cfg.dynamicSmemBytes = csmem;
       P.task_base = n_unrolled;
       if (cudaLaunchKernelEx(&cfg, rt, P, cur, (int)(k == 0)) != cudaSuccess) return BI_ERR_CUDA;
+    }
+    if (unit_mid) {
+      cfg.gridDim = dim3((unsigned)((NU + 31) / 32));
+      cfg.blockDim = dim3((unsigned)(32 * h.F));
+      cfg.dynamicSmemBytes = unit_smem;
+      if (cudaLaunchKernelEx(&cfg, A.final ? unit_last : unit_mid, (const BiDev *)md->d, P, A, UL) != cudaSuccess) return BI_ERR_CUDA;
+      continue;
     }
     cfg.gridDim = dim3((unsigned)(fw ? NU : (NU + upb - 1) / upb));
     cfg.blockDim = dim3((unsigned)(fw ? 32 * h.F : 128));
