@@ -357,16 +357,15 @@ bi_batch_contract_kernel(BatchParams P, int cur, int first) {
 }
 
 // ---- contraction for any shape: compiled for the padded last axis only ----
-// Same arithmetic as the unrolled forms.  For a row of the slice (all outer
-// indices fixed) v = sum_c L[row][c] q_c[c] and acc_c[c] += W L[row][c], with W
-// the product of the outer beliefs.  v then climbs the outer axes from the
-// innermost: at axis j the message accumulator of index s_j receives
-// (product of the beliefs of axes before j) * v, the running sum p_{j-1}
-// receives q_j[s_j] * v, and when s_j was the axis' last index that sum becomes
-// the value handed to axis j - 1.  The indices are an odometer that is the same
-// for every thread of a warp, so its branches are uniform and a slice row is a
-// broadcast load.  qs / as: per-thread columns (state-major, thread-minor: no
-// bank conflicts) holding the outer axes' beliefs and message accumulators.
+// Same arithmetic as the unrolled forms.  For a row of the slice (all outer indices fixed)
+// v = sum_c L[row][c] q_c[c] and acc_c[c] += W L[row][c], with W the product of the outer beliefs.  Consecutive
+// rows run through the innermost outer axis: along it the accumulator of index s receives (prefix product) * v
+// and a running sum receives q[s] * v; after its last index that sum climbs the other outer axes the same way.
+// All indices are the same for every thread of a warp, so the branches are uniform and a slice row is a broadcast
+// load.  qs / as: columns (state-major, thread-minor) holding the outer axes' beliefs per unit and message
+// accumulators per thread, one entry longer than the threads, so that they can also be read along the states.
+// Two rows a trip and one climb per run of rows: with an odometer over all axes advanced after every row, a warp
+// took some 290 cycles per row, nearly all of them latency.
 //
 // Small batches do not have enough units to fill the machine with one thread
 // per unit, so a CTA is tu units x rs row splits: split r contracts the rows of
@@ -380,40 +379,61 @@ template <typename R, int NCP, bool PERUNIT>
 __device__ __forceinline__ void contract_rt(const BatchMember &mm, const R *__restrict__ slice, R *Lbuf, int lbuf,
                                             R *qs, R *as, int *unit_s, const BatchParams &P, int cur, int4 tk,
                                             int mi) {
-  const int tid = threadIdx.x, nt = blockDim.x, tu = P.tu, rs = nt / tu;
+  constexpr int VE = 16 / (int)sizeof(R);
+  const int tid = threadIdx.x, nt = blockDim.x, tu = P.tu, rs = nt / tu, nts = nt + 1, tus = tu + 1;
   const int u = tid % tu, r = tid / tu;
   const bool has_unit = u < tk.z;
   const int unit = has_unit ? P.perm[(size_t)mi * P.NU + tk.y + u] : 0;
   if (r == 0) unit_s[u] = unit;
-  const R *q = (const R *)P.qbuf + ((size_t)cur * P.NU + unit) * P.Sp;
+  const R *qbase = (const R *)P.qbuf + (size_t)cur * P.NU * P.Sp;
   const int K1 = mm.rank - 1, NC = mm.dim[K1];
   R qc[NCP], accc[NCP];
+  {
+    const R *q = qbase + (size_t)unit * P.Sp + mm.offp[K1];   // (offsets of factors are multiples of four: whole vectors)
 #pragma unroll
-  for (int c = 0; c < NCP; ++c) {
-    qc[c] = (has_unit && c < NC) ? q[mm.offp[K1] + c] : (R)0;
-    accc[c] = (R)0;
-  }
-  // (the outer axes' beliefs once per unit: the splits of a unit read the same column)
-  for (int j = 0; j < K1; ++j)
-    for (int sj = 0; sj < mm.dim[j]; ++sj) {
-      if (r == 0) qs[(mm.ooff[j] + sj) * tu + u] = has_unit ? q[mm.offp[j] + sj] : (R)0;
-      as[(mm.ooff[j] + sj) * nt + tid] = (R)0;
+    for (int c = 0; c < NCP; c += VE) {
+      R v[VE];
+      if (c < bi_pad4(NC)) {
+        if constexpr (sizeof(R) == 8) { const double2 x = *reinterpret_cast<const double2 *>(q + c); v[0] = x.x; v[1] = x.y; }
+        else { const float4 x = *reinterpret_cast<const float4 *>(q + c); v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w; }
+      }
+#pragma unroll
+      for (int e = 0; e < VE; ++e) {
+        qc[c + e] = (has_unit && c + e < NC) ? v[e] : (R)0;
+        accc[c + e] = (R)0;
+      }
     }
+  }
+  constexpr bool stage = !PERUNIT;
+  __shared__ __align__(8) unsigned long long bar[8];   // one per split
+  if (stage && tid < rs) bi_mbar_init(&bar[tid], 1);
+  const int so = mm.ooff[K1];   // outer states of this member
+  for (int i = 0; i < so; ++i) as[i * nts + tid] = (R)0;
+  __syncthreads();              // (unit_s, the barriers)
+  // the outer axes' beliefs, once per unit: consecutive threads read consecutive states of one unit
+  for (int j = 0; j < K1; ++j) {
+    const int d = mm.dim[j];
+    for (int i = tid; i < d * tu; i += nt) {
+      const int uu = i / d, sj = i - uu * d;
+      qs[(mm.ooff[j] + sj) * tus + uu] = uu < tk.z ? qbase[(size_t)unit_s[uu] * P.Sp + mm.offp[j] + sj] : (R)0;
+    }
+  }
   __syncthreads();
   // this split's range of the first axis, and of rows
   const int d0 = mm.dim[0], rps = mm.rows / d0;
   const int s0a = (int)((long long)r * d0 / rs), s0b = (int)((long long)(r + 1) * d0 / rs);
   const int row_a = s0a * rps, row_b = s0b * rps;
   const int most = ((d0 + rs - 1) / rs) * rps;   // rows of the largest split: the common trip count
-  int dig[4] = {s0a < d0 ? s0a : 0, 0, 0, 0};
-  R p[4] = {(R)0, (R)0, (R)0, (R)0}, Wp[4] = {(R)1, (R)1, (R)1, (R)1};
+  const int din = mm.dim[K1 - 1], oin = mm.ooff[K1 - 1];   // the innermost outer axis
+  int sin = K1 == 1 ? s0a : 0;                             // ... and the current index along it
+  int dig[3] = {s0a < d0 ? s0a : 0, 0, 0};                 // indices of the other outer axes
+  R p[3] = {(R)0, (R)0, (R)0}, Wp[3] = {(R)1, (R)1, (R)1}, pin = (R)0;
 #pragma unroll
-  for (int lv = 0; lv < 4; ++lv)
-    if (lv < K1) Wp[lv] = (lv > 0 ? Wp[lv > 0 ? lv - 1 : 0] : (R)1) * qs[(mm.ooff[lv] + dig[lv]) * tu + u];
+  for (int lv = 0; lv < 3; ++lv)
+    if (lv < K1 - 1) Wp[lv] = (lv > 0 ? Wp[lv > 0 ? lv - 1 : 0] : (R)1) * qs[(mm.ooff[lv] + dig[lv]) * tus + u];
+  R wpre = K1 == 1 ? (R)1 : K1 == 2 ? Wp[0] : K1 == 3 ? Wp[1] : Wp[2];
   const int lrows = PERUNIT ? most : lbuf / rs / NCP;   // rows of one split's staging area (PERUNIT: all at once)
   R *Lr = Lbuf + (size_t)r * (PERUNIT ? 0 : lrows) * NCP;
-  __shared__ __align__(8) unsigned long long bar[8];   // one per split
-  if (!PERUNIT && tid < rs) bi_mbar_init(&bar[tid], 1);
   uint32_t phase = 0;
   bool failed = false;
   const R *mine = nullptr;   // PERUNIT: this unit's slice
@@ -421,6 +441,28 @@ __device__ __forceinline__ void contract_rt(const BatchMember &mm, const R *__re
     const int o = clamp_flag(P.obs[(size_t)unit * P.M + mm.modality], mm.m, P.status, BI_FLAG_OBS_RANGE);
     mine = (const R *)mm.logA + (size_t)(unit / P.T) * mm.gstride + (size_t)o * mm.P_pad;
   }
+  auto one_row = [&](const R *row, int s) {
+    const R qv = qs[(oin + s) * tus + u];
+    const R wf = wpre * qv;
+    R *acc = as + (oin + s) * nts + tid;
+    const R before = *acc;
+    R v0 = (R)0, v1 = (R)0;
+#pragma unroll
+    for (int cc = 0; cc < NCP; cc += VE) {
+      R x[VE];
+      if (PERUNIT) ldg_vec(row + cc, x);
+      else lds_vec(row + cc, x);
+#pragma unroll
+      for (int i = 0; i < VE; ++i) {
+        if (i & 1) v1 = fma(x[i], qc[cc + i], v1);
+        else v0 = fma(x[i], qc[cc + i], v0);
+        accc[cc + i] = fma(wf, x[i], accc[cc + i]);
+      }
+    }
+    const R val = v0 + v1;
+    *acc = fma(wpre, val, before);
+    pin = fma(qv, val, pin);
+  };
   for (int c0 = 0; c0 < most; c0 += lrows) {
     const int ra = row_a + c0;
     const int nr = max(0, min(lrows, row_b - ra));
@@ -435,34 +477,31 @@ __device__ __forceinline__ void contract_rt(const BatchMember &mm, const R *__re
       phase ^= 1u;
     }
     if (!has_unit || failed) continue;
-    for (int rr = 0; rr < nr; ++rr) {
-      constexpr int VE = 16 / (int)sizeof(R);
-      const R *row = PERUNIT ? mine + (size_t)(ra + rr) * NCP : Lr + rr * NCP;
-      const R wf = K1 == 1 ? Wp[0] : K1 == 2 ? Wp[1] : K1 == 3 ? Wp[2] : Wp[3];
-      R v0 = (R)0, v1 = (R)0;
-#pragma unroll
-      for (int cc = 0; cc < NCP; cc += VE) {
-        R x[VE];
-        if (PERUNIT) ldg_vec(row + cc, x);
-        else lds_vec(row + cc, x);
-#pragma unroll
-        for (int i = 0; i < VE; ++i) {
-          if (i & 1) v1 = fma(x[i], qc[cc + i], v1);
-          else v0 = fma(x[i], qc[cc + i], v0);
-          accc[cc + i] = fma(wf, x[i], accc[cc + i]);
-        }
+    const R *row = PERUNIT ? mine + (size_t)ra * NCP : Lr;
+    for (int left = nr; left > 0;) {
+      const int run = min(left, din - sin);   // rows to the end of the innermost axis, or of the staged rows
+      int i = 0;
+      for (; i + 1 < run; i += 2, row += 2 * NCP) {
+        one_row(row, sin + i);
+        one_row(row + NCP, sin + i + 1);
       }
-      R val = v0 + v1;
+      if (i < run) { one_row(row, sin + i); row += NCP; }
+      left -= run;
+      sin += run;
+      if (sin < din) continue;
+      // the axis is through: its sum climbs the others
+      sin = 0;
+      R val = pin;
+      pin = (R)0;
       bool act = true;
-      int top = K1;
+      int top = K1 - 1;
 #pragma unroll
-      for (int lv = 3; lv >= 0; --lv) {
-        if (lv < K1 && act) {
+      for (int lv = 2; lv >= 0; --lv) {
+        if (lv < K1 - 1 && act) {
           const int sj = dig[lv];
-          const int idx = (mm.ooff[lv] + sj) * nt + tid;
-          const R wprev = lv > 0 ? Wp[lv > 0 ? lv - 1 : 0] : (R)1;
-          as[idx] = fma(wprev, val, as[idx]);
-          if (lv > 0) p[lv > 0 ? lv - 1 : 0] = fma(qs[(mm.ooff[lv] + sj) * tu + u], val, p[lv > 0 ? lv - 1 : 0]);
+          R *acc = as + (mm.ooff[lv] + sj) * nts + tid;
+          *acc = fma(lv > 0 ? Wp[lv > 0 ? lv - 1 : 0] : (R)1, val, *acc);
+          if (lv > 0) p[lv > 0 ? lv - 1 : 0] = fma(qs[(mm.ooff[lv] + sj) * tus + u], val, p[lv > 0 ? lv - 1 : 0]);
           if (sj + 1 == mm.dim[lv]) {
             dig[lv] = 0;
             if (lv > 0) {
@@ -478,33 +517,34 @@ __device__ __forceinline__ void contract_rt(const BatchMember &mm, const R *__re
       }
       // prefix products of the outer beliefs, from the first axis whose index changed
 #pragma unroll
-      for (int lv = 0; lv < 4; ++lv)
-        if (lv < K1 && lv >= top)
-          Wp[lv] = (lv > 0 ? Wp[lv > 0 ? lv - 1 : 0] : (R)1) * qs[(mm.ooff[lv] + dig[lv]) * tu + u];
+      for (int lv = 0; lv < 3; ++lv)
+        if (lv < K1 - 1 && lv >= top)
+          Wp[lv] = (lv > 0 ? Wp[lv > 0 ? lv - 1 : 0] : (R)1) * qs[(mm.ooff[lv] + dig[lv]) * tus + u];
+      wpre = K1 == 1 ? (R)1 : K1 == 2 ? Wp[0] : K1 == 3 ? Wp[1] : Wp[2];
     }
   }
-  // ---- add the splits' partial messages and write them out: the outer axes' from the accumulator
-  // columns, then the last axis' through the same columns (they are free by then)
+  // ---- add the splits' partial messages and write them out (consecutive threads: consecutive states of one unit):
+  // the outer axes' from the accumulator columns, then the last axis' through the same columns (free by then)
   __syncthreads();
-  const int so = mm.ooff[K1];   // outer states of this member
-  for (int i = tid; i < so * tu; i += nt) {
-    const int uu = i % tu, st = i / tu;
-    if (uu >= tk.z) continue;
-    const R *col = as + (size_t)st * nt + uu;
-    R sum = col[0];
-    for (int k = 1; k < rs; ++k) sum += col[k * tu];
-    int j = 0;
-    while (j + 1 < K1 && st >= mm.ooff[j + 1]) ++j;
-    ((R *)P.ellp)[(int64_t)((size_t)mi * P.NU + unit_s[uu]) * P.Sp + mm.oout[j] + (st - mm.ooff[j])] = sum;
+  for (int j = 0; j < K1; ++j) {
+    const int d = mm.dim[j];
+    for (int i = tid; i < d * tu; i += nt) {
+      const int uu = i / d, sj = i - uu * d;
+      if (uu >= tk.z) continue;
+      const R *col = as + (size_t)(mm.ooff[j] + sj) * nts + uu;
+      R sum = col[0];
+      for (int k = 1; k < rs; ++k) sum += col[k * tu];
+      ((R *)P.ellp)[(int64_t)((size_t)mi * P.NU + unit_s[uu]) * P.Sp + mm.oout[j] + sj] = sum;
+    }
   }
   __syncthreads();
 #pragma unroll
-  for (int c = 0; c < NCP; ++c) as[c * nt + tid] = accc[c];
+  for (int c = 0; c < NCP; ++c) as[c * nts + tid] = accc[c];
   __syncthreads();
   for (int i = tid; i < NC * tu; i += nt) {
-    const int uu = i % tu, st = i / tu;
+    const int uu = i / NC, st = i - uu * NC;
     if (uu >= tk.z) continue;
-    const R *col = as + (size_t)st * nt + uu;
+    const R *col = as + (size_t)st * nts + uu;
     R sum = col[0];
     for (int k = 1; k < rs; ++k) sum += col[k * tu];
     ((R *)P.ellp)[(int64_t)((size_t)mi * P.NU + unit_s[uu]) * P.Sp + mm.oout[K1] + st] = sum;
@@ -523,9 +563,9 @@ bi_batch_contract_rt_kernel(BatchParams P, int cur, int first) {
   (void)first;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   R *Lbuf = reinterpret_cast<R *>(smem_raw);
-  R *qs = Lbuf + P.lbuf;                                   // [so_max][tu] beliefs of the outer axes, per unit
-  R *as = qs + (size_t)P.so_max * P.tu;                     // [so_max][threads] message accumulators, per thread
-  int *unit_s = reinterpret_cast<int *>(as + (size_t)P.so_max * blockDim.x);
+  R *qs = Lbuf + P.lbuf;                                   // [so_max][tu + 1] beliefs of the outer axes, per unit
+  R *as = qs + (size_t)P.so_max * (P.tu + 1);               // [so_max][threads + 1] message accumulators, per thread
+  int *unit_s = reinterpret_cast<int *>(as + (size_t)P.so_max * (blockDim.x + 1));
   int mi = 0;
   const int slot = (int)blockIdx.x + P.task_base;
   while (mi + 1 < P.nmem && slot >= P.mem[mi + 1].task0) ++mi;
@@ -1096,7 +1136,7 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
     // issued on 29 % of the cycles); fewer splits, then fewer units, when even that does not fit
     P.so_max = std::max(so_max, 32);
     for (;;) {
-      const size_t cols = ((size_t)P.so_max * tu + (size_t)P.so_max * tu * rs) * sizeof(R) + (size_t)tu * sizeof(int);
+      const size_t cols = ((size_t)P.so_max * (tu + 1) + (size_t)P.so_max * (tu * rs + 1)) * sizeof(R) + (size_t)tu * sizeof(int);
       size_t stage = std::min<size_t>(max_slice, 48 * 1024);
       const size_t half_sm = ((size_t)md->max_smem_optin + 1024) / 2 - 1024 - 1024;   // two CTAs, their reserved 1 KB each
       if (ncp_max <= 16 && cols + stage > half_sm && cols + 8 * 1024 <= half_sm) stage = half_sm - cols;
