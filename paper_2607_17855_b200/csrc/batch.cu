@@ -663,8 +663,9 @@ __device__ __forceinline__ R lane_group_max(R v) {
 // of latencies per unit, not a matter of throughput.
 // FINAL: the call's last iteration (the only one that writes outputs); DAMPED: the damped update.  Both
 // are instantiations of their own: the plain iteration in between runs sixteen times a call and is
-// bound by instruction issue, so it carries none of their code.
-template <typename R, int ALGO, int LW, bool FW, bool FINAL, bool DAMPED>
+// bound by instruction issue, so it carries none of their code.  BDEP: transitions with several parents, whose
+// messages were contracted with the slices (as a run-time test it cost the others a third of their time).
+template <typename R, int ALGO, int LW, bool FW, bool FINAL, bool DAMPED, bool BDEP>
 __global__ void __launch_bounds__(FW ? 32 * BI_MAX_F : 128)
 bi_batch_update_kernel(const BiDev *__restrict__ mdp, BatchParams P, UpdateArgs A) {
   static_assert(!FW || LW == 32, "a warp per factor needs a whole warp per unit");
@@ -711,7 +712,7 @@ bi_batch_update_kernel(const BiDev *__restrict__ mdp, BatchParams P, UpdateArgs 
       const R *ep = (const R *)P.ellp + (size_t)unit * Sp + p;   // member j's entry: NU * Sp elements further per j
       const size_t mstride = (size_t)NU * Sp;
       for (uint32_t mk = I.fmask; mk; mk &= mk - 1) x += ep[(__ffs(mk) - 1) * mstride];
-      if (A.child_plane >= 0) {   // transitions with several parents: their messages were contracted with the slices
+      if (BDEP) {
         if (t > 0) x += ep[A.child_plane * mstride];
         if (t + 1 < T)
           for (uint32_t mk = A.pmask[f]; mk; mk &= mk - 1) x += ep[(__ffs(mk) - 1) * mstride];
@@ -735,10 +736,9 @@ bi_batch_update_kernel(const BiDev *__restrict__ mdp, BatchParams P, UpdateArgs 
     const FactorInfo I = fi[f];
     const int n = I.n, np = I.np, op = I.op;
     R x = -bi_inf<R>();
-    if (s < n) {
+    if (BDEP && s < n) x = base[op + s];
+    if (!BDEP && s < n) {
       x = base[op + s];
-    }
-    if (s < n && A.child_plane < 0) {
       // both edges are evaluated (a window's end reads zeros and discards the result)
       const int up = t > 0 ? clamp_flag(acp[f], I.U, md.status, BI_FLAG_ACT_RANGE) : 0;
       const int uf = t + 1 < T ? clamp_flag(acp[F + f], I.U, md.status, BI_FLAG_ACT_RANGE) : 0;
@@ -1248,16 +1248,18 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
   const bool fw = lw == 32 && NU <= 64 * md->sm_count;   // a few thousand units: a warp per factor (see the kernel)
   const bool damped = A.xprev != nullptr;
   auto pick = [&](bool fin) -> UpdateKernel {
-#define BI_UPD(AL, LWV, FWV) \
-    (fin ? (damped ? (UpdateKernel)bi_batch_update_kernel<R, AL, LWV, FWV, true, true>   \
-                   : (UpdateKernel)bi_batch_update_kernel<R, AL, LWV, FWV, true, false>) \
-         : (damped ? (UpdateKernel)bi_batch_update_kernel<R, AL, LWV, FWV, false, true>  \
-                   : (UpdateKernel)bi_batch_update_kernel<R, AL, LWV, FWV, false, false>))
-    if (c.algo == BI_ALGO_VMP)
-      return fw ? BI_UPD(BI_ALGO_VMP, 32, true)
-                : lw == 8 ? BI_UPD(BI_ALGO_VMP, 8, false) : lw == 16 ? BI_UPD(BI_ALGO_VMP, 16, false) : BI_UPD(BI_ALGO_VMP, 32, false);
-    return fw ? BI_UPD(BI_ALGO_MMP, 32, true)
-              : lw == 8 ? BI_UPD(BI_ALGO_MMP, 8, false) : lw == 16 ? BI_UPD(BI_ALGO_MMP, 16, false) : BI_UPD(BI_ALGO_MMP, 32, false);
+#define BI_UPD(AL, LWV, FWV, BD) \
+    (fin ? (damped ? (UpdateKernel)bi_batch_update_kernel<R, AL, LWV, FWV, true, true, BD>   \
+                   : (UpdateKernel)bi_batch_update_kernel<R, AL, LWV, FWV, true, false, BD>) \
+         : (damped ? (UpdateKernel)bi_batch_update_kernel<R, AL, LWV, FWV, false, true, BD>  \
+                   : (UpdateKernel)bi_batch_update_kernel<R, AL, LWV, FWV, false, false, BD>))
+#define BI_UPL(AL, BD) \
+    (fw ? BI_UPD(AL, 32, true, BD) : lw == 8 ? BI_UPD(AL, 8, false, BD) \
+                                   : lw == 16 ? BI_UPD(AL, 16, false, BD) : BI_UPD(AL, 32, false, BD))
+    if (h.has_bdep) return BI_UPL(BI_ALGO_VMP, true);
+    if (c.algo == BI_ALGO_VMP) return BI_UPL(BI_ALGO_VMP, false);
+    return BI_UPL(BI_ALGO_MMP, false);
+#undef BI_UPL
 #undef BI_UPD
   };
   const UpdateKernel update_mid = pick(false), update_last = pick(true);
