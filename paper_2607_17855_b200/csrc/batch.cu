@@ -1264,13 +1264,14 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
   };
   const UpdateKernel update_mid = pick(false), update_last = pick(true);
   // a lane per unit and a warp per factor: shared models of up to 16 states per factor whose matrices fit beside
-  // the units' rows twice per SM, from about two CTAs per SM on (below that the form above has more warps)
+  // the units' rows twice per SM, from about two CTAs per SM on (below that the form above has more warps); not in
+  // float32 with zeros in A, where the order of sums is kept (see bi_block_serves)
   typedef void (*UnitKernel)(const BiDev *, BatchParams, UpdateArgs, UnitUpdate);
   UnitKernel unit_mid = nullptr, unit_last = nullptr;
   UnitUpdate UL;
   memset(&UL, 0, sizeof(UL));
   size_t unit_smem = 0;
-  if (h.G == 1 && nmax <= 16 && NU >= 64 * md->sm_count) {
+  if (h.G == 1 && nmax <= 16 && NU >= 64 * md->sm_count && !(sizeof(R) == 4 && md->has_zeros)) {
     constexpr int VE = 16 / (int)sizeof(R);
     size_t o = 0;
     for (int f = 0; f < h.F; ++f) {
@@ -1370,7 +1371,7 @@ int bi_launch_batch(const BiCall &c, bi_model *mut) {
     return BI_ERR_UNSUPPORTED;   // (with zeros in A the order of float32 sums is kept, see bi_block_serves)
   if (md->h.G != 1) {
     // per-agent models: the slices are re-read every iteration, which pays only while they stay in L2
-    // (measured on config 3's model with per-step slices: faster than the warp-per-step kernels at
+    // (measured on a three-factor model with per-step slices: faster than the warp-per-step kernels at
     // 112 MB of slices, slower at 224 MB)
     double bytes = 0;
     for (int gi = 0; gi < md->h.ngroups; ++gi)

@@ -673,6 +673,49 @@ bool bi_block_serves(const bi_model *md, int algo, int T) {
   return md->blk_plan[window ? 1 : 0] && !(md->has_zeros && (md->arith == BI_ARITH_F32 || (!window && T > 2)));
 }
 
+namespace {
+
+// Microseconds a window call would take here and on the batched kernels (batch.cu), for the choice between them.
+// Linear in what each spends its time on -- here block entries, warps and finishing passes per unit, there a
+// pair of launches per iteration, the longest slice's serial walk, slice entries and states per unit -- with
+// coefficients fitted to 113 structures of two to five factors, 2 048 to 62 000 units (12 and 17 % rms error).
+// Neither side wins by size alone: [8,13,10] under two rank-3 slices, 34 124 units, 2234 us here and 1844 us there;
+// [14,14,2,12] under a rank-4 slice, 2 472 units, 342 and 595 us.
+struct WindowCost { double block, batch; };
+WindowCost window_cost(const BiCall &c, const Plan &pl, const Variant &v) {
+  const BiDev &h = c.model->h;
+  const bool f64 = c.model->arith == BI_ARITH_F64;
+  const double per_sm = (double)c.N * c.T / c.model->sm_count * 1e-3, k = c.K * per_sm;   // thousands of units; unit-iterations
+  const double ent = pl.NB * (double)(pl.BR * pl.BC) * 1e-3, warps = v.LT / 32.0;
+  double slices = 0, longest = 0, states = 0, lanes = 0;
+  int members = 0, nmax = 1;
+  for (int gi = 0; gi < h.ngroups; ++gi) {
+    const BiGroup &g = h.grp[gi];
+    if (g.rank < 2) continue;
+    double e = 1;
+    for (int j = 0; j < g.rank; ++j) e *= j + 1 < g.rank ? g.dim[j] : bi_pad4(g.dim[j]);
+    longest = std::max(longest, e * 1e-3);
+    for (int mi = g.mem_begin; mi < g.mem_end; ++mi)
+      if (g.dim[g.rank - 1] > 32 || h.mem[mi].m > 4096) return {0.0, 1.0};   // (nothing the batched kernels take)
+    slices += e * 1e-3 * (g.mem_end - g.mem_begin);
+    members += g.mem_end - g.mem_begin;
+  }
+  for (int f = 0; f < h.F; ++f) {
+    nmax = std::max(nmax, (int)h.n[f]);
+    states += h.npad[f];
+  }
+  const bool lane_per_unit = nmax <= 16 && (double)c.N * c.T >= 64.0 * c.model->sm_count;   // (the update's form, see batch.cu)
+  if (!lane_per_unit) lanes = (double)h.F * (nmax <= 8 ? 8 : nmax <= 16 ? 16 : 32) * nmax;
+  WindowCost w;
+  w.block = f64 ? 13 + k * (56 * ent + (12 + 12 * v.nbpt) * warps + 89 * v.npass) + 1270 * per_sm * ent
+                : k * (1.6 * ent + (66 + 1.1 * v.nbpt) * warps + 42 * v.npass) + 1920 * per_sm * ent;
+  w.batch = f64 ? c.K * (6.3 * (members ? 2 : 1) + 2.9 * longest) + k * (35 * slices + 1.13 * states * (members + 2) + 0.106 * lanes) + 568 * per_sm * members
+                : 31 + c.K * (4.3 * (members ? 2 : 1) + 6.4 * longest) + k * (21 * slices + 1.27 * states * (members + 2) + 0.129 * lanes) + 63 * per_sm * members;
+  return w;
+}
+
+}  // namespace
+
 // Any model whose groups span at most four factors (transitions over at most three parents in window
 // calls), either arithmetic, as long as a step's blocks fit the register file and shared memory of an SM
 // (window calls: of a cluster); BI_ERR_UNSUPPORTED otherwise.
@@ -747,6 +790,10 @@ int bi_launch_block(const BiCall &c, bi_model *mut) {
       }
     }
     if (bv < 0) return BI_ERR_UNSUPPORTED;
+    if (!md->h.has_bdep && md->h.G == 1 && (long long)c.N * c.T >= 2048 && md->test_family == BI_FAMILY_ANY && !md->soft_shadow) {
+      const WindowCost w = window_cost(c, pl, pl.var[bv]);
+      if (w.batch < 0.9 * w.block) return BI_ERR_UNSUPPORTED;
+    }
     use_variant(pl.var[bv], p);
     p.W = 0;
     p.UC = buc; p.CS = bcs;
