@@ -12,16 +12,17 @@
 //             themselves.  The BR + BC + 2 results go to the message area, every state's entries in one
 //             contiguous run.  In window calls the transition matrices of the step's two edges are blocks
 //             as well, against the neighbouring steps' beliefs.
-//   finish    a lane (or 2, 4, 8 lanes) per state adds the state's run, the log-prior and the slices of
-//             single-factor modalities, and takes the softmax inside a segment of a warp; several small
-//             factors share a pass of one warp, large ones have a warp each.
+//   finish    one to sixteen lanes per state add the state's run, the log-prior and the slices of
+//             single-factor modalities and exponentiate; a factor's numerators are summed from a small exchange
+//             area.  Several small factors share a pass of one warp, large ones have a warp each.
 //
 // Why this shape: the kernels it replaced re-read the slices from shared memory or L1 in every
 // iteration, decoded row indices as they went and reduced column sums with shuffle trees; they ran at
 // 0.5 to 1.5 of the 36 TFLOP/s a float64 unit can do, bound by instruction issue and by serial phases
 // of single warps.  Here an iteration's shared-memory traffic is (BR + BC + 2) / (BR BC) of the slice
-// instead of all of it, all offsets are loop invariants in registers, and nothing is reduced by shuffles
-// except the softmax.
+// instead of all of it, and all offsets are loop invariants in registers.  Bound: the latency of the two
+// phases' dependent chains where few teams share an SM, issue and shared-memory throughput where many do.  Five
+// coupled factors filtered by 256 agents: 2116 -> 418 us; 1000 agents in float32: 1201 -> 433 us.
 #pragma once
 #include "bi_internal.h"
 #include "block.h"
