@@ -542,11 +542,18 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
   md->batch_unrolled = 1;
   for (int gi = 0; gi < h.ngroups; ++gi)
     if (h.grp[gi].rank >= 2 && (h.grp[gi].rank > 4 || bi_batch_shape(h.grp[gi].rank, h.grp[gi].dim) < 0)) md->batch_unrolled = 0;
-  bi_block_choose_shape(md);
+  // (register-tile models have kernels of their own for every call, and per-agent ones are large: no block-ordered copy)
+  if (md->tile_sb <= 0) bi_block_choose_shape(md);
 
   // ---- allocate and pack
   rc = dev_alloc(md, (void **)&h.status, 3 * sizeof(uint32_t));   // the flags, and two marks on A
   if (rc == BI_OK && cudaMemsetAsync(h.status, 0, 3 * sizeof(uint32_t), stream) != cudaSuccess) rc = BI_ERR_CUDA;
+  size_t blk_bytes = 0;   // every modality's block-ordered copy: one allocation
+  auto blk_size = [&](int gi, const BiMember &mm) { return ((size_t)G * mm.m * bi_block_slice_elems(md, gi) * esz + 255) & ~(size_t)255; };
+  for (int gi = 0; gi < h.ngroups; ++gi)
+    for (int mi = h.grp[gi].mem_begin; mi < h.grp[gi].mem_end; ++mi) blk_bytes += blk_size(gi, h.mem[mi]);
+  unsigned char *blk_mem = nullptr;
+  if (rc == BI_OK && blk_bytes) rc = dev_alloc(md, (void **)&blk_mem, blk_bytes);
   for (int gi = 0; gi < h.ngroups && rc == BI_OK; ++gi) {
     BiGroup &g = h.grp[gi];
     for (int mi = g.mem_begin; mi < g.mem_end && rc == BI_OK; ++mi) {
@@ -602,12 +609,10 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
         if (cudaGetLastError() != cudaSuccess) rc = BI_ERR_CUDA;
         mm.logA_T = tdst;
       }
-      if (const int per = rc == BI_OK ? bi_block_slice_elems(md, gi) : 0) {
-        void *bdst = nullptr;
-        rc = dev_alloc(md, &bdst, (size_t)G * mm.m * per * esz);
-        if (rc != BI_OK) break;
-        mm.logA_blk = bdst;
-        rc = bi_block_pack_member(md, gi, desc->A[i], mm.m, p.sstride, p.P, bdst, stream);
+      if (rc == BI_OK && bi_block_slice_elems(md, gi)) {
+        mm.logA_blk = blk_mem;
+        rc = bi_block_pack_member(md, gi, desc->A[i], mm.m, p.sstride, p.P, blk_mem, stream);
+        blk_mem += blk_size(gi, mm);
       }
       if (rc == BI_OK && md->tile_sb > 0) {
         PackTile q;
@@ -865,7 +870,7 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
     if (cudaMemcpyAsync(md->d, &md->h, sizeof(BiDev), cudaMemcpyHostToDevice, stream) != cudaSuccess)
       rc = BI_ERR_CUDA;
   }
-  if (rc == BI_OK && md->blk_BR) {   // (the dispatcher needs to know on the host: making a handle synchronises the stream)
+  if (rc == BI_OK && (md->blk_BR || arith == BI_ARITH_F32)) {   // (the dispatcher needs to know on the host: making a handle synchronises the stream)
     uint32_t z = 0;
     if (cudaMemcpyAsync(&z, h.status + 2, sizeof(z), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
         cudaStreamSynchronize(stream) != cudaSuccess)

@@ -94,7 +94,10 @@ __global__ void __launch_bounds__(WARPS * 32) bi_pair_filter_kernel(const PairPa
   __shared__ __align__(16) R exp_tab[EXP_TAB];
   __shared__ __align__(16) R sm_q[WARPS * UPW][QS];
   __shared__ __align__(16) R sm_e[WARPS * UPW][2 * LPU];   // e_a, e_b of the pair
-  bi_exp_tab_copy(exp_tab, p.exp_tab, threadIdx.x, blockDim.x);
+  // (asynchronously: a call of a few sweeps would wait half a microsecond for it here)
+  for (int j = threadIdx.x; j < EXP_TAB / 2; j += WARPS * 32)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(exp_tab + 2 * j)),
+                 "l"(p.exp_tab + 2 * j) : "memory");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int unit = lane / LPU, u = lane % LPU;
   int agent = (blockIdx.x * WARPS + warp) * UPW + unit;
@@ -109,7 +112,7 @@ __global__ void __launch_bounds__(WARPS * 32) bi_pair_filter_kernel(const PairPa
       v = p.carry_in ? p.carry_in[(size_t)agent * p.S + p.off[f] + u] : (R)p.q_prev[(size_t)agent * p.S + p.off[f] + u];
     sq[f * LPU + u] = v;
   }
-  __syncthreads();   // the table; every later exchange stays inside a warp
+  __syncwarp();
 
   const bool pair = p.fa >= 0;
   const bool a_ok = pair && u < p.na, b_ok = pair && u < p.nb;
@@ -145,6 +148,10 @@ __global__ void __launch_bounds__(WARPS * 32) bi_pair_filter_kernel(const PairPa
       for (int j = p.r1_begin[f]; j < p.r1_begin[f + 1]; ++j) {
         const int o = clamp_flag(__ldg(obs_t + p.r1_mod[j]), p.r1_m[j], p.status, BI_FLAG_OBS_RANGE);
         if (ok) c += __ldg(p.r1_logA[j] + (size_t)g * p.r1_gstride[j] + (size_t)o * p.r1_P[j] + u);
+      }
+      if (t == 0 && f == 0) {   // the table; every other exchange stays inside a warp
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
       }
       if (pair && f == p.fa) { ca = c; continue; }
       if (pair && f == p.fb) { cb = c; continue; }
