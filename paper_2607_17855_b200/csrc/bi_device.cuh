@@ -130,6 +130,15 @@ __device__ __forceinline__ void bi_exp_tab_copy(double *exp_tab, const double *_
   for (int j = tid; j < BI_EXP_TAB / 2; j += nthreads)
     reinterpret_cast<double2 *>(exp_tab)[j] = __ldg(reinterpret_cast<const double2 *>(src) + j);
 }
+// The same asynchronously, for kernels that have loads of their own to wait for first: after bi_exp_tab_wait and a
+// barrier of the threads that fetched it the table can be read.  (After a kernel that streamed through L2 the table
+// comes from memory.)
+__device__ __forceinline__ void bi_exp_tab_fetch(double *exp_tab, const double *src, int tid, int nthreads) {
+  for (int j = tid; j < BI_EXP_TAB / 2; j += nthreads)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(exp_tab + 2 * j)),
+                 "l"(src + 2 * j) : "memory");
+}
+__device__ __forceinline__ void bi_exp_tab_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ void bi_fast_tabs_init(double *exp_tab, double2 *log_tab, const double *__restrict__ src, int tid, int nthreads) {
   bi_exp_tab_copy(exp_tab, src, tid, nthreads);
   for (int j = tid; j < BI_LOG_TAB; j += nthreads) log_tab[j] = __ldg(reinterpret_cast<const double2 *>(src + BI_EXP_TAB) + j);

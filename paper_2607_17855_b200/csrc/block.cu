@@ -667,9 +667,12 @@ bool allow_smem(const void *kern, int slot, int device, size_t bytes) {
 // A model with zeros in A amplifies a rounding by up to 1e9 within sixteen iterations, and a trajectory carries
 // the result on from step to step: in float32, and in float64 over more than two filtered steps, another
 // order of summation gives other beliefs (measured: one in five such trajectories differs in the first
-// digit from the CTA kernel's).  Those calls stay with the kernels that have served them, bit for bit.
+// digit from the CTA kernel's).  Those calls stay with the kernels that have served them, bit for bit.  So does
+// float32 filtering of models coupled in one pair of factors: several sharp modalities on one pair carry float32
+// roundings to 2e-3 in a belief over thirty steps, and these kernels gain only 1.1 to 1.2 there.
 bool bi_block_serves(const bi_model *md, int algo, int T) {
   const bool window = algo != BI_ALGO_FILTER;
+  if (!window && md->pair_ok && md->arith == BI_ARITH_F32) return false;
   return md->blk_plan[window ? 1 : 0] && !(md->has_zeros && (md->arith == BI_ARITH_F32 || (!window && T > 2)));
 }
 

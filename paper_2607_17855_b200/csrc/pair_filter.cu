@@ -95,9 +95,7 @@ __global__ void __launch_bounds__(WARPS * 32) bi_pair_filter_kernel(const PairPa
   __shared__ __align__(16) R sm_q[WARPS * UPW][QS];
   __shared__ __align__(16) R sm_e[WARPS * UPW][2 * LPU];   // e_a, e_b of the pair
   // (asynchronously: a call of a few sweeps would wait half a microsecond for it here)
-  for (int j = threadIdx.x; j < EXP_TAB / 2; j += WARPS * 32)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(exp_tab + 2 * j)),
-                 "l"(p.exp_tab + 2 * j) : "memory");
+  bi_exp_tab_fetch(exp_tab, p.exp_tab, threadIdx.x, WARPS * 32);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int unit = lane / LPU, u = lane % LPU;
   int agent = (blockIdx.x * WARPS + warp) * UPW + unit;
@@ -150,7 +148,7 @@ __global__ void __launch_bounds__(WARPS * 32) bi_pair_filter_kernel(const PairPa
         if (ok) c += __ldg(p.r1_logA[j] + (size_t)g * p.r1_gstride[j] + (size_t)o * p.r1_P[j] + u);
       }
       if (t == 0 && f == 0) {   // the table; every other exchange stays inside a warp
-        asm volatile("cp.async.wait_all;" ::: "memory");
+        bi_exp_tab_wait();
         __syncthreads();
       }
       if (pair && f == p.fa) { ca = c; continue; }

@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(32) bi_tile3_filter_f64_kernel(const Tile3Para
   __shared__ __align__(16) R sm_tp[UPW][LPU * G::TPR + 2];
   __shared__ __align__(16) R sm_se[UPW][G::SE];
   const int lane = threadIdx.x;
-  bi_exp_tab_copy(exp_tab, p.exp_tab, lane, 32);
+  bi_exp_tab_fetch(exp_tab, p.exp_tab, lane, 32);
   // One warp-wide reduction finds the softmax shift of all the warp's agents at once, unless the model's
   // logits can lie too far apart for a common shift (many modalities, entries of A above 1, observation
   // vectors with the caller's weights): then every agent takes its own.
@@ -390,6 +390,10 @@ __global__ void __launch_bounds__(32) bi_tile3_filter_f64_kernel(const Tile3Para
       lpa = bi_log_inline(bi_max(row_dot<NA>(ra, sq, 0), (R)BI_EPS));
       lpb = bi_log_inline(bi_max(row_dot<NB>(rb, sq, NA), (R)BI_EPS));
       lpc = bi_log_inline(bi_max(row_dot<NC>(rc, sq, NA + NB), (R)BI_EPS));
+    }
+    if (t == 0) {
+      bi_exp_tab_wait();
+      __syncwarp();
     }
     sw.lpa = a_ok ? lpa : 0.0;
     sw.lpb = b_ok ? lpb : 0.0;
