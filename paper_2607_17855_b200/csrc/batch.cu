@@ -1314,14 +1314,15 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
   };
   const UpdateKernel update_mid = pick(false), update_last = pick(true);
   // a lane per unit and a warp per factor: shared models of up to 16 states per factor whose matrices fit beside
-  // the units' rows twice per SM, from about two CTAs per SM on (below that the form above has more warps); not in
+  // the units' rows twice per SM, from about two CTAs and six warps per SM on (below that the form above has
+  // more warps: one factor of four states, 12 405 units, 86 against 107 us a call); not in
   // float32 with zeros in A, where the order of sums is kept (see bi_block_serves)
   typedef void (*UnitKernel)(const BiDev *, BatchParams, UpdateArgs, UnitUpdate);
   UnitKernel unit_mid = nullptr, unit_last = nullptr;
   UnitUpdate UL;
   memset(&UL, 0, sizeof(UL));
   size_t unit_smem = 0;
-  if (h.G == 1 && nmax <= 16 && NU >= 64 * md->sm_count && !(sizeof(R) == 4 && md->has_zeros)) {
+  if (h.G == 1 && nmax <= 16 && NU >= 64 * md->sm_count && (long long)NU * h.F >= 192LL * md->sm_count && !(sizeof(R) == 4 && md->has_zeros)) {
     constexpr int VE = 16 / (int)sizeof(R);
     size_t o = 0;
     for (int f = 0; f < h.F; ++f) {

@@ -707,7 +707,7 @@ WindowCost window_cost(const BiCall &c, const Plan &pl, const Variant &v) {
     nmax = std::max(nmax, (int)h.n[f]);
     states += h.npad[f];
   }
-  const bool lane_per_unit = nmax <= 16 && (double)c.N * c.T >= 64.0 * c.model->sm_count;   // (the update's form, see batch.cu)
+  const bool lane_per_unit = nmax <= 16 && (double)c.N * c.T * std::min(1.0, h.F / 3.0) >= 64.0 * c.model->sm_count;   // (the update's form, see batch.cu)
   if (!lane_per_unit) lanes = (double)h.F * (nmax <= 8 ? 8 : nmax <= 16 ? 16 : 32) * nmax;
   WindowCost w;
   w.block = f64 ? 13 + k * (56 * ent + (12 + 12 * v.nbpt) * warps + 89 * v.npass) + 1270 * per_sm * ent
