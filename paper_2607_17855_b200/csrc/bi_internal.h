@@ -197,7 +197,7 @@ int bi_launch_block(const BiCall &c, bi_model *mut);        // any structure of 
 // elements of one outcome's slice of group gi in the block kernels' order (0: the model has none)
 int bi_block_slice_elems(const bi_model *md, int gi);
 // whether the block kernels may serve such calls on this model (they may still decline one that does not fit)
-bool bi_block_serves(const bi_model *md, int algo, int T);
+bool bi_block_serves(const bi_model *md, int algo);
 // tries the kernel families in order (the dispatcher behind every inference call)
 int bi_dispatch(const BiCall &c, bi_model *mut);
 // inference with observations given as categorical vectors [N][T][sum m_i]

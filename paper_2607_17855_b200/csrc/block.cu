@@ -665,15 +665,16 @@ bool allow_smem(const void *kern, int slot, int device, size_t bytes) {
 }  // namespace
 
 // A model with zeros in A amplifies a rounding by up to 1e9 within sixteen iterations, and a trajectory carries
-// the result on from step to step: in float32, and in float64 over more than two filtered steps, another
-// order of summation gives other beliefs (measured: one in five such trajectories differs in the first
-// digit from the CTA kernel's).  Those calls stay with the kernels that have served them, bit for bit.  So does
-// float32 filtering of models coupled in one pair of factors: several sharp modalities on one pair carry float32
-// roundings to 2e-3 in a belief over thirty steps, and these kernels gain only 1.1 to 1.2 there.
-bool bi_block_serves(const bi_model *md, int algo, int T) {
+// the result on from step to step: in float32, and in filtering, another order of summation gives other beliefs
+// (measured: one in five such trajectories differs in the first digit from the CTA kernel's).  Those calls stay
+// with the kernels that have served them, bit for bit.  The number of steps has no say in it: a trajectory
+// filtered in blocks of steps is the single call's (bi_filter_continue), and a stream of ticks is a trajectory too.
+// Float32 filtering of models coupled in one pair of factors stays as well: several sharp modalities on one pair
+// carry float32 roundings to 2e-3 in a belief over thirty steps, and these kernels gain only 1.1 to 1.2 there.
+bool bi_block_serves(const bi_model *md, int algo) {
   const bool window = algo != BI_ALGO_FILTER;
   if (!window && md->pair_ok && md->arith == BI_ARITH_F32) return false;
-  return md->blk_plan[window ? 1 : 0] && !(md->has_zeros && (md->arith == BI_ARITH_F32 || (!window && T > 2)));
+  return md->blk_plan[window ? 1 : 0] && !(md->has_zeros && (md->arith == BI_ARITH_F32 || !window));
 }
 
 namespace {
@@ -728,7 +729,7 @@ int bi_launch_block(const BiCall &c, bi_model *mut) {
   const Plan *plp = static_cast<const Plan *>(md->blk_plan[window ? 1 : 0]);
   if (!plp || !plp->ok) return BI_ERR_UNSUPPORTED;
   if (window && md->h.has_bdep && (c.algo == BI_ALGO_MMP || c.lnprior)) return BI_ERR_UNSUPPORTED;
-  if (!bi_block_serves(md, c.algo, c.T)) return BI_ERR_UNSUPPORTED;
+  if (!bi_block_serves(md, c.algo)) return BI_ERR_UNSUPPORTED;
   if (plp->NB == 0) return BI_ERR_UNSUPPORTED;   // nothing to contract: the CTA kernel's warp per factor does that
   if (window && !md->h.has_bdep && md->batch_unrolled && (long long)c.N * c.T >= 4096) return BI_ERR_UNSUPPORTED;   // (see batch_unrolled)
   const Plan &pl = *plp;

@@ -231,7 +231,7 @@ int run_soft_t(const bi_model *model, int algo, int N, int T, const float *obs_s
   }
   // A call that the block kernels serve: their groups' slices are formed in block order instead (a rank-1
   // group's stay packed; the packed ones of the others follow only if those kernels decline the call).
-  const bool block = !tile && bi_block_serves(model, algo, T) &&
+  const bool block = !tile && bi_block_serves(model, algo) &&
                      (sizeof(R) == 4 || !(algo == BI_ALGO_FILTER ? model->pair_ok : model->rank2_ok));
   size_t off_blk[BI_MAX_GROUPS] = {};
   for (int k = 0; k < h.ngroups && block; ++k)

@@ -91,3 +91,26 @@ def test_float32(algo):
     # (dense and few iterations: the tolerance of check_workload's strict=False form is not a numerical one)
     res = check_workload(_workload(50, [9, 5, 7, 6], [[0, 1, 2], [1, 3]], N=21, T=5, K=4), algo, arith="f32", strict=False)
     assert res["q_max_err"] < 1e-3, res   # four undamped float32 iterations: 1e-6 of the logits' sums, amplified below 1e3
+
+
+@pytest.mark.parametrize("bdep", [None, [[0, 1], [1], [2, 3], [3]]], ids=["one_parent", "several_parents"])
+def test_filtering_in_blocks_of_steps_on_sparse_models(bdep):
+    """bi_filter_continue promises the single call's beliefs bit for bit.  Zeros in A amplify the last bit of a
+    belief to its first digit, so the kernel must not depend on how many steps a call has."""
+    import torch
+    import paper_2607_17855_b200 as bi
+    from test_gpu_parity import _blockwise
+    n, dep, U = [5, 7, 6, 4], [[0, 1, 2], [2, 3, 1], [3]], [2, 1, 3, 2]
+    rng = np.random.default_rng(71)
+    m = [9, 11, 5]
+    A, B, D = make_model(rng, n, m, dep, U, 1, sparsity=0.7, d_alpha=1.0, bdep=bdep)
+    obs, act = sample_streams(rng, n, m, dep, U, 1, A, B, D, 96, 10, bdep=bdep)
+    w = Workload(name="sparse", algo="filter", n=np.asarray(n, np.int32), m=np.asarray(m, np.int32), dep=dep,
+                 U=np.asarray(U, np.int32), G=1, A=A, B=B, D=D, N=96, T=10, K=16, obs=obs, act=act, bdep=bdep)
+    md = bi.model_from_workload(w)
+    whole = md.bi_filter(torch.from_numpy(w.obs).cuda(), torch.from_numpy(w.act).cuda(), w.K).cpu().numpy()
+    for cuts in (list(range(11)), [0, 2, 4, 6, 8, 10], [0, 5, 6, 8, 10]):
+        q, _ = _blockwise(md, w, cuts, w.K)
+        assert np.array_equal(q, whole), (cuts, np.abs(q - whole).max())
+    assert md.status() == 0
+    md.close()
