@@ -870,7 +870,7 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
     if (cudaMemcpyAsync(md->d, &md->h, sizeof(BiDev), cudaMemcpyHostToDevice, stream) != cudaSuccess)
       rc = BI_ERR_CUDA;
   }
-  if (rc == BI_OK && (md->blk_BR || arith == BI_ARITH_F32)) {   // (the dispatcher needs to know on the host: making a handle synchronises the stream)
+  if (rc == BI_OK) {   // the marks on A choose kernels on the host; the caller's arrays are free from here on (for every kind of model)
     uint32_t z = 0;
     if (cudaMemcpyAsync(&z, h.status + 2, sizeof(z), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
         cudaStreamSynchronize(stream) != cudaSuccess)

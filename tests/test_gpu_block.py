@@ -114,3 +114,24 @@ def test_filtering_in_blocks_of_steps_on_sparse_models(bdep):
         assert np.array_equal(q, whole), (cuts, np.abs(q - whole).max())
     assert md.status() == 0
     md.close()
+
+
+@pytest.mark.parametrize("case", ["tile", "rank5", "block", "pair"])
+def test_the_model_is_packed_when_the_call_returns(case):
+    """The caller may reuse A, B and D (on any stream) once bi_model_create has returned: whatever the kind of
+    model, the packing is then done, also behind work that the stream had queued before."""
+    import torch
+    import paper_2607_17855_b200 as bi
+    n, dep = {"tile": ([8, 8, 6], [[0, 1, 2]]), "rank5": ([3, 2, 4, 2, 3], [[0, 1, 2, 3, 4]]),
+              "block": ([5, 4, 7], [[0, 1, 2]]), "pair": ([4, 3], [[0, 1]])}[case]
+    w = _workload(80, n, dep, N=3, T=2, K=2)
+    arrays = [[torch.from_numpy(x).cuda() for x in part] for part in (w.A, w.B, w.D)]
+    x = torch.randn(4096, 4096, device="cuda")
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s):
+        for _ in range(40):   # some milliseconds each
+            x = torch.mm(x, x).clamp_(-1, 1)
+        md = bi.Model(w.n, w.m, w.dep, w.U, w.G, *arrays)
+        assert s.query()
+    md.close()
