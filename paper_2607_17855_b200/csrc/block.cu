@@ -564,11 +564,18 @@ void fill_params(const BiCall &c, const Plan &pl, Params &p) {
   p.mmp = c.algo == BI_ALGO_MMP;
   p.has_bdep = h.has_bdep;
   p.lambda = c.lambda;
-  // No softmax shift in float64: with probabilities in A and B a logit is at least
-  // (modalities + 3) ln 1e-16 below zero, 53.2 binary orders each; beyond that, or with the caller's own
-  // weights or starting beliefs (used as given), every segment shifts by its own maximum (a model with
-  // entries above 1 is marked in status[1]).
-  p.common = !md->soft_shadow && !(c.q_init && c.lambda != 1.0) && (h.M + 3) * 54 < 960;
+  // No softmax shift in float64: with probabilities in A and B none of the terms of a logit is below ln 1e-16,
+  // 53.2 binary orders below zero.  They are one per modality, the prior or past message and the future message; with
+  // several parents per transition a future message from every factor whose transition reads this one.
+  // Beyond seventeen of them, or with the caller's own weights or starting beliefs (used as given), every
+  // segment shifts by its own maximum (a model with entries above 1 is marked in status[1]).
+  int terms = h.M + 3;
+  if (window && h.has_bdep) {
+    int readers[BI_MAX_F] = {};
+    for (int f = 0; f < h.F; ++f)
+      for (int j = 0; j < h.bdep_len[f]; ++j) terms = std::max(terms, h.M + 1 + ++readers[h.bdep[f][j]]);
+  }
+  p.common = !md->soft_shadow && !(c.q_init && c.lambda != 1.0) && terms * 54 < 960;
   for (int f = 0; f < h.F; ++f) {
     p.n[f] = h.n[f]; p.off[f] = h.off[f]; p.qo[f] = pl.qo[f]; p.npad[f] = h.npad[f]; p.U[f] = h.U[f];
     p.logD[f] = h.logD[f];

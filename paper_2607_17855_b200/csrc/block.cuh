@@ -297,8 +297,8 @@ struct StepOut {          // where a unit's results go (pointers already at the 
 // The sum of the numerators is taken by every lane itself from the exchange area (in shared memory, one
 // 16-byte load and two additions per two states, all lanes of a factor reading one address): states need no
 // alignment to powers of two within a pass, and nothing is shuffled.
-// The exponentials need no shift where the logits are sums of logarithms of probabilities (`common`): none
-// is above zero and, with up to 14 modalities, none below -640, so the numerators and their sum are normal
+// The exponentials need no shift where the logits are sums of at most seventeen logarithms of probabilities (`common`,
+// decided by the launcher): none is above zero and none below -640, so the numerators and their sum are normal
 // numbers.  Otherwise they are relative to the factor's largest logit (starting beliefs are used as
 // given, which counts for the first iteration, and under damping for all).
 template <typename R, bool WIN, bool FINAL>

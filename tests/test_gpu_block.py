@@ -135,3 +135,33 @@ def test_the_model_is_packed_when_the_call_returns(case):
         md = bi.Model(w.n, w.m, w.dep, w.U, w.G, *arrays)
         assert s.query()
     md.close()
+
+
+@pytest.mark.parametrize("K", [1, 2])
+def test_improbable_states_under_many_future_messages(K):
+    """A factor whose thirteen impossible outcomes put every state at the floor, ln 1e-16 each, and whose state is
+    read by eight transitions that the uniform next beliefs contradict (K = 1: 15/16 of ln 1e-16 each): logits near
+    -740, where exp underflows, so the softmax must be relative to the largest of them."""
+    M, n, F = 14, [3] + [16] * 7, 8
+    rng = np.random.default_rng(90)
+    A = []
+    for i in range(M):
+        a = np.zeros((1, 4, 3), np.float32)   # (outcome 3 has probability zero in every state)
+        a[0, :3] = rng.dirichlet(np.ones(3), 3).T
+        if i == 0:
+            a[0, 3], a[0, :3] = 0.25, 0.75 * a[0, :3]
+        A.append(a)
+    B, D = [], []
+    for f, nf in enumerate(n):
+        b = np.zeros((1, nf, 3, 2), np.float32)
+        if f == 0:
+            b[:] = 1.0 / 3.0
+        else:
+            b[:, 0] = 1.0
+        B.append(b)
+        D.append(np.full((1, nf), 1.0 / nf, np.float32))
+    N, T = 4, 4
+    w = Workload(name="improbable", algo="vmp", n=np.asarray(n, np.int32), m=np.full(M, 4, np.int32), dep=[[0]] * M,
+                 U=np.full(F, 2, np.int32), G=1, A=A, B=B, D=D, N=N, T=T, K=K, obs=np.full((N, T, M), 3, np.int32),
+                 act=np.zeros((N, T - 1, F), np.int32), bdep=[[0]] * F)
+    print(check_workload(w, "vmp"))
