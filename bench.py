@@ -214,7 +214,7 @@ def bench_config(torch, bi, w, algo, arith, steps, warmup, flush):
     launches = (md.launch_count - l0) // (steps + warmup)
     assert md.status() == 0
     res = {"seconds": sum(times) / len(times), "best": min(times), "median": sorted(times)[len(times) // 2],
-           "pack_ms": pack_ms, "kernel": md.last_kernel,
+           "pack_ms": pack_ms, "kernel": md.last_family,
            "launches_per_step": launches, "model": md, "obs": obs, "act": act, "q": q}
     return res
 
@@ -286,7 +286,7 @@ def run_case(args):
     ms = a.elapsed_time(b)
     assert md.status() == 0
     print(json.dumps({"workload": w.name, "algo": algo, "agents": w.N, "T": w.T, "K": w.K, "arith": args.arith,
-                      "soft": bool(args.soft), "kernel": md.last_kernel, "ms": ms,
+                      "soft": bool(args.soft), "kernel": md.last_family, "ms": ms,
                       "updates_per_s": w.updates / (ms * 1e-3)}), flush=True)
 
 
@@ -479,7 +479,7 @@ def main():
             qd = torch.empty((w.N, w.T, w.S), dtype=torch.float32, device="cuda")
             ts = time_steps(lambda: mdd.bi_filter(head["obs"], head["act"], w.K, q_out=qd), max(3, args.steps // 2),
                             3, flush, torch)
-            damped[ar] = (sum(ts) / len(ts), qd, mdd.last_kernel)
+            damped[ar] = (sum(ts) / len(ts), qd, mdd.last_family)
             mdd.close()
         dd = (damped["f32"][1] - damped["f64"][1]).abs().reshape(w.N, -1).max(dim=1).values
         others["config2_filter_damped_0.5"] = {
@@ -531,7 +531,7 @@ def main():
         sec_s = sum(ts) / len(ts)
         slice_flops = 2.0 * w.N * w.T * float(off[-1]) * sum(int(np.prod([w.n[f] for f in d])) for d in w.dep[:1])
         others[f"config2_filter_soft_{args.arith}"] = {
-            "value": w.updates / sec_s, "unit": UNIT, "ms_per_step": sec_s * 1e3, "kernel": md_s.last_kernel,
+            "value": w.updates / sec_s, "unit": UNIT, "ms_per_step": sec_s * 1e3, "kernel": md_s.last_family,
             "launches_per_step": (md_s.launch_count - l0) // (max(3, args.steps // 4) + 3),
             "slice_forming_gflop": slice_flops / 1e9}
         md_s.close()
@@ -548,7 +548,7 @@ def main():
             ts = time_steps(lambda: md4.bi_mmp(d_obs4, d_act4, w4.K, q_out=q4), max(3, args.steps // 4), 3, flush, torch)
             sec4 = sum(ts) / len(ts)
             others[f"config4_mmp_compressed_{args.arith}"] = {
-                "value": w4.updates / sec4, "unit": UNIT, "ms_per_step": sec4 * 1e3, "kernel": md4.last_kernel,
+                "value": w4.updates / sec4, "unit": UNIT, "ms_per_step": sec4 * 1e3, "kernel": md4.last_family,
                 "slice_bytes_dense": int(dense_b), "slice_bytes_compressed": int(comp_b)}
         md4.close()
         del d_obs4, d_act4, q4, w4

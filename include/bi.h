@@ -377,9 +377,14 @@ int bi_filter_static(const bi_model_desc *desc, int32_t N, int32_t T, const int3
  * call in *flags (HOST) and clears them. */
 int bi_status(const bi_model_t *model, void *cuda_stream, uint32_t *flags);
 
-/* Name of the kernel family the dispatcher picked for the most recent
- * inference call on this handle ("" before the first call).  Static storage. */
+/* The class of the most recent inference call on this handle, as the name of a kernel family ("" before the
+ * first call): the family that ran it, except that the block kernels -- which take calls of the "cta", "warp" and
+ * "batch" classes -- are reported under the class of the call.  Static storage. */
 const char *bi_last_kernel(const bi_model_t *model);
+
+/* Name of the kernel family that ran the most recent inference call on this handle: as bi_last_kernel, with
+ * the block kernels under their own name ("block_filter_f64", "block_vmp_f32", ...).  Static storage. */
+const char *bi_last_family(const bi_model_t *model);
 
 /* Number of kernel launches issued by inference calls on this handle so far. */
 int64_t bi_launch_count(const bi_model_t *model);

@@ -29,7 +29,7 @@ BI_ARITH_F32 = 1
 ARITH = {"f64": BI_ARITH_F64, "f32": BI_ARITH_F32}
 
 EXPORTS = ["bi_model_create", "bi_model_create_arith", "bi_model_create_bdep", "bi_model_slice_bytes", "bi_model_set_compressed", "bi_model_arith", "bi_model_destroy", "bi_filter", "bi_filter_from", "bi_filter_continue", "bi_vmp", "bi_mmp", "bi_vmp_warm", "bi_mmp_warm", "bi_vmp_from", "bi_mmp_from", "bi_filter_soft", "bi_vmp_soft", "bi_mmp_soft", "bi_model_set_damping", "bi_status",
-           "bi_last_kernel", "bi_launch_count", "bi_strerror", "bi_filter_static"]
+           "bi_last_kernel", "bi_last_family", "bi_launch_count", "bi_strerror", "bi_filter_static"]
 BI_STATIC_SCRATCH_BYTES = 4 << 20
 
 
@@ -95,6 +95,8 @@ def lib():
         L.bi_status.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.POINTER(ctypes.c_uint32)]
         L.bi_last_kernel.restype = ctypes.c_char_p
         L.bi_last_kernel.argtypes = [ctypes.c_void_p]
+        L.bi_last_family.restype = ctypes.c_char_p
+        L.bi_last_family.argtypes = [ctypes.c_void_p]
         L.bi_launch_count.restype = ctypes.c_int64
         L.bi_launch_count.argtypes = [ctypes.c_void_p]
         L.bi_strerror.restype = ctypes.c_char_p
@@ -323,6 +325,11 @@ class Model:
     @property
     def last_kernel(self) -> str:
         return lib().bi_last_kernel(self._h).decode()
+
+    @property
+    def last_family(self) -> str:
+        """The kernel family that ran the latest call (``last_kernel`` names the class of the call)."""
+        return lib().bi_last_family(self._h).decode()
 
     @property
     def launch_count(self) -> int:

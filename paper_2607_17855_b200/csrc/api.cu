@@ -921,6 +921,7 @@ __global__ void bi_predictive_prior_kernel(const BiDev *__restrict__ mdp, int N,
 }
 
 int bi_dispatch(const BiCall &c, bi_model *mut) {
+  mut->last_block = nullptr;
   if (c.model->h.has_bdep) {
     // Transition tensors with several parents.  In filtering they enter only the prior, formed once per
     // step, which the CTA-per-agent filtering kernel computes; window calls (VMP) need them in every
@@ -1153,6 +1154,10 @@ extern "C" int bi_status(const bi_model_t *model, void *cuda_stream, uint32_t *f
 }
 
 extern "C" const char *bi_last_kernel(const bi_model_t *model) { return model ? model->last_kernel : ""; }
+
+extern "C" const char *bi_last_family(const bi_model_t *model) {
+  return !model ? "" : model->last_block ? model->last_block : model->last_kernel;
+}
 
 extern "C" int64_t bi_launch_count(const bi_model_t *model) { return model ? model->launches : 0; }
 

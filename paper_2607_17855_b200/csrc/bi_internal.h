@@ -133,6 +133,7 @@ struct bi_model {
   int rows_max;     // largest first-level row count over groups
   int64_t launches;
   const char *last_kernel;
+  const char *last_block;   // the block kernels' own name when they ran the most recent call, else NULL
   void *ws;         // workspace of the batched window path (stream-ordered allocation), or NULL
   size_t ws_bytes;
   void *ws_soft;    // workspace of the calls that take observation vectors, or NULL

@@ -836,8 +836,11 @@ int bi_launch_block(const BiCall &c, bi_model *mut) {
     return BI_ERR_CUDA;
   }
   mut->launches += 1;
-  // family names: by the class of call the kernels of each family serve
   const bool f64 = esz == 8;
+  if (!window) mut->last_block = f64 ? "block_filter_f64" : "block_filter_f32";
+  else if (c.algo == BI_ALGO_VMP) mut->last_block = f64 ? "block_vmp_f64" : "block_vmp_f32";
+  else mut->last_block = f64 ? "block_mmp_f64" : "block_mmp_f32";
+  // bi_last_kernel names the class of call: the family whose calls of this size these are
   if (!window) mut->last_kernel = f64 ? "cta_filter_f64" : "cta_filter_f32";
   else if (md->h.has_bdep || (long long)c.N * c.T < 2048)
     mut->last_kernel = c.algo == BI_ALGO_VMP ? (f64 ? "warp_vmp_f64" : "warp_vmp_f32") : (f64 ? "warp_mmp_f64" : "warp_mmp_f32");

@@ -329,6 +329,7 @@ int run_soft_t(const bi_model *model, int algo, int N, int T, const float *obs_s
   }
   // (a group of one modality is its own pre-summed table: the shadow's T per-agent slices)
   sh.soft_shadow = 1;
+  sh.last_block = nullptr;
   if (!block) sh.blk_plan[0] = sh.blk_plan[1] = nullptr;
   sh.pair_ok = kpair >= 0 || (model->pair_ok && sizeof(R) == 8 && algo == BI_ALGO_FILTER);
   // (the pair filtering kernel needs the transposed slices formed above, or no pair at all; the pair
@@ -373,6 +374,7 @@ int run_soft_t(const bi_model *model, int algo, int N, int T, const float *obs_s
   mut->ws_bytes = sh.ws_bytes;
   mut->launches += launches + (sh.launches - before);
   mut->last_kernel = sh.last_kernel;
+  mut->last_block = sh.last_block;
   return rc;
 }
 

@@ -288,6 +288,6 @@ def check_workload(w, algo=None, agents=None, arith="f64", strict=True, conditio
         out.update(strict_checks(sub, algo, ref=ref, arith=arith))
     else:
         out = compare(sub, q, lq, am, *ref) if strict else error_stats(sub, q, ref[0])
-    out["kernel"] = md.last_kernel
+    out["kernel"], out["family"] = md.last_kernel, md.last_family
     md.close()
     return out

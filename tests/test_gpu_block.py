@@ -36,12 +36,14 @@ FILTER = {
 @pytest.mark.parametrize("case", sorted(FILTER))
 def test_filtering(case, N):
     n, dep = FILTER[case]
-    print(check_workload(_workload(10 + N, n, dep, N=N, T=4, K=7), "filter"))
+    res = check_workload(_workload(10 + N, n, dep, N=N, T=4, K=7), "filter")
+    assert res["family"] == "block_filter_f64", res
 
 
 def test_filtering_large_batches_share_a_cta():
-    print(check_workload(_workload(3, [5, 4, 3], [[0, 1, 2], [1, 0, 2]], N=3701, T=2, K=3), "filter",
-                         agents=range(0, 3701, 97)))
+    res = check_workload(_workload(3, [5, 4, 3], [[0, 1, 2], [1, 0, 2]], N=3701, T=2, K=3), "filter",
+                         agents=range(0, 3701, 97))
+    assert res["family"] == "block_filter_f64", res
 
 
 WINDOW = {   # (n, dep, T): one CTA, idle steps in the last one of a cluster, the longest window, blocks in shared memory
@@ -58,18 +60,21 @@ WINDOW = {   # (n, dep, T): one CTA, idle steps in the last one of a cluster, th
 @pytest.mark.parametrize("case", sorted(WINDOW))
 def test_windows(case, algo):
     n, dep, T = WINDOW[case]
-    print(check_workload(_workload(20, n, dep, N=5, T=T, K=6), algo))
+    res = check_workload(_workload(20, n, dep, N=5, T=T, K=6), algo)
+    assert res["family"] == f"block_{algo}_f64", res
 
 
 @pytest.mark.parametrize("algo", ["filter", "vmp", "mmp"])
 def test_models_of_their_own(algo):
-    print(check_workload(_workload(30, [6, 5, 9], [[0, 1, 2], [2, 1]], N=9, T=7, K=5, G=9), algo))
+    res = check_workload(_workload(30, [6, 5, 9], [[0, 1, 2], [2, 1]], N=9, T=7, K=5, G=9), algo)
+    assert res["family"] == f"block_{algo}_f64", res
 
 
 @pytest.mark.parametrize("algo", ["filter", "vmp"])
 @pytest.mark.parametrize("bdep", [[[0, 1], [1, 2], [2, 0]], [[2], [0, 1, 2], [1, 2]], [[1, 0, 2], [2, 1], [2]]])
 def test_transitions_with_several_parents(bdep, algo):
-    print(check_workload(_workload(40, [9, 4, 7], [[0, 1], [1, 2, 0]], N=7, T=6, K=5, bdep=bdep), algo))
+    res = check_workload(_workload(40, [9, 4, 7], [[0, 1], [1, 2, 0]], N=7, T=6, K=5, bdep=bdep), algo)
+    assert res["family"] == f"block_{algo}_f64", res
 
 
 @pytest.mark.parametrize("n, dep, bdep, T", [
@@ -83,13 +88,14 @@ def test_batched_transitions_with_several_parents(n, dep, bdep, T):
     N = 2100 if T == 1 else 2100 // T + 60
     with family_forced("batch"):
         res = check_workload(_workload(60 + T, n, dep, N=N, T=T, K=5, bdep=bdep), "vmp", agents=range(0, N, 23))
-    assert res["kernel"] == "batch_vmp_f64", res
+    assert res["family"] == "batch_vmp_f64", res
 
 
 @pytest.mark.parametrize("algo", ["filter", "vmp", "mmp"])
 def test_float32(algo):
     # (dense and few iterations: the tolerance of check_workload's strict=False form is not a numerical one)
     res = check_workload(_workload(50, [9, 5, 7, 6], [[0, 1, 2], [1, 3]], N=21, T=5, K=4), algo, arith="f32", strict=False)
+    assert res["family"] == f"block_{algo}_f32", res
     assert res["q_max_err"] < 1e-3, res   # four undamped float32 iterations: 1e-6 of the logits' sums, amplified below 1e3
 
 
@@ -164,4 +170,5 @@ def test_improbable_states_under_many_future_messages(K):
     w = Workload(name="improbable", algo="vmp", n=np.asarray(n, np.int32), m=np.full(M, 4, np.int32), dep=[[0]] * M,
                  U=np.full(F, 2, np.int32), G=1, A=A, B=B, D=D, N=N, T=T, K=K, obs=np.full((N, T, M), 3, np.int32),
                  act=np.zeros((N, T - 1, F), np.int32), bdep=[[0]] * F)
-    print(check_workload(w, "vmp"))
+    res = check_workload(w, "vmp")
+    assert res["family"] == "block_vmp_f64", res
