@@ -924,14 +924,16 @@ int bi_dispatch(const BiCall &c, bi_model *mut) {
   mut->last_block = nullptr;
   if (c.model->h.has_bdep) {
     // Transition tensors with several parents.  In filtering they enter only the prior, formed once per
-    // step, which the CTA-per-agent filtering kernel computes; window calls (VMP) need them in every
-    // message: the warp-per-step kernel's lanes sum them, the general kernel where that one does not fit.
+    // step; window calls (VMP) need them in every message: blocks in registers, or members of the batched
+    // contraction, where they fit, then the warp-per-step kernel, whose lanes sum them.  (The testing aid
+    // starts at the named family here too.)
+    const int only = c.model->test_family;
+    const bool any = only == BI_FAMILY_ANY;
     int rc = BI_ERR_UNSUPPORTED;
-    if (c.model->test_family == BI_FAMILY_ANY) rc = bi_launch_block(c, mut);
-    if ((c.model->test_family == BI_FAMILY_ANY && rc == BI_ERR_UNSUPPORTED) || c.model->test_family == BI_FAMILY_BATCH)
-      rc = bi_launch_batch(c, mut);
-    if (rc == BI_ERR_UNSUPPORTED && c.model->test_family == BI_FAMILY_ANY)
-      rc = c.algo == BI_ALGO_FILTER ? bi_launch_cta_filter(c, mut) : bi_launch_warp(c, mut);
+    if (any || only == BI_FAMILY_BLOCK) rc = bi_launch_block(c, mut);
+    if (rc == BI_ERR_UNSUPPORTED && (any || only == BI_FAMILY_BATCH)) rc = bi_launch_batch(c, mut);
+    if (rc == BI_ERR_UNSUPPORTED && c.algo == BI_ALGO_FILTER && (any || only == BI_FAMILY_CTA)) rc = bi_launch_cta_filter(c, mut);
+    if (rc == BI_ERR_UNSUPPORTED && c.algo != BI_ALGO_FILTER && (any || only == BI_FAMILY_WARP)) rc = bi_launch_warp(c, mut);
     return rc == BI_ERR_UNSUPPORTED ? bi_launch_generic(c, mut) : rc;
   }
   const int only = c.model->test_family;   // testing aid: start at the named family

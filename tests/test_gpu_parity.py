@@ -16,7 +16,7 @@ ALGOS = ["filter", "vmp", "mmp"]
 
 @contextlib.contextmanager
 def family_forced(name):
-    """The library's testing aid BI_TEST_FAMILY ("batch", "cta", "warp" or "generic"), read when a handle is made: its
+    """The library's testing aid BI_TEST_FAMILY ("block", "batch", "cta", "warp" or "generic"), read when a handle is made: its
     calls skip the kernel families ahead of the named one, so that the general kernels can be checked
     on oracle-sized inputs that would otherwise go to a specialised kernel."""
     old = os.environ.get("BI_TEST_FAMILY")
@@ -898,6 +898,47 @@ def test_b_dependencies(case, algo):
         with family_forced("generic"):
             res = check_workload(w, algo)
         assert res["kernel"].startswith("generic_"), res
+
+
+@pytest.mark.parametrize("case", sorted(BDEP_CASES))
+def test_b_dependencies_on_every_family(case):
+    """Each family that takes transitions with several parents, by the name of the kernel that ran: the dispatcher
+    gives most of these calls to the block kernels."""
+    w = _bdep_workload(1200 + sorted(BDEP_CASES).index(case), **BDEP_CASES[case])
+    for algo, forced in (("filter", "cta"), ("vmp", "warp"), ("filter", "block"), ("vmp", "block")):
+        with family_forced(forced):
+            res = check_workload(w, algo)
+        # (the block kernels decline filtering without a group to contract or with zeros in A, windows with more than three
+        # parents per transition and windows whose tensors do not fit)
+        declined = ("ragged_edge", "cross", "per_agent") if algo == "filter" else ("wide", "five_parents", "long_window")
+        want = "generic" if forced == "block" and case in declined else forced
+        assert res["family"].startswith(f"{want}_{algo}") and res["family"].endswith("f64"), res
+
+
+@pytest.mark.parametrize("algo", ["vmp", "mmp"])
+def test_batched_kernels_where_the_estimate_prefers_blocks(algo):
+    """The batched window kernels on calls that the dispatcher may give to the block kernels, by the name of the kernel
+    that ran: shared models on unrolled and any-shape slices, models of the agents' own."""
+    cases = [(make_config(3, N=128, T=16, K=9), 5),
+             (_custom(41, [3, 4, 2, 5, 3], [3, 2, 4, 3], [[0, 1, 2], [3, 4], [1], [2, 0, 1]], [2, 1, 3, 2, 2],
+                      N=171, T=12, K=7, sparsity=0.5), 7),
+             (_custom(44, [7, 13, 32, 9], [5, 3, 2, 6], [[0, 1], [1, 2], [0, 3, 2], [3, 0]], [2, 2, 1, 3],
+                      N=128, T=16, K=5), 5),
+             (_custom(52, [5, 7, 3, 4], [4, 3, 5], [[0, 1, 3], [1, 2], [2]], [2, 1, 3, 2], N=140, T=16, K=5, G=140,
+                      sparsity=0.5), 7)]
+    for w, step in cases:
+        with family_forced("batch"):
+            res = check_workload(w, algo, agents=range(0, w.N, step))
+        assert res["family"] == f"batch_{algo}_f64", res
+
+
+@pytest.mark.parametrize("algo", ["vmp", "mmp"])
+def test_warp_window_kernels_behind_the_block_kernels(algo):
+    for w in (_custom(54, [5, 4, 3, 6], [3, 4, 5], [[0, 1], [1, 2, 3], [3]], [2, 2, 1, 3], N=9, T=7, K=6),
+              _custom(55, [9, 5, 7], [4, 6], [[0, 1, 2], [2, 1]], [2, 1, 3], N=6, T=13, K=4, G=6)):
+        with family_forced("warp"):
+            res = check_workload(w, algo)
+        assert res["family"] == f"warp_{algo}_f64", res
 
 
 @pytest.mark.parametrize("algo", ["filter", "vmp"])
