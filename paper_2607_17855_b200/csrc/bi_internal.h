@@ -199,6 +199,8 @@ int bi_launch_block(const BiCall &c, bi_model *mut);        // any structure of 
 int bi_block_slice_elems(const bi_model *md, int gi);
 // whether the block kernels may serve such calls on this model (they may still decline one that does not fit)
 bool bi_block_serves(const bi_model *md, int algo);
+// whether bi_launch_block would take this call (for callers that lay data out for it first)
+bool bi_block_accepts(const BiCall &c);
 // tries the kernel families in order (the dispatcher behind every inference call)
 int bi_dispatch(const BiCall &c, bi_model *mut);
 // inference with observations given as categorical vectors [N][T][sum m_i]

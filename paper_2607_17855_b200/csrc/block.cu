@@ -725,27 +725,32 @@ WindowCost window_cost(const BiCall &c, const Plan &pl, const Variant &v) {
   return w;
 }
 
-}  // namespace
+// How a call would run here.
+struct Route {
+  Params p;
+  const Plan *plan;
+  unsigned grid, threads;
+  size_t bytes;
+};
 
-// Any model whose groups span at most four factors (transitions over at most three parents in window
-// calls), either arithmetic, as long as a step's blocks fit the register file and shared memory of an SM
-// (window calls: of a cluster); BI_ERR_UNSUPPORTED otherwise.
-int bi_launch_block(const BiCall &c, bi_model *mut) {
+// Whether these kernels take a call, and in which shape.  Any model whose groups span at most four factors
+// (transitions over at most three parents in window calls), either arithmetic, as long as a step's blocks fit the
+// register file and shared memory of an SM (window calls: of a cluster).
+bool choose_route(const BiCall &c, Route &L) {
   const bi_model *md = c.model;
   const bool window = c.algo != BI_ALGO_FILTER;
   const Plan *plp = static_cast<const Plan *>(md->blk_plan[window ? 1 : 0]);
-  if (!plp || !plp->ok) return BI_ERR_UNSUPPORTED;
-  if (window && md->h.has_bdep && (c.algo == BI_ALGO_MMP || c.lnprior)) return BI_ERR_UNSUPPORTED;
-  if (!bi_block_serves(md, c.algo)) return BI_ERR_UNSUPPORTED;
-  if (plp->NB == 0) return BI_ERR_UNSUPPORTED;   // nothing to contract: the CTA kernel's warp per factor does that
-  if (window && !md->h.has_bdep && md->batch_unrolled && (long long)c.N * c.T >= 4096) return BI_ERR_UNSUPPORTED;   // (see batch_unrolled)
+  if (!plp || !plp->ok) return false;
+  if (window && md->h.has_bdep && (c.algo == BI_ALGO_MMP || c.lnprior)) return false;
+  if (!bi_block_serves(md, c.algo)) return false;
   const Plan &pl = *plp;
+  L.plan = plp;
+  if (pl.NB == 0) return false;   // nothing to contract: the CTA kernel's warp per factor does that
+  if (window && !md->h.has_bdep && md->batch_unrolled && (long long)c.N * c.T >= 4096) return false;   // (see batch_unrolled)
   const int esz = md->arith == BI_ARITH_F64 ? 8 : 4;
   const size_t budget = (size_t)md->max_smem_optin - 1024;
-  Params p;
+  Params &p = L.p;
   fill_params(c, pl, p);
-  unsigned grid = 0, threads = 0;
-  size_t bytes = 0;
   if (!window) {
     // Team size: cycles of an iteration (a phase for each round of blocks and of passes), plus what the teams
     // beside it on the SM add, times the waves of teams.  (Five coupled factors, 204 blocks, 256 agents: teams
@@ -764,16 +769,16 @@ int bi_launch_block(const BiCall &c, bi_model *mut) {
       const double t = waves * (alone + (on_sm - 1) * beside);
       if (t < best) { best = t; v0 = v; }
     }
-    if (best >= 1e300) return BI_ERR_UNSUPPORTED;
+    if (best >= 1e300) return false;
     use_variant(pl.var[v0], p);
     // agents per CTA (one-warp teams): one while the batch fits the machine anyway, so that no SM gets
     // four more warps than another; four for large batches, which share the CTA's exponential table
     p.W = p.LT == 32 ? (c.N > 24 * md->sm_count ? 4 : 1) : 1;
     p.UC = p.W; p.CS = 1;
-    bytes = layout(pl, p, esz, p.W, p.W);
-    if (bytes > budget) return BI_ERR_UNSUPPORTED;
-    grid = (unsigned)((c.N + p.W - 1) / p.W);
-    threads = (unsigned)(p.W * p.LT);
+    L.bytes = layout(pl, p, esz, p.W, p.W);
+    if (L.bytes > budget) return false;
+    L.grid = (unsigned)((c.N + p.W - 1) / p.W);
+    L.threads = (unsigned)(p.W * p.LT);
   } else {
     // Steps per CTA and CTAs per agent: the cheapest by a small model of an iteration -- the larger of a
     // dependent chain of about a thousand cycles (more when it crosses CTAs) and the throughput of
@@ -800,29 +805,47 @@ int bi_launch_block(const BiCall &c, bi_model *mut) {
         if (t < best) { best = t; bv = v; buc = uc; bcs = cs; }
       }
     }
-    if (bv < 0) return BI_ERR_UNSUPPORTED;
+    if (bv < 0) return false;
     if (!md->h.has_bdep && md->h.G == 1 && (long long)c.N * c.T >= 2048 && md->test_family == BI_FAMILY_ANY && !md->soft_shadow) {
       const WindowCost w = window_cost(c, pl, pl.var[bv]);
-      if (w.batch < 0.9 * w.block) return BI_ERR_UNSUPPORTED;
+      if (w.batch < 0.9 * w.block) return false;
     }
     use_variant(pl.var[bv], p);
     p.W = 0;
     p.UC = buc; p.CS = bcs;
-    bytes = layout(pl, p, esz, buc, 2 * (buc + 2));
-    grid = (unsigned)(c.N * bcs);
-    threads = (unsigned)(buc * p.LT);
+    L.bytes = layout(pl, p, esz, buc, 2 * (buc + 2));
+    L.grid = (unsigned)(c.N * bcs);
+    L.threads = (unsigned)(buc * p.LT);
   }
+  return true;
+}
+
+}  // namespace
+
+bool bi_block_accepts(const BiCall &c) {
+  Route L;
+  return choose_route(c, L);
+}
+
+int bi_launch_block(const BiCall &c, bi_model *mut) {
+  const bi_model *md = c.model;
+  const bool window = c.algo != BI_ALGO_FILTER;
+  Route L;
+  if (!choose_route(c, L)) return BI_ERR_UNSUPPORTED;
+  const Plan &pl = *L.plan;
+  Params &p = L.p;
+  const int esz = md->arith == BI_ARITH_F64 ? 8 : 4;
   const bool hass = p.nbpt > 1;
   const int sync = p.LT == 32 ? 0 : (window && p.UC > 1) ? 2 : 1;   // (SYNC_WARP, SYNC_CTA, SYNC_NAMED)
   const void *kern = esz == 8 ? bi_block_kernel_f64(pl.BR, pl.BC, window, sync, hass)
                               : bi_block_kernel_f32(pl.BR, pl.BC, window, sync, hass);
   if (!kern) return BI_ERR_UNSUPPORTED;
   const int slot = (((pl.BR == 4 ? 0 : pl.BC == 4 ? 1 : 2) * 2 + window) * 3 + sync) * 4 + hass * 2 + (esz == 8);
-  if (!allow_smem(kern, slot, md->device, bytes)) return BI_ERR_CUDA;
+  if (!allow_smem(kern, slot, md->device, L.bytes)) return BI_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = bytes;
+  cfg.gridDim = dim3(L.grid);
+  cfg.blockDim = dim3(L.threads);
+  cfg.dynamicSmemBytes = L.bytes;
   cfg.stream = c.stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;

@@ -209,6 +209,35 @@ int run_soft_t(const bi_model *model, int algo, int N, int T, const float *obs_s
   const bool tile = model->tile_sb > 0;
   const size_t NT = (size_t)N * T;
 
+  // ---- the shadow model: one modality per group, T outcomes per agent, selected by the step index
+  bi_model sh = *model;
+  sh.h.G = N;
+  sh.h.M = h.ngroups;
+  sh.h.nmem = h.ngroups;
+  for (int k = 0; k < h.ngroups; ++k) {
+    BiGroup &g = sh.h.grp[k];
+    g.mem_begin = k;
+    g.mem_end = k + 1;
+    BiMember &mm = sh.h.mem[k];
+    mm.cmask = nullptr; mm.cvals = nullptr; mm.coff = nullptr;   // (the slices formed below are dense)
+    mm.gstride = (int64_t)T * g.P_pad;
+    mm.m = T;
+    mm.modality = k;
+    mm.P_pad = g.P_pad;
+    sh.h.m[k] = T;
+  }
+  // (a group of one modality is its own pre-summed table: the shadow's T per-agent slices)
+  sh.soft_shadow = 1;
+  sh.last_block = nullptr;
+  sh.tile_ncomb = T;
+  sh.tile_comb_mul[0] = 1;
+  BiCall c;
+  c.carry_in = nullptr; c.carry_out = nullptr;
+  c.model = &sh; c.algo = algo; c.N = N; c.T = T; c.K = iters;
+  c.obs = nullptr; c.act = act; c.q_prev = nullptr; c.act_prev = nullptr; c.q_init = nullptr; c.lnprior = nullptr; c.lambda = model->damping;
+  c.q_out = q_out; c.logq_out = logq_out; c.argmax_out = argmax_out;
+  c.stream = stream;
+
   // ---- workspace: per group the packed slices (and the lane-interleaved ones of a tile model),
   // the step-index "observations", the shadow descriptor
   size_t off_pack[BI_MAX_GROUPS], off_tile = 0, need = 0;
@@ -229,10 +258,10 @@ int run_soft_t(const bi_model *model, int algo, int N, int T, const float *obs_s
     off_packT = need;
     need += up256(NT * PT * sizeof(R));
   }
-  // A call that the block kernels serve: their groups' slices are formed in block order instead (a rank-1
-  // group's stay packed; the packed ones of the others follow only if those kernels decline the call).
-  const bool block = !tile && bi_block_serves(model, algo) &&
-                     (sizeof(R) == 4 || !(algo == BI_ALGO_FILTER ? model->pair_ok : model->rank2_ok));
+  // A call that the block kernels take: their groups' slices are formed in block order instead (a rank-1
+  // group's stay packed).  Asked before anything is formed: a call that they decline has its slices formed once too.
+  const bool block = !tile && (sizeof(R) == 4 || !(algo == BI_ALGO_FILTER ? model->pair_ok : model->rank2_ok)) &&
+                     (model->test_family == BI_FAMILY_ANY || model->test_family == BI_FAMILY_BLOCK) && bi_block_accepts(c);
   size_t off_blk[BI_MAX_GROUPS] = {};
   for (int k = 0; k < h.ngroups && block; ++k)
     if (h.grp[k].rank >= 2) {
@@ -306,47 +335,23 @@ int run_soft_t(const bi_model *model, int algo, int N, int T, const float *obs_s
   ++launches;
   if (cudaGetLastError() != cudaSuccess) return BI_ERR_CUDA;
 
-  // ---- the shadow model: one modality per group, T outcomes per agent, selected by the step index
-  bi_model sh = *model;
-  sh.h.G = N;
-  sh.h.M = h.ngroups;
-  sh.h.nmem = h.ngroups;
+  // ---- the shadow model's slices
   for (int k = 0; k < h.ngroups; ++k) {
-    BiGroup &g = sh.h.grp[k];
-    g.mem_begin = k;
-    g.mem_end = k + 1;
     BiMember &mm = sh.h.mem[k];
     mm.logA = w + off_pack[k];
     mm.logA_tile = tile && k == 0 ? w + off_tile : nullptr;
-    mm.logA_blk = block && g.rank >= 2 ? w + off_blk[k] : nullptr;
+    mm.logA_blk = block && h.grp[k].rank >= 2 ? w + off_blk[k] : nullptr;
     mm.logA_T = k == kpair ? w + off_packT : nullptr;
-    mm.cmask = nullptr; mm.cvals = nullptr; mm.coff = nullptr;   // (the slices formed above are dense)
-    mm.gstride = (int64_t)T * g.P_pad;
-    mm.m = T;
-    mm.modality = k;
-    mm.P_pad = g.P_pad;
-    sh.h.m[k] = T;
   }
-  // (a group of one modality is its own pre-summed table: the shadow's T per-agent slices)
-  sh.soft_shadow = 1;
-  sh.last_block = nullptr;
   if (!block) sh.blk_plan[0] = sh.blk_plan[1] = nullptr;
   sh.pair_ok = kpair >= 0 || (model->pair_ok && sizeof(R) == 8 && algo == BI_ALGO_FILTER);
   // (the pair filtering kernel needs the transposed slices formed above, or no pair at all; the pair
   // window kernel reads rows only)
   sh.tile_comb = tile ? w + off_tile : nullptr;
-  sh.tile_ncomb = T;
-  sh.tile_comb_mul[0] = 1;
   sh.d = reinterpret_cast<BiDev *>(w + off_desc);
   // (the shadow borrows the handle's batched-path workspace and hands it back below)
   if (cudaMemcpyAsync(sh.d, &sh.h, sizeof(BiDev), cudaMemcpyHostToDevice, stream) != cudaSuccess) return BI_ERR_CUDA;
-
-  BiCall c;
-  c.carry_in = nullptr; c.carry_out = nullptr;
-  c.model = &sh; c.algo = algo; c.N = N; c.T = T; c.K = iters;
-  c.obs = obs_idx; c.act = act; c.q_prev = nullptr; c.act_prev = nullptr; c.q_init = nullptr; c.lnprior = nullptr; c.lambda = model->damping;
-  c.q_out = q_out; c.logq_out = logq_out; c.argmax_out = argmax_out;
-  c.stream = stream;
+  c.obs = obs_idx;
   const int64_t before = sh.launches;
   int rc;
   if (tile) {
@@ -359,16 +364,7 @@ int run_soft_t(const bi_model *model, int algo, int N, int T, const float *obs_s
       if (rc == BI_ERR_UNSUPPORTED) rc = bi_launch_generic(c, &sh);
     }
   } else {
-    rc = BI_ERR_UNSUPPORTED;
-    if (block && model->test_family == BI_FAMILY_ANY) rc = bi_launch_block(c, &sh);
-    if (rc == BI_ERR_UNSUPPORTED) {
-      if (block) {
-        form(0);
-        if (cudaGetLastError() != cudaSuccess) return BI_ERR_CUDA;
-        sh.blk_plan[0] = sh.blk_plan[1] = nullptr;
-      }
-      rc = bi_dispatch(c, &sh);
-    }
+    rc = block ? bi_launch_block(c, &sh) : bi_dispatch(c, &sh);
   }
   mut->ws = sh.ws;
   mut->ws_bytes = sh.ws_bytes;

@@ -172,3 +172,29 @@ def test_improbable_states_under_many_future_messages(K):
                  act=np.zeros((N, T - 1, F), np.int32), bdep=[[0]] * F)
     res = check_workload(w, "vmp")
     assert res["family"] == "block_vmp_f64", res
+
+
+@pytest.mark.parametrize("case", ["every_slice_unrolled", "too_large_for_blocks"])
+def test_observation_vectors_form_every_slice_once(case):
+    """Which kernels will read the slices is known before they are formed: one launch per group, one for the step
+    indices, and the inference call's own (batched windows: the two at the start and two per iteration)."""
+    import torch
+    import oracle
+    import paper_2607_17855_b200 as bi
+    from test_gpu_parity import _soft_vectors
+    if case == "every_slice_unrolled":
+        n, dep, N, T, step = [10, 10, 8, 6], [[0, 1], [1, 2], [0, 2, 3]], 260, 16, 20
+    else:
+        n, dep, N, T, step = [32, 31, 30], [[0, 1, 2], [2]], 3, 4, 1
+    w = _workload(100, n, dep, N=N, T=T, K=3)
+    md = bi.model_from_workload(w)
+    soft = _soft_vectors(w, 7)
+    q = md.run_soft("vmp", torch.from_numpy(soft).cuda(), torch.from_numpy(w.act).cuda(), w.K).cpu().numpy()
+    own = md.launch_count - (len(dep) + 1)
+    sel = list(range(0, N, step))
+    sub = w.take_agents(sel)
+    ref = oracle.run("vmp", sub.n, sub.m, sub.dep, sub.U, sub.G, sub.A, sub.B, sub.D, None, sub.act, sub.K, obs_soft=soft[sel])[0]
+    assert np.abs(q[sel] - ref).max() <= 1e-5
+    kernel = md.last_kernel
+    md.close()
+    assert own in (1, 2 + 2 * w.K), (kernel, own)
