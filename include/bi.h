@@ -324,8 +324,9 @@ int bi_mmp_from(const bi_model_t *model, int32_t N, int32_t T, const int32_t *ob
  *   others    as for bi_filter / bi_vmp / bi_mmp
  * The call first forms the weighted slices of every (agent, step) in a workspace
  * of N * T * (sum over dependency groups of the padded slice size) elements of
- * the handle's arithmetic type (twice that for register-tile models), obtained
- * from the stream-ordered allocator on first use and kept in the handle, then
+ * the handle's arithmetic type (twice that for register-tile models; in whole blocks of up
+ * to 8 x 6 where kernels that hold such blocks in registers serve the call and the workspace can be obtained),
+ * obtained from the stream-ordered allocator on first use and kept in the handle, then
  * runs the same inference kernels on them.  BI_ERR_ALLOC if the workspace cannot
  * be obtained; BI_ERR_UNSUPPORTED if sum_i m_i exceeds 768 (1536 in float32 arithmetic).
  */

@@ -238,40 +238,34 @@ int run_soft_t(const bi_model *model, int algo, int N, int T, const float *obs_s
   c.q_out = q_out; c.logq_out = logq_out; c.argmax_out = argmax_out;
   c.stream = stream;
 
-  // ---- workspace: per group the packed slices (and the lane-interleaved ones of a tile model),
-  // the step-index "observations", the shadow descriptor
-  size_t off_pack[BI_MAX_GROUPS], off_tile = 0, need = 0;
-  for (int k = 0; k < h.ngroups; ++k) {
-    off_pack[k] = need;
-    need += up256(NT * h.grp[k].P_pad * sizeof(R));
-  }
-  if (tile) { off_tile = need; need += up256(NT * model->tile_P * sizeof(R)); }
+  // A call that the block kernels take: their groups' slices are formed in block order (a rank-1 group's stay
+  // packed).  Asked before anything is formed: a call that they decline has its slices formed once too.
+  bool block = !tile && (sizeof(R) == 4 || !(algo == BI_ALGO_FILTER ? model->pair_ok : model->rank2_ok)) &&
+               (model->test_family == BI_FAMILY_ANY || model->test_family == BI_FAMILY_BLOCK) && bi_block_accepts(c);
   // a filtering call on a model the pair filtering kernel serves: that kernel also reads the pair's
   // slices with the two axes exchanged, so those are formed too (from the handle's transposed copies)
   int kpair = -1;
-  size_t off_packT = 0, PT = 0;
   if (algo == BI_ALGO_FILTER && model->pair_ok && sizeof(R) == 8)
     for (int k = 0; k < h.ngroups; ++k)
       if (h.grp[k].rank == 2 && h.mem[h.grp[k].mem_begin].logA_T) kpair = k;
-  if (kpair >= 0) {
-    PT = (size_t)h.grp[kpair].dim[1] * bi_pad4(h.grp[kpair].dim[0]);
-    off_packT = need;
-    need += up256(NT * PT * sizeof(R));
-  }
-  // A call that the block kernels take: their groups' slices are formed in block order instead (a rank-1
-  // group's stay packed).  Asked before anything is formed: a call that they decline has its slices formed once too.
-  const bool block = !tile && (sizeof(R) == 4 || !(algo == BI_ALGO_FILTER ? model->pair_ok : model->rank2_ok)) &&
-                     (model->test_family == BI_FAMILY_ANY || model->test_family == BI_FAMILY_BLOCK) && bi_block_accepts(c);
-  size_t off_blk[BI_MAX_GROUPS] = {};
-  for (int k = 0; k < h.ngroups && block; ++k)
-    if (h.grp[k].rank >= 2) {
-      off_blk[k] = need;
-      need += up256(NT * bi_block_slice_elems(model, k) * sizeof(R));
+  const size_t PT = kpair >= 0 ? (size_t)h.grp[kpair].dim[1] * bi_pad4(h.grp[kpair].dim[0]) : 0;
+
+  // ---- workspace: per group its slices in the one layout that will be read (a tile model's in both that may be),
+  // the step-index "observations", the shadow descriptor
+  size_t off_pack[BI_MAX_GROUPS] = {}, off_blk[BI_MAX_GROUPS] = {}, off_tile = 0, off_packT = 0, off_obs = 0, off_desc = 0, need = 0;
+  auto reserve = [&](size_t bytes) { const size_t at = need; need += up256(bytes); return at; };
+  auto lay_out = [&] {
+    need = 0;
+    for (int k = 0; k < h.ngroups; ++k) {
+      const bool blk = block && h.grp[k].rank >= 2;
+      (blk ? off_blk : off_pack)[k] = reserve(NT * (blk ? bi_block_slice_elems(model, k) : h.grp[k].P_pad) * sizeof(R));
     }
-  const size_t off_obs = need;
-  need += up256(NT * h.ngroups * sizeof(int32_t));
-  const size_t off_desc = need;
-  need += up256(sizeof(BiDev));
+    if (tile) off_tile = reserve(NT * model->tile_P * sizeof(R));
+    if (kpair >= 0) off_packT = reserve(NT * PT * sizeof(R));
+    off_obs = reserve(NT * h.ngroups * sizeof(int32_t));
+    off_desc = reserve(sizeof(BiDev));
+  };
+  lay_out();
   if (mut->ws_soft_bytes < need) {
     if (mut->ws_soft && cudaFreeAsync(mut->ws_soft, stream) != cudaSuccess) return BI_ERR_CUDA;
     mut->ws_soft = nullptr;
@@ -279,7 +273,15 @@ int run_soft_t(const bi_model *model, int algo, int N, int T, const float *obs_s
     void *pnew = nullptr;
     if (cudaMallocAsync(&pnew, need, stream) != cudaSuccess) {
       cudaGetLastError();
-      return BI_ERR_ALLOC;
+      const size_t wanted = need;
+      if (block) {   // (padded to whole blocks; the packed slices are smaller)
+        block = false;
+        lay_out();
+      }
+      if (need >= wanted || cudaMallocAsync(&pnew, need, stream) != cudaSuccess) {
+        cudaGetLastError();
+        return BI_ERR_ALLOC;
+      }
     }
     mut->ws_soft = pnew;
     mut->ws_soft_bytes = need;

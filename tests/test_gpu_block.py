@@ -198,3 +198,22 @@ def test_observation_vectors_form_every_slice_once(case):
     kernel = md.last_kernel
     md.close()
     assert own in (1, 2 + 2 * w.K), (kernel, own)
+
+
+def test_observation_vectors_reserve_one_layout():
+    """The workspace of a call with observation vectors holds the slices in the layout that is read, not beside another
+    one: [9,10,11] in blocks of 8 x 6 is 2 x 2 x 9 of them per step (the axes of ten and eleven states cut)."""
+    import torch
+    import paper_2607_17855_b200 as bi
+    w = _workload(110, [9, 10, 11], [[0, 1, 2]], N=1000, T=20, K=2)
+    md = bi.model_from_workload(w)
+    soft = torch.rand((w.N, w.T, int(w.m.sum())), device="cuda")
+    act, q = torch.from_numpy(w.act).cuda(), torch.empty((w.N, w.T, w.S), device="cuda")
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    md.run_soft("vmp", soft, act, w.K, q_out=q)
+    torch.cuda.synchronize()
+    used = before - torch.cuda.mem_get_info()[0]
+    md.close()
+    slices = w.N * w.T * 36 * 48 * 8
+    assert used <= slices + (80 << 20), (used, slices)   # (the allocator takes whole chunks of 32 MB; kernels are loaded on first use)
