@@ -102,7 +102,9 @@ typedef struct {
  * outcome's slice contiguously with modalities of equal dependency set sharing
  * one axis order; B is re-laid per action as forward, log, log-transposed and
  * column-normalised-transposed matrices; D as ln D.  The packed copies live in
- * device memory owned by the handle.  The call waits for the packing on the
+ * device memory owned by the handle.  Models whose calls may run on kernels that hold blocks of a slice in
+ * registers get a second copy of the slices in that order (in whole blocks of up to 8 x 6), unless it would take
+ * more than half of the memory still free; without it the other kernels serve all calls.  The call waits for the packing on the
  * stream (later calls choose their kernels by whether A has zeros), so the
  * caller's A, B, D may be released when it returns.  Returns BI_OK and *out, or
  * an error code with *out = NULL.

@@ -16,6 +16,7 @@ int bi_block_pack_member(const bi_model *md, int gi, const float *src, int m, co
 void bi_block_build(bi_model *md, std::vector<unsigned char> &blob);
 void bi_block_bind(bi_model *md, unsigned char *dev);
 void bi_block_free(bi_model *md);
+bool bi_block_copies(const bi_model *md);
 int bi_block_exp_table(double *dst, cudaStream_t stream);
 
 namespace {
@@ -542,18 +543,12 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
   md->batch_unrolled = 1;
   for (int gi = 0; gi < h.ngroups; ++gi)
     if (h.grp[gi].rank >= 2 && (h.grp[gi].rank > 4 || bi_batch_shape(h.grp[gi].rank, h.grp[gi].dim) < 0)) md->batch_unrolled = 0;
-  // (register-tile models have kernels of their own for every call, and per-agent ones are large: no block-ordered copy)
-  if (md->tile_sb <= 0) bi_block_choose_shape(md);
+  if (md->tile_sb <= 0) bi_block_choose_shape(md);   // (register-tile models have kernels of their own for every call)
 
   // ---- allocate and pack
   rc = dev_alloc(md, (void **)&h.status, 3 * sizeof(uint32_t));   // the flags, and two marks on A
   if (rc == BI_OK && cudaMemsetAsync(h.status, 0, 3 * sizeof(uint32_t), stream) != cudaSuccess) rc = BI_ERR_CUDA;
-  size_t blk_bytes = 0;   // every modality's block-ordered copy: one allocation
-  auto blk_size = [&](int gi, const BiMember &mm) { return ((size_t)G * mm.m * bi_block_slice_elems(md, gi) * esz + 255) & ~(size_t)255; };
-  for (int gi = 0; gi < h.ngroups; ++gi)
-    for (int mi = h.grp[gi].mem_begin; mi < h.grp[gi].mem_end; ++mi) blk_bytes += blk_size(gi, h.mem[mi]);
-  unsigned char *blk_mem = nullptr;
-  if (rc == BI_OK && blk_bytes) rc = dev_alloc(md, (void **)&blk_mem, blk_bytes);
+  PackA packed[BI_MAX_M];   // (the members' sources, for the block-ordered copies at the end)
   for (int gi = 0; gi < h.ngroups && rc == BI_OK; ++gi) {
     BiGroup &g = h.grp[gi];
     for (int mi = g.mem_begin; mi < g.mem_end && rc == BI_OK; ++mi) {
@@ -609,11 +604,7 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
         if (cudaGetLastError() != cudaSuccess) rc = BI_ERR_CUDA;
         mm.logA_T = tdst;
       }
-      if (rc == BI_OK && bi_block_slice_elems(md, gi)) {
-        mm.logA_blk = blk_mem;
-        rc = bi_block_pack_member(md, gi, desc->A[i], mm.m, p.sstride, p.P, blk_mem, stream);
-        blk_mem += blk_size(gi, mm);
-      }
+      packed[mi] = p;
       if (rc == BI_OK && md->tile_sb > 0) {
         PackTile q;
         memset(&q, 0, sizeof(q));
@@ -849,12 +840,34 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
     }
     if (cudaGetLastError() != cudaSuccess) rc = BI_ERR_CUDA;
   }
+  if (rc == BI_OK) rc = dev_alloc(md, (void **)&md->d, sizeof(BiDev));
   if (rc == BI_OK) {   // the block kernels' plans and table, one upload (from pageable memory: the call returns when it is staged)
     std::vector<unsigned char> blob;
     bi_block_build(md, blob);
+    // Their copy of the slices, every modality's in one allocation.  It comes last and only into memory that leaves
+    // as much free again: a model that fits without it is made without it, and runs on the other kernels.
+    auto blk_size = [&](int gi, const BiMember &mm) { return ((size_t)G * mm.m * bi_block_slice_elems(md, gi) * esz + 255) & ~(size_t)255; };
+    size_t blk_bytes = 0, free_bytes = 0, total_bytes = 0;
+    for (int gi = 0; gi < h.ngroups; ++gi)
+      for (int mi = h.grp[gi].mem_begin; mi < h.grp[gi].mem_end; ++mi) blk_bytes += blk_size(gi, h.mem[mi]);
+    unsigned char *blk_mem = nullptr;
+    if (blk_bytes > (64u << 20) && (cudaMemGetInfo(&free_bytes, &total_bytes) != cudaSuccess || free_bytes / 2 < blk_bytes)) blk_bytes = 0;
+    if (md->blk_BR && bi_block_copies(md) && (!blk_bytes || dev_alloc(md, (void **)&blk_mem, blk_bytes) != BI_OK)) {
+      bi_block_free(md);
+      md->blk_BR = md->blk_BC = 0;
+      blob.clear();
+    }
+    for (int gi = 0; gi < h.ngroups && rc == BI_OK; ++gi)
+      for (int mi = h.grp[gi].mem_begin; mi < h.grp[gi].mem_end && rc == BI_OK; ++mi) {
+        if (!bi_block_slice_elems(md, gi)) continue;
+        BiMember &mm = h.mem[mi];
+        mm.logA_blk = blk_mem;
+        rc = bi_block_pack_member(md, gi, packed[mi].src, mm.m, packed[mi].sstride, packed[mi].P, blk_mem, stream);
+        blk_mem += blk_size(gi, mm);
+      }
     unsigned char *dev = nullptr;
     const size_t tab = (512 + 256) * sizeof(double);   // 2^(j/512), then 128 pairs (1/c, ln c)
-    rc = dev_alloc(md, (void **)&dev, tab + blob.size());
+    if (rc == BI_OK) rc = dev_alloc(md, (void **)&dev, tab + blob.size());
     if (rc == BI_OK) {
       rc = bi_block_exp_table((double *)dev, stream);
       md->exp_tab = (const double *)dev;
@@ -864,7 +877,6 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
         rc = BI_ERR_CUDA;
     }
   }
-  if (rc == BI_OK) rc = dev_alloc(md, (void **)&md->d, sizeof(BiDev));
   if (rc == BI_OK) {
     // the host copy outlives the asynchronous copy: it is a member of the handle
     if (cudaMemcpyAsync(md->d, &md->h, sizeof(BiDev), cudaMemcpyHostToDevice, stream) != cudaSuccess)

@@ -191,6 +191,7 @@ int bi_launch_warp(const BiCall &c, bi_model *mut);
 int bi_launch_cta_filter(const BiCall &c, bi_model *mut);   // filtering only; slices staged per step
 int bi_launch_pair_filter(const BiCall &c, bi_model *mut);  // filtering only; models coupled in at most one pair of factors
 int bi_launch_pair_window(const BiCall &c, bi_model *mut);  // window calls on the same models; a CTA per agent
+bool bi_pair_window_always(const bi_model *md);             // whether that one takes every window call on a model
 int bi_launch_tile3(const BiCall &c, bi_model *mut);
 int bi_launch_tile3_window(const BiCall &c, bi_model *mut);
 int bi_launch_batch(const BiCall &c, bi_model *mut);

@@ -80,6 +80,13 @@ __global__ void bi_pack_block_kernel(PackBlk p) {
 }
 __global__ void bi_exp_table_kernel(double *tab) { bi_fast_tabs_compute(tab, threadIdx.x, blockDim.x); }
 
+// Whether the handle keeps a block-ordered copy of any slice.
+bool bi_block_copies(const bi_model *md) {
+  for (int gi = 0; gi < md->h.ngroups; ++gi)
+    if (bi_block_slice_elems(md, gi)) return true;
+  return false;
+}
+
 // Elements of one outcome's slice of group gi in block order (0: the model has no block plan).
 int bi_block_slice_elems(const bi_model *md, int gi) {
   if (!md->blk_BR || md->h.grp[gi].rank < 2) return 0;
@@ -508,7 +515,53 @@ bool build_plan(const bi_model *md, bool window, HostPlan &hp) {
 
 }  // namespace
 
-// Builds the filtering and the window plan of a model and appends their tables to the upload buffer; the
+namespace {
+
+void use_variant(const Variant &v, Params &p) {
+  p.lane = v.lane; p.pass = v.pass; p.npass = v.npass; p.LT = v.LT; p.nbpt = v.nbpt;
+}
+
+// shared-memory layout for `units` teams and `slots` belief slots (behind the exponential table); returns bytes
+size_t layout(const Plan &pl, Params &p, int esz, int units, int slots) {
+  auto up16 = [](int x) { return (x + 15) & ~15; };
+  int u = up16(pl.Ysz * esz);
+  p.o_cst = u; u += pl.SQ * 8;
+  p.o_xp = u; u += p.lambda != 1.0 ? pl.SQ * 8 : 0;
+  p.o_e = u; u += pl.Esz * 8;
+  p.unit_sz = u;
+  size_t o = (512 + (p.mmp ? 256 : 0)) * sizeof(double);
+  p.o_unit = (int)o; o += (size_t)units * p.unit_sz;
+  p.o_q = (int)o; o += (size_t)slots * pl.SQ * esz;
+  p.o_par = (int)o; o += (size_t)p.W * up16(p.wpar * esz);
+  // the blocks beyond a thread each: whole rounds of the team, the last one only as far as it goes
+  const int extra = p.nbpt > 1 ? (pl.NB - p.LT + 31) / 32 * 32 : 0;
+  p.extra = extra;
+  p.o_L = (int)o; o += (size_t)units * extra * pl.BR * pl.BC * esz;
+  p.o_ref = (int)o; o += (size_t)extra * 48;
+  p.o_lane = (int)o; o += (size_t)p.npass * 33 * 16;
+  return o;
+}
+
+// Whether one unit of a plan fits an SM under some team size (filtering one agent, a window of one step).
+bool smallest_fits(const bi_model *md, const Plan &pl, bool window) {
+  if (pl.NB == 0) return false;
+  Params p;
+  memset(&p, 0, sizeof(p));
+  p.lambda = 1.0;
+  p.W = window ? 0 : 1;
+  for (int f = 0; f < md->h.F && md->h.has_bdep && !window; ++f) p.wpar = std::max(p.wpar, (md->h.PB[f] + 3) & ~3);
+  for (int v = 0; v < pl.nv; ++v) {
+    use_variant(pl.var[v], p);
+    if (layout(pl, p, md->arith == BI_ARITH_F64 ? 8 : 4, 1, window ? 6 : 1) <= (size_t)md->max_smem_optin - 1024) return true;
+  }
+  return false;
+}
+
+}  // namespace
+
+// Builds the filtering and the window plan of a model (those that some call can run: a plan whose smallest call does
+// not fit an SM, and a plan for calls that the pair kernels take ahead of these, are not kept, and a model without
+// plans has no block shape and so no copies of its slices) and appends their tables to the upload buffer; the
 // device pointers in the plans are offsets until bi_block_bind turns them into addresses.
 void bi_block_build(bi_model *md, std::vector<unsigned char> &blob) {
   auto put = [&](const void *src, size_t bytes) {
@@ -520,7 +573,8 @@ void bi_block_build(bi_model *md, std::vector<unsigned char> &blob) {
   md->blk_plan[0] = md->blk_plan[1] = nullptr;
   for (int k = 0; k < 2; ++k) {
     HostPlan hp;
-    if (!build_plan(md, k == 1, hp)) continue;
+    if (md->arith == BI_ARITH_F64 && md->test_family == BI_FAMILY_ANY && (k == 0 ? md->pair_ok : bi_pair_window_always(md))) continue;
+    if (!build_plan(md, k == 1, hp) || !smallest_fits(md, hp.p, k == 1)) continue;
     hp.p.desc = reinterpret_cast<const Desc *>(put(hp.desc.data(), hp.desc.size() * sizeof(Desc)));
     for (int v = 0; v < hp.p.nv; ++v) {
       hp.p.var[v].lane = reinterpret_cast<const Lane *>(put(hp.lane[v].data(), hp.lane[v].size() * sizeof(Lane)));
@@ -528,6 +582,7 @@ void bi_block_build(bi_model *md, std::vector<unsigned char> &blob) {
     }
     md->blk_plan[k] = new Plan(hp.p);
   }
+  if (!md->blk_plan[0] && !md->blk_plan[1]) md->blk_BR = md->blk_BC = 0;
 }
 void bi_block_bind(bi_model *md, unsigned char *dev) {
   for (int k = 0; k < 2; ++k) {
@@ -628,31 +683,6 @@ void fill_params(const BiCall &c, const Plan &pl, Params &p) {
   p.obs = c.obs; p.act = c.act; p.act_prev = c.act_prev;
   p.q_prev = c.q_prev; p.q_init = c.q_init; p.carry_in = c.carry_in; p.carry_out = c.carry_out; p.lnprior = c.lnprior;
   p.q_out = c.q_out; p.logq_out = c.logq_out; p.argmax_out = c.argmax_out; p.status = h.status;
-}
-
-void use_variant(const Variant &v, Params &p) {
-  p.lane = v.lane; p.pass = v.pass; p.npass = v.npass; p.LT = v.LT; p.nbpt = v.nbpt;
-}
-
-// shared-memory layout for `units` teams and `slots` belief slots (behind the exponential table); returns bytes
-size_t layout(const Plan &pl, Params &p, int esz, int units, int slots) {
-  auto up16 = [](int x) { return (x + 15) & ~15; };
-  int u = up16(pl.Ysz * esz);
-  p.o_cst = u; u += pl.SQ * 8;
-  p.o_xp = u; u += p.lambda != 1.0 ? pl.SQ * 8 : 0;
-  p.o_e = u; u += pl.Esz * 8;
-  p.unit_sz = u;
-  size_t o = (512 + (p.mmp ? 256 : 0)) * sizeof(double);
-  p.o_unit = (int)o; o += (size_t)units * p.unit_sz;
-  p.o_q = (int)o; o += (size_t)slots * pl.SQ * esz;
-  p.o_par = (int)o; o += (size_t)p.W * up16(p.wpar * esz);
-  // the blocks beyond a thread each: whole rounds of the team, the last one only as far as it goes
-  const int extra = p.nbpt > 1 ? (pl.NB - p.LT + 31) / 32 * 32 : 0;
-  p.extra = extra;
-  p.o_L = (int)o; o += (size_t)units * extra * pl.BR * pl.BC * esz;
-  p.o_ref = (int)o; o += (size_t)extra * 48;
-  p.o_lane = (int)o; o += (size_t)p.npass * 33 * 16;
-  return o;
 }
 
 // The attribute is set once per kernel and device and only ever raised.

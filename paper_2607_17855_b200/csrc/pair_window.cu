@@ -282,15 +282,22 @@ __global__ void __launch_bounds__(MAXT, MAXT <= 320 ? 2 : 1) bi_pair_window_kern
   }
 }
 
+// Threads of a CTA and its shared memory in bytes, for windows of T steps with LPU lanes each.
+constexpr int kMaxThreads = 512;   // (the kernel's register budget is set for this)
+int window_threads(int T, int LPU) { return ((T * LPU + 31) / 32) * 32; }
+size_t window_bytes(int units, int LPU, int F, int ng, int nar, int ls, bool damped) {
+  const size_t slot = (size_t)F * LPU;
+  const size_t elems = EXP_TAB + 2 * (units + 2) * slot + (damped ? 2 : 1) * units * slot + (((size_t)units * ng * nar * ls + 1) & ~(size_t)1);
+  return elems * sizeof(R) + (size_t)units * F * 2 * sizeof(int32_t) + 16;
+}
+
 template <int LPU>
 int launch(PairWinParams &p, const bi_model *md, cudaStream_t stream) {
-  const int threads = ((p.T * LPU + 31) / 32) * 32;
-  if (threads > 512) return BI_ERR_UNSUPPORTED;   // (the kernel's register budget is set for this)
+  const int threads = window_threads(p.T, LPU);
+  if (threads > kMaxThreads) return BI_ERR_UNSUPPORTED;
   p.units = threads / LPU;
-  const size_t slot = (size_t)p.F * LPU;
   const bool damped = p.lambda != 1.0;
-  size_t elems = EXP_TAB + 2 * (p.units + 2) * slot + (damped ? 2 : 1) * p.units * slot + (((size_t)p.units * p.ng * p.nar * p.ls + 1) & ~(size_t)1);
-  const size_t bytes = elems * sizeof(R) + (size_t)p.units * p.F * 2 * sizeof(int32_t) + 16;
+  const size_t bytes = window_bytes(p.units, LPU, p.F, p.ng, p.nar, p.ls, damped);
   if (bytes > (size_t)md->max_smem_optin - 1024) return BI_ERR_UNSUPPORTED;
   void (*kern)(const PairWinParams);
   if (threads <= 320) {
@@ -309,6 +316,22 @@ int launch(PairWinParams &p, const bi_model *md, cudaStream_t stream) {
 }
 
 }  // namespace
+
+// Whether bi_launch_pair_window takes every window call on a model: the longest window, damped, fits one CTA.
+bool bi_pair_window_always(const bi_model *md) {
+  const BiDev &h = md->h;
+  if (md->arith != BI_ARITH_F64 || h.has_bdep || !md->rank2_ok) return false;
+  int nmax = 1, ng = 0, nar = 2, ls = 3;
+  for (int f = 0; f < h.F; ++f) nmax = std::max(nmax, (int)h.n[f]);
+  for (int gi = 0; gi < h.ngroups; ++gi) {
+    if (h.grp[gi].rank != 2) continue;
+    ++ng;
+    nar = std::max(nar, (h.grp[gi].dim[0] + 1) & ~1);
+    ls = std::max(ls, bi_pad4(h.grp[gi].dim[1]) + 1);
+  }
+  const int LPU = nmax <= 4 ? 4 : nmax <= 8 ? 8 : nmax <= 16 ? 16 : 32, threads = window_threads(BI_MAX_T, LPU);
+  return threads <= kMaxThreads && window_bytes(threads / LPU, LPU, h.F, ng, nar, ls, true) <= (size_t)md->max_smem_optin - 1024;
+}
 
 // Applicable to float64 handles, plain and damped updates, trivial B-dependencies, window calls (also warm
 // starts and continued windows) on models with no group over more than two factors, and to windows

@@ -217,3 +217,52 @@ def test_observation_vectors_reserve_one_layout():
     md.close()
     slices = w.N * w.T * 36 * 48 * 8
     assert used <= slices + (80 << 20), (used, slices)   # (the allocator takes whole chunks of 32 MB; kernels are loaded on first use)
+
+
+def test_pair_models_keep_no_copy_that_no_call_reads():
+    """The pair kernels take every call on a float64 model with one pair of factors of up to eight states."""
+    import dataclasses
+    import torch
+    import paper_2607_17855_b200 as bi
+    G = 120000
+    w = _workload(120, [8, 7], [[0, 1]], N=1, T=2, K=2)
+    rep = lambda x: np.broadcast_to(x, (G,) + x.shape[1:]).copy()
+    w = dataclasses.replace(w, G=G, N=G, A=[rep(x) for x in w.A], B=[rep(x) for x in w.B], D=[rep(x) for x in w.D])
+    arrays = [[torch.from_numpy(x).cuda() for x in part] for part in (w.A, w.B, w.D)]
+    bi.Model(w.n, w.m, w.dep, w.U, w.G, *arrays).close()   # (the kernels of the packing are loaded)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    md = bi.Model(w.n, w.m, w.dep, w.U, w.G, *arrays)
+    torch.cuda.synchronize()
+    used = before - torch.cuda.mem_get_info()[0]
+    md.close()
+    slices = G * int(w.m[0]) * 8 * 8 * 8 * 2                          # rows and, for the filtering kernel, columns
+    matrices = G * sum(6 * int(u) * int(k) * 8 * 8 for u, k in zip(w.U, w.n)) + G * 2 * 8 * 8
+    assert used <= slices + matrices + (48 << 20), (used, slices, matrices)   # (sixteen allocations in whole 2 MB)
+
+
+def test_a_model_that_fits_without_its_second_copy_is_made():
+    """With room for the packed slices but not for the block-ordered ones beside them the handle is made without the
+    latter, and the call runs on another kernel."""
+    import torch
+    import oracle
+    import paper_2607_17855_b200 as bi
+    G = 16000
+    w = _workload(121, [9, 10, 11], [[0, 1, 2]], N=G, T=2, K=2)
+    shared = [[torch.from_numpy(x).cuda() for x in part] for part in (w.A, w.B, w.D)]
+    arrays = [[x.expand(G, *x.shape[1:]).contiguous() for x in part] for part in shared]
+    bi.Model(w.n, w.m, w.dep, w.U, 1, *shared).close()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    packed = G * int(w.m[0]) * 9 * 10 * 12 * 8
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - (packed * 5 // 4 + (200 << 20)), dtype=torch.uint8, device="cuda")
+    try:
+        md = bi.Model(w.n, w.m, w.dep, w.U, G, *arrays)
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+    q = md.bi_filter(torch.from_numpy(w.obs).cuda(), torch.from_numpy(w.act).cuda(), w.K).cpu().numpy()
+    assert md.last_family == "cta_filter_f64" and md.status() == 0
+    md.close()
+    sel = list(range(0, G, 799))
+    assert np.abs(q[sel] - oracle.run_workload(w.take_agents(sel), "filter")[0]).max() <= 1e-5
