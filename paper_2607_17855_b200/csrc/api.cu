@@ -38,6 +38,7 @@ struct PackA {
   int64_t sstride[BI_MAX_RANK];  // source stride of each packed axis
   int32_t npad;                  // padded size of the last packed axis (rank > 0)
   uint32_t *wide;                // [0] set when an entry exceeds 1, [1] when one is at or below 1e-16 (BiDev::status)
+  int32_t mark_floor;            // whether [1] is wanted (some call of the model chooses its kernel by it)
 };
 
 // ln(max(A, eps)) in float64, rounded once; outcome slices contiguous, axes in
@@ -49,12 +50,13 @@ __global__ void bi_pack_A_kernel(PackA p) {
   int64_t go = e / p.P_pad;  // g * m + o
   int32_t idx = (int32_t)(e - go * p.P_pad);
   R out = (R)0;
+  bool floor = false;
   if (p.rank == 0) {
     // every axis has a single state: the slice is one number (padded to 4)
     if (idx == 0) {
       const float v = p.src[go * p.P];
       if (v > 1.0f) atomicOr(p.wide, 1u);
-      if (v <= 1e-16f) p.wide[1] = 1u;
+      floor = v <= 1e-16f;
       out = (R)log(fmax((double)v, 1e-16));
     }
   } else {
@@ -68,11 +70,17 @@ __global__ void bi_pack_A_kernel(PackA p) {
       }
       const float v = p.src[s];
       if (v > 1.0f) atomicOr(p.wide, 1u);
-      if (v <= 1e-16f) p.wide[1] = 1u;
+      floor = v <= 1e-16f;
       out = (R)log(fmax((double)v, 1e-16));
     }
   }
   ((R *)p.dst)[e] = out;
+  // one vote per warp and one store, while the mark is still clear: a store by every zero of a sparse per-agent
+  // model is a hundred million of them to one word
+  if (p.mark_floor) {
+    const unsigned zeros = __ballot_sync(__activemask(), floor);
+    if (zeros && (threadIdx.x & 31) == __ffs(zeros) - 1 && *(volatile uint32_t *)(p.wide + 1) == 0u) p.wide[1] = 1u;
+  }
 }
 
 // B[g][s_next][s_prev][u] -> four [g][u][row][npad] matrices
@@ -564,6 +572,7 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
       p.src = desc->A[i];
       p.dst = dst;
       p.wide = h.status + 1;
+      p.mark_floor = md->blk_BR || arith == BI_ARITH_F32;
       p.total = (int64_t)count;
       p.P_pad = g.P_pad;
       p.rank = g.rank;
@@ -595,6 +604,7 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
         rc = dev_alloc(md, &tdst, tcount * esz);
         if (rc != BI_OK) break;
         t.dst = tdst;
+        t.mark_floor = 0;
         t.total = (int64_t)tcount;
         t.P_pad = g.dim[1] * bi_pad4(g.dim[0]);
         t.dim[0] = g.dim[1]; t.dim[1] = g.dim[0];

@@ -266,3 +266,17 @@ def test_a_model_that_fits_without_its_second_copy_is_made():
     md.close()
     sel = list(range(0, G, 799))
     assert np.abs(q[sel] - oracle.run_workload(w.take_agents(sel), "filter")[0]).max() <= 1e-5
+
+
+@pytest.mark.parametrize("where", [None, "first", "last", "middle"])
+def test_a_single_zero_in_a_is_seen(where):
+    """Filtering on a model with zeros in A stays on the CTA kernel; one zero anywhere is enough (the packing kernel's
+    last warp is a partial one here)."""
+    w = _workload(130, [5, 3, 7], [[0, 1, 2], [2]], N=3, T=2, K=3)
+    for a in w.A:
+        a[:] = np.maximum(a, 1e-6)
+    if where:
+        a = w.A[0] if where != "last" else w.A[1]
+        a.reshape(-1)[{"first": 0, "last": -1, "middle": a.size // 2}[where]] = 0.0
+    res = check_workload(w, "filter")
+    assert res["family"] == ("cta_filter_f64" if where else "block_filter_f64"), res
