@@ -646,6 +646,7 @@ void fill_params(const BiCall &c, const Plan &pl, Params &p) {
       p.Mp[f] = h.logBfull[f];
       p.wpar = std::max(p.wpar, (h.PB[f] + 3) & ~3);
     } else if (window) {
+      if (h.n[f] == 1) p.ones |= 1u << f;
       p.Mp[f] = c.algo == BI_ALGO_VMP ? h.logBt[f] : h.BfT[f];     // [previous][next]
       p.Mf[f] = c.algo == BI_ALGO_VMP ? h.logB[f] : h.BdagT[f];    // [next][previous]
     } else {

@@ -683,6 +683,11 @@ __global__ void __launch_bounds__(max_threads(BR * BC * (int)sizeof(R) / 4), 1) 
     if (xp >= 0 && p.q_init && real)
       at<double>(xp + (p.qo[f] + s) * 8) = (double)bi_log(bi_max((R)__ldg(p.q_init + ((size_t)agent * T + t) * p.S + i), (R)BI_EPS));
   }
+  if (t > 0)
+    for (uint32_t mk = p.ones; mk; mk &= mk - 1) {
+      const int f = __ffs(mk) - 1;
+      clamp_flag(__ldg(p.act + ((size_t)agent * (T - 1) + (t - 1)) * p.F + f), p.U[f], p.status, BI_FLAG_ACT_RANGE);
+    }
   // ---- this thread's block: a group's summed slice, or part of an edge's transition (both are read and one
   // is taken where a warp holds blocks of both kinds: see gather_group on why the warp must not split)
   const bool has_prev = t > 0, has_next = t + 1 < T;

@@ -90,6 +90,7 @@ struct Params {
   int32_t max_mem, n_max;      // most modalities of a group, most states of a factor
   int32_t g_any;               // a group over several factors (valid to read from)
   int32_t extra;               // blocks beyond one per thread, in whole warps (kept in shared memory)
+  uint32_t ones;               // window: factors of one state (no transition blocks: their actions are only checked)
   int32_t common;              // the softmax needs no shift
   double lambda;
   int32_t n[BI_MAX_F], off[BI_MAX_F], qo[BI_MAX_F], npad[BI_MAX_F], U[BI_MAX_F];

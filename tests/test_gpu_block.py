@@ -280,3 +280,22 @@ def test_a_single_zero_in_a_is_seen(where):
         a.reshape(-1)[{"first": 0, "last": -1, "middle": a.size // 2}[where]] = 0.0
     res = check_workload(w, "filter")
     assert res["family"] == ("cta_filter_f64" if where else "block_filter_f64"), res
+
+
+@pytest.mark.parametrize("algo", ["filter", "vmp", "mmp"])
+def test_actions_of_every_factor_are_checked(algo):
+    """An action out of range raises the status flag whichever factor and step it is of, a factor of one state included."""
+    import torch
+    import paper_2607_17855_b200 as bi
+    w = _workload(140, [3, 1, 4, 2], [[0, 2, 3], [0]], N=6, T=9, K=2)
+    md = bi.model_from_workload(w)
+    obs = torch.from_numpy(w.obs).cuda()
+    for f in range(4):
+        for step, bad in ((0, -1), (3, 9), (7, int(w.U[f]))):
+            act = w.act.copy()
+            act[2, step, f] = bad
+            md.run(algo, obs, torch.from_numpy(act).cuda(), w.K)
+            assert md.status() == 2, (f, step)
+    md.run(algo, obs, torch.from_numpy(w.act).cuda(), w.K)
+    assert md.status() == 0 and md.last_family == f"block_{algo}_f64"
+    md.close()
