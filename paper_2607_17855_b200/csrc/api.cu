@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -312,6 +313,26 @@ int validate_desc(const bi_model_desc *d) {
 }
 
 }  // namespace
+
+cudaError_t bi_allow_smem(const void *kern, size_t bytes, bool carveout) {
+  struct Limit { const void *kern; int device; size_t bytes; };
+  constexpr size_t kSlots = 4096;   // (open addressing; some two hundred kernels per device)
+  static Limit limits[kSlots];
+  static std::mutex lock;
+  int device = 0;
+  cudaError_t e = cudaGetDevice(&device);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> hold(lock);
+  size_t at = (((size_t)kern >> 4) * 31 + (size_t)device * 509) % kSlots, probes = 0;
+  while (limits[at].kern && (limits[at].kern != kern || limits[at].device != device) && ++probes < kSlots) at = (at + 1) % kSlots;
+  const bool known = limits[at].kern == kern && limits[at].device == device;
+  if (known && limits[at].bytes >= bytes) return cudaSuccess;
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess && carveout) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  if (e != cudaSuccess) cudaGetLastError();
+  else if (probes < kSlots) limits[at] = {kern, device, bytes};
+  return e;
+}
 
 // ------------------------------------------------------------------ public API
 

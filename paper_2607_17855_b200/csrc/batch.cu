@@ -1271,7 +1271,7 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
     cfg.blockDim = dim3(1024);
     cfg.dynamicSmemBytes = 4 * max_m * sizeof(int32_t);
     if (cfg.dynamicSmemBytes > 48 * 1024 &&
-        cudaFuncSetAttribute((const void *)bi_batch_bucket_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes) != cudaSuccess)
+        bi_allow_smem((const void *)bi_batch_bucket_kernel, cfg.dynamicSmemBytes) != cudaSuccess)
       return BI_ERR_CUDA;
     cfg.stream = c.stream;
     cfg.attrs = early;
@@ -1282,9 +1282,9 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
   const ContractKernel rt = per_unit ? (ncp_max <= 16 ? bi_batch_contract_rt_kernel<R, true, 16> : bi_batch_contract_rt_kernel<R, true, 32>)
                                      : (ncp_max <= 16 ? bi_batch_contract_rt_kernel<R, false, 16> : bi_batch_contract_rt_kernel<R, false, 32>);
   const ContractKernel unrolled = bi_batch_contract_kernel<R>;
-  if (use_rt && cudaFuncSetAttribute((const void *)rt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem) != cudaSuccess)
+  if (use_rt && bi_allow_smem((const void *)rt, csmem) != cudaSuccess)
     return BI_ERR_CUDA;
-  if (!any_shape && cudaFuncSetAttribute((const void *)unrolled, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)usmem) != cudaSuccess)
+  if (!any_shape && bi_allow_smem((const void *)unrolled, usmem) != cudaSuccess)
     return BI_ERR_CUDA;
   for (int gi = 0; gi < h.ngroups; ++gi) {
     const BiGroup &g = h.grp[gi];
@@ -1348,7 +1348,7 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
       unit_mid = pick_unit(false);
       unit_last = pick_unit(true);
       for (UnitKernel k : {unit_mid, unit_last})
-        if (cudaFuncSetAttribute((const void *)k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)unit_smem) != cudaSuccess)
+        if (bi_allow_smem((const void *)k, unit_smem) != cudaSuccess)
           return BI_ERR_CUDA;
     }
   }

@@ -184,6 +184,11 @@ struct BiCall {
   cudaStream_t stream;
 };
 
+// Raises a kernel's dynamic shared memory limit on the current device to at least `bytes` (and, with `carveout`, asks for
+// the largest shared-memory share of L1).  The limit belongs to the kernel, not to the launch: threads that each set
+// their own size before launching can lower it under one another, so it is only ever raised, behind a lock.
+cudaError_t bi_allow_smem(const void *kern, size_t bytes, bool carveout = false);
+
 // kernel families; each returns BI_OK, BI_ERR_UNSUPPORTED (not applicable to
 // this model / call: the dispatcher tries the next one) or an error.
 int bi_launch_generic(const BiCall &c, bi_model *mut);

@@ -1,6 +1,5 @@
 // Planner and launcher of the block kernels (block.cuh).
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -686,20 +685,6 @@ void fill_params(const BiCall &c, const Plan &pl, Params &p) {
   p.q_out = c.q_out; p.logq_out = c.logq_out; p.argmax_out = c.argmax_out; p.status = h.status;
 }
 
-// The attribute is set once per kernel and device and only ever raised.
-bool allow_smem(const void *kern, int slot, int device, size_t bytes) {
-  constexpr int kDev = 32;
-  static std::atomic<int> have[72][kDev];
-  if (device < kDev && have[slot][device].load(std::memory_order_relaxed) >= (int)bytes) return true;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess ||
-      cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  if (device < kDev) have[slot][device].store((int)bytes, std::memory_order_relaxed);
-  return true;
-}
-
 }  // namespace
 
 // A model with zeros in A amplifies a rounding by up to 1e9 within sixteen iterations, and a trajectory carries
@@ -871,8 +856,7 @@ int bi_launch_block(const BiCall &c, bi_model *mut) {
   const void *kern = esz == 8 ? bi_block_kernel_f64(pl.BR, pl.BC, window, sync, hass)
                               : bi_block_kernel_f32(pl.BR, pl.BC, window, sync, hass);
   if (!kern) return BI_ERR_UNSUPPORTED;
-  const int slot = (((pl.BR == 4 ? 0 : pl.BC == 4 ? 1 : 2) * 2 + window) * 3 + sync) * 4 + hass * 2 + (esz == 8);
-  if (!allow_smem(kern, slot, md->device, L.bytes)) return BI_ERR_CUDA;
+  if (bi_allow_smem(kern, L.bytes, true) != cudaSuccess) return BI_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(L.grid);
   cfg.blockDim = dim3(L.threads);

@@ -700,8 +700,7 @@ int launch_cta_filter_t(const BiCall &c, bi_model *mut) {
   if ((size_t)o * sizeof(R) > (size_t)md->max_smem_optin - 1024) return BI_ERR_UNSUPPORTED;
 
   auto kern = bi_cta_filter_kernel<R>;
-  if (cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sm.total_bytes) !=
-      cudaSuccess)
+  if (bi_allow_smem((const void *)kern, sm.total_bytes) != cudaSuccess)
     return BI_ERR_CUDA;
   kern<<<c.N, NT, sm.total_bytes, c.stream>>>(md->d, c.T, c.obs, c.act, c.q_prev, c.act_prev, c.carry_in, c.carry_out, c.lambda, c.K, c.q_out,
                                                c.logq_out, c.argmax_out, md->exp_tab, sm);

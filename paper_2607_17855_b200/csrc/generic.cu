@@ -525,8 +525,7 @@ int launch_generic_t(const BiCall &c, bi_model *mut) {
     name = f64 ? (sm.staged ? "generic_mmp_staged_f64" : "generic_mmp_global_f64")
                : (sm.staged ? "generic_mmp_staged_f32" : "generic_mmp_global_f32");
   }
-  if (cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sm.total_bytes) !=
-      cudaSuccess)
+  if (bi_allow_smem((const void *)kern, sm.total_bytes) != cudaSuccess)
     return BI_ERR_CUDA;
   kern<<<c.N, NT, sm.total_bytes, c.stream>>>(md->d, c.N, c.T, c.obs, c.act, c.q_prev, c.act_prev, c.carry_in,
                                                c.carry_out, c.q_init, c.lnprior, c.lambda, c.K, c.q_out, c.logq_out, c.argmax_out, sm);

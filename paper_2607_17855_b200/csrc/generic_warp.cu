@@ -706,7 +706,7 @@ int launch_warp_t(const BiCall &c, bi_model *mut) {
   cudaError_t e;
   if (!window) {
     auto kern = bi_warp_filter_kernel<R>;
-    e = cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sm.total_bytes);
+    e = bi_allow_smem((const void *)kern, sm.total_bytes);
     if (e != cudaSuccess) return BI_ERR_CUDA;
     kern<<<(c.N + W - 1) / W, W * 32, sm.total_bytes, c.stream>>>(md->d, c.N, c.T, c.obs, c.act, c.q_prev,
                                                                    c.act_prev, c.carry_in, c.carry_out, c.lambda, c.K,
@@ -714,14 +714,14 @@ int launch_warp_t(const BiCall &c, bi_model *mut) {
     name = f64 ? "warp_filter_f64" : "warp_filter_f32";
   } else if (c.algo == BI_ALGO_VMP) {
     auto kern = bi_warp_window_kernel<R, BI_ALGO_VMP>;
-    e = cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sm.total_bytes);
+    e = bi_allow_smem((const void *)kern, sm.total_bytes);
     if (e != cudaSuccess) return BI_ERR_CUDA;
     kern<<<c.N, W * 32, sm.total_bytes, c.stream>>>(md->d, c.N, c.T, c.obs, c.act, c.q_init, c.lnprior, c.lambda, c.K,
                                                     c.q_out, c.logq_out, c.argmax_out, sm);
     name = f64 ? "warp_vmp_f64" : "warp_vmp_f32";
   } else {
     auto kern = bi_warp_window_kernel<R, BI_ALGO_MMP>;
-    e = cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sm.total_bytes);
+    e = bi_allow_smem((const void *)kern, sm.total_bytes);
     if (e != cudaSuccess) return BI_ERR_CUDA;
     kern<<<c.N, W * 32, sm.total_bytes, c.stream>>>(md->d, c.N, c.T, c.obs, c.act, c.q_init, c.lnprior, c.lambda, c.K,
                                                     c.q_out, c.logq_out, c.argmax_out, sm);

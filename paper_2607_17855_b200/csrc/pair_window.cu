@@ -307,7 +307,7 @@ int launch(PairWinParams &p, const bi_model *md, cudaStream_t stream) {
     if (damped) kern = p.algo == BI_ALGO_VMP ? bi_pair_window_kernel<LPU, BI_ALGO_VMP, 512, true> : bi_pair_window_kernel<LPU, BI_ALGO_MMP, 512, true>;
     else kern = p.algo == BI_ALGO_VMP ? bi_pair_window_kernel<LPU, BI_ALGO_VMP, 512, false> : bi_pair_window_kernel<LPU, BI_ALGO_MMP, 512, false>;
   }
-  if (cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) {
+  if (bi_allow_smem((const void *)kern, bytes) != cudaSuccess) {
     cudaGetLastError();
     return BI_ERR_CUDA;
   }

@@ -294,7 +294,7 @@ int run_soft_t(const bi_model *model, int algo, int N, int T, const float *obs_s
   void (*kerns[4])(const SoftJob) = {bi_soft_slices_kernel<R, 1>, bi_soft_slices_kernel<R, 2>,
                                      bi_soft_slices_kernel<R, 3>, bi_soft_slices_kernel<R, 4>};
   for (auto kf : kerns)
-    if (cudaFuncSetAttribute((const void *)kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsmem) != cudaSuccess)
+    if (bi_allow_smem((const void *)kf, wsmem) != cudaSuccess)
       return BI_ERR_CUDA;
   int launches = 0;
   // layout 0: every group's packed slices; 1: the lane-interleaved slices of a tile model; 2: the

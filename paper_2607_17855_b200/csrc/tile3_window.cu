@@ -533,7 +533,7 @@ int launch_window(const Tile3Params &p, int smem_budget, cudaStream_t stream) {
     // CTAs that fit an SM together (shared memory and registers), as the runtime counts them
     const void *kf = pick(cs > 1);
     int per_sm = 0;
-    if (cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b) != cudaSuccess ||
+    if (bi_allow_smem(kf, b) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kf, warps * 32, b) != cudaSuccess) {
       cudaGetLastError();
       continue;
@@ -574,7 +574,7 @@ int launch_window(const Tile3Params &p, int smem_budget, cudaStream_t stream) {
   cfg.numAttrs = geo.CS > 1 ? 1 : 0;
   const void *kern = pick(geo.CS > 1);
   void *args[2] = {(void *)&p, (void *)&geo};
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  cudaError_t e = bi_allow_smem(kern, bytes);
   if (e == cudaSuccess) e = cudaLaunchKernelExC(&cfg, kern, args);
   if (e != cudaSuccess) {
     cudaGetLastError();

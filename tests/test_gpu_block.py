@@ -299,3 +299,47 @@ def test_actions_of_every_factor_are_checked(algo):
     md.run(algo, obs, torch.from_numpy(w.act).cuda(), w.K)
     assert md.status() == 0 and md.last_family == f"block_{algo}_f64"
     md.close()
+
+
+@pytest.mark.parametrize("family", ["batch", "cta", "warp", "block"])
+def test_threads_with_models_of_different_sizes(family):
+    """Calls of several threads, each on a handle and stream of its own, on kernels that they share with different
+    amounts of shared memory."""
+    import threading
+    import torch
+    import paper_2607_17855_b200 as bi
+    from test_gpu_parity import family_forced
+    algo = "filter" if family == "cta" else "vmp"
+    with family_forced(family):
+        jobs = []
+        for i, n in enumerate(([12, 12, 12], [3, 4, 5], [9, 7, 11], [6, 5, 3])):
+            w = _workload(150 + i, n, [[0, 1, 2], [1, 2]], N=140, T=16, K=3)
+            md = bi.model_from_workload(w)
+            obs, act = torch.from_numpy(w.obs).cuda(), torch.from_numpy(w.act).cuda()
+            jobs.append((md, obs, act, w.K, md.run(algo, obs, act, w.K)))
+    torch.cuda.synchronize()
+    failures, go = [], threading.Barrier(len(jobs))
+
+    def work(md, obs, act, K, want):
+        s = torch.cuda.Stream()
+        with torch.cuda.stream(s):
+            q = torch.empty_like(want)
+            go.wait()
+            try:
+                for _ in range(300):
+                    md.run(algo, obs, act, K, q_out=q)
+                s.synchronize()
+                if not torch.equal(q, want):
+                    failures.append("other beliefs")
+            except Exception as e:
+                failures.append(repr(e))
+
+    threads = [threading.Thread(target=work, args=j) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    for j in jobs:
+        j[0].close()
+    assert not failures, failures
