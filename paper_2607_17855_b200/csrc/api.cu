@@ -359,14 +359,25 @@ extern "C" int bi_model_slice_bytes(const bi_model_t *model, int64_t *dense, int
 static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep_len, const int32_t *bdep,
                        void *cuda_stream, bi_model_t **out);
 
+// Planning and grouping use the host's allocator: its failure is an error code like the device's, not an exception
+// that crosses the C interface.
+static int create(const bi_model_desc *desc, int arith, const int32_t *bdep_len, const int32_t *bdep, void *cuda_stream,
+                  bi_model_t **out) {
+  try {
+    return create_impl(desc, arith, bdep_len, bdep, cuda_stream, out);
+  } catch (const std::bad_alloc &) {
+    return BI_ERR_ALLOC;
+  }
+}
+
 extern "C" int bi_model_create_arith(const bi_model_desc *desc, int arith, void *cuda_stream, bi_model_t **out) {
-  return create_impl(desc, arith, nullptr, nullptr, cuda_stream, out);
+  return create(desc, arith, nullptr, nullptr, cuda_stream, out);
 }
 
 extern "C" int bi_model_create_bdep(const bi_model_desc *desc, const int32_t *bdep_len, const int32_t *bdep, int arith,
                                     void *cuda_stream, bi_model_t **out) {
   if (!bdep_len || !bdep) return BI_ERR_INVALID_ARG;
-  return create_impl(desc, arith, bdep_len, bdep, cuda_stream, out);
+  return create(desc, arith, bdep_len, bdep, cuda_stream, out);
 }
 
 static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep_len, const int32_t *bdep,
@@ -400,6 +411,17 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
   bi_model *md = new (std::nothrow) bi_model();
   if (!md) return BI_ERR_ALLOC;
   memset(md, 0, sizeof(*md));
+  struct Undo {   // (whichever way this function is left without a handle)
+    bi_model *md;
+    cudaStream_t stream;
+    ~Undo() {
+      if (!md) return;
+      cudaStreamSynchronize(stream);
+      free_all(md);
+      bi_block_free(md);
+      delete md;
+    }
+  } undo = {md, stream};
   md->damping = 1.0;
   if (const char *e = getenv("BI_TEST_NO_COMPRESS")) md->test_no_compress = atoi(e) != 0;
   if (const char *e = getenv("BI_TEST_DROP_COPY")) md->test_drop_copy = atoi(e) > 0 ? atoi(e) : 0;   // testing aids,
@@ -410,10 +432,7 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
   }
   md->last_kernel = "";
   md->arith = arith;
-  if (cudaGetDevice(&md->device) != cudaSuccess) {
-    delete md;
-    return BI_ERR_CUDA;
-  }
+  if (cudaGetDevice(&md->device) != cudaSuccess) return BI_ERR_CUDA;
   cudaDeviceGetAttribute(&md->sm_count, cudaDevAttrMultiProcessorCount, md->device);
   cudaDeviceGetAttribute(&md->max_smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, md->device);
 
@@ -920,13 +939,8 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
       rc = BI_ERR_CUDA;
     md->has_zeros = z != 0;
   }
-  if (rc != BI_OK) {
-    cudaStreamSynchronize(stream);
-    free_all(md);
-    bi_block_free(md);
-    delete md;
-    return rc;
-  }
+  if (rc != BI_OK) return rc;
+  undo.md = nullptr;
   *out = md;
   return BI_OK;
 }
