@@ -343,3 +343,53 @@ def test_threads_with_models_of_different_sizes(family):
     for j in jobs:
         j[0].close()
     assert not failures, failures
+
+
+@pytest.mark.parametrize("damping", [1.0, 0.5])
+@pytest.mark.parametrize("case", ["warps_of_one_cta", "cluster", "shared_memory_blocks"])
+def test_every_call_form(case, damping):
+    """Continued, warm-started and damped calls and observation vectors, on teams of one and of several warps, windows over
+    one CTA and over a cluster, blocks left over for shared memory; all by the name of the kernel that ran."""
+    import torch
+    import oracle
+    import paper_2607_17855_b200 as bi
+    from test_gpu_parity import _soft_vectors
+    n, dep, T = {"warps_of_one_cta": ([3, 4, 2, 5], [[0, 1, 2], [1, 3]], 4), "cluster": ([9, 6, 12, 4], [[0, 1], [1, 2, 3], [0, 1, 2]], 13),
+                 "shared_memory_blocks": ([18, 29, 11], [[0, 1, 2], [0, 2]], 7)}[case]
+    N = 5
+    w = _workload(160, n, dep, N=N, T=T, K=5)
+    rng = np.random.default_rng(161)
+    simplex = lambda *size: np.concatenate([rng.dirichlet(np.full(k, 1.5), size=size) for k in n], axis=-1).astype(np.float32)
+    q_prev, q_init, soft = simplex(N), simplex(N, T), _soft_vectors(w, 162)
+    act_prev = np.stack([rng.integers(0, int(u), size=N) for u in w.U], axis=1).astype(np.int32)
+    cuda = lambda x: torch.from_numpy(x).cuda()
+    obs, act = cuda(w.obs), cuda(w.act)
+    md = bi.model_from_workload(w)
+    md.set_damping(damping)
+    for algo in ("filter", "vmp", "mmp"):
+        prev = dict(q_prev=q_prev.astype(np.float64), act_prev=act_prev)
+        start = dict(q_init=q_init.astype(np.float64))
+        calls = [("from", lambda: md.run_from(algo, obs, act, cuda(q_prev), cuda(act_prev), w.K), prev),
+                 ("soft", lambda: md.run_soft(algo, cuda(soft), act, w.K), dict(obs_soft=soft))]
+        if algo != "filter":
+            warm = md.bi_vmp_warm if algo == "vmp" else md.bi_mmp_warm
+            calls += [("warm", lambda: warm(obs, act, cuda(q_init), w.K), start),
+                      ("from, warm", lambda: md.run_from(algo, obs, act, cuda(q_prev), cuda(act_prev), w.K, q_init=cuda(q_init)),
+                       {**prev, **start})]
+        for name, call, kw in calls:
+            q = call().cpu().numpy()
+            assert md.last_family == f"block_{algo}_f64", (algo, name, md.last_family)
+            ref = oracle.run(algo, w.n, w.m, w.dep, w.U, w.G, w.A, w.B, w.D, None if "obs_soft" in kw else w.obs, w.act, w.K,
+                             damping=damping, **kw)[0]
+            assert np.abs(q - ref).max() <= 1e-5, (algo, name, np.abs(q - ref).max())
+    assert md.status() == 0
+    md.close()
+
+
+@pytest.mark.parametrize("algo", ["filter", "vmp", "mmp"])
+def test_sixteen_modalities(algo):
+    """More modalities than the softmax without a shift allows: log-beliefs and most probable states relative to the
+    largest logit."""
+    dep = [[0, 1, 2], [1, 2], [0, 2], [0]] * 4
+    res = check_workload(_workload(170, [5, 4, 7], dep, N=6, T=5, K=4), algo)
+    assert res["family"] == f"block_{algo}_f64", res
