@@ -255,7 +255,8 @@ def test_a_model_that_fits_without_its_second_copy_is_made():
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
     packed = G * int(w.m[0]) * 9 * 10 * 12 * 8
-    fill = torch.empty(torch.cuda.mem_get_info()[0] - (packed * 5 // 4 + (200 << 20)), dtype=torch.uint8, device="cuda")
+    matrices = G * sum(6 * int(u) * int(k) * 12 * 8 for u, k in zip(w.U, w.n))   # (six forms of every action's, rows padded to 12)
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - (packed * 5 // 4 + matrices + (200 << 20)), dtype=torch.uint8, device="cuda")
     try:
         md = bi.Model(w.n, w.m, w.dep, w.U, G, *arrays)
     finally:
