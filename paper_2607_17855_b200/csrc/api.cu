@@ -1002,6 +1002,7 @@ int bi_dispatch(const BiCall &c, bi_model *mut) {
     if (rc == BI_ERR_UNSUPPORTED) rc = bi_launch_pair_window(c, mut);
     if (rc == BI_ERR_UNSUPPORTED && c.model->test_drop_copy == 0) rc = bi_launch_block(c, mut);
     if (rc == BI_ERR_UNSUPPORTED) rc = bi_launch_batch(c, mut);
+    if (rc == BI_ERR_UNSUPPORTED && c.algo != BI_ALGO_FILTER && c.model->test_drop_copy == 0) rc = bi_launch_block(c, mut, false);
     // Filtering exposes one unit per agent, so a CTA per agent keeps more of the machine busy than
     // a warp per agent, and its staged slices and per-factor warps pay at every batch size measured
     // on the 128 random structures (sum of times, CTA against warp kernel): 44 against 99 ms at 256

@@ -200,7 +200,9 @@ bool bi_pair_window_always(const bi_model *md);             // whether that one 
 int bi_launch_tile3(const BiCall &c, bi_model *mut);
 int bi_launch_tile3_window(const BiCall &c, bi_model *mut);
 int bi_launch_batch(const BiCall &c, bi_model *mut);
-int bi_launch_block(const BiCall &c, bi_model *mut);        // any structure of rank up to 4; blocks of the slices in registers
+// any structure of rank up to 4; blocks of the slices in registers.  `estimate`: declines what another family is
+// estimated to run faster (should that one then decline, the call comes back without)
+int bi_launch_block(const BiCall &c, bi_model *mut, bool estimate = true);
 // elements of one outcome's slice of group gi in the block kernels' order (0: the model has none)
 int bi_block_slice_elems(const bi_model *md, int gi);
 // whether the block kernels may serve such calls on this model (they may still decline one that does not fit)

@@ -705,8 +705,9 @@ namespace {
 // Microseconds a window call would take here and on the batched kernels (batch.cu), for the choice between them.
 // Linear in what each spends its time on -- here block entries, warps and finishing passes per unit, there a
 // pair of launches per iteration, the longest slice's serial walk, slice entries and states per unit -- with
-// coefficients fitted to 113 structures of two to five factors, 2 048 to 62 000 units (12 and 17 % rms error).
-// Neither side wins by size alone: [8,13,10] under two rank-3 slices, 34 124 units, 2234 us here and 1844 us there;
+// coefficients fitted to 204 structures of one to five factors, 2 100 to 62 000 units, 6 and 16 iterations (in
+// cross-validation 13 and 17 % rms error here, 19 % there, float64 and float32).  Neither side wins by size alone:
+// [9,32,19] under two rank-2 slices, float32, 59 508 units, 4463 us here and 2407 us there;
 // [14,14,2,12] under a rank-4 slice, 2 472 units, 342 and 595 us.
 struct WindowCost { double block, batch; };
 WindowCost window_cost(const BiCall &c, const Plan &pl, const Variant &v) {
@@ -734,10 +735,12 @@ WindowCost window_cost(const BiCall &c, const Plan &pl, const Variant &v) {
   const bool lane_per_unit = nmax <= 16 && (double)c.N * c.T * std::min(1.0, h.F / 3.0) >= 64.0 * c.model->sm_count;   // (the update's form, see batch.cu)
   if (!lane_per_unit) lanes = (double)h.F * (nmax <= 8 ? 8 : nmax <= 16 ? 16 : 32) * nmax;
   WindowCost w;
-  w.block = f64 ? 13 + k * (56 * ent + (12 + 12 * v.nbpt) * warps + 89 * v.npass) + 1270 * per_sm * ent
-                : k * (1.6 * ent + (66 + 1.1 * v.nbpt) * warps + 42 * v.npass) + 1920 * per_sm * ent;
-  w.batch = f64 ? c.K * (6.3 * (members ? 2 : 1) + 2.9 * longest) + k * (35 * slices + 1.13 * states * (members + 2) + 0.106 * lanes) + 568 * per_sm * members
-                : 31 + c.K * (4.3 * (members ? 2 : 1) + 6.4 * longest) + k * (21 * slices + 1.27 * states * (members + 2) + 0.129 * lanes) + 63 * per_sm * members;
+  const double mmp = c.algo == BI_ALGO_MMP;   // (two logarithms per state)
+  w.block = f64 ? 19 + k * (81 * ent + (80 + 39 * v.nbpt) * warps + 3 * mmp * v.npass) + 675 * per_sm * ent
+                : 9 + 0.2 * c.K + k * (88 * ent + 4.7 * v.nbpt * warps + (73 + 9.4 * mmp) * v.npass) + per_sm * (117 * ent + 358 * warps);
+  const double launches = members ? 2 : 1;
+  w.batch = f64 ? 21 + c.K * (8.1 * launches + 3.6 * longest) + k * (86 * slices + states * (1.28 * members + 0.33 + 0.62 * mmp) + 0.103 * lanes) + 16 * per_sm * members
+                : c.K * (6.6 * launches + 4.4 * longest) + k * (38 * slices + states * (0.81 * members + 0.38 + 0.38 * mmp) + 0.093 * lanes) + 13 * per_sm * members;
   return w;
 }
 
@@ -752,7 +755,8 @@ struct Route {
 // Whether these kernels take a call, and in which shape.  Any model whose groups span at most four factors
 // (transitions over at most three parents in window calls), either arithmetic, as long as a step's blocks fit the
 // register file and shared memory of an SM (window calls: of a cluster).
-bool choose_route(const BiCall &c, Route &L) {
+// `estimate`: declines calls that another family is estimated to run faster.
+bool choose_route(const BiCall &c, Route &L, bool estimate = true) {
   const bi_model *md = c.model;
   const bool window = c.algo != BI_ALGO_FILTER;
   const Plan *plp = static_cast<const Plan *>(md->blk_plan[window ? 1 : 0]);
@@ -822,9 +826,9 @@ bool choose_route(const BiCall &c, Route &L) {
       }
     }
     if (bv < 0) return false;
-    if (!md->h.has_bdep && md->h.G == 1 && (long long)c.N * c.T >= 2048 && md->test_family == BI_FAMILY_ANY && !md->soft_shadow) {
+    if (estimate && !md->h.has_bdep && md->h.G == 1 && (long long)c.N * c.T >= 2048 && md->test_family == BI_FAMILY_ANY && !md->soft_shadow) {
       const WindowCost w = window_cost(c, pl, pl.var[bv]);
-      if (w.batch < 0.9 * w.block) return false;
+      if (w.batch < w.block) return false;
     }
     use_variant(pl.var[bv], p);
     p.W = 0;
@@ -843,11 +847,11 @@ bool bi_block_accepts(const BiCall &c) {
   return choose_route(c, L);
 }
 
-int bi_launch_block(const BiCall &c, bi_model *mut) {
+int bi_launch_block(const BiCall &c, bi_model *mut, bool estimate) {
   const bi_model *md = c.model;
   const bool window = c.algo != BI_ALGO_FILTER;
   Route L;
-  if (!choose_route(c, L)) return BI_ERR_UNSUPPORTED;
+  if (!choose_route(c, L, estimate)) return BI_ERR_UNSUPPORTED;
   const Plan &pl = *L.plan;
   Params &p = L.p;
   const int esz = md->arith == BI_ARITH_F64 ? 8 : 4;
