@@ -990,6 +990,7 @@ int bi_dispatch(const BiCall &c, bi_model *mut) {
     if (any || only == BI_FAMILY_BLOCK) rc = bi_launch_block(c, mut);
     if (rc == BI_ERR_UNSUPPORTED && (any || only == BI_FAMILY_BATCH)) rc = bi_launch_batch(c, mut);
     if (rc == BI_ERR_UNSUPPORTED && c.algo == BI_ALGO_FILTER && (any || only == BI_FAMILY_CTA)) rc = bi_launch_cta_filter(c, mut);
+    if (rc == BI_ERR_UNSUPPORTED && any) rc = bi_launch_block(c, mut, false);
     if (rc == BI_ERR_UNSUPPORTED && c.algo != BI_ALGO_FILTER && (any || only == BI_FAMILY_WARP)) rc = bi_launch_warp(c, mut);
     return rc == BI_ERR_UNSUPPORTED ? bi_launch_generic(c, mut) : rc;
   }

@@ -744,6 +744,44 @@ WindowCost window_cost(const BiCall &c, const Plan &pl, const Variant &v) {
   return w;
 }
 
+// Microseconds a step of a filtering call with several parents per transition would take here and on the CTA kernel (a
+// step, not the call: a trajectory filtered in blocks of steps has to stay on one kernel).  The prior of a step
+// is a contraction of every tensor with its parents' beliefs; a team here may be a single warp where the CTA
+// kernel has eight, and with few iterations or small slices that outweighs the faster ones.  Linear in the
+// dependent trips of a step (a team alone) and in the work of the teams that share an SM, fitted to 347
+// structures, 4 to 2 048 agents (12 and 21 % rms error in cross-validation).  [16,7,19] under three parents,
+// 4 agents, six iterations: 2.9 times slower here; [4,6,2,7] under a rank-4 slice, 654 agents: 131 us
+// here and 544 us there.
+struct FilterCost { double block, cta; };
+FilterCost filter_cost(const BiCall &c, const Plan &pl, const Variant &v) {
+  const BiDev &h = c.model->h;
+  const int NW = v.LT / 32;
+  double dots = 0, prods = 0, tensors = 0, slices = 0, rows = 0;
+  int groups = 0, deep = 0;
+  for (int f = 0; f < h.F; ++f) {
+    dots += (double)ceil_div(h.n[f], 4 * NW) * ceil_div(h.PB[f], 8);
+    prods += (double)ceil_div(h.PB[f], v.LT) * h.bdep_len[f];
+    tensors += (double)h.n[f] * h.PB[f];
+    rows += h.n[f];
+  }
+  for (int gi = 0; gi < h.ngroups; ++gi) {
+    const BiGroup &g = h.grp[gi];
+    if (g.rank < 2) continue;
+    double e = 1;
+    for (int j = 0; j < g.rank; ++j) e *= g.dim[j];
+    slices += e;
+    groups += 1;
+    if (g.rank > 2) deep = 1;
+  }
+  const double beside = std::max(0.0, (double)c.N / c.model->sm_count - 1.0);
+  const double ent = pl.NB * (double)(pl.BR * pl.BC) / 32.0 * (c.model->arith == BI_ARITH_F64 ? 1.0 : 0.5);
+  FilterCost w;
+  w.block = 2.4 + 0.68 * c.K * v.nbpt + 0.061 * dots + 0.052 * prods + 0.74 * h.F + beside * (0.0052 * c.K * ent + 9.1e-5 * tensors);
+  w.cta = 1.6 + c.K * (0.43 + 0.29 * groups + 3.4e-4 * slices + 0.66 * deep) + 1.46e-4 * tensors + 1.63 * h.F +
+          beside * (c.K * (4.4e-4 * slices + 6.1e-3 * rows + 0.095) + 6.9e-5 * tensors);
+  return w;
+}
+
 // How a call would run here.
 struct Route {
   Params p;
@@ -790,6 +828,10 @@ bool choose_route(const BiCall &c, Route &L, bool estimate = true) {
       if (t < best) { best = t; v0 = v; }
     }
     if (best >= 1e300) return false;
+    if (estimate && md->h.has_bdep && md->test_family == BI_FAMILY_ANY) {
+      const FilterCost w = filter_cost(c, pl, pl.var[v0]);
+      if (w.cta < 0.95 * w.block) return false;
+    }
     use_variant(pl.var[v0], p);
     // agents per CTA (one-warp teams): one while the batch fits the machine anyway, so that no SM gets
     // four more warps than another; four for large batches, which share the CTA's exponential table

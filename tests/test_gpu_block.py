@@ -394,3 +394,23 @@ def test_sixteen_modalities(algo):
     dep = [[0, 1, 2], [1, 2], [0, 2], [0]] * 4
     res = check_workload(_workload(170, [5, 4, 7], dep, N=6, T=5, K=4), algo)
     assert res["family"] == f"block_{algo}_f64", res
+
+
+@pytest.mark.parametrize("case, family", [("large_tensors", "cta"), ("large_slices", "block")])
+def test_filtering_with_several_parents_by_the_cost_of_a_step(case, family):
+    """The prior of large transition tensors is cheaper on the CTA kernel, the iterations of large slices on the block
+    kernels; which it is does not depend on the number of steps, so blocks of steps are the single call bit for bit."""
+    import torch
+    import paper_2607_17855_b200 as bi
+    from test_gpu_parity import _blockwise
+    n, dep, bdep, N, K = {"large_tensors": ([16, 7, 19], [[0, 1], [2]], [[2, 1, 0], [2, 1], [1, 0]], 4, 6),
+                          "large_slices": ([4, 6, 2, 7], [[0, 1, 2, 3]], [[0, 3], [1, 2, 3], [1, 2], [0, 1, 3]], 300, 16)}[case]
+    w = _workload(180, n, dep, N=N, T=7, K=K, bdep=bdep)
+    res = check_workload(w, "filter", agents=range(0, N, max(1, N // 8)))
+    assert res["family"] == f"{family}_filter_f64", res
+    md = bi.model_from_workload(w)
+    whole = md.bi_filter(torch.from_numpy(w.obs).cuda(), torch.from_numpy(w.act).cuda(), K).cpu().numpy()
+    for cuts in (list(range(8)), [0, 2, 3, 7]):
+        q, _ = _blockwise(md, w, cuts, K)
+        assert np.array_equal(q, whole), cuts
+    md.close()
