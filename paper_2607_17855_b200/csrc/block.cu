@@ -703,26 +703,25 @@ bool bi_block_serves(const bi_model *md, int algo) {
 namespace {
 
 // Microseconds a window call would take here and on the batched kernels (batch.cu), for the choice between them.
-// Linear in what each spends its time on -- here block entries, warps and finishing passes per unit, there a
-// pair of launches per iteration, the longest slice's serial walk, slice entries and states per unit -- with
-// coefficients fitted to 204 structures of one to five factors, 2 100 to 62 000 units, 6 and 16 iterations (in
-// cross-validation 13 and 17 % rms error here, 19 % there, float64 and float32).  Neither side wins by size alone:
-// [9,32,19] under two rank-2 slices, float32, 59 508 units, 4463 us here and 2407 us there;
-// [14,14,2,12] under a rank-4 slice, 2 472 units, 342 and 595 us.
+// Linear in what each spends its time on -- here the launcher's own cost of an iteration (`cycles`, waves included),
+// block entries and finishing passes per unit and the preparation of both, there launches and members per
+// iteration, slice entries and states per unit -- with coefficients fitted to 204 structures of one to five
+// factors, 2 100 to 62 000 units, 6 and 16 iterations (in cross-validation 9 and 14 % rms error here, 15 and 16 % there,
+// float64 and float32).  Neither side wins by size alone: [9,32,19] under two rank-2 slices, float32, 59 508 units,
+// 4463 us here and 2407 us there; [14,14,2,12] under a rank-4 slice, 2 472 units, 342 and 595 us.
 struct WindowCost { double block, batch; };
-WindowCost window_cost(const BiCall &c, const Plan &pl, const Variant &v) {
+WindowCost window_cost(const BiCall &c, const Plan &pl, const Variant &v, double cycles) {
   const BiDev &h = c.model->h;
   const bool f64 = c.model->arith == BI_ARITH_F64;
   const double per_sm = (double)c.N * c.T / c.model->sm_count * 1e-3, k = c.K * per_sm;   // thousands of units; unit-iterations
   const double ent = pl.NB * (double)(pl.BR * pl.BC) * 1e-3, warps = v.LT / 32.0;
-  double slices = 0, longest = 0, states = 0, lanes = 0;
+  double slices = 0, states = 0, lanes = 0;
   int members = 0, nmax = 1;
   for (int gi = 0; gi < h.ngroups; ++gi) {
     const BiGroup &g = h.grp[gi];
     if (g.rank < 2) continue;
     double e = 1;
     for (int j = 0; j < g.rank; ++j) e *= j + 1 < g.rank ? g.dim[j] : bi_pad4(g.dim[j]);
-    longest = std::max(longest, e * 1e-3);
     for (int mi = g.mem_begin; mi < g.mem_end; ++mi)
       if (g.dim[g.rank - 1] > 32 || h.mem[mi].m > 4096) return {0.0, 1.0};   // (nothing the batched kernels take)
     slices += e * 1e-3 * (g.mem_end - g.mem_begin);
@@ -735,12 +734,11 @@ WindowCost window_cost(const BiCall &c, const Plan &pl, const Variant &v) {
   const bool lane_per_unit = nmax <= 16 && (double)c.N * c.T * std::min(1.0, h.F / 3.0) >= 64.0 * c.model->sm_count;   // (the update's form, see batch.cu)
   if (!lane_per_unit) lanes = (double)h.F * (nmax <= 8 ? 8 : nmax <= 16 ? 16 : 32) * nmax;
   WindowCost w;
-  const double mmp = c.algo == BI_ALGO_MMP;   // (two logarithms per state)
-  w.block = f64 ? 19 + k * (81 * ent + (80 + 39 * v.nbpt) * warps + 3 * mmp * v.npass) + 675 * per_sm * ent
-                : 9 + 0.2 * c.K + k * (88 * ent + 4.7 * v.nbpt * warps + (73 + 9.4 * mmp) * v.npass) + per_sm * (117 * ent + 358 * warps);
-  const double launches = members ? 2 : 1;
-  w.batch = f64 ? 21 + c.K * (8.1 * launches + 3.6 * longest) + k * (86 * slices + states * (1.28 * members + 0.33 + 0.62 * mmp) + 0.103 * lanes) + 16 * per_sm * members
-                : c.K * (6.6 * launches + 4.4 * longest) + k * (38 * slices + states * (0.81 * members + 0.38 + 0.38 * mmp) + 0.093 * lanes) + 13 * per_sm * members;
+  const double mmp = c.algo == BI_ALGO_MMP, launches = members ? 2 : 1;   // (MMP: two logarithms per state)
+  w.block = f64 ? 12 + 2.06 * c.K * cycles / 1965 + k * (42 * ent + 5.8 * v.nbpt * warps + 6.3 * mmp * v.npass) + per_sm * (648 * ent + 97 * warps)
+                : 7 + 1.77 * c.K * cycles / 1965 + k * (29 * ent + (14 + 6.8 * mmp) * v.npass) + per_sm * (245 * ent + 386 * warps);
+  w.batch = f64 ? 19 + c.K * (3.1 * launches + 3.9 * members + 4.1 * slices) + k * (78 * slices + states * (0.29 * members + 2.85 + mmp) + 0.095 * lanes)
+                : 5 + c.K * (4.8 * launches + 2.2 * members + 3.7 * slices) + k * (29 * slices + states * (0.23 * members + 1.28 + 0.45 * mmp) + 0.092 * lanes);
   return w;
 }
 
@@ -804,7 +802,25 @@ bool choose_route(const BiCall &c, Route &L, bool estimate = true) {
   const Plan &pl = *plp;
   L.plan = plp;
   if (pl.NB == 0) return false;   // nothing to contract: the CTA kernel's warp per factor does that
-  if (window && !md->h.has_bdep && md->batch_unrolled && (long long)c.N * c.T >= 4096) return false;   // (see batch_unrolled)
+  if (window && !md->h.has_bdep && estimate) {
+    const long long units = (long long)c.N * c.T;
+    const bool shared = md->h.G == 1 && !md->soft_shadow;
+    if (shared && md->batch_unrolled && units >= 4096) return false;   // (see batch_unrolled)
+    // Models of the agents' own and observation vectors have a slice per unit, which the batched kernels contract in
+    // their any-shape form: slower at nearly every size ([10,10,8,6], three groups, 20 480 units: 1246 us here, 1890 us
+    // there).  What crosses are large float32 calls without a group over three factors.  With observation
+    // vectors, whose softmax is relative to the largest logit: pairs of some size, and no pair at all ([10,10] and
+    // [10,8], 4 160 units 182 and 377 us, 20 000 units 821 and 653 us; single factors 91 and 138, 303 and 259 us; but slices
+    // of 56 entries in all, 20 000 units, 297 and 349 us).  With models of the agents' own: the pairs
+    // first named alone (659 and 625 us; [20,25] and [25,4] 975 and 1323 us).
+    if (!shared && md->arith == BI_ARITH_F32 && md->rank2_ok && units >= 16000) {
+      double entries = 0;
+      for (int gi = 0; gi < md->h.ngroups; ++gi)
+        if (md->h.grp[gi].rank >= 2) entries += (double)md->h.grp[gi].P_pad * (md->h.grp[gi].mem_end - md->h.grp[gi].mem_begin);
+      const bool crosses = md->soft_shadow ? entries == 0 || entries >= 128 : entries > 0 && md->batch_unrolled;
+      if (crosses && entries * 4.0 * (double)units <= 120e6) return false;   // (the batched kernels take no more)
+    }
+  }
   const int esz = md->arith == BI_ARITH_F64 ? 8 : 4;
   const size_t budget = (size_t)md->max_smem_optin - 1024;
   Params &p = L.p;
@@ -869,8 +885,8 @@ bool choose_route(const BiCall &c, Route &L, bool estimate = true) {
     }
     if (bv < 0) return false;
     if (estimate && !md->h.has_bdep && md->h.G == 1 && (long long)c.N * c.T >= 2048 && md->test_family == BI_FAMILY_ANY && !md->soft_shadow) {
-      const WindowCost w = window_cost(c, pl, pl.var[bv]);
-      if (w.batch < w.block) return false;
+      const WindowCost w = window_cost(c, pl, pl.var[bv], best);
+      if (w.batch < 0.95 * w.block) return false;
     }
     use_variant(pl.var[bv], p);
     p.W = 0;

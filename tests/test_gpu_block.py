@@ -414,3 +414,15 @@ def test_filtering_with_several_parents_by_the_cost_of_a_step(case, family):
         q, _ = _blockwise(md, w, cuts, K)
         assert np.array_equal(q, whole), cuts
     md.close()
+
+
+@pytest.mark.parametrize("case, family", [("pairs_float32_many", "batch"), ("tiny_float32_many", "batch"),
+                                          ("rank4_few", "block"), ("own_models_many", "block")])
+def test_windows_by_the_estimate_of_both(case, family):
+    n, dep, N, T, G, arith = {"pairs_float32_many": ([9, 32, 19], [[0, 2], [2]], 2975, 20, 1, "f32"),
+                              "tiny_float32_many": ([5, 5, 2, 2, 4], [[3], [0, 1, 2], [0, 2, 3], [1, 2, 4], [0, 2, 3]], 2746, 20, 1, "f32"),
+                              "rank4_few": ([14, 14, 2, 12], [[0, 1, 2, 3]], 206, 12, 1, "f64"),
+                              "own_models_many": ([10, 10, 8, 6], [[0, 1], [1, 2], [0, 2, 3]], 260, 16, 260, "f64")}[case]
+    res = check_workload(_workload(190, n, dep, N=N, T=T, K=6 if arith == "f32" else 16, G=G), "mmp", agents=range(0, N, N // 10), arith=arith, strict=arith == "f64")
+    assert res["family"] == f"{family}_mmp_{arith}", res
+    assert res["q_max_err"] < 1e-2, res   # (float32: six undamped iterations amplify 1e-6 of the logits by 1e3 at most)
