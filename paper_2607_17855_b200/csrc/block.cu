@@ -704,10 +704,11 @@ namespace {
 
 // Microseconds a window call would take here and on the batched kernels (batch.cu), for the choice between them.
 // Linear in what each spends its time on -- here the launcher's own cost of an iteration (`cycles`, waves included),
-// block entries and finishing passes per unit and the preparation of both, there launches and members per
-// iteration, slice entries and states per unit -- with coefficients fitted to 204 structures of one to five
-// factors, 2 100 to 62 000 units, 6 and 16 iterations (in cross-validation 9 and 14 % rms error here, 15 and 16 % there,
-// float64 and float32).  Neither side wins by size alone: [9,32,19] under two rank-2 slices, float32, 59 508 units,
+// block entries and finishing passes per unit and the preparation of both, there launches, members and slices
+// per iteration, slice entries and states per unit -- with coefficients fitted to 960 calls on structures of one to
+// five factors, 2 100 to 62 000 units, 6 and 16 iterations (9 and 14 % rms error here, 14 and 15 % there, float64 and
+// float32).  On those the choice costs 1.2 % over the faster of the two; 49 calls take over 5 % more, 2.4 times at
+// most.  Neither side wins by size alone: [9,32,19] under two rank-2 slices, float32, 59 508 units,
 // 4463 us here and 2407 us there; [14,14,2,12] under a rank-4 slice, 2 472 units, 342 and 595 us.
 struct WindowCost { double block, batch; };
 WindowCost window_cost(const BiCall &c, const Plan &pl, const Variant &v, double cycles) {
@@ -715,13 +716,14 @@ WindowCost window_cost(const BiCall &c, const Plan &pl, const Variant &v, double
   const bool f64 = c.model->arith == BI_ARITH_F64;
   const double per_sm = (double)c.N * c.T / c.model->sm_count * 1e-3, k = c.K * per_sm;   // thousands of units; unit-iterations
   const double ent = pl.NB * (double)(pl.BR * pl.BC) * 1e-3, warps = v.LT / 32.0;
-  double slices = 0, states = 0, lanes = 0;
+  double slices = 0, longest = 0, states = 0;   // (thousands of entries)
   int members = 0, nmax = 1;
   for (int gi = 0; gi < h.ngroups; ++gi) {
     const BiGroup &g = h.grp[gi];
     if (g.rank < 2) continue;
     double e = 1;
     for (int j = 0; j < g.rank; ++j) e *= j + 1 < g.rank ? g.dim[j] : bi_pad4(g.dim[j]);
+    longest = std::max(longest, e * 1e-3);
     for (int mi = g.mem_begin; mi < g.mem_end; ++mi)
       if (g.dim[g.rank - 1] > 32 || h.mem[mi].m > 4096) return {0.0, 1.0};   // (nothing the batched kernels take)
     slices += e * 1e-3 * (g.mem_end - g.mem_begin);
@@ -732,13 +734,12 @@ WindowCost window_cost(const BiCall &c, const Plan &pl, const Variant &v, double
     states += h.npad[f];
   }
   const bool lane_per_unit = nmax <= 16 && (double)c.N * c.T * std::min(1.0, h.F / 3.0) >= 64.0 * c.model->sm_count;   // (the update's form, see batch.cu)
-  if (!lane_per_unit) lanes = (double)h.F * (nmax <= 8 ? 8 : nmax <= 16 ? 16 : 32) * nmax;
-  WindowCost w;
   const double mmp = c.algo == BI_ALGO_MMP, launches = members ? 2 : 1;   // (MMP: two logarithms per state)
-  w.block = f64 ? 12 + 2.06 * c.K * cycles / 1965 + k * (42 * ent + 5.8 * v.nbpt * warps + 6.3 * mmp * v.npass) + per_sm * (648 * ent + 97 * warps)
-                : 7 + 1.77 * c.K * cycles / 1965 + k * (29 * ent + (14 + 6.8 * mmp) * v.npass) + per_sm * (245 * ent + 386 * warps);
-  w.batch = f64 ? 19 + c.K * (3.1 * launches + 3.9 * members + 4.1 * slices) + k * (78 * slices + states * (0.29 * members + 2.85 + mmp) + 0.095 * lanes)
-                : 5 + c.K * (4.8 * launches + 2.2 * members + 3.7 * slices) + k * (29 * slices + states * (0.23 * members + 1.28 + 0.45 * mmp) + 0.092 * lanes);
+  WindowCost w;
+  w.block = f64 ? 10 + 2.11 * c.K * cycles / 1965 + k * (36 * ent + 1.9 * v.nbpt * warps + 15 * mmp * v.npass) + per_sm * (637 * ent + 142 * warps)
+                : 6 + 1.93 * c.K * cycles / 1965 + k * (16 * ent + (15.6 + 9.4 * mmp) * v.npass) + per_sm * (333 * ent + 282 * warps);
+  w.batch = f64 ? 7 + c.K * (5.3 * launches + 2.3 * members + 1.2 * longest) + k * (101 * slices + states * (0.56 * members + (lane_per_unit ? 1.9 : 6.6) + 1.2 * mmp))
+                : 10 + c.K * (3.4 * launches + 2.3 * members + 2.3 * slices) + k * (36 * slices + states * (0.26 * members + (lane_per_unit ? 1.3 : 5.9) + 0.63 * mmp));
   return w;
 }
 
@@ -886,7 +887,7 @@ bool choose_route(const BiCall &c, Route &L, bool estimate = true) {
     if (bv < 0) return false;
     if (estimate && !md->h.has_bdep && md->h.G == 1 && (long long)c.N * c.T >= 2048 && md->test_family == BI_FAMILY_ANY && !md->soft_shadow) {
       const WindowCost w = window_cost(c, pl, pl.var[bv], best);
-      if (w.batch < 0.95 * w.block) return false;
+      if (w.batch < w.block) return false;
     }
     use_variant(pl.var[bv], p);
     p.W = 0;
