@@ -716,7 +716,7 @@ WindowCost window_cost(const BiCall &c, const Plan &pl, const Variant &v, double
   const bool f64 = c.model->arith == BI_ARITH_F64;
   const double per_sm = (double)c.N * c.T / c.model->sm_count * 1e-3, k = c.K * per_sm;   // thousands of units; unit-iterations
   const double ent = pl.NB * (double)(pl.BR * pl.BC) * 1e-3, warps = v.LT / 32.0;
-  double slices = 0, longest = 0, states = 0;   // (thousands of entries)
+  double slices = 0, longest = 0, states = 0;   // (slices in thousands of entries)
   int members = 0, nmax = 1;
   for (int gi = 0; gi < h.ngroups; ++gi) {
     const BiGroup &g = h.grp[gi];
