@@ -17,7 +17,7 @@
 // shapes in BI_BATCH_SHAPES (every accumulator in registers), and a form for any
 // shape of rank 2..5 that is compiled only for the padded size of the last axis
 // (its accumulators in registers, those of the outer axes in per-thread columns
-// of shared memory, the outer loops an odometer shared by the whole CTA).
+// of shared memory; a plain loop along the innermost outer axis, one climb of the others per run of rows).
 #include <algorithm>
 #include <climits>
 #include <cstring>

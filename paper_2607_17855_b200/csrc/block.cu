@@ -692,6 +692,7 @@ void fill_params(const BiCall &c, const Plan &pl, Params &p) {
 // (measured: one in five such trajectories differs in the first digit from the CTA kernel's).  Those calls stay
 // with the kernels that have served them, bit for bit.  The number of steps has no say in it: a trajectory
 // filtered in blocks of steps is the single call's (bi_filter_continue), and a stream of ticks is a trajectory too.
+// (It costs such ticks: 26 agents on [5,12,12,3], 68 us there and 24 us here.)
 // Float32 filtering of models coupled in one pair of factors stays as well: several sharp modalities on one pair
 // carry float32 roundings to 2e-3 in a belief over thirty steps, and these kernels gain only 1.1 to 1.2 there.
 bool bi_block_serves(const bi_model *md, int algo) {

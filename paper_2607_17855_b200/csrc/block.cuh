@@ -22,7 +22,7 @@
 // of single warps.  Here an iteration's shared-memory traffic is (BR + BC + 2) / (BR BC) of the slice
 // instead of all of it, and all offsets are loop invariants in registers.  Bound: the latency of the two
 // phases' dependent chains where few teams share an SM, issue and shared-memory throughput where many do.  Five
-// coupled factors filtered by 256 agents: 2116 -> 418 us; 1000 agents in float32: 1201 -> 433 us.
+// coupled factors filtered by 256 agents: 2116 -> 414 us; 1000 agents in float32: 1201 -> 435 us.
 #pragma once
 #include "bi_internal.h"
 #include "block.h"
