@@ -426,3 +426,19 @@ def test_windows_by_the_estimate_of_both(case, family):
     res = check_workload(_workload(190, n, dep, N=N, T=T, K=6 if arith == "f32" else 16, G=G), "mmp", agents=range(0, N, N // 10), arith=arith, strict=arith == "f64")
     assert res["family"] == f"{family}_mmp_{arith}", res
     assert res["q_max_err"] < 1e-2, res   # (float32: six undamped iterations amplify 1e-6 of the logits by 1e3 at most)
+
+
+@pytest.mark.parametrize("algo", ["filter", "vmp", "mmp"])
+def test_float32_damped(algo):
+    """The fast mode as it is used.  Logits are sums of some ten logarithms and messages, at most 60 in size: 60 x 6e-8 x 10
+    roundings, 4e-5, and the damped iteration does not amplify; the bound is twice that."""
+    import oracle
+    import torch
+    import paper_2607_17855_b200 as bi
+    w = _workload(200, [9, 5, 7, 6], [[0, 1, 2], [1, 3]], N=21, T=5, K=12)
+    md = bi.model_from_workload(w, arith="f32")
+    md.set_damping(0.5)
+    q = md.run(algo, torch.from_numpy(w.obs).cuda(), torch.from_numpy(w.act).cuda(), w.K).cpu().numpy()
+    assert md.last_family == f"block_{algo}_f32"
+    md.close()
+    assert np.abs(q - oracle.run_workload(w, algo, damping=0.5)[0]).max() <= 8e-5
