@@ -442,3 +442,31 @@ def test_float32_damped(algo):
     assert md.last_family == f"block_{algo}_f32"
     md.close()
     assert np.abs(q - oracle.run_workload(w, algo, damping=0.5)[0]).max() <= 8e-5
+
+
+def test_long_trajectories_in_blocks_of_steps_on_the_cta_kernel():
+    """The CTA filtering kernel keeps a trajectory's first observations in shared memory; a trajectory too long for that
+    stays on it all the same, and equals its blocks bit for bit."""
+    import torch
+    import paper_2607_17855_b200 as bi
+    from test_gpu_parity import _blockwise
+    n, dep, T = [5, 4, 3], [[0, 1, 2]] + [[i % 3] for i in range(9)], 3000
+    rng = np.random.default_rng(210)
+    m, U = [9] + [3] * 9, [2, 1, 3]
+    A, B, D = make_model(rng, n, m, dep, U, 1, sparsity=0.6, d_alpha=1.0)
+    obs, act = sample_streams(rng, n, m, dep, U, 1, A, B, D, 3, T)
+    w = Workload(name="long", algo="filter", n=np.asarray(n, np.int32), m=np.asarray(m, np.int32), dep=dep,
+                 U=np.asarray(U, np.int32), G=1, A=A, B=B, D=D, N=3, T=T, K=16, obs=obs, act=act)
+    md = bi.model_from_workload(w)
+    whole = md.bi_filter(torch.from_numpy(obs).cuda(), torch.from_numpy(act).cuda(), w.K).cpu().numpy()
+    assert md.last_family == "cta_filter_f64"
+    for cuts in ([0, 1500, T], [0, 7, 900, T]):
+        q, names = _blockwise(md, w, cuts, w.K)
+        assert names == {"cta_filter_f64"} and np.array_equal(q, whole), cuts
+    bad = obs.copy()
+    bad[1, T - 1, 4] = 77   # (beyond the kept ones: clamped and flagged)
+    q = md.bi_filter(torch.from_numpy(bad).cuda(), torch.from_numpy(act).cuda(), w.K).cpu().numpy()
+    assert md.status() == 1 and np.array_equal(q[:, :T - 1], whole[:, :T - 1])
+    bad[1, T - 1, 4] = 2
+    assert np.array_equal(q, md.bi_filter(torch.from_numpy(bad).cuda(), torch.from_numpy(act).cuda(), w.K).cpu().numpy())
+    md.close()
