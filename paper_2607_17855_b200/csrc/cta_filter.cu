@@ -40,7 +40,7 @@ namespace {
 
 struct CtaGeom {   // element offsets (units of R) into dynamic shared memory
   int desc, q0, q1, lpri, xp, ellg, part, obs;
-  int obs_n;                 // observations kept in shared memory: the trajectory's first ones
+  int obs_T;                 // steps whose observations are in shared memory at a time
   int Lst[BI_MAX_GROUPS];    // per group: its staged slice, rows `lstride` apart
   int lstride[BI_MAX_GROUPS];
   int V[BI_MAX_GROUPS][2];   // per group: the two buffers its levels alternate between
@@ -278,11 +278,8 @@ bi_cta_filter_kernel(const BiDev *__restrict__ mdp, int T, const int32_t *__rest
   int32_t *obs_s = reinterpret_cast<int32_t *>(smem + sm.obs);
   const R lam = (R)lambda;
 
-  obs += (size_t)a * T * M;
-  for (int i = tid; i < T * M; i += NT) {
-    const int o = clamp_flag(__ldg(obs + i), md.m[i % M], md.status, BI_FLAG_OBS_RANGE);
-    if (i < sm.obs_n) obs_s[i] = o;
-  }
+  for (int i = tid; i < min(T, sm.obs_T) * M; i += NT)
+    obs_s[i] = clamp_flag(__ldg(obs + (size_t)a * T * M + i), md.m[i % M], md.status, BI_FLAG_OBS_RANGE);
   for (int i = tid; i < 2 * Sp; i += NT) cur[i] = (R)0;   // q0 and q1 are adjacent
   for (int i = tid; i < NG * Sp; i += NT) ellg[i] = (R)0;  // entries of factors outside a group stay zero
   for (int i = sm.vtot_begin + tid; i < sm.vtot_end; i += NT) smem[i] = (R)0;
@@ -337,7 +334,16 @@ bi_cta_filter_kernel(const BiDev *__restrict__ mdp, int T, const int32_t *__rest
     __syncthreads();
   }
 
+  int refill = sm.obs_T;
   for (int t = 0; t < T; ++t) {
+    if (t == refill) {   // (long trajectories) the next steps' observations
+      refill += sm.obs_T;
+      obs_s -= sm.obs_T * M;
+      __syncthreads();
+      for (int i = t * M + tid; i < min(T, t + sm.obs_T) * M; i += NT)
+        obs_s[i] = clamp_flag(__ldg(obs + (size_t)a * T * M + i), md.m[i % M], md.status, BI_FLAG_OBS_RANGE);
+      __syncthreads();
+    }
     // ln prior: D at the first step, else B_u q_{t-1} (cur still holds step t-1)
     if (md.has_bdep && (t > 0 || from_prev)) {
       // The expectation of the transition tensor under the parents' beliefs.  The parents' outer product
@@ -431,9 +437,7 @@ bi_cta_filter_kernel(const BiDev *__restrict__ mdp, int T, const int32_t *__rest
       const R *src[BI_MAX_M];
       for (int mi = 0; mi < nm; ++mi) {
         const BiMember &mm = md.mem[gr.mem_begin + mi];
-        const int at = t * M + mm.modality;   // (those beyond the kept ones were flagged above)
-        const int o = at < sm.obs_n ? obs_s[at] : min(max(__ldg(obs + at), 0), mm.m - 1);
-        src[mi] = (const R *)mm.logA + (size_t)g * mm.gstride + (size_t)o * mm.P_pad;
+        src[mi] = (const R *)mm.logA + (size_t)g * mm.gstride + (size_t)obs_s[t * M + mm.modality] * mm.P_pad;
       }
       const int npad4 = gr.rank > 1 ? gr.lev[0].last_npad4 : bi_pad4(gr.first_n) / 4;
       R *dst = smem + sm.Lst[gi];
@@ -701,14 +705,15 @@ int launch_cta_filter_t(const BiCall &c, bi_model *mut) {
     sm.wpar_cap = std::min(bi_pad4(sm.wpar_cap), 4096);
     o += sm.wpar_cap;
   }
-  // The observations take what is left, 32 KB at most: whether the model fits does not depend on the number of steps
+  // The observations take what is left, those of as many steps as 32 KB hold: whether the model fits does not depend on the number of steps
   // (a trajectory filtered in blocks of steps has to stay on one kernel).
   const size_t budget = (size_t)md->max_smem_optin - 1024, used = (size_t)o * sizeof(R);
   if (used > budget) return BI_ERR_UNSUPPORTED;
   sm.obs = o;
-  sm.obs_n = (int)std::min({(long long)c.T * h.M, (long long)(32 * 1024 / sizeof(int32_t)), (long long)((budget - used) / sizeof(int32_t))});
-  sm.total_bytes = (int)(used + (((size_t)sm.obs_n * sizeof(int32_t) + 15) & ~(size_t)15));
-  if ((size_t)sm.total_bytes > budget) { sm.total_bytes = (int)used; sm.obs_n = 0; }
+  const size_t step = (size_t)std::max(h.M, 1) * sizeof(int32_t), room = std::min<size_t>(budget - used, 32 * 1024);
+  if (room < step + 16) return BI_ERR_UNSUPPORTED;
+  sm.obs_T = (int)std::min<size_t>((size_t)c.T, (room - 16) / step);
+  sm.total_bytes = (int)(used + ((sm.obs_T * step + 15) & ~(size_t)15));
 
   auto kern = bi_cta_filter_kernel<R>;
   if (bi_allow_smem((const void *)kern, sm.total_bytes) != cudaSuccess)
