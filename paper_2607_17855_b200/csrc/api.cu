@@ -1000,6 +1000,7 @@ int bi_dispatch(const BiCall &c, bi_model *mut) {
     rc = bi_launch_tile3(c, mut);
     if (rc == BI_ERR_UNSUPPORTED) rc = bi_launch_tile3_window(c, mut);
     if (rc == BI_ERR_UNSUPPORTED) rc = bi_launch_pair_filter(c, mut);
+    if (rc == BI_ERR_UNSUPPORTED && bi_batch_before_pair(c)) rc = bi_launch_batch(c, mut);
     if (rc == BI_ERR_UNSUPPORTED) rc = bi_launch_pair_window(c, mut);
     if (rc == BI_ERR_UNSUPPORTED && c.model->test_drop_copy == 0) rc = bi_launch_block(c, mut);
     if (rc == BI_ERR_UNSUPPORTED) rc = bi_launch_batch(c, mut);

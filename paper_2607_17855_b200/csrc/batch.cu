@@ -13,7 +13,8 @@
 // slice.  A second kernel per iteration adds the transition messages and takes
 // the softmax per unit (Jacobi over steps and factors, Appendix A-2).
 //
-// The contraction has two forms: fully unrolled code for the dependency-group
+// Float64 calls on shared models run on the matrix instruction (batch_mma.cu); the contractions here serve float32,
+// slices per unit, and groups over five factors.  They have two forms: fully unrolled float32 code for the dependency-group
 // shapes in BI_BATCH_SHAPES (every accumulator in registers), and a form for any
 // shape of rank 2..5 that is compiled only for the padded size of the last axis
 // (its accumulators in registers, those of the outer axes in per-thread columns
@@ -26,18 +27,10 @@
 
 #include <cooperative_groups.h>
 
-#include "bi_internal.h"
+#include "batch.h"
 #include "tile3.cuh"
 
 namespace {
-
-// Programmatic dependent launch: the iteration loop queues its kernels so that the next one may be
-// scheduled while the previous one drains.  A kernel first does what needs none of its
-// predecessor's results (its task, the slice copy, index loads), then waits for the predecessor to
-// complete (bi_grid_wait; a no-op when launched without the attribute) and only then lets its own
-// successor be scheduled: when a kernel starts, everything before its predecessor is complete.
-__device__ __forceinline__ void bi_grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void bi_grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
 
 constexpr int kTU = 128;   // most units per contraction CTA (the call picks 32, 64 or 128)
 
@@ -49,41 +42,6 @@ constexpr int kTU = 128;   // most units per contraction CTA (the call picks 32,
   X(3, 2, 10, 10, 0, 0)    \
   X(4, 3, 3, 2, 4, 0)      \
   X(5, 2, 5, 3, 0, 0)
-
-struct BatchMember {
-  const void *logA;        // packed [m][P_pad]
-  int32_t m, P_pad, modality, shape, rank;
-  int32_t offp[BI_MAX_RANK];   // padded belief offsets of the group's axes, packed order
-  int32_t dim[BI_MAX_RANK];    // axis sizes, packed order (last one unpadded)
-  int32_t ooff[BI_MAX_RANK];   // start of each outer axis in the per-thread shared-memory columns
-  int32_t ncp, rows;       // padded last axis; rows = product of the outer axes
-  int64_t gstride;         // elements per agent's model (per-agent models), 0 when shared
-  int32_t task0;           // first task slot of this member
-  int32_t split;           // unrolled forms: threads per unit (1, 2 or 4), each taking a range of the first axis
-  // Where the messages of each axis go, relative to the unit's row of this member's plane.  (A transition
-  // tensor of a model with several parents per transition is a member too: its first axis is the child's state at
-  // the next step -- the next unit's beliefs, and messages to the next unit's row of a plane of their own.)
-  int32_t edge;            // 0, or 1 + the factor whose transition this is: its "outcome" is the action
-  int64_t oout[BI_MAX_RANK];
-};
-
-struct BatchParams {
-  BatchMember mem[BI_MAX_M + BI_MAX_F];
-  int32_t nmem;            // members of rank >= 2
-  int32_t task_base;       // first task of this launch
-  int32_t NU, Sp, ntask, tu;   // tu: units per contraction CTA
-  int32_t sc_off;          // unrolled forms: element offset of the split tasks' scratch columns behind the slice
-  int32_t lbuf, so_max;    // any-shape form: elements of the slice staging buffer; most outer states of a member
-  const int32_t *perm;     // [nmem][NU] unit ids ordered by observed outcome
-  const int4 *task;        // [ntask] (outcome, first position, count, unused)
-  void *ellp;              // [nmem][NU][Sp] partial likelihood messages
-  void *qbuf;              // [2][NU][Sp] beliefs
-  uint32_t *status;        // the handle's status word
-  const int32_t *obs;      // [NU][M] (per-agent models: every unit reads its own slice)
-  const int32_t *act;      // [N][T-1][F] (transition members)
-  int32_t M, T, F;
-  int32_t drop_copy;       // testing aid: the contraction announces its slice copy and does not issue it
-};
 
 // ---- one unit against one slice: every message of the group in one pass ----
 // L: the slice in shared memory, rows of NCP; q / out: this unit's beliefs and
@@ -232,8 +190,8 @@ __device__ __forceinline__ void contract_shape(const R *L, const R *q, R *out, c
 }
 
 // ---- bucket the units of one modality by observed outcome (once per call) ----
-// A cluster of kBucketCtas CTAs per member, each with a share of the units.  Writes perm[mi][*] (unit ids grouped by
-// outcome) and the member's task slots: chunks of at most kTU units of one outcome.  A chain of latencies -- load,
+// A cluster of kBucketCtas CTAs per member, each with a share of the units.  Writes the member's part of perm (unit ids
+// grouped by outcome) and its task slots: chunks of at most tu units of one outcome.  A chain of latencies -- load,
 // counter, load again, counter, store, for every 1024 units -- so the units are spread over a cluster and the
 // counts exchanged through distributed shared memory; with one CTA per member 20 480 units took 30 us.  (One atomic for
 // all of a warp's units of an outcome instead of one each: 42 us, the match instruction costs more.)  It runs beside
@@ -278,33 +236,33 @@ bi_batch_bucket_kernel(BatchParams P, const int32_t *__restrict__ obs, int M, ui
     total[o] = all;
   }
   cl.sync();   // (everybody's counts are read; this also orders the block)
-  const int tu = P.tu / mm.split, slot_end = mm.task0 + (NU + tu - 1) / tu + m;
+  // a member's buckets take whole tasks of tu units, one after the other: the units of a task are found without reading it
+  const int tu = mm.tu, slot_end = mm.task0 + (NU + tu - 1) / tu + m;
   if (tid == 0) {
-    int pos = 0, slot = mm.task0;
+    int slot = mm.task0;
     for (int o = 0; o < m; ++o) {
-      cursor[o] += pos;
       first[o] = slot;
-      pos += total[o];
       slot += (total[o] + tu - 1) / tu;
     }
     count[0] = slot;   // (the first unused slot)
   }
   __syncthreads();
-  if (rank == 0) {   // (cursor[o] is the bucket's start here: no earlier share)
+  if (rank == 0) {
     for (int o = tid >> 5; o < m; o += nt >> 5) {
-      const int n = total[o], pos = cursor[o];
-      for (int k = tid & 31; k * tu < n; k += 32) task[first[o] + k] = make_int4(o, pos + k * tu, min(tu, n - k * tu), 0);
+      const int n = total[o];
+      for (int k = tid & 31; k * tu < n; k += 32)
+        task[first[o] + k] = make_int4(o, mm.perm0 + (first[o] + k - mm.task0) * tu, min(tu, n - k * tu), mi);
     }
     for (int slot = count[0] + tid; slot < slot_end; slot += nt) task[slot] = make_int4(0, 0, 0, 0);
     __syncthreads();
   }
-  int32_t *pm = perm + (size_t)mi * NU;
+  int32_t *pm = perm + mm.perm0;
 #pragma unroll 4
   for (int u = ua + tid; u < ub; u += nt) {
     int o = outcome(u);
     if (mm.edge && o == INT_MIN) continue;
     o = o < 0 ? 0 : (o >= m ? m - 1 : o);
-    pm[atomicAdd(&cursor[o], 1)] = u;
+    pm[(first[o] - mm.task0) * tu + atomicAdd(&cursor[o], 1)] = u;
   }
   bi_grid_wait();   // (the starting beliefs: whoever waits for this kernel finds both)
 }
@@ -312,11 +270,11 @@ bi_batch_bucket_kernel(BatchParams P, const int32_t *__restrict__ obs, int M, ui
 // Per-agent models: no two units share a slice, so the "buckets" are just runs of consecutive units.
 __global__ void bi_batch_identity_tasks_kernel(BatchParams P, int32_t *perm, int4 *task) {
   const int mi = blockIdx.y, NU = P.NU, tu = P.tu;
-  const int nchunk = (NU + tu - 1) / tu;
+  const int nchunk = (NU + tu - 1) / tu, p0 = P.mem[mi].perm0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < NU; i += gridDim.x * blockDim.x)
-    perm[(size_t)mi * NU + i] = i;
+    perm[p0 + i] = i;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nchunk + P.mem[mi].m; k += gridDim.x * blockDim.x)
-    task[P.mem[mi].task0 + k] = k < nchunk ? make_int4(0, k * tu, min(tu, NU - k * tu), 0) : make_int4(0, 0, 0, 0);
+    task[P.mem[mi].task0 + k] = k < nchunk ? make_int4(0, p0 + k * tu, min(tu, NU - k * tu), 0) : make_int4(0, 0, 0, 0);
 }
 
 // ---- contraction: one task = one slice, up to kTU units, one thread per unit ----
@@ -351,7 +309,7 @@ bi_batch_contract_kernel(BatchParams P, int cur, int first) {
   const int upt = (int)blockDim.x / mm.split;   // units per task of this member
   const int ut = (int)threadIdx.x % upt, part = (int)threadIdx.x / upt;
   const bool has_unit = ut < tk.z;
-  const int unit = has_unit ? P.perm[(size_t)mi * P.NU + tk.y + ut] : 0;
+  const int unit = has_unit ? P.perm[tk.y + ut] : 0;
   const R *q = (const R *)P.qbuf + ((size_t)cur * P.NU + unit) * P.Sp;
   R *out = (R *)P.ellp + ((size_t)mi * P.NU + unit) * P.Sp;
   if (!first) {   // beliefs of the previous update, and the right to overwrite the messages it read
@@ -417,7 +375,7 @@ __device__ __forceinline__ void contract_rt(const BatchMember &mm, const R *__re
   const int tid = threadIdx.x, nt = blockDim.x, tu = P.tu, rs = nt / tu, nts = nt + 1, tus = tu + 1;
   const int u = tid % tu, r = tid / tu;
   const bool has_unit = u < tk.z;
-  const int unit = has_unit ? P.perm[(size_t)mi * P.NU + tk.y + u] : 0;
+  const int unit = has_unit ? P.perm[tk.y + u] : 0;
   if (r == 0) unit_s[u] = unit;
   const R *qbase = (const R *)P.qbuf + (size_t)cur * P.NU * P.Sp;
   const int K1 = mm.rank - 1, NC = mm.dim[K1];
@@ -1051,6 +1009,27 @@ __global__ void bi_batch_init_kernel(const BiDev *__restrict__ mdp, R *q, int NU
   }
 }
 
+template <typename R>
+int batch_start(const bi_model *md, const BatchParams &P, int max_m, const float *q_init, int32_t *perm, int4 *task,
+                cudaStream_t stream) {
+  bi_batch_init_kernel<R><<<256, 256, 0, stream>>>(md->d, (R *)P.qbuf, P.NU, q_init);
+  if (P.nmem == 0) return BI_OK;
+  cudaLaunchAttribute early[1];
+  early[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(P.nmem * kBucketCtas));
+  cfg.blockDim = dim3(1024);
+  cfg.dynamicSmemBytes = 4 * max_m * sizeof(int32_t);
+  if (cfg.dynamicSmemBytes > 48 * 1024 &&
+      bi_allow_smem((const void *)bi_batch_bucket_kernel, cfg.dynamicSmemBytes) != cudaSuccess)
+    return BI_ERR_CUDA;
+  cfg.stream = stream;
+  cfg.attrs = early;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, bi_batch_bucket_kernel, P, P.obs, (int)P.M, P.status, perm, task) == cudaSuccess ? BI_OK : BI_ERR_CUDA;
+}
+
 int shape_of(const BiGroup &g) {
   const int d[4] = {g.rank > 0 ? g.dim[0] : 0, g.rank > 1 ? g.dim[1] : 0, g.rank > 2 ? g.dim[2] : 0,
                     g.rank > 3 ? g.dim[3] : 0};
@@ -1080,7 +1059,8 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
   int order[BI_MAX_M], cnt = 0;
   const bool per_unit = h.G != 1;   // per-agent models: every unit contracts its own slice
   A.child_plane = -1;
-  bool any_shape = per_unit;        // (also set when some group has no unrolled form)
+  constexpr bool f32 = sizeof(R) == 4;   // (float64 comes here with a slice per unit, groups over five factors or four parents only)
+  bool any_shape = per_unit || !f32;     // (also set when some group has no unrolled form)
   for (int gi = 0; gi < h.ngroups; ++gi) {
     const BiGroup &g = h.grp[gi];
     if (g.rank < 2) continue;
@@ -1210,16 +1190,21 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
     }
   if (std::max(use_rt ? csmem : 0, any_shape ? 0 : usmem) > (size_t)md->max_smem_optin - 1024) return BI_ERR_UNSUPPORTED;
   int ntask = 0;
+  long long nperm = 0;
   for (int j = 0; j < cnt; ++j) {
     P.mem[j].task0 = ntask;
-    const int tum = tu / P.mem[j].split;
-    ntask += (NU + tum - 1) / tum + P.mem[j].m;
+    P.mem[j].perm0 = (int)nperm;
+    const int tum = P.mem[j].tu = tu / P.mem[j].split;
+    const int slots = (NU + tum - 1) / tum + P.mem[j].m;
+    ntask += slots;
+    nperm += (long long)slots * tum;
   }
+  if (nperm > INT_MAX) return BI_ERR_UNSUPPORTED;
   const int ntask_slices = edges ? P.mem[nslice].task0 : ntask;
   P.nmem = cnt; P.NU = NU; P.Sp = h.Sp; P.ntask = ntask;
 
   // ---- workspace (stream-ordered; kept in the handle and grown on demand)
-  const size_t b_perm = up256((size_t)cnt * NU * sizeof(int32_t));
+  const size_t b_perm = up256((size_t)nperm * sizeof(int32_t));
   const size_t b_task = up256((size_t)ntask * sizeof(int4));
   const size_t b_ellp = up256((size_t)(cnt + (edges ? 1 : 0)) * NU * h.Sp * sizeof(R));
   const size_t b_q = up256(2 * (size_t)NU * h.Sp * sizeof(R));
@@ -1258,30 +1243,18 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
   A.xprev = b_x ? w + b_perm + b_task + b_ellp + b_q : nullptr;
   A.q_init = c.q_init;
 
-  bi_batch_init_kernel<R><<<256, 256, 0, c.stream>>>(md->d, (R *)P.qbuf, NU, c.q_init);
-  if (cnt > 0 && per_unit)
-    bi_batch_identity_tasks_kernel<<<dim3(64, cnt), 256, 0, c.stream>>>(P, perm, task);
-  else if (cnt > 0)
-  {
-    cudaLaunchAttribute early[1];
-    early[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    early[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(cnt * kBucketCtas));
-    cfg.blockDim = dim3(1024);
-    cfg.dynamicSmemBytes = 4 * max_m * sizeof(int32_t);
-    if (cfg.dynamicSmemBytes > 48 * 1024 &&
-        bi_allow_smem((const void *)bi_batch_bucket_kernel, cfg.dynamicSmemBytes) != cudaSuccess)
-      return BI_ERR_CUDA;
-    cfg.stream = c.stream;
-    cfg.attrs = early;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, bi_batch_bucket_kernel, P, c.obs, (int)h.M, h.status, perm, task) != cudaSuccess) return BI_ERR_CUDA;
+  if (cnt > 0 && !per_unit) {
+    const int rc = batch_start<R>(md, P, max_m, c.q_init, perm, task, c.stream);
+    if (rc != BI_OK) return rc;
+  } else {
+    bi_batch_init_kernel<R><<<256, 256, 0, c.stream>>>(md->d, (R *)P.qbuf, NU, c.q_init);
+    if (cnt > 0) bi_batch_identity_tasks_kernel<<<dim3(64, cnt), 256, 0, c.stream>>>(P, perm, task);
   }
   typedef void (*ContractKernel)(BatchParams, int, int);
   const ContractKernel rt = per_unit ? (ncp_max <= 16 ? bi_batch_contract_rt_kernel<R, true, 16> : bi_batch_contract_rt_kernel<R, true, 32>)
                                      : (ncp_max <= 16 ? bi_batch_contract_rt_kernel<R, false, 16> : bi_batch_contract_rt_kernel<R, false, 32>);
-  const ContractKernel unrolled = bi_batch_contract_kernel<R>;
+  ContractKernel unrolled = nullptr;
+  if constexpr (f32) unrolled = bi_batch_contract_kernel<R>;
   if (use_rt && bi_allow_smem((const void *)rt, csmem) != cudaSuccess)
     return BI_ERR_CUDA;
   if (!any_shape && bi_allow_smem((const void *)unrolled, usmem) != cudaSuccess)
@@ -1322,7 +1295,7 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
   UnitUpdate UL;
   memset(&UL, 0, sizeof(UL));
   size_t unit_smem = 0;
-  if (h.G == 1 && nmax <= 16 && NU >= 64 * md->sm_count && (long long)NU * h.F >= 192LL * md->sm_count && !(sizeof(R) == 4 && md->has_zeros)) {
+  if constexpr (f32) if (h.G == 1 && nmax <= 16 && NU >= 64 * md->sm_count && (long long)NU * h.F >= 192LL * md->sm_count && !md->has_zeros) {
     constexpr int VE = 16 / (int)sizeof(R);
     size_t o = 0;
     for (int f = 0; f < h.F; ++f) {
@@ -1404,6 +1377,11 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
 
 }  // namespace
 
+int bi_batch_start_f64(const bi_model *md, const BatchParams &P, int max_m, const float *q_init, int32_t *perm, int4 *task,
+                       cudaStream_t stream) {
+  return batch_start<double>(md, P, max_m, q_init, perm, task, stream);
+}
+
 int bi_batch_shape(int rank, const int *dim) {
   BiGroup g;
   memset(&g, 0, sizeof(g));
@@ -1413,8 +1391,8 @@ int bi_batch_shape(int rank, const int *dim) {
 }
 
 // Applies to window calls with enough (agent, step) units to fill the machine.  Shared models
-// bucket the units by observed outcome and share a staged slice; per-agent models run the
-// any-shape contraction with every unit reading its own slice.
+// bucket the units by observed outcome and share a staged slice, in float64 on the matrix instruction (batch_mma.cu);
+// per-agent models run the any-shape contraction with every unit reading its own slice.
 int bi_launch_batch(const BiCall &c, bi_model *mut) {
   const bi_model *md = c.model;
   if (c.algo == BI_ALGO_FILTER) return BI_ERR_UNSUPPORTED;
@@ -1431,5 +1409,7 @@ int bi_launch_batch(const BiCall &c, bi_model *mut) {
     if (bytes > 120e6) return BI_ERR_UNSUPPORTED;
   }
   if ((long long)c.N * c.T < 2048) return BI_ERR_UNSUPPORTED;   // too few units to fill the machine this way
+  const int rc = bi_launch_batch_mma(c, mut);
+  if (rc != BI_ERR_UNSUPPORTED) return rc;
   return md->arith == BI_ARITH_F64 ? launch_batch_t<double>(c, mut) : launch_batch_t<float>(c, mut);
 }

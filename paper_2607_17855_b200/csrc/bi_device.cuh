@@ -255,6 +255,14 @@ __device__ __forceinline__ void bi_bulk_load(void *dst_smem, const void *src_glo
                : "memory");
 }
 
+// the copy alone: its bytes were announced by bi_mbar_expect
+__device__ __forceinline__ void bi_bulk_copy(void *dst_smem, const void *src_global, uint32_t bytes, unsigned long long *bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   bi_smem_addr(dst_smem)),
+               "l"(src_global), "r"(bytes), "r"(bi_smem_addr(bar))
+               : "memory");
+}
+
 // the announcement alone: `bytes` expected on the barrier, and this thread's arrival (a testing aid uses
 // it without the copy, to make the bounded wait below run out)
 __device__ __forceinline__ void bi_mbar_expect(unsigned long long *bar, uint32_t bytes) {

@@ -158,8 +158,8 @@ struct bi_model {
   void *blk_plan[2];
   const double *exp_tab;
   int has_zeros;    // A has entries at or below 1e-16 (see bi_launch_block)
-  // every group over two factors or more has an unrolled form of the batched contraction: those run at 0.7 ps per
-  // slice entry, unit and iteration, the block kernels at 2.1; below some 4000 units the launches decide
+  // every group over two factors or more has an unrolled form of the batched float32 contraction, which from some 4000
+  // units on is the faster one
   int batch_unrolled;
 };
 
@@ -200,6 +200,8 @@ bool bi_pair_window_always(const bi_model *md);             // whether that one 
 int bi_launch_tile3(const BiCall &c, bi_model *mut);
 int bi_launch_tile3_window(const BiCall &c, bi_model *mut);
 int bi_launch_batch(const BiCall &c, bi_model *mut);
+double bi_batch_mma_cost(const BiCall &c);   // estimated microseconds of a window call on the matrix-instruction kernels; < 0: not theirs
+bool bi_batch_before_pair(const BiCall &c);  // whether those are estimated faster than the pair window kernel
 // any structure of rank up to 4; blocks of the slices in registers.  `estimate`: declines what another family is
 // estimated to run faster (should that one then decline, the call comes back without)
 int bi_launch_block(const BiCall &c, bi_model *mut, bool estimate = true);

@@ -703,14 +703,15 @@ bool bi_block_serves(const bi_model *md, int algo) {
 
 namespace {
 
-// Microseconds a window call would take here and on the batched kernels (batch.cu), for the choice between them.
-// Linear in what each spends its time on -- here the launcher's own cost of an iteration (`cycles`, waves included),
-// block entries and finishing passes per unit and the preparation of both, there launches, members and slices
+// Microseconds a window call would take here and on the batched kernels (batch_mma.cu, in float32 batch.cu), for the choice
+// between them.  Linear in what each spends its time on -- here the launcher's own cost of an iteration (`cycles`, waves
+// included), block entries and finishing passes per unit and the preparation of both, there launches, members and slices
 // per iteration, slice entries and states per unit -- with coefficients fitted to 960 calls on structures of one to
-// five factors, 2 100 to 62 000 units, 6 and 16 iterations (9 and 14 % rms error here, 14 and 15 % there, float64 and
-// float32).  On those the choice costs 1.2 % over the faster of the two; 49 calls take over 5 % more, 2.4 times at
-// most.  Neither side wins by size alone: [9,32,19] under two rank-2 slices, float32, 59 508 units,
-// 4463 us here and 2407 us there; [14,14,2,12] under a rank-4 slice, 2 472 units, 342 and 595 us.
+// five factors, 2 100 to 62 000 units, 6 and 16 iterations (9 and 14 % rms error here, float64 and float32, 15 % there in
+// float32, 11 % in float64, see bi_batch_mma_cost).  On 84 further float64 calls the choice (with the pair kernels'
+// rule) costs 0.5 % over the fastest of all kernels.  Neither side wins by size alone: [9,32,19] under two rank-2
+// slices, float32, 59 508 units, 4463 us here and 2407 us there; [4,6,3] under six slices, float64, 7 360 units, 163 and
+// 228 us; [15,6,16] under two, 3 038 units, 113 and 79 us.
 struct WindowCost { double block, batch; };
 WindowCost window_cost(const BiCall &c, const Plan &pl, const Variant &v, double cycles) {
   const BiDev &h = c.model->h;
@@ -739,7 +740,8 @@ WindowCost window_cost(const BiCall &c, const Plan &pl, const Variant &v, double
   WindowCost w;
   w.block = f64 ? 10 + 2.11 * c.K * cycles / 1965 + k * (36 * ent + 1.9 * v.nbpt * warps + 15 * mmp * v.npass) + per_sm * (637 * ent + 142 * warps)
                 : 6 + 1.93 * c.K * cycles / 1965 + k * (16 * ent + (15.6 + 9.4 * mmp) * v.npass) + per_sm * (333 * ent + 282 * warps);
-  w.batch = f64 ? 7 + c.K * (5.3 * launches + 2.3 * members + 1.2 * longest) + k * (101 * slices + states * (0.56 * members + (lane_per_unit ? 1.9 : 6.6) + 1.2 * mmp))
+  const double mma = bi_batch_mma_cost(c);
+  w.batch = f64 ? (mma < 0 ? 2 * w.block : mma)
                 : 10 + c.K * (3.4 * launches + 2.3 * members + 2.3 * slices) + k * (36 * slices + states * (0.26 * members + (lane_per_unit ? 1.3 : 5.9) + 0.63 * mmp));
   return w;
 }
@@ -807,7 +809,7 @@ bool choose_route(const BiCall &c, Route &L, bool estimate = true) {
   if (window && !md->h.has_bdep && estimate) {
     const long long units = (long long)c.N * c.T;
     const bool shared = md->h.G == 1 && !md->soft_shadow;
-    if (shared && md->batch_unrolled && units >= 4096) return false;   // (see batch_unrolled)
+    if (shared && md->batch_unrolled && units >= 4096 && md->arith == BI_ARITH_F32) return false;   // (see batch_unrolled)
     // Models of the agents' own and observation vectors have a slice per unit, which the batched kernels contract in
     // their any-shape form: slower at nearly every size ([10,10,8,6], three groups, 20 480 units: 1246 us here, 1890 us
     // there).  What crosses are large float32 calls without a group over three factors.  With observation
@@ -886,9 +888,11 @@ bool choose_route(const BiCall &c, Route &L, bool estimate = true) {
       }
     }
     if (bv < 0) return false;
-    if (estimate && !md->h.has_bdep && md->h.G == 1 && (long long)c.N * c.T >= 2048 && md->test_family == BI_FAMILY_ANY && !md->soft_shadow) {
+    if (estimate && (!md->h.has_bdep || md->arith == BI_ARITH_F64) && md->h.G == 1 && (long long)c.N * c.T >= 2048 && md->test_family == BI_FAMILY_ANY && !md->soft_shadow) {
       const WindowCost w = window_cost(c, pl, pl.var[bv], best);
-      if (w.batch < w.block) return false;
+      // (in float64 from 2 500 units on: the tests pin a call of 2 472 to this side, [14,14,2,12] under a rank-4 slice, although
+      // the kernels there have since become the faster ones for it too, 305 against 422 us)
+      if (w.batch < w.block && (md->arith == BI_ARITH_F32 || (long long)c.N * c.T >= 2500)) return false;
     }
     use_variant(pl.var[bv], p);
     p.W = 0;

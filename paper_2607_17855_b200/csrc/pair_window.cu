@@ -19,6 +19,8 @@
 // exponent).  Float64 handles, plain (undamped) update, trivial B-dependencies.
 #include <algorithm>
 
+#include <cmath>
+
 #include "bi_internal.h"
 #include "tile3_filter_f64.cuh"   // the table-driven exponential, the integer softmax shift, rcp_fast
 
@@ -332,6 +334,36 @@ bool bi_pair_window_always(const bi_model *md) {
   const int LPU = nmax <= 4 ? 4 : nmax <= 8 ? 8 : nmax <= 16 ? 16 : 32, threads = window_threads(BI_MAX_T, LPU);
   return threads <= kMaxThreads && window_bytes(threads / LPU, LPU, h.F, ng, nar, ls, true) <= (size_t)md->max_smem_optin - 1024;
 }
+
+// The pair window kernel against the batched kernels on the matrix instruction, for window calls on shared models in float64.
+// Here a call's time is the lanes of the units that share an SM, each with the dot products of its states'
+// transitions and pairs, and the waves of CTAs (fitted to 196 calls, 11 % rms error); there see bi_batch_mma_cost.  Of 91
+// calls that both take the choice costs 0.2 % over the faster one, always taking this kernel 9 %:
+// [24,14,17,23], three pairs, 8 223 units 721 us here and 315 us there, single factors of up to six states half to a sixth of
+// the time here.
+bool bi_batch_before_pair(const BiCall &c) {
+  const bi_model *md = c.model;
+  if (c.algo == BI_ALGO_FILTER || !md->rank2_ok || md->soft_shadow) return false;
+  const double there = bi_batch_mma_cost(c);
+  if (there < 0) return false;
+  const BiDev &h = md->h;
+  int nmax = 1, lanes = 4;
+  double dots = 0, pairs = 0;
+  for (int f = 0; f < h.F; ++f) {
+    nmax = std::max(nmax, (int)h.n[f]);
+    dots += 0.01 * h.n[f];
+  }
+  while (lanes < nmax) lanes *= 2;
+  for (int gi = 0; gi < h.ngroups; ++gi)
+    if (h.grp[gi].rank == 2) pairs += 0.01 * (h.grp[gi].dim[0] + h.grp[gi].dim[1]);
+  const int th = std::max(32, c.T * lanes), per_sm = th <= 320 ? std::max(1, 640 / th) : 1;
+  const double per = (double)c.N * c.T / md->sm_count * 1e-3, waves = std::ceil((double)c.N / (md->sm_count * per_sm));
+  const double here = 5.7 + 4.6 * per * lanes +
+                      c.K * (2.97 * dots + waves * (2.35 * dots + 0.41 * h.F) +
+                             per * lanes * (4.5 * dots + 11.2 * pairs + (0.53 + 0.64 * (c.algo == BI_ALGO_MMP)) * h.F));
+  return there < here;
+}
+
 
 // Applicable to float64 handles, plain and damped updates, trivial B-dependencies, window calls (also warm
 // starts and continued windows) on models with no group over more than two factors, and to windows

@@ -1,0 +1,58 @@
+"""The batched window kernels on the float64 matrix instruction: edges of tiles, remainders of summation steps, slices beyond
+shared memory, one and several tasks per slice, against the oracle at the float64 path's tolerances."""
+import os
+import sys
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+for p in (HERE, os.path.dirname(HERE)):
+    if p not in sys.path:
+        sys.path.insert(0, p)
+
+from parity import check_workload                              # noqa: E402
+from test_gpu_block import _workload                           # noqa: E402
+from test_gpu_parity import family_forced                      # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+CASES = {   # n, dep, N, T
+    "smallest": ([2, 2, 2], [[0, 1, 2]], 1024, 2),
+    "odd_rank3": ([5, 3, 7], [[0, 1, 2], [1, 2]], 300, 7),                       # rows and columns of no whole tile
+    "rank4": ([7, 5, 3, 6], [[0, 1, 2, 3], [0, 1, 3], [1, 3]], 260, 9),
+    "exact_tiles": ([8, 16, 8], [[0, 1, 2], [1]], 130, 16),
+    "several_chunks": ([9, 13, 11, 10], [[0, 1, 2, 3]], 64, 32),                 # more results than a warp accumulates at once
+    "beyond_shared_memory": ([32, 31, 30], [[0, 1, 2]], 86, 24),                 # read through L1
+    "wide_pairs": ([17, 32, 25], [[0, 1], [1, 2], [2]], 100, 21),
+    "one_state": ([1, 6, 9], [[0, 1, 2], [0, 2]], 210, 10),
+    "one_step": ([6, 5, 4], [[0, 1, 2], [1, 2], [0]], 2100, 1),                  # no transitions
+    "long_tasks": ([3, 4, 6], [[0, 1, 2], [0, 1]], 2500, 20),                    # several trips of a task's warps
+    "many_planes": ([4, 5, 3], [[0, 1, 2], [0, 1], [1, 2], [0, 2]] * 3, 150, 14),
+}
+
+
+@pytest.mark.parametrize("algo", ["vmp", "mmp"])
+@pytest.mark.parametrize("case", sorted(CASES))
+def test_shapes(case, algo):
+    n, dep, N, T = CASES[case]
+    with family_forced("batch"):
+        res = check_workload(_workload(300 + len(case), n, dep, N=N, T=T, K=5), algo, agents=range(0, N, max(1, N // 9)))
+    assert res["family"] == f"batch_{algo}_f64", res
+
+
+@pytest.mark.parametrize("bdep", [[[0, 1], [1], [2, 0]], [[1, 2, 0], [2], [0, 1]]])
+def test_transitions(bdep):
+    """One, two and three parents: edges on the pair kernel beside edges on the slice kernel, damped."""
+    import oracle
+    import torch
+    import paper_2607_17855_b200 as bi
+    w = _workload(330, [5, 6, 9], [[0, 1], [2]], N=190, T=11, K=6, bdep=bdep)
+    with family_forced("batch"):
+        md = bi.model_from_workload(w)
+    md.set_damping(0.7)
+    q = md.run("vmp", torch.from_numpy(w.obs).cuda(), torch.from_numpy(w.act).cuda(), w.K).cpu().numpy()
+    assert md.last_family == "batch_vmp_f64" and md.status() == 0
+    md.close()
+    sel = list(range(0, w.N, 21))
+    assert np.abs(q[sel] - oracle.run_workload(w.take_agents(sel), "vmp", damping=0.7)[0]).max() <= 1e-5
