@@ -481,6 +481,11 @@ bi_block_filter_kernel(const __grid_constant__ Params p) {
   const int2 src0 = __ldg(reinterpret_cast<const int2 *>(&(p.desc + (has ? lt : 0))->grp));
   const int any0 = (int)__reduce_or_sync(0xffffffffu, (unsigned)b0.kind);
   const bool lanes0 = warp < p.npass;
+  // the description of the warp's first pass, kept where the blocks are small enough to leave the registers for it
+  // (a description read again in every iteration is 40 instructions and a round trip to shared memory; 1000 agents, [7,9,5],
+  // float32, 8 x 4 blocks: 436 -> 414 us; 585 agents, [8,5], 4 x 4: 262 -> 246 us; beside 8 x 6 in float64 it spills)
+  constexpr bool kKeepLanes = BR * BC * E <= 256;
+  const LaneRef l0 = lane_ref<R>(p, lanes0 ? warp : 0, lane, unit, ex);
   const bool common = p.common != 0 && __ldg(p.status + 1) == 0;
 
   const bool from_prev = p.q_prev != nullptr || p.carry_in != nullptr;
@@ -596,7 +601,7 @@ bi_block_filter_kernel(const __grid_constant__ Params p) {
 #pragma unroll 1
     for (int k = 0; k < p.K; ++k) {
       contract_all<R, BR, BC, HASS>(p, L, own, b0, any0, lt, LT, unit, p.o_L);
-      LaneRef l = lane_ref<R>(p, lanes0 ? warp : 0, lane, unit, ex);
+      LaneRef l = kKeepLanes ? l0 : lane_ref<R>(p, lanes0 ? warp : 0, lane, unit, ex);
       team_sync<SYNC>(LT, team);
       if (k < p.K - 1) {
         if (lanes0) {
