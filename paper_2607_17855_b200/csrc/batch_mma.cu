@@ -27,7 +27,6 @@ namespace {
 
 constexpr int kWarps = 4;          // warps of a CTA of the pair kernel: two (V and W) for each of two groups of units
 constexpr int kPairTiles = 2;      // eights of units that one of its warps takes at a time
-constexpr int kSliceWarps = 4;     // warps of a CTA of the slice kernel, eight units at a time each
 constexpr int kTiles = 8;          // most 8-wide tiles of results a warp accumulates at once
 constexpr int kChunk = 8 * kTiles;
 constexpr int kChunkStride = kChunk + 4;   // (4 modulo 16: a half warp's 4 units x 32 bytes fall on different banks)
@@ -287,8 +286,8 @@ __device__ __forceinline__ void mma_side(const MmaParams &P, const MmaMember &mm
 // that overlaps the kernel before (tasks of 32 units, three waves: 15 of 35 us went into starting them).  The
 // warps take eight units at a time, their beliefs gathered by asynchronous copies.  SPLIT: half
 // of the warps does V, half W, for batches with fewer units than that fills the machine with.
-template <bool GLOBAL, bool SPLIT>
-__global__ void __launch_bounds__(32 * kSliceWarps, 4) bi_mma_slice_kernel(const __grid_constant__ MmaParams P, int cur, int first) {
+template <bool GLOBAL, bool SPLIT, int NW>
+__global__ void __launch_bounds__(32 * NW, 16 / NW) bi_mma_slice_kernel(const __grid_constant__ MmaParams P, int cur, int first) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long bar;
   double *Ls = reinterpret_cast<double *>(smem_raw);
@@ -317,15 +316,15 @@ __global__ void __launch_bounds__(32 * kSliceWarps, 4) bi_mma_slice_kernel(const
   }
   // index tables: summation index -> two entries of a unit's beliefs
   uint32_t *ctab = tab, *rtab = tab + C;
-  for (int c = tid; c < C; c += 32 * kSliceWarps) {
+  for (int c = tid; c < C; c += 32 * NW) {
     const int x = c / mm.np[3], y = c - x * mm.np[3];
     ctab[c] = (uint32_t)((mm.n[2] > 1 ? mm.lo[2] + x : P.one) | ((mm.lo[3] + y) << 16)) * 8u;
   }
-  for (int r = tid; r < ((R + 3) & ~3); r += 32 * kSliceWarps) {
+  for (int r = tid; r < ((R + 3) & ~3); r += 32 * NW) {
     const int x = r / mm.np[1], y = r - x * mm.np[1];
     rtab[r] = (r < R ? (uint32_t)((mm.n[0] > 1 ? mm.lo[0] + x : P.one) | ((mm.lo[1] + y) << 16)) : (uint32_t)((P.one + 1) | ((P.one + 1) << 16))) * 8u;
   }
-  constexpr int GRP = SPLIT ? kSliceWarps / 2 : kSliceWarps;   // groups of units at a time
+  constexpr int GRP = SPLIT ? NW / 2 : NW;   // groups of units at a time
   const int side = SPLIT ? warp & 1 : 0;
   int u0 = 8 * (SPLIT ? warp >> 1 : warp);
   double *own = reinterpret_cast<double *>(tab + P.tabs) + (size_t)warp * 8 * (P.sq + kChunkStride);
@@ -394,7 +393,7 @@ struct MmaUpdate {
 // added up before the wait for the messages.
 constexpr int kUpdThreads = 128;
 template <bool FINAL, bool DAMPED>
-__global__ void __launch_bounds__(kUpdThreads) bi_mma_update_kernel(const BiDev *__restrict__ mdp, const __grid_constant__ MmaUpdate A,
+__global__ void __launch_bounds__(kUpdThreads, 9) bi_mma_update_kernel(const BiDev *__restrict__ mdp, const __grid_constant__ MmaUpdate A,
                                                                     const double *__restrict__ ell, double *__restrict__ qbuf, int NU, int upb) {
   __shared__ double part[2][kUpdThreads];
   __shared__ double2 logit[FINAL ? kUpdThreads : 1];
@@ -679,14 +678,20 @@ int bi_launch_batch_mma(const BiCall &c, bi_model *mut) {
   P.sq = (own + 2 + 3) & ~3;
   if (P.sq % 8 == 0) P.sq += 4;
   P.tabs = (int)((tabs + 3) & ~(size_t)3);
-  const size_t fixed = (size_t)P.tabs * sizeof(uint32_t) + (size_t)kSliceWarps * 8 * (P.sq + kChunkStride) * sizeof(double);
-  const bool global = fixed + lsz * sizeof(double) > (size_t)md->max_smem_optin - 1024;
+  auto slice_smem = [&](int nw, size_t slice) { return (size_t)P.tabs * sizeof(uint32_t) + ((size_t)nw * 8 * (P.sq + kChunkStride) + slice) * sizeof(double); };
+  auto fit = [&](int nw, size_t bytes) { return std::max(1, std::min(16 / nw, (int)(((size_t)md->max_smem_optin + 1024) / (bytes + 1024 + 64)))); };
+  const bool global = slice_smem(4, lsz) > (size_t)md->max_smem_optin - 1024;
   P.lsz = global ? 0 : (int)((lsz + 1) & ~(size_t)1);
-  const size_t smem = fixed + (size_t)P.lsz * sizeof(double);
+  // Warps of a CTA of the slice kernel, eight units at a time each: four, or eight around one staged slice where that leaves
+  // more warps on an SM and the units are enough for them (a slice of 5236 entries, 12 222 units: 713 -> 557 us a call; of 3528,
+  // 10 674 units: 750 -> 678; with 2 478 to 7 218 units up to 5 % slower)
+  const int nw = !global && NU >= 8192 && slice_smem(8, P.lsz) <= (size_t)md->max_smem_optin - 1024 &&
+                         8 * fit(8, slice_smem(8, P.lsz)) > 4 * fit(4, slice_smem(4, P.lsz)) ? 8 : 4;
+  const size_t smem = slice_smem(nw, P.lsz);
   if (nheavy && smem > (size_t)md->max_smem_optin - 1024) return BI_ERR_UNSUPPORTED;
   // Units per task: a wave of CTAs is shared out between the members by the cost of a unit, a matrix instruction taking
   // sixteen cycles and the rest of eight units' work about 1500; every outcome may leave one partial task.
-  const int per_sm = std::max(1, std::min(4, (int)(((size_t)md->max_smem_optin + 1024) / (smem + 1024 + 64))));
+  const int per_sm = fit(nw, smem);
   double cost[BI_MAX_M + BI_MAX_F], heavy_cost = 0;
   for (int j = 0; j < cnt; ++j) {
     const MmaMember &mm = P.mem[j];
@@ -696,12 +701,12 @@ int bi_launch_batch_mma(const BiCall &c, bi_model *mut) {
   // V and W by different warps where the units do not fill a wave with eight to a warp, and the slices are large enough to be worth
   // the second set of beliefs (a slice of 5742 entries, 2560 units: 18.5 against 21.8 us an iteration; of 648, 7500
   // units: 18.5 against 15.6)
-  const bool split = NU <= 4 * kSliceWarps * per_sm * md->sm_count && nheavy && P.mem[0].ostride >= 2048;
+  const bool split = NU <= 4 * nw * per_sm * md->sm_count && nheavy && P.mem[0].ostride >= 2048;
   int ntask = 0, ntask_heavy = 0;
   long long nperm = 0;
   for (int j = 0; j < cnt; ++j) {
     const double wave = j < nheavy ? per_sm * md->sm_count * cost[j] / heavy_cost : (nmax <= 16 ? 8.0 : 4.0) * md->sm_count / (cnt - nheavy);
-    const int trip = j < nheavy ? 8 * (split ? kSliceWarps / 2 : kSliceWarps) : 8 * kPairTiles * kWarps / 2;
+    const int trip = j < nheavy ? 8 * (split ? nw / 2 : nw) : 8 * kPairTiles * kWarps / 2;
     const double tasks = std::max(wave - B.mem[j].m, 0.5 * wave);
     const int unit_step = j < nheavy ? 8 : trip;
     const int tu = std::max(trip, ceil_div((int)std::ceil(NU / std::max(tasks, 1.0)), unit_step) * unit_step);
@@ -764,8 +769,9 @@ int bi_launch_batch_mma(const BiCall &c, bi_model *mut) {
   typedef void (*SliceKernel)(MmaParams, int, int);
   typedef void (*PairKernel)(MmaParams, int, int, int);
   typedef void (*UpdateKernel)(const BiDev *, MmaUpdate, const double *, double *, int, int);
-  const SliceKernel ks = split ? (global ? bi_mma_slice_kernel<true, true> : bi_mma_slice_kernel<false, true>)
-                               : (global ? bi_mma_slice_kernel<true, false> : bi_mma_slice_kernel<false, false>);
+  const SliceKernel ks = nw == 8 ? (split ? bi_mma_slice_kernel<false, true, 8> : bi_mma_slice_kernel<false, false, 8>)
+                         : split ? (global ? bi_mma_slice_kernel<true, true, 4> : bi_mma_slice_kernel<false, true, 4>)
+                                 : (global ? bi_mma_slice_kernel<true, false, 4> : bi_mma_slice_kernel<false, false, 4>);
   const PairKernel kp = nmax <= 16 ? bi_mma_pair_kernel<kPairTiles, 4> : bi_mma_pair_kernel<kPairTiles, 8>;
   const bool damped = A.xprev != nullptr;
   const UpdateKernel mid = damped ? bi_mma_update_kernel<false, true> : bi_mma_update_kernel<false, false>;
@@ -792,7 +798,7 @@ int bi_launch_batch_mma(const BiCall &c, bi_model *mut) {
     if (nheavy) {
       cfg.gridDim = dim3((unsigned)ntask_heavy);
       cfg.dynamicSmemBytes = smem;
-      cfg.blockDim = dim3(32 * kSliceWarps);
+      cfg.blockDim = dim3((unsigned)(32 * nw));
       P.task0 = 0;
       if (cudaLaunchKernelEx(&cfg, ks, P, cur, (int)(k == 0)) != cudaSuccess) return BI_ERR_CUDA;
     }
@@ -803,7 +809,8 @@ int bi_launch_batch_mma(const BiCall &c, bi_model *mut) {
       P.task0 = ntask_heavy;
       if (cudaLaunchKernelEx(&cfg, kp, P, cur, (int)(k == 0), (int)(nheavy > 0)) != cudaSuccess) return BI_ERR_CUDA;
     }
-    cfg.gridDim = dim3((unsigned)std::min(ceil_div(NU, upb), 12 * md->sm_count));
+    // (the CTAs that are resident at once, by registers: a wave of 12 an SM waited for its last quarter, 762 -> 735 us on 20 480 units of 34 states)
+    cfg.gridDim = dim3((unsigned)std::min(ceil_div(NU, upb), 9 * md->sm_count));
     cfg.blockDim = dim3((unsigned)upd_threads);
     A.common = terms * 54 < 960 && !(c.q_init && (k == 0 || damped));   // (starting beliefs are used as given)
     if (cudaLaunchKernelEx(&cfg, k == c.K - 1 ? last : mid, (const BiDev *)md->d, A, (const double *)P.ell, q, NU, upb) != cudaSuccess)
