@@ -392,8 +392,10 @@ struct MmaUpdate {
 // go out together, and what does not change between the iterations (the slices of single-factor modalities, the prior) is
 // added up before the wait for the messages.
 constexpr int kUpdThreads = 128;
-template <bool FINAL, bool DAMPED>
-__global__ void __launch_bounds__(kUpdThreads, 9) bi_mma_update_kernel(const BiDev *__restrict__ mdp, const __grid_constant__ MmaUpdate A,
+// PER_SM: CTAs resident on an SM.  Twelve cost some spilled registers and hide more of the loads, which pays where the units are
+// more than one wave of nine (20 480 units of 34 states: 751 -> 738 us a call; with fewer it costs up to 6 %).
+template <int PER_SM, bool FINAL, bool DAMPED>
+__global__ void __launch_bounds__(kUpdThreads, PER_SM) bi_mma_update_kernel(const BiDev *__restrict__ mdp, const __grid_constant__ MmaUpdate A,
                                                                     const double *__restrict__ ell, double *__restrict__ qbuf, int NU, int upb) {
   __shared__ double part[2][kUpdThreads];
   __shared__ double2 logit[FINAL ? kUpdThreads : 1];
@@ -774,11 +776,17 @@ int bi_launch_batch_mma(const BiCall &c, bi_model *mut) {
                                  : (global ? bi_mma_slice_kernel<true, false, 4> : bi_mma_slice_kernel<false, false, 4>);
   const PairKernel kp = nmax <= 16 ? bi_mma_pair_kernel<kPairTiles, 4> : bi_mma_pair_kernel<kPairTiles, 8>;
   const bool damped = A.xprev != nullptr;
-  const UpdateKernel mid = damped ? bi_mma_update_kernel<false, true> : bi_mma_update_kernel<false, false>;
-  const UpdateKernel last = damped ? bi_mma_update_kernel<true, true> : bi_mma_update_kernel<true, false>;
   int terms = h.M + 3;   // (see MmaUpdate::common; with several parents a future message from every child)
   for (int f = 0; f < h.F; ++f) terms = std::max(terms, h.M + 1 + __builtin_popcount(A.emask[f]));
   const int upb = std::max(1, kUpdThreads / (h.Sp / 2)), upd_threads = (upb * (h.Sp / 2) + 31) / 32 * 32;
+  const int upd_per_sm = ceil_div(NU, upb) > 9 * md->sm_count ? 12 : 9;
+  auto pick = [&](bool fin) -> UpdateKernel {
+#define BI_UPD(PER) (fin ? (damped ? bi_mma_update_kernel<PER, true, true> : bi_mma_update_kernel<PER, true, false>) \
+                         : (damped ? bi_mma_update_kernel<PER, false, true> : bi_mma_update_kernel<PER, false, false>))
+    return upd_per_sm == 12 ? BI_UPD(12) : BI_UPD(9);
+#undef BI_UPD
+  };
+  const UpdateKernel mid = pick(false), last = pick(true);
   if (nheavy && bi_allow_smem((const void *)ks, smem) != cudaSuccess) return BI_ERR_CUDA;
   // every launch of the loop may be scheduled while its predecessor drains (see bi_grid_wait)
   // ... and they share SMs, so they ask for one split of L1 and shared memory
@@ -809,8 +817,8 @@ int bi_launch_batch_mma(const BiCall &c, bi_model *mut) {
       P.task0 = ntask_heavy;
       if (cudaLaunchKernelEx(&cfg, kp, P, cur, (int)(k == 0), (int)(nheavy > 0)) != cudaSuccess) return BI_ERR_CUDA;
     }
-    // (the CTAs that are resident at once, by registers: a wave of 12 an SM waited for its last quarter, 762 -> 735 us on 20 480 units of 34 states)
-    cfg.gridDim = dim3((unsigned)std::min(ceil_div(NU, upb), 9 * md->sm_count));
+    // (the CTAs that are resident at once: twelve an SM where nine fit waited for the last quarter, 762 against 735 us on 20 480 units of 34 states)
+    cfg.gridDim = dim3((unsigned)std::min(ceil_div(NU, upb), upd_per_sm * md->sm_count));
     cfg.blockDim = dim3((unsigned)upd_threads);
     A.common = terms * 54 < 960 && !(c.q_init && (k == 0 || damped));   // (starting beliefs are used as given)
     if (cudaLaunchKernelEx(&cfg, k == c.K - 1 ? last : mid, (const BiDev *)md->d, A, (const double *)P.ell, q, NU, upb) != cudaSuccess)
