@@ -977,6 +977,14 @@ __global__ void bi_predictive_prior_kernel(const BiDev *__restrict__ mdp, int N,
   out[i] = bi_log(bi_max(acc, (R)BI_EPS));
 }
 
+// Window calls of fewer units than the batched kernels otherwise take, on models too large for the block kernels (and with too many
+// steps for the pair window kernel), float64.  The warp kernel re-reads a slice per unit, these once per task: a slice of 29 760
+// entries, 256 units 1365 us a call here and 3019 there, 1800 units 1656 and 5844; of 49 152 entries 1685 and 16319, 1876 and
+// 12444.  Below 256 units the two come together (128 units of the first: 1468 there).
+static bool few_units_batched(const BiCall &c) {
+  return c.algo != BI_ALGO_FILTER && !c.model->soft_shadow && c.model->test_drop_copy == 0 && (long long)c.N * c.T >= 256;
+}
+
 int bi_dispatch(const BiCall &c, bi_model *mut) {
   mut->last_block = nullptr;
   if (c.model->h.has_bdep) {
@@ -991,6 +999,7 @@ int bi_dispatch(const BiCall &c, bi_model *mut) {
     if (rc == BI_ERR_UNSUPPORTED && (any || only == BI_FAMILY_BATCH)) rc = bi_launch_batch(c, mut);
     if (rc == BI_ERR_UNSUPPORTED && c.algo == BI_ALGO_FILTER && (any || only == BI_FAMILY_CTA)) rc = bi_launch_cta_filter(c, mut);
     if (rc == BI_ERR_UNSUPPORTED && any) rc = bi_launch_block(c, mut, false);
+    if (rc == BI_ERR_UNSUPPORTED && any && few_units_batched(c)) rc = bi_launch_batch_mma(c, mut);
     if (rc == BI_ERR_UNSUPPORTED && c.algo != BI_ALGO_FILTER && (any || only == BI_FAMILY_WARP)) rc = bi_launch_warp(c, mut);
     return rc == BI_ERR_UNSUPPORTED ? bi_launch_generic(c, mut) : rc;
   }
@@ -1005,6 +1014,7 @@ int bi_dispatch(const BiCall &c, bi_model *mut) {
     if (rc == BI_ERR_UNSUPPORTED && c.model->test_drop_copy == 0) rc = bi_launch_block(c, mut);
     if (rc == BI_ERR_UNSUPPORTED) rc = bi_launch_batch(c, mut);
     if (rc == BI_ERR_UNSUPPORTED && c.algo != BI_ALGO_FILTER && c.model->test_drop_copy == 0) rc = bi_launch_block(c, mut, false);
+    if (rc == BI_ERR_UNSUPPORTED && few_units_batched(c)) rc = bi_launch_batch_mma(c, mut);
     // Filtering exposes one unit per agent, so a CTA per agent keeps more of the machine busy than
     // a warp per agent, and its staged slices and per-factor warps pay at every batch size measured
     // on the 128 random structures (sum of times, CTA against warp kernel): 44 against 99 ms at 256

@@ -53,5 +53,3 @@ struct BatchParams {
 // models; perm and task are P.perm and P.task, writable).  max_m: most outcomes of a member.
 int bi_batch_start_f64(const bi_model *md, const BatchParams &P, int max_m, const float *q_init, int32_t *perm, int4 *task,
                        cudaStream_t stream);
-// The whole call on the matrix instruction: float64, one model for all agents, groups over at most four factors.
-int bi_launch_batch_mma(const BiCall &c, bi_model *mut);

@@ -200,6 +200,8 @@ bool bi_pair_window_always(const bi_model *md);             // whether that one 
 int bi_launch_tile3(const BiCall &c, bi_model *mut);
 int bi_launch_tile3_window(const BiCall &c, bi_model *mut);
 int bi_launch_batch(const BiCall &c, bi_model *mut);
+// its float64 form on the matrix instruction: one model for all agents, groups over at most four factors, any number of units
+int bi_launch_batch_mma(const BiCall &c, bi_model *mut);
 double bi_batch_mma_cost(const BiCall &c);   // estimated microseconds of a window call on the matrix-instruction kernels; < 0: not theirs
 bool bi_batch_before_pair(const BiCall &c);  // whether those are estimated faster than the pair window kernel
 // any structure of rank up to 4; blocks of the slices in registers.  `estimate`: declines what another family is

@@ -56,3 +56,9 @@ def test_transitions(bdep):
     md.close()
     sel = list(range(0, w.N, 21))
     assert np.abs(q[sel] - oracle.run_workload(w.take_agents(sel), "vmp", damping=0.7)[0]).max() <= 1e-5
+
+
+@pytest.mark.parametrize("N, family", [(32, "batch"), (31, "warp")])
+def test_few_units_of_a_model_too_large_for_the_block_kernels(N, family):
+    res = check_workload(_workload(340, [32, 31, 30], [[0, 1, 2], [0]], N=N, T=8, K=3), "vmp", agents=range(0, N, 5))
+    assert res["family"] == f"{family}_vmp_f64", res
