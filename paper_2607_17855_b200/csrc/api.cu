@@ -425,6 +425,7 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
   md->damping = 1.0;
   if (const char *e = getenv("BI_TEST_NO_COMPRESS")) md->test_no_compress = atoi(e) != 0;
   if (const char *e = getenv("BI_TEST_DROP_COPY")) md->test_drop_copy = atoi(e) > 0 ? atoi(e) : 0;   // testing aids,
+  if (const char *e = getenv("BI_TEST_WORKSPACE")) md->test_workspace = !strcmp(e, "nan") ? BI_WORKSPACE_NAN : 0;
   if (const char *e = getenv("BI_TEST_FAMILY")) {                                                  // read here only
     md->test_family = !strcmp(e, "warp") ? BI_FAMILY_WARP : !strcmp(e, "generic") ? BI_FAMILY_GENERIC
                       : !strcmp(e, "cta") ? BI_FAMILY_CTA : !strcmp(e, "batch") ? BI_FAMILY_BATCH

@@ -36,10 +36,11 @@ struct MmaMember {
   int64_t ostride;
   int32_t R, C;
   int32_t logs;              // both messages enter as 1/2 ln max(., eps)
-  // up to two axes of each side, slow and fast (a side of one axis has a slow axis of size 1): 0, 1 rows; 2, 3 columns
+  // up to two axes of each side, slow and fast: 0, 1 rows; 2, 3 columns.  A side of one axis has no slow one: sizes 1, lo -1.
+  // (A slow axis that is there may have one state too, in a transition: its messages are summed and written like any other's.)
   int32_t n[4], np[4];       // states; length along its side (the last axis is padded)
   int32_t q[4];              // beliefs, from the unit's row
-  int32_t lo[4];             // beliefs in the warp's copy
+  int32_t lo[4];             // beliefs in the warp's copy, or -1
   int64_t out[4];            // messages, from the unit's row of the first plane
 };
 
@@ -227,7 +228,7 @@ __device__ __forceinline__ void mma_side(const MmaParams &P, const MmaMember &mm
 #undef X
       default: break;
     }
-    if (nx == 1) {   // one axis: the results are its messages
+    if (mm.lo[2 * SIDE] < 0) {   // one axis: the results are its messages
 #pragma unroll
       for (int t = 0; t < kTiles; ++t)
         if (live && 8 * t + 2 * l < ((cnt + 3) & ~3)) *reinterpret_cast<double2 *>(oy + 8 * t + 2 * l) = make_double2(c[t][0], c[t][1]);
@@ -318,11 +319,11 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) bi_mma_slice_kernel(const __
   uint32_t *ctab = tab, *rtab = tab + C;
   for (int c = tid; c < C; c += 32 * NW) {
     const int x = c / mm.np[3], y = c - x * mm.np[3];
-    ctab[c] = (uint32_t)((mm.n[2] > 1 ? mm.lo[2] + x : P.one) | ((mm.lo[3] + y) << 16)) * 8u;
+    ctab[c] = (uint32_t)((mm.lo[2] >= 0 ? mm.lo[2] + x : P.one) | ((mm.lo[3] + y) << 16)) * 8u;
   }
   for (int r = tid; r < ((R + 3) & ~3); r += 32 * NW) {
     const int x = r / mm.np[1], y = r - x * mm.np[1];
-    rtab[r] = (r < R ? (uint32_t)((mm.n[0] > 1 ? mm.lo[0] + x : P.one) | ((mm.lo[1] + y) << 16)) : (uint32_t)((P.one + 1) | ((P.one + 1) << 16))) * 8u;
+    rtab[r] = (r < R ? (uint32_t)((mm.lo[0] >= 0 ? mm.lo[0] + x : P.one) | ((mm.lo[1] + y) << 16)) : (uint32_t)((P.one + 1) | ((P.one + 1) << 16))) * 8u;
   }
   constexpr int GRP = SPLIT ? NW / 2 : NW;   // groups of units at a time
   const int side = SPLIT ? warp & 1 : 0;
@@ -346,7 +347,7 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) bi_mma_slice_kernel(const __
     const int size = unit >= 0 ? 16 : 0;
 #pragma unroll
     for (int j = 0; j < 4; ++j)   // 16 bytes a copy (rows and offsets are multiples of four entries; zeros where there is no unit)
-      if ((j & 1) != 0 || mm.n[j] > 1)
+      if (mm.lo[j] >= 0)
         for (int s = 2 * l; s < ((mm.n[j] + 3) & ~3); s += 8)
           asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(bi_smem_addr(q + mm.lo[j] + s)), "l"(qr + mm.q[j] + s), "r"(size) : "memory");
     const int unit2 = u0 + 8 * GRP + g < tk.z ? __ldcg(pm + u0 + 8 * GRP) : -1;
@@ -633,7 +634,10 @@ int bi_launch_batch_mma(const BiCall &c, bi_model *mut) {
     for (int k = 0; k < x.rank; ++k) dim[k] = h.n[x.fac[k]];
     int rows = x.rank == 4 ? 2 : 1;
     if (x.rank == 3 && cut_cost(dim, 3, 2) < cut_cost(dim, 3, 1)) rows = 2;
-    for (int k = 0; k < 4; ++k) mm.n[k] = mm.np[k] = 1;
+    for (int k = 0; k < 4; ++k) {
+      mm.n[k] = mm.np[k] = 1;
+      mm.lo[k] = -1;
+    }
     int lo = 0;
     for (int k = 0; k < x.rank; ++k) {
       const int side = k < rows ? 0 : 1, slot = side == 0 ? 2 - rows + k : 4 - x.rank + k, f = x.fac[k];
@@ -741,6 +745,7 @@ int bi_launch_batch_mma(const BiCall &c, bi_model *mut) {
     mut->ws = pnew;
     mut->ws_bytes = need;
   }
+  if (mut->test_workspace == BI_WORKSPACE_NAN && cudaMemsetAsync(mut->ws, 0xff, need, c.stream) != cudaSuccess) return BI_ERR_CUDA;
   unsigned char *w = static_cast<unsigned char *>(mut->ws);
   int32_t *perm = reinterpret_cast<int32_t *>(w);
   int4 *task = reinterpret_cast<int4 *>(w + b_perm);

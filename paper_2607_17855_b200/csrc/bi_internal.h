@@ -103,6 +103,8 @@ struct alignas(16) BiDev {
   uint32_t *status;
 };
 
+enum { BI_WORKSPACE_NAN = 1 };   // bi_model::test_workspace
+
 // host-side handle
 struct bi_model {
   BiDev h;          // host copy (device pointers inside)
@@ -152,6 +154,9 @@ struct bi_model {
   // announce their slice copies without issuing them, so that the bounded wait on the copy runs out and
   // the status flag BI_FLAG_COPY_TIMEOUT is raised; nothing faults, nothing is left in flight.
   int test_drop_copy;
+  // Testing aid (BI_TEST_WORKSPACE, read when the handle is made): "nan" fills the workspace of the matrix-instruction window
+  // kernels with NaN before each call, so that a message that is read and was not written shows.
+  int test_workspace;
   // block kernels: the block shape the slices are laid out for (0: none), the filtering and the window plan
   // (bi_block::Plan), the device table 2^(j/512)
   int blk_BR, blk_BC;

@@ -1,5 +1,6 @@
 """The batched window kernels on the float64 matrix instruction: edges of tiles, remainders of summation steps, slices beyond
 shared memory, one and several tasks per slice, against the oracle at the float64 path's tolerances."""
+import contextlib
 import os
 import sys
 
@@ -11,11 +12,21 @@ for p in (HERE, os.path.dirname(HERE)):
     if p not in sys.path:
         sys.path.insert(0, p)
 
-from parity import check_workload                              # noqa: E402
+from parity import check_workload, compare, run_gpu           # noqa: E402
 from test_gpu_block import _workload                           # noqa: E402
 from test_gpu_parity import family_forced                      # noqa: E402
 
 pytestmark = pytest.mark.gpu
+
+
+@contextlib.contextmanager
+def workspace(what):
+    """The library's testing aid BI_TEST_WORKSPACE, read when a handle is made."""
+    os.environ["BI_TEST_WORKSPACE"] = what
+    try:
+        yield
+    finally:
+        del os.environ["BI_TEST_WORKSPACE"]
 
 CASES = {   # n, dep, N, T
     "smallest": ([2, 2, 2], [[0, 1, 2]], 1024, 2),
@@ -56,6 +67,29 @@ def test_transitions(bdep):
     md.close()
     sel = list(range(0, w.N, 21))
     assert np.abs(q[sel] - oracle.run_workload(w.take_agents(sel), "vmp", damping=0.7)[0]).max() <= 1e-5
+
+
+@pytest.mark.parametrize("n, bdep", [
+    ([1, 5, 6], [[0, 1], [1, 0], [2]]),                     # a one-state factor as the slow column; as the only one
+    ([6, 1, 9], [[0, 1, 2], [0, 1, 2], [2, 1]]),            # ... as the middle parent, as the child
+    ([5, 1, 9], [[1, 2], [1], [1, 0]]),                     # ... as its own only parent
+    ([1, 6, 9, 4], [[1, 2, 3], [2, 0, 3], [0, 2], [3]]),    # ... as the slow axis of either side of four
+])
+def test_one_state_factors_in_transitions(n, bdep):
+    """Every message that the update reads is written: the workspace holds NaN before each call.  Also on a
+    second call with fewer units, whose planes lie elsewhere."""
+    import oracle
+    import paper_2607_17855_b200 as bi
+    dep = [[0, 1], list(range(len(n)))]
+    w = _workload(350, n, dep, N=300, T=9, K=5, bdep=bdep)
+    first = _workload(350, n, dep, N=270, T=13, K=5, bdep=bdep)
+    with family_forced("batch"), workspace("nan"):
+        md = bi.model_from_workload(w)
+    for c in (first, w):
+        *out, _ = run_gpu(c, "vmp", model=md)
+        assert md.last_family == "batch_vmp_f64"
+        compare(c, *out, *oracle.run_workload(c, "vmp"))
+    md.close()
 
 
 @pytest.mark.parametrize("N, family", [(32, "batch"), (31, "warp")])
