@@ -219,7 +219,7 @@ __device__ __forceinline__ void mma_side(const MmaParams &P, const MmaMember &mm
     int off[kTiles];
 #pragma unroll
     for (int t = 0; t < kTiles; ++t) off[t] = GLOBAL ? min(n0 + 8 * t + g, len - 1) * (SIDE == 0 ? S : 1) : 0;
-    // (in shared memory rows beyond the last are there to be read: what comes of them is not used)
+    // (in shared memory rows beyond the last are there to be read, see staged_elements: what comes of them is not used)
     const double *b = GLOBAL ? L + (SIDE == 0 ? l : 0) : L + (SIDE == 0 ? (n0 + g) * S + l : l * S + n0 + g);
     double c[kTiles][2];
     switch (T) {
@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) bi_mma_slice_kernel(const __
     const int size = unit >= 0 ? 16 : 0;
 #pragma unroll
     for (int j = 0; j < 4; ++j)   // 16 bytes a copy (rows and offsets are multiples of four entries; zeros where there is no unit)
-      if (mm.lo[j] >= 0)
+      if ((j & 1) != 0 || mm.lo[j] >= 0)
         for (int s = 2 * l; s < ((mm.n[j] + 3) & ~3); s += 8)
           asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(bi_smem_addr(q + mm.lo[j] + s)), "l"(qr + mm.q[j] + s), "r"(size) : "memory");
     const int unit2 = u0 + 8 * GRP + g < tk.z ? __ldcg(pm + u0 + 8 * GRP) : -1;
@@ -525,6 +525,18 @@ long long cut_cost(const int *dim, int rank, int rows) {
   return cost;
 }
 
+// Elements of a staged slice's buffer: up to the last that either side's tiles read.  A chunk takes whole tiles of eight results
+// from its first one on, which need not be a multiple of eight: rows of 8 x 9 states are read as 0 to 63 and 63 to 78.
+size_t staged_elements(const MmaMember &mm) {
+  const int S = (mm.C & 4) ? mm.C : mm.C + 4, rows = bi_pad4(mm.R);   // (row stride, rows summed over: see the kernel)
+  int end[2] = {0, 0};
+  for (int side = 0; side < 2; ++side) {
+    const int nx = mm.n[2 * side], ny = mm.np[2 * side + 1], xs = std::max(1, kChunk / ny);
+    for (int x0 = 0; x0 < nx; x0 += xs) end[side] = std::max(end[side], x0 * ny + 8 * ceil_div(std::min(xs, nx - x0) * ny, 8));
+  }
+  return std::max((size_t)std::max(rows, end[0]) * S, (size_t)(rows - 1) * S + end[1]);
+}
+
 // matrix instructions per eight units of one member
 double member_instructions(int R, int C) {
   return (double)ceil_div(R, 8) * ceil_div(C, 4) + (double)ceil_div(C, 8) * ceil_div(R, 4);
@@ -659,7 +671,7 @@ int bi_launch_batch_mma(const BiCall &c, bi_model *mut) {
     heavy[j] = x.rank > 2;
     if (heavy[j]) {
       tabs = std::max(tabs, (size_t)(mm.C + bi_pad4(mm.R)));
-      lsz = std::max(lsz, (size_t)((mm.R + 7) & ~7) * ((mm.C & 4) ? mm.C : mm.C + 4) + 4);   // (whole tiles of rows are read)
+      lsz = std::max(lsz, staged_elements(mm));
       own = std::max(own, lo);
     } else {
       for (int k = 0; k < 2; ++k) nmax = std::max(nmax, dim[k]);

@@ -34,6 +34,7 @@ CASES = {   # n, dep, N, T
     "rank4": ([7, 5, 3, 6], [[0, 1, 2, 3], [0, 1, 3], [1, 3]], 260, 9),
     "exact_tiles": ([8, 16, 8], [[0, 1, 2], [1]], 130, 16),
     "several_chunks": ([9, 13, 11, 10], [[0, 1, 2, 3]], 64, 32),                 # more results than a warp accumulates at once
+    "chunks_across_tiles": ([8, 9, 7, 10], [[0, 1, 2, 3], [1, 2, 3]], 90, 25),    # chunks that start within a tile, on either side
     "beyond_shared_memory": ([32, 31, 30], [[0, 1, 2]], 86, 24),                 # read through L1
     "wide_pairs": ([17, 32, 25], [[0, 1], [1, 2], [2]], 100, 21),
     "one_state": ([1, 6, 9], [[0, 1, 2], [0, 2]], 210, 10),
