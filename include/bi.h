@@ -180,7 +180,8 @@ int bi_model_set_damping(bi_model_t *model, double lambda);
  * its workspaces (of the batched window path for shared models, of the calls that
  * take observation vectors and of the continued window calls; all obtained from the stream-ordered allocator
  * on first need, grown on demand and kept until bi_model_destroy) belong to the
- * handle.  Issue a handle's calls on one stream, or order the streams with
+ * handle.  (A window call that would run on the batched kernels and finds no memory for their workspace
+ * runs on the kernels that need none.)  Issue a handle's calls on one stream, or order the streams with
  * events; for concurrent inference on one model create one handle per stream.
  * All other calls allocate nothing.
  */

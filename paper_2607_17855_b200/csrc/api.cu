@@ -425,7 +425,7 @@ static int create_impl(const bi_model_desc *desc, int arith, const int32_t *bdep
   md->damping = 1.0;
   if (const char *e = getenv("BI_TEST_NO_COMPRESS")) md->test_no_compress = atoi(e) != 0;
   if (const char *e = getenv("BI_TEST_DROP_COPY")) md->test_drop_copy = atoi(e) > 0 ? atoi(e) : 0;   // testing aids,
-  if (const char *e = getenv("BI_TEST_WORKSPACE")) md->test_workspace = !strcmp(e, "nan") ? BI_WORKSPACE_NAN : 0;
+  if (const char *e = getenv("BI_TEST_WORKSPACE")) md->test_workspace = !strcmp(e, "nan") ? BI_WORKSPACE_NAN : !strcmp(e, "none") ? BI_WORKSPACE_NONE : 0;
   if (const char *e = getenv("BI_TEST_FAMILY")) {                                                  // read here only
     md->test_family = !strcmp(e, "warp") ? BI_FAMILY_WARP : !strcmp(e, "generic") ? BI_FAMILY_GENERIC
                       : !strcmp(e, "cta") ? BI_FAMILY_CTA : !strcmp(e, "batch") ? BI_FAMILY_BATCH
@@ -986,8 +986,36 @@ static bool few_units_batched(const BiCall &c) {
   return c.algo != BI_ALGO_FILTER && !c.model->soft_shadow && c.model->test_drop_copy == 0 && (long long)c.N * c.T >= 256;
 }
 
+int bi_workspace(bi_model *mut, size_t need, cudaStream_t stream) {
+  if (mut->test_workspace == BI_WORKSPACE_NONE) return BI_ERR_ALLOC;
+  if (mut->ws_bytes >= need) return BI_OK;
+  if (mut->ws && cudaFreeAsync(mut->ws, stream) != cudaSuccess) return BI_ERR_CUDA;
+  mut->ws = nullptr;
+  mut->ws_bytes = 0;
+  void *pnew = nullptr;
+  if (cudaMallocAsync(&pnew, need, stream) != cudaSuccess) {
+    cudaGetLastError();
+    return BI_ERR_ALLOC;
+  }
+  mut->ws = pnew;
+  mut->ws_bytes = need;
+  return BI_OK;
+}
+
 int bi_dispatch(const BiCall &c, bi_model *mut) {
   mut->last_block = nullptr;
+  // The batched window kernels are mostly a choice, not a need: where their workspace cannot be had the call goes on to the
+  // families behind them, which need none.
+  bool no_room = false;
+  auto batched = [&](int (*launch)(const BiCall &, bi_model *)) {
+    int rc = no_room ? BI_ERR_UNSUPPORTED : launch(c, mut);
+    if (rc == BI_ERR_ALLOC) {
+      no_room = true;
+      rc = BI_ERR_UNSUPPORTED;
+    }
+    return rc;
+  };
+  auto last = [&](int rc) { return rc == BI_ERR_UNSUPPORTED && no_room ? BI_ERR_ALLOC : rc; };
   if (c.model->h.has_bdep) {
     // Transition tensors with several parents.  In filtering they enter only the prior, formed once per
     // step; window calls (VMP) need them in every message: blocks in registers, or members of the batched
@@ -997,12 +1025,12 @@ int bi_dispatch(const BiCall &c, bi_model *mut) {
     const bool any = only == BI_FAMILY_ANY;
     int rc = BI_ERR_UNSUPPORTED;
     if (any || only == BI_FAMILY_BLOCK) rc = bi_launch_block(c, mut);
-    if (rc == BI_ERR_UNSUPPORTED && (any || only == BI_FAMILY_BATCH)) rc = bi_launch_batch(c, mut);
+    if (rc == BI_ERR_UNSUPPORTED && (any || only == BI_FAMILY_BATCH)) rc = batched(bi_launch_batch);
     if (rc == BI_ERR_UNSUPPORTED && c.algo == BI_ALGO_FILTER && (any || only == BI_FAMILY_CTA)) rc = bi_launch_cta_filter(c, mut);
     if (rc == BI_ERR_UNSUPPORTED && any) rc = bi_launch_block(c, mut, false);
-    if (rc == BI_ERR_UNSUPPORTED && any && few_units_batched(c)) rc = bi_launch_batch_mma(c, mut);
+    if (rc == BI_ERR_UNSUPPORTED && any && few_units_batched(c)) rc = batched(bi_launch_batch_mma);
     if (rc == BI_ERR_UNSUPPORTED && c.algo != BI_ALGO_FILTER && (any || only == BI_FAMILY_WARP)) rc = bi_launch_warp(c, mut);
-    return rc == BI_ERR_UNSUPPORTED ? bi_launch_generic(c, mut) : rc;
+    return last(rc == BI_ERR_UNSUPPORTED ? bi_launch_generic(c, mut) : rc);
   }
   const int only = c.model->test_family;   // testing aid: start at the named family
   int rc = BI_ERR_UNSUPPORTED;
@@ -1010,12 +1038,12 @@ int bi_dispatch(const BiCall &c, bi_model *mut) {
     rc = bi_launch_tile3(c, mut);
     if (rc == BI_ERR_UNSUPPORTED) rc = bi_launch_tile3_window(c, mut);
     if (rc == BI_ERR_UNSUPPORTED) rc = bi_launch_pair_filter(c, mut);
-    if (rc == BI_ERR_UNSUPPORTED && bi_batch_before_pair(c)) rc = bi_launch_batch(c, mut);
+    if (rc == BI_ERR_UNSUPPORTED && bi_batch_before_pair(c)) rc = batched(bi_launch_batch);
     if (rc == BI_ERR_UNSUPPORTED) rc = bi_launch_pair_window(c, mut);
     if (rc == BI_ERR_UNSUPPORTED && c.model->test_drop_copy == 0) rc = bi_launch_block(c, mut);
-    if (rc == BI_ERR_UNSUPPORTED) rc = bi_launch_batch(c, mut);
+    if (rc == BI_ERR_UNSUPPORTED) rc = batched(bi_launch_batch);
     if (rc == BI_ERR_UNSUPPORTED && c.algo != BI_ALGO_FILTER && c.model->test_drop_copy == 0) rc = bi_launch_block(c, mut, false);
-    if (rc == BI_ERR_UNSUPPORTED && few_units_batched(c)) rc = bi_launch_batch_mma(c, mut);
+    if (rc == BI_ERR_UNSUPPORTED && few_units_batched(c)) rc = batched(bi_launch_batch_mma);
     // Filtering exposes one unit per agent, so a CTA per agent keeps more of the machine busy than
     // a warp per agent, and its staged slices and per-factor warps pay at every batch size measured
     // on the 128 random structures (sum of times, CTA against warp kernel): 44 against 99 ms at 256
@@ -1027,12 +1055,12 @@ int bi_dispatch(const BiCall &c, bi_model *mut) {
   if (only == BI_FAMILY_BLOCK) rc = bi_launch_block(c, mut);
   if (only == BI_FAMILY_CTA && c.algo == BI_ALGO_FILTER) rc = bi_launch_cta_filter(c, mut);
   if (only == BI_FAMILY_BATCH) {   // the batched window kernels and what follows them
-    rc = bi_launch_batch(c, mut);
+    rc = batched(bi_launch_batch);
     if (rc == BI_ERR_UNSUPPORTED && c.algo == BI_ALGO_FILTER) rc = bi_launch_cta_filter(c, mut);
   }
   if (rc == BI_ERR_UNSUPPORTED && only != BI_FAMILY_GENERIC) rc = bi_launch_warp(c, mut);
   if (rc == BI_ERR_UNSUPPORTED) rc = bi_launch_generic(c, mut);
-  return rc;
+  return last(rc);
 }
 
 static int run_call(const bi_model_t *model, int algo, int32_t N, int32_t T, const int32_t *obs,

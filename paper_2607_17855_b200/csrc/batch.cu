@@ -1210,18 +1210,7 @@ int launch_batch_t(const BiCall &c, bi_model *mut) {
   const size_t b_q = up256(2 * (size_t)NU * h.Sp * sizeof(R));
   const size_t b_x = c.lambda != 1.0 ? up256((size_t)NU * h.Sp * sizeof(R)) : 0;
   const size_t need = b_perm + b_task + b_ellp + b_q + b_x;
-  if (mut->ws_bytes < need) {
-    if (mut->ws && cudaFreeAsync(mut->ws, c.stream) != cudaSuccess) return BI_ERR_CUDA;
-    mut->ws = nullptr;
-    mut->ws_bytes = 0;
-    void *pnew = nullptr;
-    if (cudaMallocAsync(&pnew, need, c.stream) != cudaSuccess) {
-      cudaGetLastError();
-      return BI_ERR_ALLOC;
-    }
-    mut->ws = pnew;
-    mut->ws_bytes = need;
-  }
+  if (const int rc = bi_workspace(mut, need, c.stream)) return rc;
   unsigned char *w = static_cast<unsigned char *>(mut->ws);
   int32_t *perm = reinterpret_cast<int32_t *>(w);
   int4 *task = reinterpret_cast<int4 *>(w + b_perm);

@@ -745,18 +745,8 @@ int bi_launch_batch_mma(const BiCall &c, bi_model *mut) {
   const size_t b_q = up256(2 * (size_t)NU * h.Sp * sizeof(double));
   const size_t b_x = c.lambda != 1.0 ? up256((size_t)NU * h.Sp * sizeof(double)) : 0;
   const size_t need = b_perm + b_task + b_ell + b_q + b_x;
-  if (mut->ws_bytes < need) {
-    if (mut->ws && cudaFreeAsync(mut->ws, c.stream) != cudaSuccess) return BI_ERR_CUDA;
-    mut->ws = nullptr;
-    mut->ws_bytes = 0;
-    void *pnew = nullptr;
-    if (cudaMallocAsync(&pnew, need, c.stream) != cudaSuccess) {
-      cudaGetLastError();
-      return BI_ERR_ALLOC;
-    }
-    mut->ws = pnew;
-    mut->ws_bytes = need;
-  }
+  int rc = bi_workspace(mut, need, c.stream);
+  if (rc != BI_OK) return rc;
   if (mut->test_workspace == BI_WORKSPACE_NAN && cudaMemsetAsync(mut->ws, 0xff, need, c.stream) != cudaSuccess) return BI_ERR_CUDA;
   unsigned char *w = static_cast<unsigned char *>(mut->ws);
   int32_t *perm = reinterpret_cast<int32_t *>(w);
@@ -783,7 +773,7 @@ int bi_launch_batch_mma(const BiCall &c, bi_model *mut) {
   A.xprev = b_x ? reinterpret_cast<double *>(w + b_perm + b_task + b_ell + b_q) : nullptr;
   A.q_init = c.q_init;
 
-  int rc = bi_batch_start_f64(md, B, max_m, c.q_init, perm, task, c.stream);
+  rc = bi_batch_start_f64(md, B, max_m, c.q_init, perm, task, c.stream);
   if (rc != BI_OK) return rc;
   typedef void (*SliceKernel)(MmaParams, int, int);
   typedef void (*PairKernel)(MmaParams, int, int, int);

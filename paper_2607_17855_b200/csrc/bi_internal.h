@@ -103,7 +103,7 @@ struct alignas(16) BiDev {
   uint32_t *status;
 };
 
-enum { BI_WORKSPACE_NAN = 1 };   // bi_model::test_workspace
+enum { BI_WORKSPACE_NAN = 1, BI_WORKSPACE_NONE = 2 };   // bi_model::test_workspace
 
 // host-side handle
 struct bi_model {
@@ -155,7 +155,8 @@ struct bi_model {
   // the status flag BI_FLAG_COPY_TIMEOUT is raised; nothing faults, nothing is left in flight.
   int test_drop_copy;
   // Testing aid (BI_TEST_WORKSPACE, read when the handle is made): "nan" fills the workspace of the matrix-instruction window
-  // kernels with NaN before each call, so that a message that is read and was not written shows.
+  // kernels with NaN before each call, so that a message that is read and was not written shows; "none": the workspace of the
+  // batched window kernels cannot be had.
   int test_workspace;
   // block kernels: the block shape the slices are laid out for (0: none), the filtering and the window plan
   // (bi_block::Plan), the device table 2^(j/512)
@@ -193,6 +194,10 @@ struct BiCall {
 // the largest shared-memory share of L1).  The limit belongs to the kernel, not to the launch: threads that each set
 // their own size before launching can lower it under one another, so it is only ever raised, behind a lock.
 cudaError_t bi_allow_smem(const void *kern, size_t bytes, bool carveout = false);
+
+// Sees to it that the workspace of the batched window kernels (mut->ws) has at least `need` bytes.  BI_ERR_ALLOC where that
+// cannot be had; the dispatcher then goes on to the kernels that need none.
+int bi_workspace(bi_model *mut, size_t need, cudaStream_t stream);
 
 // kernel families; each returns BI_OK, BI_ERR_UNSUPPORTED (not applicable to
 // this model / call: the dispatcher tries the next one) or an error.

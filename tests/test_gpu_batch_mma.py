@@ -93,6 +93,25 @@ def test_one_state_factors_in_transitions(n, bdep):
     md.close()
 
 
+FALLBACK = {   # n, dep, bdep, N, T, and who serves the call without a workspace
+    "pairs": ([25, 27, 6, 28, 17], [[0, 3], [2], [4], [3], [0, 1]], None, 256, 10, "pair"),
+    "blocks": ([14, 14, 2, 12], [[0, 1, 2, 3]], None, 300, 12, "block"),
+    "several_parents": ([10, 10, 8], [[0, 1], [1, 2]], [[0, 1], [1, 2], [2, 0]], 200, 16, "block"),
+    "few_units": ([28, 27, 26], [[0, 1, 2], [0]], None, 20, 16, "warp"),
+}
+
+
+@pytest.mark.parametrize("case", sorted(FALLBACK))
+def test_without_a_workspace(case):
+    """A call whose workspace cannot be had runs on the kernels that need none."""
+    n, dep, bdep, N, T, family = FALLBACK[case]
+    w = _workload(360, n, dep, N=N, T=T, K=3, bdep=bdep)
+    few = range(0, N, max(1, N // 8))
+    assert check_workload(w, "vmp", agents=few)["family"] == "batch_vmp_f64"
+    with workspace("none"):
+        assert check_workload(w, "vmp", agents=few)["family"] == f"{family}_vmp_f64"
+
+
 @pytest.mark.parametrize("N, family", [(32, "batch"), (31, "warp")])
 def test_few_units_of_a_model_too_large_for_the_block_kernels(N, family):
     res = check_workload(_workload(340, [32, 31, 30], [[0, 1, 2], [0]], N=N, T=8, K=3), "vmp", agents=range(0, N, 5))
