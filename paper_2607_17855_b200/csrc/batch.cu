@@ -1397,7 +1397,7 @@ int bi_launch_batch(const BiCall &c, bi_model *mut) {
     bytes *= (double)c.N * c.T * (md->arith == BI_ARITH_F64 ? 8 : 4);
     if (bytes > 120e6) return BI_ERR_UNSUPPORTED;
   }
-  if ((long long)c.N * c.T < 2048) return BI_ERR_UNSUPPORTED;   // too few units to fill the machine this way
+  if ((long long)c.N * c.T < 2048 || (long long)c.N * c.T > kMaxUnits) return BI_ERR_UNSUPPORTED;   // (too few to fill the machine this way)
   const int rc = bi_launch_batch_mma(c, mut);
   if (rc != BI_ERR_UNSUPPORTED) return rc;
   return md->arith == BI_ARITH_F64 ? launch_batch_t<double>(c, mut) : launch_batch_t<float>(c, mut);

@@ -13,6 +13,9 @@
 __device__ __forceinline__ void bi_grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void bi_grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
 
+// Most (agent, step) units of a call: the kernels and launchers count them in 32 bits.
+constexpr long long kMaxUnits = 1LL << 30;
+
 struct BatchMember {
   const void *logA;        // packed [m][P_pad]
   int32_t m, P_pad, modality, shape, rank;

@@ -555,7 +555,7 @@ double axes_instructions(const int *dim, int rank) {
 // structures of one to five factors, 2 048 to 62 000 units, 6 and 16 iterations (11 % rms error).
 double bi_batch_mma_cost(const BiCall &c) {
   const BiDev &h = c.model->h;
-  if (c.model->arith != BI_ARITH_F64 || h.G != 1 || (long long)c.N * c.T < 2048) return -1.0;
+  if (c.model->arith != BI_ARITH_F64 || h.G != 1 || (long long)c.N * c.T < 2048 || (long long)c.N * c.T > kMaxUnits) return -1.0;
   double deep = 0, longest = 0, pairs = 0, states = 0;
   int ndeep = 0, npair = 0;
   auto add = [&](const int *dim, int rank) {
