@@ -181,7 +181,9 @@ int bi_model_set_damping(bi_model_t *model, double lambda);
  * take observation vectors and of the continued window calls; all obtained from the stream-ordered allocator
  * on first need, grown on demand and kept until bi_model_destroy) belong to the
  * handle.  (A window call that would run on the batched kernels and finds no memory for their workspace
- * runs on the kernels that need none.)  Issue a handle's calls on one stream, or order the streams with
+ * runs on the kernels that need none; so does one that is captured into a CUDA graph before an uncaptured
+ * call of its size has obtained the workspace.  A workspace that captured calls use is kept until
+ * bi_model_destroy, whatever later calls need: destroy a handle after the graphs that hold its calls.)  Issue a handle's calls on one stream, or order the streams with
  * events; for concurrent inference on one model create one handle per stream.
  * All other calls allocate nothing.
  */

@@ -950,6 +950,11 @@ extern "C" int bi_model_destroy(bi_model_t *model) {
   if (!model) return BI_OK;
   cudaError_t e = cudaDeviceSynchronize();
   if (model->ws) cudaFree(model->ws);
+  while (BiKept *kept = model->ws_kept) {
+    cudaFree(kept->p);
+    model->ws_kept = kept->next;
+    delete kept;
+  }
   if (model->ws_soft) cudaFree(model->ws_soft);
   if (model->ws_prior) cudaFree(model->ws_prior);
   if (model->carry) cudaFree(model->carry);
@@ -988,10 +993,24 @@ static bool few_units_batched(const BiCall &c) {
 
 int bi_workspace(bi_model *mut, size_t need, cudaStream_t stream) {
   if (mut->test_workspace == BI_WORKSPACE_NONE) return BI_ERR_ALLOC;
-  if (mut->ws_bytes >= need) return BI_OK;
-  if (mut->ws && cudaFreeAsync(mut->ws, stream) != cudaSuccess) return BI_ERR_CUDA;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(stream, &capture) != cudaSuccess) cudaGetLastError();   // (another stream's capture: the launches report it)
+  const bool captured = capture != cudaStreamCaptureStatusNone;
+  if (mut->ws_bytes >= need) {
+    mut->ws_captured |= captured;
+    return BI_OK;
+  }
+  if (captured) return BI_ERR_ALLOC;
+  if (mut->ws_captured) {
+    BiKept *kept = new (std::nothrow) BiKept{mut->ws, mut->ws_kept};
+    if (!kept) return BI_ERR_ALLOC;
+    mut->ws_kept = kept;
+  } else if (mut->ws && cudaFreeAsync(mut->ws, stream) != cudaSuccess) {
+    return BI_ERR_CUDA;
+  }
   mut->ws = nullptr;
   mut->ws_bytes = 0;
+  mut->ws_captured = 0;
   void *pnew = nullptr;
   if (cudaMallocAsync(&pnew, need, stream) != cudaSuccess) {
     cudaGetLastError();

@@ -105,6 +105,12 @@ struct alignas(16) BiDev {
 
 enum { BI_WORKSPACE_NAN = 1, BI_WORKSPACE_NONE = 2 };   // bi_model::test_workspace
 
+// a workspace that captured calls use, kept beside its successor
+struct BiKept {
+  void *p;
+  BiKept *next;
+};
+
 // host-side handle
 struct bi_model {
   BiDev h;          // host copy (device pointers inside)
@@ -138,6 +144,10 @@ struct bi_model {
   const char *last_block;   // the block kernels' own name when they ran the most recent call, else NULL
   void *ws;         // workspace of the batched window path (stream-ordered allocation), or NULL
   size_t ws_bytes;
+  // A captured call's graph holds the workspace's address: once there is such a graph, the workspace is kept (until the
+  // handle goes) when a larger one takes its place.
+  int ws_captured;
+  struct BiKept *ws_kept;
   void *ws_soft;    // workspace of the calls that take observation vectors, or NULL
   size_t ws_soft_bytes;
   void *ws_prior;   // predictive log-priors of continued window calls, or NULL
@@ -196,7 +206,9 @@ struct BiCall {
 cudaError_t bi_allow_smem(const void *kern, size_t bytes, bool carveout = false);
 
 // Sees to it that the workspace of the batched window kernels (mut->ws) has at least `need` bytes.  BI_ERR_ALLOC where that
-// cannot be had; the dispatcher then goes on to the kernels that need none.
+// cannot be had; the dispatcher then goes on to the kernels that need none.  During a capture nothing is allocated (memory
+// that a graph allocates is there only from one of its runs on, and later calls would use it before): a call captured into a
+// graph uses the workspace of earlier calls, or none.
 int bi_workspace(bi_model *mut, size_t need, cudaStream_t stream);
 
 // kernel families; each returns BI_OK, BI_ERR_UNSUPPORTED (not applicable to

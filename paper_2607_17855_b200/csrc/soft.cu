@@ -370,6 +370,8 @@ int run_soft_t(const bi_model *model, int algo, int N, int T, const float *obs_s
   }
   mut->ws = sh.ws;
   mut->ws_bytes = sh.ws_bytes;
+  mut->ws_captured = sh.ws_captured;
+  mut->ws_kept = sh.ws_kept;
   mut->launches += launches + (sh.launches - before);
   mut->last_kernel = sh.last_kernel;
   mut->last_block = sh.last_block;

@@ -112,6 +112,46 @@ def test_without_a_workspace(case):
         assert check_workload(w, "vmp", agents=few)["family"] == f"{family}_vmp_f64"
 
 
+def test_captured_calls():
+    """A graph's calls keep their memory: the first call of a handle, captured, takes kernels without a workspace; one captured
+    after a call of its size stays valid when a larger call obtains a larger workspace."""
+    import torch
+    import paper_2607_17855_b200 as bi
+    n, dep, _, N, T, _ = FALLBACK["pairs"]
+    w, large = (_workload(370, n, dep, N=k * N, T=T, K=3) for k in (1, 4))
+    cuda = lambda x: torch.from_numpy(x).cuda()
+    obs, act, big = cuda(w.obs), cuda(w.act), (cuda(large.obs), cuda(large.act), large.K)
+    with workspace("none"):   # (and the pair kernel is loaded before the capture)
+        plain = bi.model_from_workload(w)
+    want = {"pair": plain.run("vmp", obs, act, w.K)}
+    other = bi.model_from_workload(w)
+    want["batch"] = other.run("vmp", obs, act, w.K)
+    for family in ("pair", "batch"):
+        md = bi.model_from_workload(w)
+        o, q = obs.clone(), torch.zeros_like(want[family])
+        if family == "batch":
+            md.run("vmp", o, act, w.K, q_out=q)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            md.run("vmp", o, act, w.K, q_out=q)
+        assert md.last_family == f"{family}_vmp_f64"
+        g.replay()
+        assert torch.equal(q, want[family])
+        q_big = md.run("vmp", *big)
+        assert md.last_family == "batch_vmp_f64"
+        o.zero_()
+        g.replay()
+        assert torch.equal(q, (plain if family == "pair" else other).run("vmp", torch.zeros_like(obs), act, w.K))
+        o.copy_(obs)
+        g.replay()
+        assert torch.equal(q, want[family]) and torch.equal(q_big, md.run("vmp", *big))
+        assert md.status() == 0
+        del g
+        md.close()
+    plain.close()
+    other.close()
+
+
 @pytest.mark.parametrize("N, family", [(32, "batch"), (31, "warp")])
 def test_few_units_of_a_model_too_large_for_the_block_kernels(N, family):
     res = check_workload(_workload(340, [32, 31, 30], [[0, 1, 2], [0]], N=N, T=8, K=3), "vmp", agents=range(0, N, 5))
