@@ -40,6 +40,8 @@ CASES = {   # n, dep, N, T
     "one_state": ([1, 6, 9], [[0, 1, 2], [0, 2]], 210, 10),
     "one_step": ([6, 5, 4], [[0, 1, 2], [1, 2], [0]], 2100, 1),                  # no transitions
     "long_tasks": ([3, 4, 6], [[0, 1, 2], [0, 1]], 2500, 20),                    # several trips of a task's warps
+    "eight_warps_split": ([10, 10, 8, 6], [[0, 1], [0, 1, 2, 3]], 450, 20),      # up to 9472 units: V and W by different warps
+    "eight_warps": ([10, 10, 8, 6], [[0, 1], [0, 1, 2, 3]], 620, 20),
     "many_planes": ([4, 5, 3], [[0, 1, 2], [0, 1], [1, 2], [0, 2]] * 3, 150, 14),
 }
 
@@ -90,6 +92,41 @@ def test_one_state_factors_in_transitions(n, bdep):
         *out, _ = run_gpu(c, "vmp", model=md)
         assert md.last_family == "batch_vmp_f64"
         compare(c, *out, *oracle.run_workload(c, "vmp"))
+    md.close()
+
+
+@pytest.mark.parametrize("damping", [1.0, 0.6])
+@pytest.mark.parametrize("algo", ["vmp", "mmp"])
+def test_call_forms(algo, damping):
+    """Warm-started and continued calls, plain and damped, one after the other on one handle and of fewer and fewer units; every
+    agent, with NaN in the workspace before each."""
+    import oracle
+    import torch
+    import paper_2607_17855_b200 as bi
+    n, T = [5, 1, 7, 4], 9
+    w = _workload(380, n, [[0, 1, 2], [2, 3], [0, 2, 3], [0]], N=400, T=T, K=5)
+    rng = np.random.default_rng(381)
+    simplex = lambda *size: np.concatenate([rng.dirichlet(np.full(k, 1.5), size=size) for k in n], axis=-1).astype(np.float32)
+    q_prev, q_init = simplex(w.N), simplex(w.N, T)
+    act_prev = np.stack([rng.integers(0, int(u), size=w.N) for u in w.U], axis=1).astype(np.int32)
+    cuda = lambda x: torch.from_numpy(x).cuda()
+    with family_forced("batch"), workspace("nan"):
+        md = bi.model_from_workload(w)
+    md.set_damping(damping)
+    warm = md.bi_vmp_warm if algo == "vmp" else md.bi_mmp_warm
+    for N, call in ((400, "plain"), (350, "warm"), (300, "from"), (250, "from, warm")):
+        obs, act, kw = cuda(w.obs[:N]), cuda(w.act[:N]), {}
+        if "from" in call:
+            kw = dict(q_prev=q_prev[:N].astype(np.float64), act_prev=act_prev[:N])
+        if "warm" in call:
+            kw["q_init"] = q_init[:N].astype(np.float64)
+        if "from" in call:
+            q = md.run_from(algo, obs, act, cuda(q_prev[:N]), cuda(act_prev[:N]), w.K, q_init=cuda(q_init[:N]) if "warm" in call else None)
+        else:
+            q = warm(obs, act, cuda(q_init[:N]), w.K) if call == "warm" else md.run(algo, obs, act, w.K)
+        assert md.last_family == f"batch_{algo}_f64" and md.status() == 0
+        ref = oracle.run(algo, w.n, w.m, w.dep, w.U, w.G, w.A, w.B, w.D, w.obs[:N], w.act[:N], w.K, damping=damping, **kw)[0]
+        assert np.abs(q.cpu().numpy() - ref).max() <= 1e-5, call
     md.close()
 
 
