@@ -718,14 +718,13 @@ WindowCost window_cost(const BiCall &c, const Plan &pl, const Variant &v, double
   const bool f64 = c.model->arith == BI_ARITH_F64;
   const double per_sm = (double)c.N * c.T / c.model->sm_count * 1e-3, k = c.K * per_sm;   // thousands of units; unit-iterations
   const double ent = pl.NB * (double)(pl.BR * pl.BC) * 1e-3, warps = v.LT / 32.0;
-  double slices = 0, longest = 0, states = 0;   // (slices in thousands of entries)
+  double slices = 0, states = 0;   // (slices in thousands of entries)
   int members = 0, nmax = 1;
   for (int gi = 0; gi < h.ngroups; ++gi) {
     const BiGroup &g = h.grp[gi];
     if (g.rank < 2) continue;
     double e = 1;
     for (int j = 0; j < g.rank; ++j) e *= j + 1 < g.rank ? g.dim[j] : bi_pad4(g.dim[j]);
-    longest = std::max(longest, e * 1e-3);
     for (int mi = g.mem_begin; mi < g.mem_end; ++mi)
       if (g.dim[g.rank - 1] > 32 || h.mem[mi].m > 4096) return {0.0, 1.0};   // (nothing the batched kernels take)
     slices += e * 1e-3 * (g.mem_end - g.mem_begin);
