@@ -983,10 +983,14 @@ __global__ void bi_predictive_prior_kernel(const BiDev *__restrict__ mdp, int N,
   out[i] = bi_log(bi_max(acc, (R)BI_EPS));
 }
 
-// Window calls of fewer units than the batched kernels otherwise take, on models too large for the block kernels (and with too many
-// steps for the pair window kernel), float64.  The warp kernel re-reads a slice per unit, these once per task: a slice of 29 760
-// entries, 256 units 1365 us a call here and 3019 there, 1800 units 1656 and 5844; of 49 152 entries 1685 and 16319, 1876 and
-// 12444.  Below 256 units the two come together (128 units of the first: 1468 there).
+// Float64 window calls of fewer units than the batched kernels otherwise take, which the pair window and block kernels have
+// declined: slices or transition tensors too large for an SM or a cluster, pairs or many factors over too many steps.  What would
+// follow is the warp kernel, which reads a slice or matrix per unit where these read it once per task, and it was the
+// slower one for every kind of such model, 256 to 1984 units, 16 iterations (small models do not come this far).  In us a call
+// here and there, 256 units: slices of 29 760 entries, T = 16, 1340 and 2982, T = 1 1211 and 1271; [12,11,10,12] under a rank-4
+// slice 298 and 6060; a pair [32,32], T = 64, 79 and 1272; eight single factors of sixteen states, T = 64, 83 and 967; two
+// parents per transition, eight factors of 32 states, T = 1, 60 and 171, T = 2 1820 and 27 490.  Below 256 units the two come
+// together (128 units of the first: 1468 there).
 static bool few_units_batched(const BiCall &c) {
   return c.algo != BI_ALGO_FILTER && !c.model->soft_shadow && c.model->test_drop_copy == 0 && (long long)c.N * c.T >= 256;
 }

@@ -249,7 +249,7 @@ struct LaneRef {     // byte offsets, absolute unless said otherwise
 };
 // The lanes' descriptions, in shared memory for all teams of the CTA (16 bytes each; a pass' own 16 bytes behind
 // them): read again in every iteration just before the barrier between the phases, so that they take no
-// registers beside the blocks.
+// registers beside the blocks; the filtering kernel keeps a warp's first one where the blocks are small (see kKeepLanes).
 template <typename R>
 __device__ __forceinline__ void stage_lanes(const Params &p) {
   const int n = p.npass * 32;
